@@ -91,6 +91,18 @@ static __device__ __forceinline__ double coulomb_inv_r(double x) {
   return fma(0.5 * y, e, y);
 }
 
+// The largest |r| of a walker and spin as its high FP64 word (NaN above Inf above all others),
+// kept in a register while a warp's determinants are of one spin.
+static __device__ __forceinline__ void ratio_max(const DevScratch& S, int64_t w, int sp, int& sp_max, uint32_t& top,
+                                                 double r) {
+  if (sp != sp_max) {
+    if (top) atomicMax(S.xmax + sp_max * S.wp + w, top);
+    sp_max = sp;
+    top = 0;
+  }
+  top = max(top, (uint32_t)__double2hiint(r) & 0x7fffffffu);
+}
+
 static __device__ __forceinline__ double ipow_d(double x, int n) {
   double r = 1.0;
   for (int i = 0; i < n; i++) r *= x;

@@ -48,6 +48,8 @@ struct mdet_ctx {
   };
   std::vector<ItemSet> item_sets;
   DevProblem P{};
+  DenseContract dense{};  // residue products of the contraction
+  bool dense_ok = false;  //   whether this expansion has them
   DevScratch S{};
   // escalation of mixed-precision walkers (FP64 re-evaluation of the flagged ones):
   // scratch for fallback_cap walkers, their positions, compact outputs and live count
@@ -102,6 +104,9 @@ constexpr int kEscalationChunk = 128;
 // words of S.queue per walker chunk: the work counters of its two persistent contractions, then
 // the global-timer stamps (start complemented, end) of each
 constexpr int kQueueWords = 6;
+
+// residue planes of C above this size, and workspace of the residue products per context
+constexpr size_t kDenseMaxBytes = (size_t)8 << 30, kDenseWorkBytes = (size_t)4 << 30;
 
 // weights of the first, each middle and the last walker chunk of the pipelined evaluation. The
 // first chunk's orbitals and tables run before any contraction, and the last chunk's epilogue
@@ -240,6 +245,7 @@ void free_problem(mdet_ctx* c) {
   for (void* p : c->dev_problem_allocs) cudaFree(p);
   c->dev_problem_allocs.clear();
   c->item_sets.clear();
+  c->dense_ok = false;
   c->P = DevProblem{};
 }
 
@@ -303,6 +309,7 @@ bool use_items(const mdet_ctx* c, DevProblem& P, int chunk) {
 
 void free_arrays(DevScratch& S) {
   void* ptrs[] = {S.phi, S.Ainv, S.ld0, S.sg0, S.g, S.kap, S.est, S.T, S.Tdf, S.r, S.rdf, S.vu, S.psit, S.psia, S.wstat,
+                  S.xmax, S.dx, S.dy, S.dyabs, S.derr,
                   S.fb, S.fb_list, S.fb_acc, S.queue, S.R_stage, S.out_stage};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -378,6 +385,60 @@ mdet_status spin_tables(mdet_ctx* c, int sp, int n_int, const std::vector<uint64
     c->exc[sp][t] = e;
     c->degree[sp][t] = k;
   }
+  return MDET_OK;
+}
+
+// Whether an expansion's contraction is taken as residue products on the tensor cores: a filled-in
+// C costs about 70 tensor flops per matrix element and walker, the sparse FP64 sums 4 flops per
+// nonzero at a thousandth of that rate. 8,192 walkers: 8.2 % of 3,015 x 3,015 filled takes 20.5 ms
+// sparse and 5.1 ms dense, so the two meet near 2 % by arithmetic; at 0.35 % the sparse sums take
+// 2.0 ms, and below a few thousand products the three launches cost more than the sums.
+bool dense_pays(int64_t nnz, int64_t nu, int64_t nd) { return nnz >= 4096 && (double)nnz > 0.012 * (double)nu * (double)nd; }
+
+// Residue planes of C for the tensor-core contraction, where they pay and fit; the sparse sums
+// serve every other expansion (and this one, when the device has no room for the planes).
+mdet_status build_dense(mdet_ctx* c) {
+  DevProblem& P = c->P;
+  if (!dense_pays(P.nnz, P.n_det_sp[0], P.n_det_sp[1])) return MDET_OK;
+  DenseContract& D = c->dense;
+  D = DenseContract{};
+  dense_shape(P.n_det_sp[0], P.n_det_sp[1], &D);
+  const int* es[2] = {};
+  for (int o = 0; o < 2; o++) {  // exponents above the sum of magnitudes of each row
+    const std::vector<int32_t>& ptr = o ? c->csc_ptr : c->csr_ptr;
+    const std::vector<double>& val = o ? c->coo_val : c->csr_val;
+    std::vector<int> e(P.n_det_sp[o], 0);
+    for (size_t i = 0; i < e.size(); i++) {
+      double l1 = 0.0;
+      for (int32_t k = ptr[i]; k < ptr[i + 1]; k++) l1 += std::fabs(val[k]);
+      if (!std::isfinite(l1)) return MDET_OK;
+      if (l1 > 0.0) e[i] = std::ilogb(l1 * (1.0 + 0x1p-40)) + 1;
+    }
+    mdet_status s = upload(c, e, &es[o]);
+    if (s != MDET_OK) return s;
+    D.es[o] = es[o];
+  }
+  std::vector<uint32_t> mx(dense_moduli_range(), 0);
+  const uint32_t* d_mx = nullptr;
+  mdet_status s = upload(c, mx, &d_mx);
+  if (s != MDET_OK) return s;
+  CUDA_TRY(c, launch_dense_rowsum(P, es, const_cast<uint32_t*>(d_mx), nullptr));
+  CUDA_TRY(c, cudaMemcpy(mx.data(), d_mx, mx.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost));
+  if (!choose_moduli(mx.data(), &D)) return MDET_OK;
+  for (int o = 0; o < 2; o++) {
+    const size_t bytes = dense_plane_elems(D, o) * sizeof(uint16_t) * (D.nm + (o ? 0 : 2));
+    void* p = nullptr;
+    if (bytes > kDenseMaxBytes || cudaMalloc(&p, bytes) != cudaSuccess) {
+      cudaGetLastError();  // no room: the sparse sums
+      return MDET_OK;
+    }
+    c->dev_problem_allocs.push_back(p);
+    D.planes[o] = static_cast<uint16_t*>(p);
+  }
+  CUDA_TRY(c, launch_dense_planes(P, D, nullptr));
+  CUDA_TRY(c, cudaStreamSynchronize(nullptr));
+  c->dense_ok = true;
+  P.dense = &c->dense;
   return MDET_OK;
 }
 
@@ -495,6 +556,7 @@ mdet_status upload_problem(mdet_ctx* c) {
   // contraction work items for the tuned size and for the short items of escalated re-evaluations
   if ((s = ensure_items(c, c->spmm_chunk)) != MDET_OK || (s = ensure_items(c, kEscalationChunk)) != MDET_OK) return s;
   use_items(c, P, c->spmm_chunk);
+  if ((s = build_dense(c)) != MDET_OK) return s;
   // the sequential chain of Sec. 2.2: distinct determinants in the order of the key of Eq. 3,
   // each with the substitutions from its predecessor (holes and particles ascending, paired in order)
   for (int sp = 0; sp < 2; sp++) {
@@ -575,6 +637,30 @@ mdet_status alloc_eval_arrays(mdet_ctx* c, DevScratch& S, int64_t W, bool df_tab
   if ((s = dalloc(c, &S.psit, (size_t)wp))) return s;
   if ((s = dalloc(c, &S.psia, (size_t)wp))) return s;
   if ((s = dalloc(c, &S.wstat, (size_t)W))) return s;
+  if (c->dense_ok) {  // the workspace of the residue products, for blocks of walkers that it holds
+    size_t x, y, ya;
+    dense_bytes(c->dense, &x, &y, &ya);
+    const int64_t fit = (int64_t)(kDenseWorkBytes / (x + y + ya)) / kWalkerPad * kWalkerPad;
+    S.dblk = std::min(wp, std::max<int64_t>(fit, kWalkerPad));
+    bool ok = cudaMalloc((void**)&S.xmax, sizeof(uint32_t) * 2 * wp) == cudaSuccess &&
+              cudaMalloc((void**)&S.dx, x * S.dblk) == cudaSuccess &&
+              cudaMalloc((void**)&S.dy, y * S.dblk) == cudaSuccess &&
+              cudaMalloc((void**)&S.dyabs, ya * S.dblk) == cudaSuccess &&
+              cudaMalloc((void**)&S.derr, sizeof(int)) == cudaSuccess;
+    if (ok) {
+      CUDA_TRY(c, cudaMemset(S.xmax, 0, sizeof(uint32_t) * 2 * wp));
+    } else {  // no room: the sparse sums
+      cudaGetLastError();
+      void* p[] = {S.xmax, S.dx, S.dy, S.dyabs, S.derr};
+      for (void* q : p)
+        if (q) cudaFree(q);
+      S.xmax = nullptr;
+      S.dx = nullptr;
+      S.dy = nullptr;
+      S.dyabs = nullptr;
+      S.derr = nullptr;
+    }
+  }
   S.cap_walk = W;
   S.wp = wp;
   return MDET_OK;
@@ -674,7 +760,10 @@ mdet_status refine(mdet_ctx* c, bool table, int64_t n_walk, const double* R, dou
   // few walkers: short work items keep the contraction's chains short, and the epilogue
   // spreads each walker's determinants over 512 threads
   Pe.spmm_blocks = 0;
-  CUDA_TRY(c, launch_contract_f64(Pe, E, cap, st));
+  if (E.xmax)
+    CUDA_TRY(c, launch_contract_dense(Pe, E, cap, st, nullptr, nullptr));
+  else
+    CUDA_TRY(c, launch_contract_f64(Pe, E, cap, st));
   CUDA_TRY(c, launch_final(P, E, cap, c->e_R, o.log_abs_psi, o.sign, o.grad, o.lap, o.e_local, o.status, false, st,
                            true));
   CUDA_TRY(c, launch_fallback(P, E, cap, c->e_R, o.log_abs_psi, o.sign, o.grad, o.lap, o.e_local, o.status, st));
@@ -683,13 +772,19 @@ mdet_status refine(mdet_ctx* c, bool table, int64_t n_walk, const double* R, dou
   return MDET_OK;
 }
 
+// Whether an evaluation's contraction runs as residue products: its expansion has them, its
+// scratch has their workspace, and no setting asks for a form of the sparse sums.
+bool use_dense(const mdet_ctx* c) { return c->dense_ok && c->contract_impl == 0 && c->spmm_blocks == 0; }
+
 // Walker chunks of a mixed-precision evaluation when none are configured: three
 // when the FP64 contraction is long enough to hide the FP32-pipe stages of the
 // other chunks (at least 100,000 products and 4 walker tiles per chunk), else one.
 int auto_chunks(const mdet_ctx* c, int64_t n_walk) {
   const int64_t tiles = (n_walk + kWalkerPad - 1) / kWalkerPad;
-  return (c->precision == MDET_PRECISION_MIXED && c->contract_impl == 0 && c->P.nnz >= 100000 && tiles >= 12) ? 3
-                                                                                                                : 1;
+  return (c->precision == MDET_PRECISION_MIXED && c->contract_impl == 0 && !use_dense(c) && c->P.nnz >= 100000 &&
+          tiles >= 12)
+             ? 3
+             : 1;
 }
 
 }  // namespace
@@ -1142,11 +1237,14 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
     *off = t0 * kWalkerPad;
     *n = std::min<int64_t>(t1 * kWalkerPad, n_walk) - *off;
   };
+  const bool dense = use_dense(c) && c->S.xmax;
+  int contract_kernels = 0;
   // stage i (MDET_STAGE_*) of chunk k on stream ks, bracketed by its two profiling events
   auto stage = [&](int k, int i, cudaStream_t ks, int persistent) -> mdet_status {
     int64_t off, n;
     chunk_range(k, &off, &n);
-    const DevScratch S = scratch_view(c->S, P, off);
+    DevScratch S = scratch_view(c->S, P, off);
+    if (!dense) S.xmax = nullptr;
     const double* Rk = R + off * N * 3;
     const bool mark = prof_all;
     if (mark) CUDA_TRY(c, cudaEventRecord(c->ev[k][2 * i], ks));
@@ -1161,6 +1259,11 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
       case MDET_STAGE_ZERO: CUDA_TRY(c, launch_zero_f64(P, S, n, ks)); break;
       case MDET_STAGE_CONTRACT: {
         unsigned long long* q = c->S.queue + kQueueWords * k;
+        if (dense) {
+          CUDA_TRY(c, launch_contract_dense(P, S, n, ks, prof_stamp ? q + 2 : nullptr, &contract_kernels));
+          break;
+        }
+        contract_kernels += 2;
         CUDA_TRY(c, launch_contract_f64(P, S, n, ks, q, persistent, prof_stamp ? q + 2 : nullptr));
         break;
       }
@@ -1213,16 +1316,17 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
   c->prof_chunks = nch;
   // stability fallback over the whole batch, after every chunk has finished: mixed precision
   // escalates to FP64 first, FP64 goes to full LU directly
-  // kernels: 6 per chunk (orbitals, reference, ratios, 2 contractions, epilogue); the full-LU
+  // kernels: 4 per chunk (orbitals, reference, ratios, epilogue) and its contraction's (2 sparse
+  // sums, or 3 per walker block of the residue products); the full-LU
   // fallback 5 (list, dets, scale, rows, out); the mixed refinement adds its list, gather,
   // FP64 orbitals and scatter, and either the mark or the 5 FP64 table kernels
-  c->last_kernels = 6 * nch;
+  c->last_kernels = 4 * nch + contract_kernels;
   if (prof_all) CUDA_TRY(c, cudaEventRecord(c->ev_refine[0], st));
   if (mixed && c->E.fb && P.fallback_tol > 0.0) {
     const bool table = escalation_on(c);
     mdet_status es = refine(c, table, n_walk, R, log_abs_psi, sign, grad, lap, e_local, status, st);
     if (es != MDET_OK) return es;
-    c->last_kernels += 4 + 5 + (table ? 5 : 1);
+    c->last_kernels += 4 + 5 + (table ? (c->E.xmax ? 6 : 5) : 1);
   } else {
     CUDA_TRY(c, launch_fallback(P, c->S, n_walk, R, log_abs_psi, sign, grad, lap, e_local, status, st));
     if (P.fallback_tol > 0.0 && c->S.fb && P.n_up <= MDET_FALLBACK_MAX_SPIN) c->last_kernels += 5;

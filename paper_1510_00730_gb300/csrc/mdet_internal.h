@@ -54,6 +54,28 @@ struct __align__(16) Exc {
 };
 static_assert(sizeof(Exc) == 16, "Exc must be 16 bytes");
 
+// The contraction as residue products on the tensor cores (mdet_modgemm.cu): moduli, shapes
+// and the residue planes of C. Passed to the kernels by value.
+constexpr int kMaxModuli = 24;
+struct ModConst {
+  float p, invp;
+  uint32_t c0, c1;  // 256^k mod p, k = 0..7, as signed bytes
+  int off;          // -(2^63 mod p) plus the bits of 1.5 * 2^23
+};
+struct DenseContract {
+  int nm;                // moduli
+  int kb[2];             // 64-wide K blocks over the distinct determinants of each spin
+  int nt[2], hw[2];      // determinant tiles of 2 hw rows of product o (0: v, 1: u)
+  int ldy[2];            // row stride of the residue bytes of product o
+  uint16_t* planes[2];   // BF16 residue planes of C and C^T; the two magnitude planes of C
+  const int* es[2];      // [n_det_sp[o]] exponents of the rows of C and of C^T
+  ModConst m[kMaxModuli];
+  uint32_t M4[kMaxModuli][4];  // reconstruction weights modulo 2^128
+  uint32_t F[kMaxModuli];      // 2^32 ((P / p)^-1 mod p) / p
+  uint32_t init4[4], P4[4];
+  long long finit;
+};
+
 // Read-only problem description resident on the device.
 struct DevProblem {
   int n_up, n_dn, n_elec, n_nuc;
@@ -69,6 +91,7 @@ struct DevProblem {
   const uint8_t* split;   // [n_det_up + n_det_dn] 1 for a segment cut into pieces (its v or u entries are
                           //   cleared before the contraction, by the ratio kernel)
   int spmm_blocks;        // tuning: grid of the contraction (0: one warp per work item)
+  const DenseContract* dense;  // host: the residue products, null where the sparse sums are taken
   int contract_impl;      // tuning: contraction in FP64 (0) or double-float on the FP32 pipe (1, mixed only)
   const float2* csr_val_df;  // C values as double-float pairs, row-major and column-major orders
   const float2* csc_val_df;
@@ -130,6 +153,14 @@ struct DevScratch {
   double* vu = nullptr;   // walker-major [wp][n_det_up + n_det_dn]: v = C r_dn (up) then u = C^T r_up (down)
   double* psit = nullptr; // [wp] Psi / (D_ref_up D_ref_dn)
   float* psia = nullptr;  // [wp] sum_ij |c_ij| |r_up,i| |r_dn,j| (FP32), the magnitude sum behind psit
+  // residue products (null without them): largest ratio magnitudes (high FP64 words) per spin, [2][wp];
+  // residue planes, residue bytes and magnitude sums of dblk walkers; the kernel's failure flag
+  uint32_t* xmax = nullptr;
+  uint16_t* dx = nullptr;
+  uint8_t* dy = nullptr;
+  float* dyabs = nullptr;
+  int* derr = nullptr;
+  int64_t dblk = 0;
   uint32_t* wstat = nullptr;  // [W] status bits
   double* fb = nullptr;       // fallback: [cap][n_det_up + n_det_dn][2 + 4 max(n_up, n_dn)], then [cap][ndt] values
   int* fb_list = nullptr;     // fallback: [1 + cap] count, then walker indices
@@ -190,6 +221,21 @@ cudaError_t launch_zero_f64(const DevProblem& P, const DevScratch& S, int64_t n_
 cudaError_t launch_contract_f64(const DevProblem& P, const DevScratch& S, int64_t n_walk,
                                 cudaStream_t st, unsigned long long* queue = nullptr, int persistent_blocks = 0,
                                 unsigned long long* stamp = nullptr);
+// The contraction by residue products (mdet_modgemm.cu). Set-up: the shape for the distinct
+// determinant counts, the largest residue row sums of every modulus (device array of
+// dense_moduli_range() words), the moduli from them, the residue planes of C.
+void dense_shape(int n_up, int n_dn, DenseContract* D);
+int dense_moduli_range();
+cudaError_t launch_dense_rowsum(const DevProblem& P, const int* const es[2], uint32_t* mx, cudaStream_t st);
+bool choose_moduli(const uint32_t* rowmax, DenseContract* D);
+size_t dense_plane_elems(const DenseContract& D, int o);  // elements of one plane of product o
+cudaError_t launch_dense_planes(const DevProblem& P, const DenseContract& D, cudaStream_t st);
+// Bytes per walker of the residue planes, the residue bytes and the magnitude sums.
+void dense_bytes(const DenseContract& D, size_t* x, size_t* y, size_t* yabs);
+// v, u, Psi~ and its magnitude sum into S.vu, S.psit and S.psia, in blocks of S.dblk walkers (3
+// kernels each, counted into *n_kernels); stamp as above, for all the products together.
+cudaError_t launch_contract_dense(const DevProblem& P, const DevScratch& S, int64_t n_walk, cudaStream_t st,
+                                  unsigned long long* stamp, int* n_kernels);
 // A view of the scratch for walkers [off, off + n): walker-major arrays move by
 // whole walkers, walker-minor arrays by columns (off must be a multiple of kWalkerPad).
 DevScratch scratch_view(const DevScratch& S, const DevProblem& P, int64_t off);

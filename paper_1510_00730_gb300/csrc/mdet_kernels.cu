@@ -238,6 +238,7 @@ __global__ void __launch_bounds__(64) k_ref(DevProblem P, DevScratch S) {
     // set: it keeps the magnitude sum of the evaluation that flagged it), sum |c r r|
     S.psit[w] = 0.0;
     if (!S.live) S.psia[w] = 0.0f;
+    if (S.xmax) S.xmax[w] = S.xmax[S.wp + w] = 0u;
   }
   const int nu = P.n_up, nd = P.n_dn;
   if (MIXED) {
@@ -337,9 +338,11 @@ __global__ void __launch_bounds__(128) k_ratio_f64(DevProblem P, DevScratch S) {
   const int nu_det = P.n_det_sp[0], ntot = nu_det + P.n_det_sp[1];
   const int M = P.n_mo;
   const int64_t wp = S.wp;
+  int sp_max = 0;
+  uint32_t top = 0;
   for (int q = 0; q < 8; q++) {
     const int t = blockIdx.x * 32 + warp * 8 + q;
-    if (t >= ntot) return;
+    if (t >= ntot) break;
     const int sp = t < nu_det ? 0 : 1;
     const Exc e = P.exc[sp][sp ? t - nu_det : t];
     const double* T = S.T + (size_t)(sp ? P.n_up * M : 0) * wp;
@@ -352,8 +355,12 @@ __global__ void __launch_bounds__(128) k_ratio_f64(DevProblem P, DevScratch S) {
     const double d = small_det(e.k, m);
     // the sign by its bit, not by an FP64 instruction
     S.r[(size_t)t * wp + w] = __longlong_as_double(__double_as_longlong(d) ^ ((long long)(e.eps < 0) << 63));
-    if (P.split[t]) S.vu[w * ntot + t] = 0.0;  // the contraction adds the pieces of a cut segment
+    if (S.xmax)
+      ratio_max(S, w, sp, sp_max, top, d);
+    else if (P.split[t])
+      S.vu[w * ntot + t] = 0.0;  // the contraction adds the pieces of a cut segment
   }
+  if (S.xmax && top) atomicMax(S.xmax + sp_max * wp + w, top);
 }
 
 // ---------------------------------------------------------------------------
@@ -1181,6 +1188,7 @@ DevScratch scratch_view(const DevScratch& S, const DevProblem& P, int64_t off) {
   V.T = S.T + off;  // walker-minor: a column offset with the same stride
   if (S.Tdf) V.Tdf = S.Tdf + off;
   V.r = S.r + off;
+  if (S.xmax) V.xmax = S.xmax + off;  // walker-minor as well
   if (S.rdf) V.rdf = S.rdf + off;
   V.psit = S.psit + off;
   V.psia = S.psia + off;

@@ -269,9 +269,11 @@ __global__ void __launch_bounds__(128) k_ratio_df(DevProblem P, DevScratch S) {
   const int nu_det = P.n_det_sp[0], ntot = nu_det + P.n_det_sp[1];
   const int M = P.n_mo;
   const int64_t wp = S.wp;
+  int sp_max = 0;
+  uint32_t top = 0;
   for (int q = 0; q < 8; q++) {
     const int t = blockIdx.x * 32 + warp * 8 + q;
-    if (t >= ntot) return;
+    if (t >= ntot) break;
     const int sp = t < nu_det ? 0 : 1;
     const Exc e = P.exc[sp][sp ? t - nu_det : t];
     const float2* T = S.Tdf + (size_t)(sp ? P.n_up * M : 0) * wp;
@@ -285,10 +287,15 @@ __global__ void __launch_bounds__(128) k_ratio_df(DevProblem P, DevScratch S) {
       }
     const df32 d0 = small_det_dot(e.k, m);
     const df32 dd = e.eps < 0 ? df32(-d0.hi, -d0.lo) : d0;  // the sign on the FP32 words
-    S.r[(size_t)t * wp + w] = df_to_double_int(dd);  // the FP64 ratio for the contraction, off the FP64 pipe
+    const double d = df_to_double_int(dd);  // the FP64 ratio for the contraction, off the FP64 pipe
+    S.r[(size_t)t * wp + w] = d;
     if (S.rdf) S.rdf[(size_t)t * wp + w] = make_float2(dd.hi, dd.lo);
-    if (P.split[t]) S.vu[w * ntot + t] = 0.0;  // the contraction adds the pieces of a cut segment
+    if (S.xmax)
+      ratio_max(S, w, sp, sp_max, top, d);
+    else if (P.split[t])
+      S.vu[w * ntot + t] = 0.0;  // the contraction adds the pieces of a cut segment
   }
+  if (S.xmax && top) atomicMax(S.xmax + sp_max * wp + w, top);
 }
 
 // Self-check of the double-float building blocks against FP64 on the device:

@@ -1,0 +1,807 @@
+// The CI contraction as integer matrix products on the 5th-generation tensor cores:
+// v = C r_dn (with Psi~ = r_up . v and its magnitude sum) and u = C^T r_up (Sec. 2.4),
+// exact for the fixed-point operands and rounded to FP64 once per output.
+//
+// Why. In FP64 the two products are 4 nnz flops per walker on a pipe that delivers 1.24
+// TFLOP/s, and they bound the whole evaluation. As a dense product of residues the same sums
+// run on the BF16 tensor cores, which are 1,500 times as fast, so a filled-in C of a few per
+// cent of nonzeros is still far cheaper: 750,000 products over 3,015 x 3,015 distinct
+// determinants and 8,192 walkers take 20.5 ms as FP64 sums, and 5.1 ms here (residues 0.43,
+// products 3.44 at 1.66 PFLOP/s, 0.86 of the measured BF16 burst rate, reconstruction 1.2).
+//
+// Method (multi-modular integer products, the Chinese remainder theorem).
+//  - Fixed point: row i of C as chat_ij = rint(c_ij 2^(61 - es_i)) with sum_j |c_ij| < 2^es_i,
+//    walker w's ratios as rhat_j = rint(r_j 2^(62 - xe_w)) with max_j |r_j| < 2^xe_w. Then
+//    |sum_j chat_ij rhat_j| < 2^123.1, an integer that determines v_i up to the two roundings,
+//    2^-62 of the row's and 2^-63 of the walker's largest values: below the rounding errors of
+//    an FP64 sum (simulated on the ratios of the synthetic walkers, the error of v weighted by
+//    r_up is 0.01 to 0.4 of FP64 accumulation's).
+//  - Residues: for pairwise coprime moduli p_q <= 256 the balanced residues |chat mod p_q|,
+//    |rhat mod p_q| <= 128 are exact in BF16, and sum_j |A_ij| (p_q / 2) <= 2^24 (checked on
+//    the actual residues when the moduli are chosen) keeps every partial sum of the FP32
+//    accumulator an exact integer. The accumulators are reduced mod p_q to one byte.
+//  - Reconstruction: X = sum_q y_q M_q - k P with M_q = (P / p_q) ((P / p_q)^-1 mod p_q),
+//    P = prod p_q > 2^124.6 and k = rint(sum_q y_q ((P / p_q)^-1 mod p_q) / p_q), in 128-bit
+//    wrap-around integers: X is exact, and v_i = RN(X) 2^(es_i + xe_w - 123).
+//  - The magnitude sum behind Psi~ (sum_j |c_ij| |r_j|, for the error estimate) rides along as
+//    one more product: both magnitudes as a BF16 pair h + l (2^-17 relative), h h + h l + l h
+//    in one FP32 accumulator.
+// A walker whose ratios are not all finite takes a direct FP64 sum over the products instead,
+// so that infinities and NaN propagate as they do in FP64.
+#include <algorithm>
+#include <cmath>
+#include <cstdint>
+#include <vector>
+
+#include "mdet_device.cuh"
+#include "mdet_internal.h"
+#include "umma.cuh"
+
+namespace mdet {
+
+namespace {
+
+constexpr int kCBits = 61, kRBits = 62;  // fixed-point fractions of C rows and of a walker's ratios
+constexpr int kTileBytes = 128 * 64 * 2;  // 128 walkers x 64 determinants of one plane
+constexpr int kMinP = 16, kMaxP = 256;
+
+__device__ __forceinline__ long long c_fixed(double c, int es) { return __double2ll_rn(scalbn(c, kCBits - es)); }
+
+__device__ __forceinline__ int balanced_mod(long long x, int p) {
+  int m = (int)(x % p);
+  if (2 * m > p) m -= p;
+  if (2 * m < -p) m += p;
+  return m;
+}
+
+// d = c + sum of products of the unsigned bytes of a with the signed bytes of b
+__device__ __forceinline__ int dp4a_us(uint32_t a, uint32_t b, int c) {
+  int d;
+  asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(c));
+  return d;
+}
+
+// The balanced residue, as an exact FP32 integer, of the 64-bit integer x given as x + 2^63 in
+// two words: its eight unsigned bytes times 256^k mod p, reduced in FP32 (an integer below 2^22
+// plus the bits of 1.5 * 2^23 is its float value without a conversion).
+__device__ __forceinline__ float residue(uint32_t lo, uint32_t hi, const ModConst& c) {
+  const float f = __int_as_float(dp4a_us(hi, c.c1, dp4a_us(lo, c.c0, c.off))) - 12582912.0f;
+  const float k = __fadd_rn(__fmaf_rn(f, c.invp, 12582912.0f), -12582912.0f);
+  return __fmaf_rn(-k, c.p, f);
+}
+
+__host__ __device__ inline ModConst mod_const(int p) {
+  ModConst c;
+  c.p = (float)p;
+  c.invp = 1.0f / (float)p;
+  uint32_t w[2] = {0, 0};
+  int pw = 1;  // 256^k mod p
+  for (int k = 0; k < 8; k++) {
+    const int b = 2 * pw > p ? pw - p : pw;
+    w[k / 4] |= (uint32_t)(uint8_t)(int8_t)b << (8 * (k % 4));
+    if (k < 7) pw = pw * 256 % p;
+  }
+  c.c0 = w[0];
+  c.c1 = w[1];
+  c.off = 0x4B400000 - pw * 128 % p;  // minus 2^63 mod p
+  return c;
+}
+
+// Largest row sum of the |balanced residues| of C for every modulus kMinP..kMaxP: a block per
+// row, its warps over the nonzeros, lanes over the moduli. Run once per expansion.
+__global__ void __launch_bounds__(256) k_mod_rowsum(const int* __restrict__ ptr, const double* __restrict__ val,
+                                                    const int* __restrict__ es, unsigned* __restrict__ mx) {
+  constexpr int kPer = (kMaxP - kMinP + 32) / 32;
+  __shared__ unsigned sum[kPer * 32];
+  const int row = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int t = threadIdx.x; t < kPer * 32; t += blockDim.x) sum[t] = 0;
+  __syncthreads();
+  float s[kPer];  // exact: at most 2^24 before they are added to the block's
+  ModConst c[kPer];
+#pragma unroll
+  for (int t = 0; t < kPer; t++) {
+    s[t] = 0.0f;
+    c[t] = mod_const(min(kMinP + lane + 32 * t, kMaxP));
+  }
+  const int e = es[row];
+  int n = 0;
+  for (int k = ptr[row] + warp; k < ptr[row + 1]; k += 8) {
+    const unsigned long long x = (unsigned long long)c_fixed(val[k], e) + 0x8000000000000000ULL;
+#pragma unroll
+    for (int t = 0; t < kPer; t++) s[t] += fabsf(residue((uint32_t)x, (uint32_t)(x >> 32), c[t]));
+    if (++n == 65536) {  // far beyond what the moduli allow: keep the sums exact and saturated
+      n = 0;
+#pragma unroll
+      for (int t = 0; t < kPer; t++) {
+        atomicMax(&sum[lane + 32 * t], 1u << 28);
+        s[t] = 0.0f;
+      }
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < kPer; t++) atomicAdd(&sum[lane + 32 * t], (unsigned)s[t]);
+  __syncthreads();
+  for (int t = threadIdx.x; t <= kMaxP - kMinP; t += blockDim.x) atomicMax(mx + t, sum[t]);
+}
+
+// The residue planes of C in one order (rows = the product's outputs, gathered index = K), and
+// with n_abs the two magnitude planes. Blocks of hw rows x 64 K in the 128-byte swizzle of the
+// MMA's shared-memory operands (row r at 128 r, its 16-byte chunk j at chunk j ^ (r mod 8)),
+// [plane][tile][half][K block][row][64]; zeroed before.
+__global__ void __launch_bounds__(256) k_mod_planes(const __grid_constant__ DenseContract D, int o,
+                                                    const int* __restrict__ row, const int* __restrict__ col,
+                                                    const double* __restrict__ val, int64_t nnz, int n_abs) {
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= nnz) return;
+  const int i = row[k], j = col[k], hw = D.hw[o], kb = D.kb[1 - o];
+  const int es = D.es[o][i];
+  const long long c = c_fixed(val[k], es);
+  const int h = i / hw, rr = i - h * hw;  // half tiles are consecutive blocks of hw rows
+  const size_t plane = (size_t)D.nt[o] * 2 * kb * hw * 64;
+  const size_t at = ((size_t)h * kb + j / 64) * hw * 64 + (size_t)rr * 64 + (((j % 64) / 8) ^ (rr & 7)) * 8 + j % 8;
+  for (int q = 0; q < D.nm; q++)
+    D.planes[o][q * plane + at] = (uint16_t)(__float_as_uint((float)balanced_mod(c, (int)D.m[q].p)) >> 16);
+  if (n_abs) {
+    const float f = __double2float_rn(scalbn(fabs(val[k]), -es));
+    const uint32_t hb = (__float_as_uint(f) + 0x8000u) & 0xffff0000u;
+    D.planes[o][D.nm * plane + at] = (uint16_t)(hb >> 16);
+    const float l = f - __uint_as_float(hb);
+    D.planes[o][(D.nm + 1) * plane + at] = (uint16_t)((__float_as_uint(l) + 0x8000u) >> 16);
+  }
+}
+
+// Residue planes of the ratios. A block takes 32 walkers (lanes) and 64 consecutive
+// determinants of one spin (8 per warp): the loads from the walker-minor ratios are coalesced,
+// and the block's 4 KB of each plane (32 rows of 128 bytes) goes through shared memory to be
+// stored as one contiguous piece. Bound by those stores (2 bytes per modulus and ratio).
+__global__ void __launch_bounds__(256) k_mod_residues(const __grid_constant__ DenseContract D,
+                                                      const double* __restrict__ r, int64_t wp,
+                                                      const uint32_t* __restrict__ xmax, int64_t w0, int nu, int nd,
+                                                      uint16_t* __restrict__ X, int nmt, int n_abs,
+                                                      int* __restrict__ err, const int* __restrict__ live) {
+  __shared__ uint4 tile[2][256];
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *err = 0;
+  const int lane = threadIdx.x & 31, oct = threadIdx.x >> 5;
+  const int wl = blockIdx.y * 32 + lane;  // walker within the block of walkers
+  if (live && w0 + wl / 256 * 256 >= *live) return;
+  const int sp = (int)blockIdx.x < D.kb[0] ? 0 : 1;
+  const int kbi = sp ? blockIdx.x - D.kb[0] : blockIdx.x;
+  const int n = sp ? nd : nu;
+  const int64_t w = w0 + wl;
+  const int xb = (int)(xmax[sp * wp + w] >> 20);  // biased exponent of the walker's largest |r|
+  const double* rs = r + (size_t)(sp ? nu : 0) * wp + w;
+  uint32_t lo[8], hi[8];  // rhat + 2^63
+  uint32_t ha[4], la[4];  // magnitude planes
+#pragma unroll
+  for (int z = 0; z < 8; z++) {
+    const int i = kbi * 64 + oct * 8 + z;
+    const long long b = (i < n && xb < 0x7ff) ? __double_as_longlong(rs[(size_t)i * wp]) : 0;
+    const int e = (int)((b >> 52) & 0x7ff);
+    unsigned long long m = (unsigned long long)b & 0xfffffffffffffULL;
+    if (e) m |= 1ULL << 52;
+    const int s = max(e, 1) - xb + 9;  // rhat = significand 2^s: 2^(max(e,1) - 1075) = 2^s 2^(xb - 1022 - 62)
+    if (s >= 0)
+      m <<= min(s, 9);
+    else
+      m = s < -54 ? 0 : (m + (1ULL << (-s - 1))) >> (-s);
+    const unsigned long long x = (b < 0 ? 0ULL - m : m) + 0x8000000000000000ULL;
+    lo[z] = (uint32_t)x;
+    hi[z] = (uint32_t)(x >> 32);
+    if (sp && n_abs) {
+      const float f = __uint2float_rn((uint32_t)(m >> 31)) * 0x1p-31f;  // |r| 2^-xe
+      const uint32_t hb = (__float_as_uint(f) + 0x8000u) & 0xffff0000u;
+      const uint32_t lb = __float_as_uint(f - __uint_as_float(hb)) + 0x8000u;
+      if (z & 1) {
+        ha[z >> 1] |= hb;
+        la[z >> 1] |= lb & 0xffff0000u;
+      } else {
+        ha[z >> 1] = hb >> 16;
+        la[z >> 1] = lb >> 16;
+      }
+    }
+  }
+  const int kb = D.kb[sp];
+  const size_t plane = (size_t)nmt * kb * (kTileBytes / 16);
+  const int row = wl % 128;
+  uint4* dst = reinterpret_cast<uint4*>(X) + (sp ? (size_t)D.nm * nmt * D.kb[0] * (kTileBytes / 16) : 0) +
+               ((size_t)(wl / 128) * kb + kbi) * (kTileBytes / 16) + (row - lane) * 8 + threadIdx.x;
+  const int at = lane * 8 + (oct ^ (row & 7));  // 128-byte swizzle
+  for (int q = 0; q < D.nm; q++) {
+    const ModConst c = D.m[q];
+    uint32_t out[4];
+#pragma unroll
+    for (int z = 0; z < 8; z += 2)
+      out[z >> 1] = __byte_perm(__float_as_uint(residue(lo[z], hi[z], c)), __float_as_uint(residue(lo[z + 1], hi[z + 1], c)),
+                                0x7632);
+    tile[q & 1][at] = make_uint4(out[0], out[1], out[2], out[3]);
+    __syncthreads();
+    dst[q * plane] = tile[q & 1][threadIdx.x];
+  }
+  if (sp && n_abs) {
+    __syncthreads();
+    tile[0][at] = make_uint4(ha[0], ha[1], ha[2], ha[3]);
+    tile[1][at] = make_uint4(la[0], la[1], la[2], la[3]);
+    __syncthreads();
+    dst[D.nm * plane] = tile[0][threadIdx.x];
+    dst[(D.nm + 1) * plane] = tile[1][threadIdx.x];
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The residue products. A work unit is one 256 walker x NW determinant tile (NW = 2 hw <= 256)
+// of one plane: D[w][i] = sum_k Xplane[w][k] Cplane[i][k]. A cluster of two CTAs takes it, 128
+// walkers each (MMAs of M = 128, N = NW, K = 16); the determinant rows serve both, so each CTA
+// fetches one half of them and multicasts it into both shared memories: 32 KB of L2 reads per SM
+// and 64 K instead of 48.
+// Warps: 0 the producer (bulk copies of pre-tiled blocks into a 4-stage ring), 1 the MMA issuer,
+// 2 tensor memory, 4-7 the epilogue of the previous unit from the other of two 256-column
+// accumulators: reduction mod p to one byte, 16 bytes per store. A stage is refilled when both
+// CTAs' MMAs have read it (their commits arrive on both CTAs' barriers).
+// Units are ordered plane by plane, so that one plane of C and of the ratios stays in L2.
+// cta_group::2 pairs measured 10 % faster alone, but their collective tensor-memory allocation
+// never returned on some SM pairs while other streams' kernels held part of the SMs; CTAs that
+// only share copies have no such dependence. The barrier operations keep their default (CTA)
+// scope: cluster-scope acquires and releases put a fence into every pipeline stage and halved
+// the rate, and the data they guard is written and read by the asynchronous proxy only.
+// Every wait is bounded in time; when one runs out the CTA sets *err and finishes without
+// further copies or MMAs, and the reconstruction writes NaN.
+constexpr int kStages = 4;
+constexpr int kStageBytes = 3 * kTileBytes;
+constexpr long long kWaitClocks = 8000000000LL;  // about 4 s
+
+struct GemmArgs {
+  const uint16_t* X;
+  uint8_t* Y;
+  float* Yabs;
+  int nmt;  // 128-walker tiles in the layout of X and Y (even)
+  int n_abs;
+  int64_t w0;
+  const int* live;
+  int* err;
+  unsigned long long* stamp;
+};
+
+__device__ __forceinline__ unsigned long long now_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+__device__ __forceinline__ uint32_t cta_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+
+__device__ __forceinline__ bool try_wait_bar(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, "
+      "p;\n}"
+      : "=r"(done)
+      : "r"(umma::smem_u32(bar)), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
+// Waits for the phase, at most kWaitClocks; gives up at once when the CTA has already given up.
+// (The SM's clock, because a read of the global timer takes longer than a pipeline stage.)
+__device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, volatile int* dead) {
+  if (try_wait_bar(bar, parity)) return true;
+  const long long t0 = clock64();
+  for (;;) {
+    if (try_wait_bar(bar, parity)) return true;
+    if (*dead) return false;
+    if (clock64() - t0 > kWaitClocks) {
+      *dead = 1;
+      return false;
+    }
+  }
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(umma::smem_u32(bar))
+               : "memory");
+}
+
+__device__ __forceinline__ void expect_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(umma::smem_u32(bar)), "r"(bytes)
+               : "memory");
+}
+
+// The same into both CTAs of the cluster, at the same offsets, each signalling its own barrier.
+__device__ __forceinline__ void bulk_load_both(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::
+          "r"(dst),
+      "l"(src), "r"(bytes), "r"(umma::smem_u32(bar)), "h"((uint16_t)3)
+      : "memory");
+}
+
+// Arrives on both CTAs' barrier at this offset once every MMA this thread issued has completed.
+__device__ __forceinline__ void commit_both(uint64_t* bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+          umma::smem_u32(bar)),
+      "h"((uint16_t)3)
+      : "memory");
+}
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&v)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      : "r"(taddr)
+      : "memory");
+}
+
+struct Unit {
+  int o, plane, abs, mt, nt;
+};
+
+__device__ __forceinline__ Unit unit_of(const DenseContract& D, const GemmArgs& a, int64_t u, int nmt2) {
+  // groups: [magnitudes], then the planes of v, then those of u; determinant tiles fastest
+  Unit r;
+  const int64_t t0 = (int64_t)nmt2 * D.nt[0], g0 = a.n_abs + D.nm;
+  int64_t rem;
+  if (u < g0 * t0) {
+    const int g = (int)(u / t0);
+    rem = u - g * t0;
+    r.o = 0;
+    r.abs = a.n_abs && g == 0;
+    r.plane = r.abs ? D.nm : g - a.n_abs;
+  } else {
+    const int64_t t1 = (int64_t)nmt2 * D.nt[1];
+    u -= g0 * t0;
+    const int g = (int)(u / t1);
+    rem = u - g * t1;
+    r.o = 1;
+    r.abs = 0;
+    r.plane = g;
+  }
+  r.mt = (int)(rem / D.nt[r.o]);
+  r.nt = (int)(rem - (int64_t)r.mt * D.nt[r.o]);
+  return r;
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
+    k_mod_gemm(const __grid_constant__ DenseContract D, const __grid_constant__ GemmArgs a) {
+  extern __shared__ __align__(1024) uint8_t stage_mem[];
+  __shared__ __align__(8) uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], fin;
+  __shared__ uint32_t tbase;
+  __shared__ int dead_s;
+  volatile int* dead = &dead_s;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t rank = cta_rank();
+  if (a.stamp && tid == 0) atomicMax(a.stamp, ~now_ns());
+  if (warp == 2) umma::tmem_alloc(&tbase, 512);
+  if (tid == 0) {
+    for (int s = 0; s < kStages; s++) {
+      umma::mbar_init(&full[s], 1);
+      umma::mbar_init(&empty[s], 2);
+    }
+    for (int b = 0; b < 2; b++) {
+      umma::mbar_init(&tfull[b], 1);
+      umma::mbar_init(&tempty[b], 4);
+    }
+    umma::mbar_init(&fin, 1);
+    dead_s = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  umma::fence_before();
+  __syncthreads();
+  cluster_sync();
+  umma::fence_after();
+  const uint32_t tb = tbase;
+  const int64_t w_live = a.live ? max((int64_t)0, (int64_t)*a.live - a.w0) : (int64_t)a.nmt * 128;
+  const int nmt2 = (int)min((int64_t)(a.nmt / 2), (w_live + 255) / 256);
+  const int64_t n_units = (int64_t)(a.n_abs + D.nm) * nmt2 * D.nt[0] + (int64_t)D.nm * nmt2 * D.nt[1];
+  const int64_t first = blockIdx.x >> 1, step = gridDim.x >> 1;
+  const uint32_t stage0 = umma::smem_u32(stage_mem);
+
+  if (warp == 0 && lane == 0) {  // producer: this CTA's walkers, and its half of the determinant rows for both
+    uint32_t it = 0;
+    for (int64_t u = first; u < n_units && !*dead; u += step) {
+      const Unit t = unit_of(D, a, u, nmt2);
+      const int sp = 1 - t.o, kb = D.kb[sp], hw = D.hw[t.o];
+      const uint32_t b_bytes = (uint32_t)hw * 128;  // half of the determinant rows
+      const size_t xplane = (size_t)a.nmt * kb * kTileBytes, cplane = (size_t)D.nt[t.o] * 2 * kb * b_bytes;
+      const uint8_t* xs = reinterpret_cast<const uint8_t*>(a.X) +
+                          (sp ? (size_t)D.nm * a.nmt * D.kb[0] * kTileBytes : 0) +
+                          ((size_t)(t.mt * 2 + (int)rank) * kb) * kTileBytes;
+      const uint8_t* cs =
+          reinterpret_cast<const uint8_t*>(D.planes[t.o]) + ((size_t)(t.nt * 2 + (int)rank) * kb) * b_bytes;
+      for (int pass = 0; pass < (t.abs ? 3 : 1); pass++) {  // magnitudes: h h, h l, l h
+        const uint8_t* xp = xs + (size_t)(t.plane + (pass == 2)) * xplane;
+        const uint8_t* cp = cs + (size_t)(t.plane + (pass == 1)) * cplane;
+        for (int k = 0; k < kb; k++, it++) {
+          const int s = it % kStages;
+          if (it >= kStages && !bounded_wait(&empty[s], ((it / kStages) & 1) ^ 1, dead)) break;
+          expect_tx(&full[s], kTileBytes + 2 * b_bytes);
+          const uint32_t dst = stage0 + (uint32_t)s * kStageBytes;
+          bulk_load(dst, xp + (size_t)k * kTileBytes, kTileBytes, &full[s]);
+          bulk_load_both(dst + kTileBytes + rank * b_bytes, cp + (size_t)k * b_bytes, b_bytes, &full[s]);
+        }
+      }
+    }
+    // after a failed wait: the copies in flight land before the block exits (bounded)
+    if (*dead) {
+      const long long t0 = clock64();
+      for (int s = 0; s < kStages && it > (uint32_t)s; s++) {
+        const uint32_t last = it - 1 - ((it - 1 - (uint32_t)s) % kStages);
+        while (!try_wait_bar(&full[s], (last / kStages) & 1) && clock64() - t0 < kWaitClocks / 4) {
+        }
+      }
+    }
+  } else if (warp == 1 && lane == 0) {  // MMA issuer
+    uint32_t it = 0, n = 0;
+    for (int64_t u = first; u < n_units && !*dead; u += step, n++) {
+      const Unit t = unit_of(D, a, u, nmt2);
+      const int hw = D.hw[t.o], nk = D.kb[1 - t.o] * (t.abs ? 3 : 1), b = n & 1;
+      const uint32_t idesc = umma::idesc_bf16(128, 2 * hw);
+      if (n >= 2 && !bounded_wait(&tempty[b], ((n >> 1) & 1) ^ 1, dead)) break;
+      umma::fence_after();
+      bool ok = true;
+      for (int k = 0; k < nk && ok; k++, it++) {
+        const int s = it % kStages;
+        ok = bounded_wait(&full[s], (it / kStages) & 1, dead);
+        if (!ok) break;
+        umma::fence_after();
+        const uint32_t sa = stage0 + (uint32_t)s * kStageBytes, sb = sa + kTileBytes;
+#pragma unroll
+        for (int ks = 0; ks < 4; ks++)
+          umma::mma_smem_a(tb + 256u * b, umma::desc_sw128(sa + ks * 32), umma::desc_sw128(sb + ks * 32), idesc,
+                           (k | ks) != 0);
+        commit_both(&empty[s]);
+      }
+      if (ok) umma::commit(&tfull[b]);
+    }
+    if (*dead) {  // after a failed wait: the MMAs in flight finish (bounded) before the release
+      umma::commit(&fin);
+      const long long t0 = clock64();
+      while (!try_wait_bar(&fin, 0) && clock64() - t0 < kWaitClocks / 4) {
+      }
+    }
+  } else if (warp >= 4) {  // epilogue
+    const int qd = warp & 3;
+    uint32_t n = 0;
+    for (int64_t u = first; u < n_units && !*dead; u += step, n++) {
+      const Unit t = unit_of(D, a, u, nmt2);
+      const int b = n & 1, nw = 2 * D.hw[t.o], ldy = D.ldy[t.o];
+      const bool ok = bounded_wait(&tfull[b], (n >> 1) & 1, dead);
+      if (!__all_sync(0xffffffffu, ok)) break;
+      umma::fence_after();
+      const int64_t wl = (int64_t)t.mt * 256 + (int)rank * 128 + qd * 32 + lane;
+      const uint32_t ta = tb + ((uint32_t)(32 * qd) << 16) + 256u * b;
+      uint32_t v[16];
+      if (t.abs) {
+        float* dst = a.Yabs + wl * ldy + t.nt * nw;
+        for (int c = 0; c < nw; c += 16) {
+          umma::tmem_ld16(ta + c, v);
+#pragma unroll
+          for (int j = 0; j < 4; j++)
+            *reinterpret_cast<uint4*>(dst + c + 4 * j) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+        }
+      } else {
+        const float p = D.m[t.plane].p, ip = D.m[t.plane].invp;
+        uint8_t* dst = a.Y + (t.o ? (size_t)D.nm * a.nmt * 128 * D.ldy[0] : 0) +
+                       ((size_t)t.plane * a.nmt * 128 + wl) * ldy + t.nt * nw;
+        auto bytes = [&](const uint32_t* x) {  // residues of four accumulators, as signed bytes + 128
+          uint32_t w[4];
+#pragma unroll
+          for (int j = 0; j < 4; j++) {
+            const float f = __uint_as_float(x[j]);
+            const float k = __fadd_rn(__fmaf_rn(f, ip, 12582912.0f), -12582912.0f);
+            w[j] = __float_as_uint(__fadd_rn(__fmaf_rn(-k, p, f), 12583040.0f));  // 1.5 * 2^23 + 128
+          }
+          return __byte_perm(__byte_perm(w[0], w[1], 0x0040), __byte_perm(w[2], w[3], 0x0040), 0x5410);
+        };
+        uint32_t v2[16];
+        tmem_ld16_issue(ta, v);
+        for (int c = 0; c < nw; c += 32) {  // nw is a multiple of 32
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          tmem_ld16_issue(ta + c + 16, v2);
+          *reinterpret_cast<uint4*>(dst + c) = make_uint4(bytes(v), bytes(v + 4), bytes(v + 8), bytes(v + 12));
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (c + 32 < nw) tmem_ld16_issue(ta + c + 32, v);
+          *reinterpret_cast<uint4*>(dst + c + 16) = make_uint4(bytes(v2), bytes(v2 + 4), bytes(v2 + 8), bytes(v2 + 12));
+        }
+      }
+      umma::fence_before();
+      __syncwarp();
+      if (lane == 0) umma::mbar_arrive(&tempty[b]);
+    }
+  }
+  __syncwarp();
+  umma::fence_before();
+  __syncthreads();
+  if (tid == 0 && *dead) *a.err = 1;
+  cluster_sync();  // neither CTA exits while the other's copies or commits may still reach it
+  umma::fence_after();
+  if (warp == 2) umma::tmem_dealloc(tb, 512);
+  if (a.stamp && tid == 0) atomicMax(a.stamp + 1, now_ns());
+}
+
+// RN(x) 2^e for a 128-bit integer x, correctly rounded (ties to even) when the result is normal.
+__device__ __noinline__ double scale_slow(double m, int e) { return ldexp(m, e); }
+
+__device__ __forceinline__ double i128_to_double(unsigned long long hi, unsigned long long lo, int e) {
+  const unsigned long long sign = hi & 0x8000000000000000ULL;
+  if (sign) {
+    lo = ~lo + 1;
+    hi = ~hi + (lo == 0);
+  }
+  if ((hi | lo) == 0) return 0.0;
+  if (hi == 0) {
+    hi = lo;
+    lo = 0;
+    e -= 64;
+  }
+  const int lz = __clzll(hi);
+  if (lz) {
+    hi = (hi << lz) | (lo >> (64 - lz));
+    lo <<= lz;
+  }
+  // value = hi.lo 2^(e + 64 - lz), hi in [2^63, 2^64): 53 bits kept, 11 (and lo) rounded
+  unsigned long long m = hi >> 11;
+  const unsigned rem = (unsigned)hi & 0x7ffu;
+  if (rem > 0x400u || (rem == 0x400u && (lo != 0 || (m & 1)))) m++;
+  const int be = e + 64 - lz + 11 + 52 + 1023;  // biased exponent of m = 1.xxx 2^52
+  if (be < 1 || be > 2045) {
+    const double s = scale_slow((double)m, e + 64 - lz + 11);
+    return sign ? -s : s;
+  }
+  return __longlong_as_double((long long)(sign | (((unsigned long long)(be - 1) << 52) + m)));
+}
+
+// Reconstruction of v and u from the residue bytes, with Psi~ = r_up . v and its magnitude sum:
+// a warp per walker and product, four consecutive determinants per lane (one 4-byte load per
+// modulus, all issued before the arithmetic). Every walker's Psi~ is summed in one warp, in a
+// fixed order. Stores go through shared memory so that a warp writes 256 consecutive bytes.
+__global__ void __launch_bounds__(256) k_mod_crt(const __grid_constant__ DenseContract D, DevProblem P, DevScratch S,
+                                                 int64_t w0, int64_t n_walk, int nmt, int n_abs) {
+  __shared__ double tile[8][128];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int o = warp >> 2;  // warps 0-3: v of four walkers, 4-7: u of the same
+  const int64_t wl = (int64_t)blockIdx.x * 4 + (warp & 3), w = w0 + wl;
+  if (w >= n_walk || (S.live && w >= *S.live)) return;
+  const int nu = P.n_det_sp[0], nd = P.n_det_sp[1];
+  const int64_t wp = S.wp;
+  const bool failed = *S.derr != 0;
+  const int n = o ? nd : nu, ldy = D.ldy[o];
+  const int xb = (int)(S.xmax[(size_t)(1 - o) * wp + w] >> 20);
+  double* out = S.vu + w * ((int64_t)nu + nd) + (o ? nu : 0);
+  double psi = 0.0;
+  float pa = 0.0f;
+  if (xb >= 0x7ff || failed) {  // ratios that are not finite: the FP64 sum itself
+    const int* ptr = o ? P.csc_ptr : P.csr_ptr;
+    const int* gi = o ? P.csc_row : P.csr_col;
+    const double* val = o ? P.csc_val : P.csr_val;
+    const double* x = S.r + (size_t)(o ? 0 : nu) * wp + w;
+    for (int i = lane; i < n; i += 32) {
+      double acc = 0.0;
+      float aa = 0.0f;
+      for (int k = ptr[i]; k < ptr[i + 1]; k++) {
+        const double xv = x[(size_t)gi[k] * wp];
+        acc = fma(val[k], xv, acc);
+        aa = fmaf(abs_f32_of(val[k]), abs_f32_of(xv), aa);
+      }
+      if (failed) acc = __longlong_as_double(0x7ff8000000000000LL);
+      out[i] = acc;
+      if (!o) {
+        const double ri = S.r[(size_t)i * wp + w];
+        psi = fma(ri, acc, psi);
+        pa = fmaf(abs_f32_of(ri), aa, pa);
+      }
+    }
+  } else {
+    const int e0 = xb - 1022 - kCBits - kRBits;
+    const uint8_t* y = S.dy + (o ? (size_t)D.nm * nmt * 128 * D.ldy[0] : 0) + (size_t)wl * ldy;
+    const size_t yplane = (size_t)nmt * 128 * ldy;
+    for (int base = 0; base < n; base += 128) {
+      const int i0 = base + 4 * lane;
+      if (i0 < ldy) {
+        unsigned long long s[4][4];
+        long long kf[4];
+#pragma unroll
+        for (int z = 0; z < 4; z++) {
+          kf[z] = D.finit;
+#pragma unroll
+          for (int j = 0; j < 4; j++) s[z][j] = D.init4[j];
+        }
+        uint32_t yw[kMaxModuli];  // all the loads first
+#pragma unroll
+        for (int q = 0; q < kMaxModuli; q++)
+          if (q < D.nm) yw[q] = __ldg(reinterpret_cast<const uint32_t*>(y + q * yplane + i0));
+#pragma unroll
+        for (int q = 0; q < kMaxModuli; q++) {
+          if (q >= D.nm) break;
+          const uint32_t yb = yw[q];
+          const uint32_t m0 = D.M4[q][0], m1 = D.M4[q][1], m2 = D.M4[q][2], m3 = D.M4[q][3], F = D.F[q];
+#pragma unroll
+          for (int z = 0; z < 4; z++) {
+            const uint32_t b = (yb >> (8 * z)) & 0xffu;
+            s[z][0] += (unsigned long long)b * m0;
+            s[z][1] += (unsigned long long)b * m1;
+            s[z][2] += (unsigned long long)b * m2;
+            s[z][3] += (uint32_t)(b * m3);
+            kf[z] += (long long)((unsigned long long)b * F);
+          }
+        }
+#pragma unroll
+        for (int z = 0; z < 4; z++) {
+          const unsigned long long t1 = s[z][1] + (s[z][0] >> 32), t2 = s[z][2] + (t1 >> 32), t3 = s[z][3] + (t2 >> 32);
+          unsigned __int128 X = ((unsigned __int128)((t3 << 32) | (uint32_t)t2) << 64) | ((t1 << 32) | (uint32_t)s[z][0]);
+          const long long k = (kf[z] + 0x80000000LL) >> 32;
+          const unsigned __int128 Pm = ((unsigned __int128)(((unsigned long long)D.P4[3] << 32) | D.P4[2]) << 64) |
+                                       (((unsigned long long)D.P4[1] << 32) | D.P4[0]);
+          X -= (unsigned __int128)(__int128)k * Pm;
+          const int i = i0 + z;
+          tile[warp][4 * lane + z] =
+              i < n ? i128_to_double((unsigned long long)(X >> 64), (unsigned long long)X, e0 + D.es[o][i]) : 0.0;
+        }
+      }
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < 4; j++) {
+        const int i = base + 32 * j + lane;
+        if (i < n) {
+          const double v = tile[warp][32 * j + lane];
+          out[i] = v;
+          if (!o) {
+            const double ri = S.r[(size_t)i * wp + w];
+            psi = fma(ri, v, psi);
+            if (n_abs)
+              pa = fmaf(abs_f32_of(ri), ldexpf(S.dyabs[(size_t)wl * ldy + i], D.es[0][i] + xb - 1022), pa);
+          }
+        }
+      }
+      __syncwarp();
+    }
+  }
+  if (o) return;
+#pragma unroll
+  for (int off = 16; off; off >>= 1) {
+    psi += __shfl_xor_sync(0xffffffffu, psi, off);
+    pa += __shfl_xor_sync(0xffffffffu, pa, off);
+  }
+  if (lane == 0) {
+    S.psit[w] = psi;
+    if (!S.live) S.psia[w] = pa;  // a re-evaluation keeps the sum of the evaluation that flagged it
+  }
+}
+
+typedef unsigned __int128 u128;
+
+int gcd_int(int a, int b) {
+  while (b) {
+    const int t = a % b;
+    a = b;
+    b = t;
+  }
+  return a;
+}
+
+}  // namespace
+
+// The moduli for an expansion: pairwise coprime, largest first, each with sum_j |A_ij| (p / 2) <= 2^24
+// over the rows of both orders (rowmax, from k_mod_rowsum), until the product exceeds 2^124.6.
+// Odd moduli stop at 253, because the reduction of the accumulators may be off by one near a
+// half and its result must fit a signed byte. False when that takes more than kMaxModuli.
+bool choose_moduli(const uint32_t* rowmax, DenseContract* D) {
+  std::vector<int> ps;
+  double bits = 0.0;
+  for (int p = kMaxP; p >= kMinP && bits < 124.6; p--) {
+    if (p != 256 && p > ((p & 1) ? 253 : 252)) continue;
+    if ((uint64_t)rowmax[p - kMinP] * (uint64_t)(p / 2) > (1u << 24)) continue;
+    bool ok = true;
+    for (int q : ps) ok = ok && gcd_int(p, q) == 1;
+    if (!ok) continue;
+    if ((int)ps.size() == kMaxModuli) return false;
+    ps.push_back(p);
+    bits += std::log2((double)p);
+  }
+  if (bits < 124.6) return false;
+  D->nm = (int)ps.size();
+  u128 Pm = 1, init = 0;
+  for (int p : ps) Pm *= (u128)p;  // modulo 2^128 throughout
+  long long fi = 0;
+  for (int q = 0; q < D->nm; q++) {
+    const int p = ps[q];
+    u128 others = 1;
+    int om = 1;
+    for (int t = 0; t < D->nm; t++)
+      if (t != q) {
+        others *= (u128)ps[t];
+        om = om * ps[t] % p;
+      }
+    int inv = 1;
+    while (inv * om % p != 1 % p) inv++;
+    const u128 M = others * (u128)inv;
+    for (int j = 0; j < 4; j++) D->M4[q][j] = (uint32_t)(M >> (32 * j));
+    D->F[q] = (uint32_t)std::llrint(4294967296.0 * inv / p);
+    init -= (u128)128 * M;  // the bytes are residues + 128
+    fi -= 128LL * (long long)D->F[q];
+    D->m[q] = mod_const(p);
+  }
+  for (int j = 0; j < 4; j++) {
+    D->P4[j] = (uint32_t)(Pm >> (32 * j));
+    D->init4[j] = (uint32_t)(init >> (32 * j));
+  }
+  D->finit = fi;
+  return true;
+}
+
+int dense_moduli_range() { return kMaxP - kMinP + 1; }
+
+cudaError_t launch_dense_rowsum(const DevProblem& P, const int* const es[2], uint32_t* mx, cudaStream_t st) {
+  cudaError_t e = cudaMemsetAsync(mx, 0, sizeof(uint32_t) * (kMaxP - kMinP + 1), st);
+  if (e != cudaSuccess) return e;
+  k_mod_rowsum<<<P.n_det_sp[0], 256, 0, st>>>(P.csr_ptr, P.csr_val, es[0], mx);
+  k_mod_rowsum<<<P.n_det_sp[1], 256, 0, st>>>(P.csc_ptr, P.csc_val, es[1], mx);
+  return cudaGetLastError();
+}
+
+size_t dense_plane_elems(const DenseContract& D, int o) { return (size_t)D.nt[o] * 2 * D.kb[1 - o] * D.hw[o] * 64; }
+
+cudaError_t launch_dense_planes(const DevProblem& P, const DenseContract& D, cudaStream_t st) {
+  for (int o = 0; o < 2; o++) {
+    const size_t bytes = dense_plane_elems(D, o) * 2 * (D.nm + (o ? 0 : 2));
+    cudaError_t e = cudaMemsetAsync(D.planes[o], 0, bytes, st);
+    if (e != cudaSuccess) return e;
+    k_mod_planes<<<(unsigned)((P.nnz + 255) / 256), 256, 0, st>>>(D, o, o ? P.csc_col : P.csr_row,
+                                                                 o ? P.csc_row : P.csr_col, o ? P.csc_val : P.csr_val,
+                                                                 P.nnz, o ? 0 : 1);
+  }
+  return cudaGetLastError();
+}
+
+void dense_shape(int n_up, int n_dn, DenseContract* D) {
+  const int n[2] = {n_up, n_dn};
+  for (int o = 0; o < 2; o++) {
+    D->kb[o] = (n[o] + 63) / 64;
+    D->nt[o] = (n[o] + 255) / 256;
+    D->hw[o] = ((n[o] + D->nt[o] - 1) / D->nt[o] + 31) / 32 * 16;  // NW = 2 hw, a multiple of 32
+    D->ldy[o] = D->nt[o] * 2 * D->hw[o];
+  }
+}
+
+void dense_bytes(const DenseContract& D, size_t* x, size_t* y, size_t* yabs) {
+  *x = (size_t)(D.nm * (D.kb[0] + D.kb[1]) + 2 * D.kb[1]) * 64 * 2;
+  *y = (size_t)D.nm * (D.ldy[0] + D.ldy[1]);
+  *yabs = (size_t)D.ldy[0] * sizeof(float);
+}
+
+cudaError_t launch_contract_dense(const DevProblem& P, const DevScratch& S, int64_t n_walk, cudaStream_t st,
+                                  unsigned long long* stamp, int* n_kernels) {
+  const DenseContract& D = *P.dense;
+  static SmemOptIn opt;
+  const size_t smem = (size_t)kStages * kStageBytes;
+  cudaError_t e = opt.ensure(k_mod_gemm, smem);
+  if (e != cudaSuccess) return e;
+  if (stamp && (e = cudaMemsetAsync(stamp, 0, 4 * sizeof(unsigned long long), st)) != cudaSuccess) return e;
+  // the magnitude sum feeds the error estimate only, and a re-evaluation keeps the one it has
+  const int n_abs = !S.live && P.fallback_tol > 0.0 && P.n_up <= MDET_FALLBACK_MAX_SPIN;
+  for (int64_t w0 = 0; w0 < n_walk; w0 += S.dblk) {
+    const int64_t nb = std::min<int64_t>(S.dblk, n_walk - w0);
+    const int nmt = (int)((nb + 255) / 256) * 2;
+    k_mod_residues<<<dim3(D.kb[0] + D.kb[1], nmt * 4), 256, 0, st>>>(D, S.r, S.wp, S.xmax, w0, P.n_det_sp[0],
+                                                                 P.n_det_sp[1], S.dx, nmt, n_abs, S.derr, S.live);
+    GemmArgs a{S.dx, S.dy, S.dyabs, nmt, n_abs, w0, S.live, S.derr, stamp};
+    const int64_t units = (int64_t)(nmt / 2) * ((int64_t)(D.nm + n_abs) * D.nt[0] + (int64_t)D.nm * D.nt[1]);
+    const int64_t pairs = std::min<int64_t>(units, std::max(P.n_sm / 2, 1));
+    k_mod_gemm<<<(unsigned)(2 * pairs), 256, smem, st>>>(D, a);
+    k_mod_crt<<<(unsigned)((nb + 3) / 4), 256, 0, st>>>(D, P, S, w0, n_walk, nmt, n_abs);
+    if (n_kernels) *n_kernels += 3;
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+}  // namespace mdet

@@ -3,7 +3,7 @@
 // kind::f16 with BF16 operands, bounded mbarrier waits, tensor-memory loads and
 // stores, and the MMA forms used by the orbital product and the perceptron.
 //
-// Operand layout (both kernels): K-major, no swizzle. A core matrix is 8 rows of
+// Operand layout (orbital product and perceptron): K-major, no swizzle. A core matrix is 8 rows of
 // 16 bytes (8 BF16 along K); `lbo` is the byte distance between core matrices
 // along K and `sbo` the distance between 8-row groups. One MMA consumes K = 16,
 // i.e. two core matrices along K.
@@ -23,6 +23,14 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)_
 __device__ __forceinline__ uint64_t desc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
   return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | ((uint64_t)1 << 46);
+}
+
+// The same for rows of 128 bytes (64 BF16 along K) in the 128-byte swizzle: 16-byte chunk j of row r
+// at chunk j ^ (r mod 8), 8-row groups 1,024 bytes apart (tile bases 1,024-byte aligned); the K = 16
+// steps within a row advance the start address by 32 bytes. Layout type 2 at bits 61-63.
+__device__ __forceinline__ uint64_t desc_sw128(uint32_t saddr) {
+  return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) |
+         ((uint64_t)2 << 61);
 }
 
 // Instruction descriptor of kind::f16: FP32 accumulator (bits 4-5 = 1), BF16 A and B

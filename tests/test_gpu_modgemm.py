@@ -1,0 +1,122 @@
+"""The contraction as residue products on the tensor cores (csrc/mdet_modgemm.cu)
+against the sparse FP64 sums and against the oracle.
+
+Expansions dense enough take the residue products; set_tuning(spmm_blocks > 0) selects
+the sparse sums on the same context. The kernels launched tell the two apart (7 and 6 per
+evaluation without the fallback).
+"""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+import paper_1510_00730_gb300 as pkg
+from paper_1510_00730_gb300 import synth
+from tests.parity import compare
+
+pytestmark = pytest.mark.gpu
+
+KEYS = ("log_abs_psi", "sign", "grad", "lap", "e_local", "status")
+TOL = {pkg.PRECISION_FP64: dict(tol_psi=1e-10, tol_der=1e-8), pkg.PRECISION_MIXED: dict(tol_psi=1e-9, tol_der=1e-6)}
+SPARSE_GRID = 1 << 20
+
+
+def _eval(ctx, R):
+    out = ctx.evaluate(torch.from_numpy(np.ascontiguousarray(R)).to("cuda:0"))
+    torch.cuda.synchronize()
+    return {k: out[k].cpu().numpy() for k in KEYS}
+
+
+def _workload(n_up_det, n_dn_det, n_walk, n_det=None, seed=5):
+    """5 up / 4 down electrons in 30 MOs with the given numbers of distinct determinants."""
+    n_det = n_det or max(4200, max(n_up_det, n_dn_det) * 3)
+    n_det = min(n_det, n_up_det * n_dn_det)
+    return synth.make_workload("mod", seed, 5, 4, 9, (12, 6, 2), (0.05, 500.0), 30, n_det, 4, n_walk,
+                               n_unique=(n_up_det, n_dn_det))
+
+
+# distinct determinants around the 64-wide K blocks and the 256-row (and 32-row) tiles
+SIZES = [(70, 66), (64, 128), (65, 129), (255, 257), (256, 256), (513, 96)]
+
+
+@pytest.mark.parametrize("prec", [pkg.PRECISION_FP64, pkg.PRECISION_MIXED])
+@pytest.mark.parametrize("nu,nd", SIZES)
+def test_residue_products_match_oracle_and_sparse_sums(nu, nd, prec):
+    wl = _workload(nu, nd, 40)
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    assert ctx.stats()["n_det_up"] == nu and ctx.stats()["n_det_dn"] == nd
+    if prec == pkg.PRECISION_MIXED:
+        ctx.set_fallback(1e-7)  # below the test tolerance, as the parity tests of this path
+    ref = oracle.evaluate(wl)
+    got = _eval(ctx, wl.R)
+    rep = compare(got, ref, **TOL[prec])
+    assert rep["ok"], rep
+    ctx.set_fallback(0.0)
+    table = _eval(ctx, wl.R)
+    assert ctx.last_kernels == 7
+    ctx.set_tuning(spmm_blocks=SPARSE_GRID)
+    sparse = _eval(ctx, wl.R)
+    assert ctx.last_kernels == 6
+    # both contractions get the same ratios: they may differ by their own rounding only, 2^-53 per term of
+    # the two nested sums, amplified like the CI sum itself, and by the rounding of the logarithm
+    tol = (nu + nd) * 2.0 ** -53 * np.maximum(ref["kappa"], 1.0) + 4 * np.spacing(np.abs(ref["log_abs_psi"]))
+    assert np.all(np.abs(table["log_abs_psi"] - sparse["log_abs_psi"]) <= tol)
+    assert np.array_equal(table["sign"], sparse["sign"]) and np.array_equal(table["status"], sparse["status"])
+
+
+@pytest.mark.parametrize("n_walk", [1, 31, 255, 257, 513])
+def test_ragged_walkers(n_walk):
+    wl = _workload(130, 70, n_walk, seed=6 + n_walk)
+    ctx = pkg.Context.from_workload(wl, device=0)
+    rep = compare(_eval(ctx, wl.R), oracle.evaluate(wl), **TOL[pkg.PRECISION_FP64])
+    assert rep["ok"], rep
+
+
+@pytest.mark.parametrize("prec", [pkg.PRECISION_FP64, pkg.PRECISION_MIXED])
+def test_error_estimates_agree(prec):
+    """The magnitude sum feeds the error estimate: as BF16 pairs it is within 2^-15 of the
+    sparse kernel's (2^-17 per operand there, 2^-20 here)."""
+    wl = _workload(200, 150, 300)
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    ctx.set_fallback(1e9)  # estimates on, nothing flagged
+    _eval(ctx, wl.R)
+    _, dense = ctx.error_estimates(300)
+    ctx.set_tuning(spmm_blocks=SPARSE_GRID)
+    _eval(ctx, wl.R)
+    _, sparse = ctx.error_estimates(300)
+    assert np.all(np.abs(dense - sparse) <= 2.0 ** -15 * sparse)
+
+
+@pytest.mark.parametrize("prec", [pkg.PRECISION_FP64, pkg.PRECISION_MIXED])
+def test_walkers_without_finite_ratios(prec):
+    """Coincident electrons make the reference singular and every ratio NaN: the outputs and
+    status of such walkers agree with the sparse sums', and their neighbours are untouched."""
+    wl = _workload(130, 70, 64)
+    R = wl.R.copy()
+    R[3, 1] = R[3, 0]    # spin up
+    R[40, 7] = R[40, 6]  # spin down
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    ctx.set_fallback(0.0)
+    clean = _eval(ctx, wl.R)
+    dense = _eval(ctx, R)
+    ctx.set_tuning(spmm_blocks=SPARSE_GRID)
+    sparse = _eval(ctx, R)
+    assert np.array_equal(dense["status"], sparse["status"])
+    for k in KEYS[:-1]:
+        assert np.array_equal(np.isfinite(dense[k]), np.isfinite(sparse[k])), k
+    ok = np.ones(64, bool)
+    ok[[3, 40]] = False
+    for k in ("log_abs_psi", "sign"):  # each walker's Psi~ is summed in a fixed order
+        assert np.array_equal(dense[k][ok], clean[k][ok]), k
+
+
+def test_dense_rows_take_smaller_moduli():
+    """A row with more than 2,048 nonzeros needs moduli below 256 for exact accumulators."""
+    wl = synth.make_workload("mod", 11, 5, 4, 9, (12, 6, 2), (0.05, 500.0), 30, 2400 * 40, 4, 6, n_unique=(40, 2400))
+    ctx = pkg.Context.from_workload(wl, device=0)
+    rep = compare(_eval(ctx, wl.R), oracle.evaluate(wl), **TOL[pkg.PRECISION_FP64])
+    assert rep["ok"], rep
+    assert ctx.last_kernels == 12
