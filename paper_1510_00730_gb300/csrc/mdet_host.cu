@@ -101,6 +101,14 @@ namespace {
 // items all add Psi~ of the same few walkers, and than 256)
 constexpr int kEscalationChunk = 128;
 
+// short work items for small contractions (pick_items). A warp walks its nonzeros one after the
+// other at about 0.6 us each when it has nothing to overlap with, but every piece of a cut segment
+// costs atomics: 1,000 products x 64 walkers took 570 us in items of 512 and takes 31 in items of 16,
+// 28,417 products x 8,192 walkers took 2.03 ms in items of 512, 1.47 in items of 128, 1.82 in items
+// of 64 and 4.4 in items of 16, so the items shrink only until there are a few thousand warps.
+constexpr int kSmallChunks[] = {256, 128, 64, 32, 16};
+constexpr int64_t kItemWarps = 4096;
+
 // words of S.queue per walker chunk: the work counters of its two persistent contractions, then
 // the global-timer stamps (start complemented, end) of each
 constexpr int kQueueWords = 6;
@@ -305,6 +313,17 @@ bool use_items(const mdet_ctx* c, DevProblem& P, int chunk) {
       return true;
     }
   return false;
+}
+
+// The item size of one contraction: the tuned one, or shorter items when those are too few to fill
+// the chip with warps (each walks its nonzeros one after the other). The count is over groups of 256
+// walkers.
+void pick_items(const mdet_ctx* c, DevProblem& P, int64_t n_walk) {
+  const int64_t groups = (n_walk + kWalkerPad - 1) / kWalkerPad;
+  int chunk = c->spmm_chunk;
+  for (int small : kSmallChunks)
+    if (small < chunk && P.nnz / chunk * groups < kItemWarps) chunk = small;
+  use_items(c, P, chunk);
 }
 
 void free_arrays(DevScratch& S) {
@@ -555,6 +574,8 @@ mdet_status upload_problem(mdet_ctx* c) {
   }
   // contraction work items for the tuned size and for the short items of escalated re-evaluations
   if ((s = ensure_items(c, c->spmm_chunk)) != MDET_OK || (s = ensure_items(c, kEscalationChunk)) != MDET_OK) return s;
+  for (int chunk : kSmallChunks)
+    if ((s = ensure_items(c, chunk)) != MDET_OK) return s;
   use_items(c, P, c->spmm_chunk);
   if ((s = build_dense(c)) != MDET_OK) return s;
   // the sequential chain of Sec. 2.2: distinct determinants in the order of the key of Eq. 3,
@@ -1243,8 +1264,12 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
   auto stage = [&](int k, int i, cudaStream_t ks, int persistent) -> mdet_status {
     int64_t off, n;
     chunk_range(k, &off, &n);
-    DevScratch S = scratch_view(c->S, P, off);
-    if (!dense) S.xmax = nullptr;
+    DevScratch S = scratch_view(c->S, c->P, off);
+    DevProblem P = c->P;
+    if (!dense) {
+      S.xmax = nullptr;
+      if (c->spmm_blocks == 0) pick_items(c, P, n);
+    }
     const double* Rk = R + off * N * 3;
     const bool mark = prof_all;
     if (mark) CUDA_TRY(c, cudaEventRecord(c->ev[k][2 * i], ks));
