@@ -91,6 +91,38 @@ static __device__ __forceinline__ double coulomb_inv_r(double x) {
   return fma(0.5 * y, e, y);
 }
 
+// RN(x) 2^e for a 128-bit integer x, correctly rounded (ties to even) when the result is normal.
+static __device__ __noinline__ double scale_slow(double m, int e) { return ldexp(m, e); }
+
+static __device__ __forceinline__ double i128_to_double(unsigned long long hi, unsigned long long lo, int e) {
+  const unsigned long long sign = hi & 0x8000000000000000ULL;
+  if (sign) {
+    lo = ~lo + 1;
+    hi = ~hi + (lo == 0);
+  }
+  if ((hi | lo) == 0) return 0.0;
+  if (hi == 0) {
+    hi = lo;
+    lo = 0;
+    e -= 64;
+  }
+  const int lz = __clzll(hi);
+  if (lz) {
+    hi = (hi << lz) | (lo >> (64 - lz));
+    lo <<= lz;
+  }
+  // value = hi.lo 2^(e + 64 - lz), hi in [2^63, 2^64): 53 bits kept, 11 (and lo) rounded
+  unsigned long long m = hi >> 11;
+  const unsigned rem = (unsigned)hi & 0x7ffu;
+  if (rem > 0x400u || (rem == 0x400u && (lo != 0 || (m & 1)))) m++;
+  const int be = e + 64 - lz + 11 + 52 + 1023;  // biased exponent of m = 1.xxx 2^52
+  if (be < 1 || be > 2045) {
+    const double s = scale_slow((double)m, e + 64 - lz + 11);
+    return sign ? -s : s;
+  }
+  return __longlong_as_double((long long)(sign | (((unsigned long long)(be - 1) << 52) + m)));
+}
+
 // The largest |r| of a walker and spin as its high FP64 word (NaN above Inf above all others),
 // kept in a register while a warp's determinants are of one spin.
 static __device__ __forceinline__ void ratio_max(const DevScratch& S, int64_t w, int sp, int& sp_max, uint32_t& top,

@@ -5,6 +5,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <initializer_list>
 #include <new>
 #include <string>
 #include <vector>
@@ -115,6 +116,9 @@ constexpr int kQueueWords = 6;
 
 // residue planes of C above this size, and workspace of the residue products per context
 constexpr size_t kDenseMaxBytes = (size_t)8 << 30, kDenseWorkBytes = (size_t)4 << 30;
+
+// workspace of the orbitals' AO digits
+constexpr size_t kDigitBytes = (size_t)5 << 28;
 
 // weights of the first, each middle and the last walker chunk of the pipelined evaluation. The
 // first chunk's orbitals and tables run before any contraction, and the last chunk's epilogue
@@ -257,46 +261,71 @@ void free_problem(mdet_ctx* c) {
   c->P = DevProblem{};
 }
 
-// Work items of the contraction for item size `chunk`: consecutive whole segments (rows of the
-// row-major copy of C, columns of the column-major one) packed while they hold at most `chunk`
-// nonzeros, and segments longer than `chunk` cut into pieces of at most `chunk` nonzeros, so
-// that every item costs about the same. A whole segment belongs to one item, whose warp stores
-// its (segment, walker) sums; the pieces of a cut segment add theirs atomically (flagged by a
-// negative end), into entries the ratio kernel has cleared (`split`).
-mdet_status ensure_items(mdet_ctx* c, int chunk) {
-  for (const auto& s : c->item_sets)
-    if (s.chunk == chunk) return MDET_OK;
-  mdet_ctx::ItemSet set{};
-  set.chunk = chunk;
+// Work items of the contraction for the given item sizes: consecutive whole segments (rows of the
+// row-major copy of C, columns of the column-major one) packed while they hold at most that many
+// nonzeros, and longer segments cut into pieces of at most that many, so that every item costs about
+// the same. A whole segment belongs to one item, whose warp stores its (segment, walker) sums; the
+// pieces of a cut segment add theirs atomically (flagged by a negative end), into entries the ratio
+// kernel has cleared (`split`). One allocation for all the sets that are missing.
+mdet_status ensure_items(mdet_ctx* c, std::initializer_list<int> chunks) {
+  std::vector<int2> it;
   std::vector<uint8_t> split;
-  for (int o = 0; o < 2; o++) {
-    const std::vector<int32_t>& ptr = o ? c->csc_ptr : c->csr_ptr;
-    const int64_t nseg = (int64_t)ptr.size() - 1;
-    std::vector<int2> it;
-    int32_t b = nseg > 0 ? ptr[0] : 0;  // start of the item being packed
-    for (int64_t q = 0; q < nseg; q++) {
-      const int32_t s0 = ptr[q], s1 = ptr[q + 1];
-      if (s1 - s0 > chunk) {  // a long segment: close the open item, then cut this one
-        if (s0 > b) it.push_back(make_int2(b, s0));
-        for (int32_t p = s0; p < s1; p += chunk) it.push_back(make_int2(p, (int32_t)(std::min(p + chunk, s1) | 0x80000000u)));
-        split.push_back(1);
-        b = s1;
-        continue;
+  struct Range {
+    int chunk;
+    size_t at[2], n[2], split;
+  };
+  std::vector<Range> made;
+  for (int chunk : chunks) {
+    bool have = false;
+    for (const auto& s : c->item_sets) have = have || s.chunk == chunk;
+    for (const auto& r : made) have = have || r.chunk == chunk;
+    if (have) continue;
+    Range rg{};
+    rg.chunk = chunk;
+    rg.split = split.size();
+    for (int o = 0; o < 2; o++) {
+      const std::vector<int32_t>& ptr = o ? c->csc_ptr : c->csr_ptr;
+      const int64_t nseg = (int64_t)ptr.size() - 1;
+      rg.at[o] = it.size();
+      int32_t b = nseg > 0 ? ptr[0] : 0;  // start of the item being packed
+      for (int64_t q = 0; q < nseg; q++) {
+        const int32_t s0 = ptr[q], s1 = ptr[q + 1];
+        if (s1 - s0 > chunk) {  // a long segment: close the open item, then cut this one
+          if (s0 > b) it.push_back(make_int2(b, s0));
+          for (int32_t p = s0; p < s1; p += chunk)
+            it.push_back(make_int2(p, (int32_t)(std::min(p + chunk, s1) | 0x80000000u)));
+          split.push_back(1);
+          b = s1;
+          continue;
+        }
+        split.push_back(0);
+        if (s0 > b && s1 - b > chunk) {
+          it.push_back(make_int2(b, s0));
+          b = s0;
+        }
       }
-      split.push_back(0);
-      if (s0 > b && s1 - b > chunk) {
-        it.push_back(make_int2(b, s0));
-        b = s0;
-      }
+      if (nseg > 0 && ptr[nseg] > b) it.push_back(make_int2(b, ptr[nseg]));
+      rg.n[o] = it.size() - rg.at[o];
     }
-    if (nseg > 0 && ptr[nseg] > b) it.push_back(make_int2(b, ptr[nseg]));
-    mdet_status s = upload(c, it, &set.d[o]);
-    if (s != MDET_OK) return s;
-    set.n[o] = (int)it.size();
+    made.push_back(rg);
   }
-  mdet_status s = upload(c, split, &set.split);
+  if (made.empty()) return MDET_OK;
+  const size_t words = it.size();
+  it.resize(words + (split.size() + sizeof(int2) - 1) / sizeof(int2));
+  std::memcpy(it.data() + words, split.data(), split.size());
+  const int2* d = nullptr;
+  mdet_status s = upload(c, it, &d);
   if (s != MDET_OK) return s;
-  c->item_sets.push_back(set);
+  for (const auto& r : made) {
+    mdet_ctx::ItemSet set{};
+    set.chunk = r.chunk;
+    for (int o = 0; o < 2; o++) {
+      set.d[o] = d + r.at[o];
+      set.n[o] = (int)r.n[o];
+    }
+    set.split = reinterpret_cast<const uint8_t*>(d + words) + r.split;
+    c->item_sets.push_back(set);
+  }
   return MDET_OK;
 }
 
@@ -323,12 +352,12 @@ void pick_items(const mdet_ctx* c, DevProblem& P, int64_t n_walk) {
   int chunk = c->spmm_chunk;
   for (int small : kSmallChunks)
     if (small < chunk && P.nnz / chunk * groups < kItemWarps) chunk = small;
-  use_items(c, P, chunk);
+  use_items(c, P, chunk);  // (sets that were not built leave the tuned one)
 }
 
 void free_arrays(DevScratch& S) {
   void* ptrs[] = {S.phi, S.Ainv, S.ld0, S.sg0, S.g, S.kap, S.est, S.T, S.Tdf, S.r, S.rdf, S.vu, S.psit, S.psia, S.wstat,
-                  S.xmax, S.dx, S.dy, S.dyabs, S.derr,
+                  S.xmax, S.dx, S.dy, S.dyabs, S.derr, S.xd, S.xer,
                   S.fb, S.fb_list, S.fb_acc, S.queue, S.R_stage, S.out_stage};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -405,6 +434,49 @@ mdet_status spin_tables(mdet_ctx* c, int sp, int n_int, const std::vector<uint64
     c->degree[sp][t] = k;
   }
   return MDET_OK;
+}
+
+// The digits of B as operand tiles of the tcgen05 orbital product: per chunk of 32 MOs and slice of
+// 16 AOs, [digit][AO / 8 mod 2][MO][AO mod 8]. Mixed precision: the 7 digits `dig` of B_dig; FP64: 8
+// digits of B_am 2^(62 - fexp_m) (balanced base 256, the bytes of that integer + 0x80...80 less 128).
+// *out is null when some order's sum could exceed 2^24, where the product's FP32 accumulators would
+// no longer be exact (the AO digits are at most 256, the first of 7, else 128).
+mdet_status upload_digit_tiles(mdet_ctx* c, const std::vector<double>& B, const std::vector<uint16_t>& dig,
+                               const std::vector<int>& fexp, const uint16_t** out) {
+  const int D = c->precision == MDET_PRECISION_MIXED ? 7 : 8;
+  const int K = c->n_ao, M = c->n_mo, Kp = (K + 15) / 16 * 16, Np = (M + 15) / 16 * 16, Mp = (M + 7) / 8 * 8;
+  std::vector<uint16_t> tiles((size_t)D * Np * Kp, 0);
+  *out = nullptr;
+  for (int m = 0; m < M; m++) {
+    if (fexp[m] == mo_bad_exponent()) continue;
+    const int m0 = m / 32 * 32, cw = std::min(32, Np - m0);
+    double sum[8] = {}, order[8] = {};
+    for (int mu = 0; mu < K; mu++) {
+      const uint64_t v = D == 8 ? (uint64_t)std::llrint(std::ldexp(B[(size_t)mu * M + m], 62 - fexp[m])) +
+                                      0x8080808080808080ULL
+                                : 0;
+      uint16_t* t = &tiles[(size_t)D * Kp * m0 + (size_t)(mu / 16) * D * 16 * cw + (size_t)((mu % 16) / 8) * cw * 8 +
+                           (size_t)(m - m0) * 8 + mu % 8];
+      for (int j = 0; j < D; j++, t += 16 * cw) {
+        float d;
+        uint32_t bits;
+        if (D == 8) {
+          d = (float)((int)((v >> (8 * (7 - j))) & 0xff) - 128);
+          std::memcpy(&bits, &d, 4);
+        } else {
+          bits = (uint32_t)dig[((size_t)j * Mp + m) * Kp + mu] << 16;
+          std::memcpy(&d, &bits, 4);
+        }
+        *t = (uint16_t)(bits >> 16);
+        sum[j] += std::fabs(d);
+      }
+    }
+    for (int i = 0; i < D; i++)
+      for (int j = 0; i + j < D; j++) order[i + j] += (D == 7 && i == 0 ? 256.0 : 128.0) * sum[j];
+    for (double o : order)
+      if (o > 16777216.0) return MDET_OK;
+  }
+  return upload(c, tiles, out);
 }
 
 // Whether an expansion's contraction is taken as residue products on the tensor cores: a filled-in
@@ -517,10 +589,12 @@ mdet_status upload_problem(mdet_ctx* c) {
     for (int m = 0; m < c->n_mo; m++) {
       double mx = 0.0;
       for (int mu = 0; mu < c->n_ao; mu++) mx = std::max(mx, std::fabs(B[(size_t)mu * c->n_mo + m]));
-      const int f = mx > 0.0 ? std::ilogb(mx) + 1 : 0;
-      fexp[m] = f;
+      bool finite = true;
+      for (int mu = 0; mu < c->n_ao; mu++) finite = finite && std::isfinite(B[(size_t)mu * c->n_mo + m]);
+      const int f = finite && mx > 0.0 ? std::ilogb(mx) + 1 : 0;
+      fexp[m] = finite ? f : mo_bad_exponent();
       for (int mu = 0; mu < c->n_ao; mu++) {
-        double v = std::ldexp(B[(size_t)mu * c->n_mo + m], -f);
+        double v = finite ? std::ldexp(B[(size_t)mu * c->n_mo + m], -f) : std::nan("");
         for (int j = 0; j < kDigits; j++) {
           v *= 256.0;
           const double d = std::nearbyint(v);
@@ -534,6 +608,8 @@ mdet_status upload_problem(mdet_ctx* c) {
     }
     UP(dig, P.B_dig);
     UP(fexp, P.B_exp);
+    P.B_tiles = P.B_tiles8 = nullptr;
+    if ((s = upload_digit_tiles(c, B, dig, fexp, P.phi_df ? &P.B_tiles : &P.B_tiles8)) != MDET_OK) return s;
   }
   auto split = [](const std::vector<double>& v) {
     std::vector<float2> o(v.size());
@@ -573,11 +649,12 @@ mdet_status upload_problem(mdet_ctx* c) {
     UP(b, P.csc_val_df);
   }
   // contraction work items for the tuned size and for the short items of escalated re-evaluations
-  if ((s = ensure_items(c, c->spmm_chunk)) != MDET_OK || (s = ensure_items(c, kEscalationChunk)) != MDET_OK) return s;
-  for (int chunk : kSmallChunks)
-    if ((s = ensure_items(c, chunk)) != MDET_OK) return s;
-  use_items(c, P, c->spmm_chunk);
+  // (and, where the sparse sums are what runs, for small contractions)
   if ((s = build_dense(c)) != MDET_OK) return s;
+  s = c->dense_ok ? ensure_items(c, {c->spmm_chunk, kEscalationChunk})
+                  : ensure_items(c, {c->spmm_chunk, kEscalationChunk, 256, 64, 32, 16});
+  if (s != MDET_OK) return s;
+  use_items(c, P, c->spmm_chunk);
   // the sequential chain of Sec. 2.2: distinct determinants in the order of the key of Eq. 3,
   // each with the substitutions from its predecessor (holes and particles ascending, paired in order)
   for (int sp = 0; sp < 2; sp++) {
@@ -658,6 +735,18 @@ mdet_status alloc_eval_arrays(mdet_ctx* c, DevScratch& S, int64_t W, bool df_tab
   if ((s = dalloc(c, &S.psit, (size_t)wp))) return s;
   if ((s = dalloc(c, &S.psia, (size_t)wp))) return s;
   if ((s = dalloc(c, &S.wstat, (size_t)W))) return s;
+  if (mo_digits_supported(P, df_tables)) {  // digits of the AO values, for blocks of walkers
+    const int64_t row_bytes = (int64_t)mo_digits_row_bytes(P, df_tables), per = 5 * N * row_bytes;
+    S.xd_walk = std::min(W, std::max<int64_t>(1, (int64_t)kDigitBytes / per));
+    const int64_t rows = (S.xd_walk * 5 * N + 127) / 128 * 128;
+    if (cudaMalloc((void**)&S.xd, rows * row_bytes) != cudaSuccess ||
+        cudaMalloc((void**)&S.xer, sizeof(int) * rows) != cudaSuccess) {  // no room: the CUDA-core products
+      cudaGetLastError();
+      if (S.xd) cudaFree(S.xd);
+      S.xd = nullptr;
+      S.xer = nullptr;
+    }
+  }
   if (c->dense_ok) {  // the workspace of the residue products, for blocks of walkers that it holds
     size_t x, y, ya;
     dense_bytes(c->dense, &x, &y, &ya);
@@ -762,10 +851,12 @@ mdet_status refine(mdet_ctx* c, bool table, int64_t n_walk, const double* R, dou
   CUDA_TRY(c, launch_fb_list(P, S.wstat, status, n_walk, S.fb_list, st));
   CUDA_TRY(c, cudaMemsetAsync(E.wstat, 0, sizeof(uint32_t) * cap, st));
   CUDA_TRY(c, launch_esc_gather(S.fb_list, cap, 3 * N, R, c->e_R, c->e_live, S.psia, E.psia, st));
-  // one electron per FP64 orbital block: the grid of a few hundred walkers then spreads evenly
-  // over the SMs (28.51 ms per step at 8,192 walkers, 750k products, against 28.60 with 6)
+  // The orbitals by AO values and FP64 dot products as two kernels before the ratio table, else, on
+  // the small expansions that go straight to full LU, by the one CUDA-core kernel with one electron
+  // per block, whose few live walkers spread evenly over the SMs.
   DevProblem Pe = P;
   Pe.mo_ec = 1;
+  if (!table) Pe.mo_impl = 1;
   if (!use_items(c, Pe, kEscalationChunk)) return fail(c, MDET_E_STATE, "internal: escalation items missing");
   CUDA_TRY(c, launch_mo_f64(Pe, E, cap, c->e_R, st));
   const EscOut& o = c->eo;
@@ -791,6 +882,11 @@ mdet_status refine(mdet_ctx* c, bool table, int64_t n_walk, const double* R, dou
   CUDA_TRY(c, launch_esc_scatter(S.fb_list, cap, N, o, MDET_WS_ESCALATED, log_abs_psi, sign, grad, lap, e_local,
                                  status, S.wstat, st));
   return MDET_OK;
+}
+
+// Kernels of the orbitals of one evaluation (or chunk) on scratch S.
+int mo_kernels(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df) {
+  return use_mo_digits(P, S, n_walk, df) ? 2 * (int)((n_walk + S.xd_walk - 1) / S.xd_walk) : 1;
 }
 
 // Whether an evaluation's contraction runs as residue products: its expansion has them, its
@@ -1259,7 +1355,7 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
     *n = std::min<int64_t>(t1 * kWalkerPad, n_walk) - *off;
   };
   const bool dense = use_dense(c) && c->S.xmax;
-  int contract_kernels = 0;
+  int contract_kernels = 0, orbital_kernels = 0;
   // stage i (MDET_STAGE_*) of chunk k on stream ks, bracketed by its two profiling events
   auto stage = [&](int k, int i, cudaStream_t ks, int persistent) -> mdet_status {
     int64_t off, n;
@@ -1275,6 +1371,7 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
     if (mark) CUDA_TRY(c, cudaEventRecord(c->ev[k][2 * i], ks));
     switch (i) {
       case MDET_STAGE_ORBITALS:
+        orbital_kernels += mo_kernels(P, S, n, mixed);
         CUDA_TRY(c, mixed ? launch_mo_mixed(P, S, n, Rk, ks) : launch_mo_f64(P, S, n, Rk, ks));
         break;
       case MDET_STAGE_REFERENCE: CUDA_TRY(c, launch_ref_tables(P, S, n, mixed, ks)); break;
@@ -1288,7 +1385,7 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
           CUDA_TRY(c, launch_contract_dense(P, S, n, ks, prof_stamp ? q + 2 : nullptr, &contract_kernels));
           break;
         }
-        contract_kernels += 2;
+        contract_kernels += c->contract_impl == 1 && mixed ? 2 : 1;
         CUDA_TRY(c, launch_contract_f64(P, S, n, ks, q, persistent, prof_stamp ? q + 2 : nullptr));
         break;
       }
@@ -1341,17 +1438,18 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
   c->prof_chunks = nch;
   // stability fallback over the whole batch, after every chunk has finished: mixed precision
   // escalates to FP64 first, FP64 goes to full LU directly
-  // kernels: 4 per chunk (orbitals, reference, ratios, epilogue) and its contraction's (2 sparse
-  // sums, or 3 per walker block of the residue products); the full-LU
+  // kernels: 3 per chunk (reference, ratios, epilogue), its orbitals' (2 per walker block of the digit
+  // products, else 1) and its contraction's (1 for the sparse sums, 2 in double-float, 3 per walker
+  // block of the residue products); the full-LU
   // fallback 5 (list, dets, scale, rows, out); the mixed refinement adds its list, gather,
   // FP64 orbitals and scatter, and either the mark or the 5 FP64 table kernels
-  c->last_kernels = 4 * nch + contract_kernels;
+  c->last_kernels = 3 * nch + orbital_kernels + contract_kernels;
   if (prof_all) CUDA_TRY(c, cudaEventRecord(c->ev_refine[0], st));
   if (mixed && c->E.fb && P.fallback_tol > 0.0) {
     const bool table = escalation_on(c);
     mdet_status es = refine(c, table, n_walk, R, log_abs_psi, sign, grad, lap, e_local, status, st);
     if (es != MDET_OK) return es;
-    c->last_kernels += 4 + 5 + (table ? (c->E.xmax ? 6 : 5) : 1);
+    c->last_kernels += 3 + 5 + (table ? mo_kernels(P, c->E, P.fallback_cap, false) + (c->E.xmax ? 6 : 4) : 1 + 1);
   } else {
     CUDA_TRY(c, launch_fallback(P, c->S, n_walk, R, log_abs_psi, sign, grad, lap, e_local, status, st));
     if (P.fallback_tol > 0.0 && c->S.fb && P.n_up <= MDET_FALLBACK_MAX_SPIN) c->last_kernels += 5;
@@ -1579,7 +1677,7 @@ mdet_status mdet_set_tuning(mdet_ctx* c, const mdet_tuning* t) {
   c->P.spmm_blocks = t->spmm_blocks;
   if (c->has_ci && c->device >= 0) {
     CUDA_TRY(c, cudaSetDevice(c->device));
-    mdet_status s = ensure_items(c, t->spmm_chunk);
+    mdet_status s = ensure_items(c, {t->spmm_chunk});
     if (s != MDET_OK) return s;
     use_items(c, c->P, t->spmm_chunk);
   }

@@ -103,6 +103,8 @@ struct DevProblem {
                           // FP64 re-evaluation scratch of a mixed context always holds FP64
   const uint16_t* B_dig;  // [7][tc_mp][tc_kp] BF16 digits of the MO coefficients (column-scaled)
   const int* B_exp;       // [n_mo] column exponents of B_dig
+  // 7 and 8 digits of B in the operand tiles of mdet_mo_digits.cu (null where the order sums are not exact)
+  const uint16_t *B_tiles, *B_tiles8;
   int tc_kp, tc_mp, tc_sx;  // K padded to 16, M padded to 8, shared row stride of the AO digits
   double fallback_tol;    // estimated relative error above which a walker is re-evaluated by full LU (<= 0: off)
   int fallback_cap;       // walkers re-evaluated per evaluation at most
@@ -161,6 +163,10 @@ struct DevScratch {
   float* dyabs = nullptr;
   int* derr = nullptr;
   int64_t dblk = 0;
+  // digits and row exponents of the AO values of xd_walk walkers (null: no room for them)
+  uint8_t* xd = nullptr;
+  int* xer = nullptr;
+  int64_t xd_walk = 0;
   uint32_t* wstat = nullptr;  // [W] status bits
   double* fb = nullptr;       // fallback: [cap][n_det_up + n_det_dn][2 + 4 max(n_up, n_dn)], then [cap][ndt] values
   int* fb_list = nullptr;     // fallback: [1 + cap] count, then walker indices
@@ -201,12 +207,17 @@ struct GemmEpilogue {
 cudaError_t launch_gemm_bf16(const GemmOperand& A, const GemmOperand& B, int64_t k_per_cta, const GemmEpilogue& E,
                              cudaStream_t st);
 
-// The mixed orbitals on the tcgen05 tensor cores (mdet_mo_umma.cu): supported for
-// at most 112 AOs and 128 MOs; launch_mo_mixed takes it when mo_impl is 2.
-bool mo_umma_supported(const DevProblem& P);
-size_t mo_umma_smem_bytes(const DevProblem& P);
-cudaError_t launch_mo_umma(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R, int n_sm,
-                           cudaStream_t st);
+// The orbitals by digit products on the tcgen05 tensor cores (mdet_mo_digits.cu), FP64 or (df)
+// double-float pairs; two kernels per block of S.xd_walk walkers. row_bytes: digits of one row of
+// the product (5 n_elec rows per walker); bad_exponent: B_exp of an MO whose coefficients are not
+// all finite.
+bool mo_digits_supported(const DevProblem& P, bool df);
+size_t mo_digits_row_bytes(const DevProblem& P, bool df);
+int mo_bad_exponent();
+cudaError_t launch_mo_digits(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R, bool df,
+                             cudaStream_t st);
+// Whether an evaluation of n_walk walkers takes them (mo_impl 2, a workspace, and enough work).
+bool use_mo_digits(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df);
 cudaError_t launch_ref_tables(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool mixed,
                               cudaStream_t st);
 cudaError_t launch_ratios_f64(const DevProblem& P, const DevScratch& S, int64_t n_walk,

@@ -446,11 +446,88 @@ static __device__ __forceinline__ unsigned long long global_timer_ns() {
   return t;
 }
 
+struct SpmmOrder {
+  const int* seg;
+  const int* gidx;
+  const double* val;
+  const int2* items;
+  int n_items, seg_off;
+  const double* x;
+};
+
+// One work item of order o (0: v with the sums of Psi~, 1: u) for walkers wb ..
+template <bool RDOT, bool ABS, int WPL>
+static __device__ __forceinline__ void spmm_item(const SpmmOrder& A, int it, int64_t wb, int64_t wp,
+                                                 double* __restrict__ y, int64_t ldy, const double* __restrict__ rdot,
+                                                 double* __restrict__ psit, float* __restrict__ psia) {
+  const int2 r0 = __ldg(A.items + it);
+  const int2 r = make_int2(r0.x, r0.y & 0x7fffffff);
+  const bool piece = r0.y < 0;  // one piece of a longer segment: its sums are added, not stored
+  double a[WPL];
+  float aa[WPL];  // ABS: sum |c| |x| of the segment
+#pragma unroll
+  for (int j = 0; j < WPL; j++) {
+    a[j] = 0.0;
+    aa[j] = 0.0f;
+  }
+  int cur = __ldg(A.seg + r.x);
+  auto flush = [&](int sg) {
+    double* yr = y + wb * ldy + A.seg_off + sg;
+    if (piece) {
+#pragma unroll
+      for (int j = 0; j < WPL; j++) atomicAdd(yr + j * ldy, a[j]);
+    } else {
+#pragma unroll
+      for (int j = 0; j < WPL; j++) yr[j * ldy] = a[j];
+    }
+    if (RDOT) {
+      const double2* rp = reinterpret_cast<const double2*>(rdot + (size_t)sg * wp + wb);
+#pragma unroll
+      for (int h = 0; h < WPL / 2; h++) {
+        const double2 t = __ldg(rp + h);
+        atomicAdd(psit + wb + 2 * h, t.x * a[2 * h]);
+        atomicAdd(psit + wb + 2 * h + 1, t.y * a[2 * h + 1]);
+        if (ABS) {
+          atomicAdd(psia + wb + 2 * h, abs_f32_of(t.x) * aa[2 * h]);
+          atomicAdd(psia + wb + 2 * h + 1, abs_f32_of(t.y) * aa[2 * h + 1]);
+        }
+      }
+    }
+  };
+  for (int k = r.x; k < r.y; k++) {
+    const int sg = __ldg(A.seg + k);
+    if (sg != cur) {
+      flush(cur);
+      cur = sg;
+#pragma unroll
+      for (int j = 0; j < WPL; j++) {
+        a[j] = 0.0;
+        aa[j] = 0.0f;
+      }
+    }
+    const double c = __ldg(A.val + k);
+    const double2* xp = reinterpret_cast<const double2*>(A.x + (size_t)__ldg(A.gidx + k) * wp + wb);
+    double xv[WPL];
+#pragma unroll
+    for (int h = 0; h < WPL / 2; h++) {
+      const double2 t = __ldg(xp + h);
+      xv[2 * h] = t.x;
+      xv[2 * h + 1] = t.y;
+    }
+#pragma unroll
+    for (int j = 0; j < WPL; j++) a[j] = fma(c, xv[j], a[j]);
+    if (ABS) {
+      const float ca = abs_f32_of(c);
+#pragma unroll
+      for (int j = 0; j < WPL; j++) aa[j] = fmaf(ca, abs_f32_of(xv[j]), aa[j]);
+    }
+  }
+  flush(cur);
+}
+
 template <bool QUEUE, bool ABS, int WPL>
-__global__ void __launch_bounds__(128) k_spmm_seg(const int* __restrict__ seg, const int* __restrict__ gidx,
-                                                  const double* __restrict__ val, const int2* __restrict__ items,
-                                                  int n_items, int64_t n_groups, const double* __restrict__ x,
-                                                  int64_t wp, double* __restrict__ y, int64_t ldy, int seg_off,
+__global__ void __launch_bounds__(128) k_spmm_seg(const __grid_constant__ SpmmOrder v, const __grid_constant__ SpmmOrder u,
+                                                  int64_t n_groups, int64_t wp, double* __restrict__ y, int64_t ldy,
                                                   const double* __restrict__ rdot, double* __restrict__ psit,
                                                   float* __restrict__ psia, unsigned long long* __restrict__ queue,
                                                   const int* __restrict__ live, unsigned long long* __restrict__ stamp) {
@@ -458,7 +535,7 @@ __global__ void __launch_bounds__(128) k_spmm_seg(const int* __restrict__ seg, c
   const int lane = threadIdx.x & 31;
   if (stamp && threadIdx.x == 0) atomicMax(stamp, ~global_timer_ns());
   const int64_t ng = live ? min(n_groups, (int64_t)(*live + G - 1) / G) : n_groups;
-  const int64_t n_work = (int64_t)n_items * ng;
+  const int64_t n_v = (int64_t)v.n_items * ng, n_work = n_v + (int64_t)u.n_items * ng;
   auto next_item = [&]() -> int64_t {
     unsigned long long t = 0;
     if (lane == 0) t = atomicAdd(queue, 1ULL);
@@ -466,72 +543,14 @@ __global__ void __launch_bounds__(128) k_spmm_seg(const int* __restrict__ seg, c
   };
   const int64_t first = QUEUE ? next_item() : (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   for (int64_t q = first; q < n_work; q = QUEUE ? next_item() : n_work) {
-    const int it = (int)(q % n_items);
-    const int64_t grp = q / n_items;
-    const int2 r0 = __ldg(items + it);
-    const int2 r = make_int2(r0.x, r0.y & 0x7fffffff);
-    const bool piece = r0.y < 0;  // one piece of a longer segment: its sums are added, not stored
-    const int64_t wb = grp * G + lane * WPL;
-    double a[WPL];
-    float aa[WPL];  // ABS: sum |c| |x| of the segment
-#pragma unroll
-    for (int j = 0; j < WPL; j++) {
-      a[j] = 0.0;
-      aa[j] = 0.0f;
+    if (q < n_v) {
+      const int64_t grp = q / v.n_items;
+      spmm_item<true, ABS, WPL>(v, (int)(q - grp * v.n_items), grp * G + lane * WPL, wp, y, ldy, rdot, psit, psia);
+    } else {
+      const int64_t p = q - n_v, grp = p / u.n_items;
+      spmm_item<false, false, WPL>(u, (int)(p - grp * u.n_items), grp * G + lane * WPL, wp, y, ldy, nullptr, nullptr,
+                                   nullptr);
     }
-    int cur = __ldg(seg + r.x);
-    auto flush = [&](int sg) {
-      double* yr = y + wb * ldy + seg_off + sg;
-      if (piece) {
-#pragma unroll
-        for (int j = 0; j < WPL; j++) atomicAdd(yr + j * ldy, a[j]);
-      } else {
-#pragma unroll
-        for (int j = 0; j < WPL; j++) yr[j * ldy] = a[j];
-      }
-      if (rdot) {
-        const double2* rp = reinterpret_cast<const double2*>(rdot + (size_t)sg * wp + wb);
-#pragma unroll
-        for (int h = 0; h < WPL / 2; h++) {
-          const double2 t = __ldg(rp + h);
-          atomicAdd(psit + wb + 2 * h, t.x * a[2 * h]);
-          atomicAdd(psit + wb + 2 * h + 1, t.y * a[2 * h + 1]);
-          if (ABS) {
-            atomicAdd(psia + wb + 2 * h, abs_f32_of(t.x) * aa[2 * h]);
-            atomicAdd(psia + wb + 2 * h + 1, abs_f32_of(t.y) * aa[2 * h + 1]);
-          }
-        }
-      }
-    };
-    for (int k = r.x; k < r.y; k++) {
-      const int sg = __ldg(seg + k);
-      if (sg != cur) {
-        flush(cur);
-        cur = sg;
-#pragma unroll
-        for (int j = 0; j < WPL; j++) {
-          a[j] = 0.0;
-          aa[j] = 0.0f;
-        }
-      }
-      const double c = __ldg(val + k);
-      const double2* xp = reinterpret_cast<const double2*>(x + (size_t)__ldg(gidx + k) * wp + wb);
-      double xv[WPL];
-#pragma unroll
-      for (int h = 0; h < WPL / 2; h++) {
-        const double2 t = __ldg(xp + h);
-        xv[2 * h] = t.x;
-        xv[2 * h + 1] = t.y;
-      }
-#pragma unroll
-      for (int j = 0; j < WPL; j++) a[j] = fma(c, xv[j], a[j]);
-      if (ABS) {
-        const float ca = abs_f32_of(c);
-#pragma unroll
-        for (int j = 0; j < WPL; j++) aa[j] = fmaf(ca, abs_f32_of(xv[j]), aa[j]);
-      }
-    }
-    flush(cur);
   }
   if (stamp && lane == 0) atomicMax(stamp + 1, global_timer_ns());
 }
@@ -1075,6 +1094,7 @@ static cudaError_t launch_mo_f64_ec(const DevProblem& P, const DevScratch& S, in
 
 cudaError_t launch_mo_f64(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R,
                           cudaStream_t st) {
+  if (use_mo_digits(P, S, n_walk, false)) return launch_mo_digits(P, S, n_walk, R, false, st);
   switch (P.mo_ec) {
     case 1: return launch_mo_f64_ec<1>(P, S, n_walk, R, st);
     case 2: return launch_mo_f64_ec<2>(P, S, n_walk, R, st);
@@ -1120,12 +1140,12 @@ cudaError_t launch_contract_f64(const DevProblem& P, const DevScratch& S, int64_
   // an escalated re-evaluation (few walkers, live count on the device) uses 4 walkers per lane
   const bool narrow = narrow_contraction(P, S);
   const int64_t n_groups = narrow ? (n_walk + 127) / 128 : (n_walk + 255) / 256;
-  const int64_t work_max = (int64_t)std::max(P.n_items[0], P.n_items[1]) * n_groups;
+  const int64_t work_max = ((int64_t)P.n_items[0] + P.n_items[1]) * n_groups;
   // one work item per warp (full occupancy hides the L2 latency of the gathers), or a
-  // persistent grid whose warps draw items from a queue (two counters, one per launch)
+  // persistent grid whose warps draw items from a queue
   const int cap = P.spmm_blocks > 0 ? P.spmm_blocks : persistent_blocks;
   const bool q = queue && cap > 0 && cap < (work_max + 3) / 4;
-  // the two counters, and the four stamp words (with one memset when they follow the counters)
+  // the counter (of two words), and the four stamp words (with one memset when they follow it)
   const bool adjacent = q && stamp == queue + 2;
   if (q) {
     cudaError_t e = cudaMemsetAsync(queue, 0, (adjacent ? 6 : 2) * sizeof(unsigned long long), st);
@@ -1135,10 +1155,6 @@ cudaError_t launch_contract_f64(const DevProblem& P, const DevScratch& S, int64_
     cudaError_t e = cudaMemsetAsync(stamp, 0, 4 * sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
   }
-  auto grid = [&](int o) -> unsigned {
-    const int64_t full = ((int64_t)P.n_items[o] * n_groups + 3) / 4;
-    return (unsigned)std::max<int64_t>(1, q ? std::min<int64_t>(full, cap) : full);
-  };
   const int64_t ndt = (int64_t)P.n_det_sp[0] + P.n_det_sp[1];
   const double* r_up = S.r;
   const double* r_dn = S.r + (size_t)P.n_det_sp[0] * S.wp;
@@ -1158,17 +1174,16 @@ cudaError_t launch_contract_f64(const DevProblem& P, const DevScratch& S, int64_
     return cudaGetLastError();
   }
   // v = C r_dn (rows = up determinants) with Psi~ = r_up . v and its magnitude sum (an escalated
-  // re-evaluation reuses the magnitude sum of the evaluation that flagged it)
-  auto* kv = narrow ? k_spmm_seg<false, false, 4> : (q ? k_spmm_seg<true, true, 8> : k_spmm_seg<false, true, 8>);
-  kv<<<grid(0), 128, 0, st>>>(P.csr_row, P.csr_col, P.csr_val, P.items[0], P.n_items[0], n_groups, r_dn, S.wp, S.vu,
-                              ndt, 0, r_up, S.psit, narrow ? nullptr : S.psia, queue, S.live, stamp);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // u = C^T r_up (columns = down determinants), in the paper's column-major order
-  auto* ku = narrow ? k_spmm_seg<false, false, 4> : (q ? k_spmm_seg<true, false, 8> : k_spmm_seg<false, false, 8>);
-  ku<<<grid(1), 128, 0, st>>>(P.csc_col, P.csc_row, P.csc_val, P.items[1], P.n_items[1], n_groups, r_up, S.wp, S.vu,
-                              ndt, P.n_det_sp[0], nullptr, nullptr, nullptr, q ? queue + 1 : nullptr, S.live,
-                              stamp ? stamp + 2 : nullptr);
+  // re-evaluation reuses the magnitude sum of the evaluation that flagged it), then u = C^T r_up
+  // (columns = down determinants, the paper's column-major order), in one launch: neither needs
+  // the other, and the items of both fill the chip better than one after the other
+  const SpmmOrder v{P.csr_row, P.csr_col, P.csr_val, P.items[0], P.n_items[0], 0, r_dn};
+  const SpmmOrder u{P.csc_col, P.csc_row, P.csc_val, P.items[1], P.n_items[1], P.n_det_sp[0], r_up};
+  const int64_t full = (work_max + 3) / 4;
+  const unsigned grid = (unsigned)std::max<int64_t>(1, q ? std::min<int64_t>(full, cap) : full);
+  auto* k = narrow ? k_spmm_seg<false, false, 4> : (q ? k_spmm_seg<true, true, 8> : k_spmm_seg<false, true, 8>);
+  k<<<grid, 128, 0, st>>>(v, u, n_groups, S.wp, S.vu, ndt, r_up, S.psit, narrow ? nullptr : S.psia, queue, S.live,
+                          stamp);
   return cudaGetLastError();
 }
 

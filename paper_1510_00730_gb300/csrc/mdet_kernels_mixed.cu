@@ -357,7 +357,7 @@ cudaError_t launch_mo_mixed(const DevProblem& P, const DevScratch& S, int64_t n_
                             cudaStream_t st) {
   // tcgen05 digit products by default; warp-level MMA digits (mo_impl 0) or the compensated
   // CUDA-core product when asked for, or when the problem exceeds what the tcgen05 kernel holds
-  if (P.mo_impl == 2 && mo_umma_supported(P)) return launch_mo_umma(P, S, n_walk, R, P.n_sm, st);
+  if (use_mo_digits(P, S, n_walk, true)) return launch_mo_digits(P, S, n_walk, R, true, st);
   const size_t kSmemMax = 200 * 1024;
   if (P.mo_impl == 0 && P.B_dig && mo_tc_smem_bytes(P, P.mo_ec) <= kSmemMax) {
     switch (P.mo_ec) {

@@ -247,7 +247,6 @@ __global__ void __launch_bounds__(256) k_mod_residues(const __grid_constant__ De
 // further copies or MMAs, and the reconstruction writes NaN.
 constexpr int kStages = 4;
 constexpr int kStageBytes = 3 * kTileBytes;
-constexpr long long kWaitClocks = 8000000000LL;  // about 4 s
 
 struct GemmArgs {
   const uint16_t* X;
@@ -273,44 +272,7 @@ __device__ __forceinline__ uint32_t cta_rank() {
   return r;
 }
 
-__device__ __forceinline__ bool try_wait_bar(uint64_t* bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, "
-      "p;\n}"
-      : "=r"(done)
-      : "r"(umma::smem_u32(bar)), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
-// Waits for the phase, at most kWaitClocks; gives up at once when the CTA has already given up.
-// (The SM's clock, because a read of the global timer takes longer than a pipeline stage.)
-__device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, volatile int* dead) {
-  if (try_wait_bar(bar, parity)) return true;
-  const long long t0 = clock64();
-  for (;;) {
-    if (try_wait_bar(bar, parity)) return true;
-    if (*dead) return false;
-    if (clock64() - t0 > kWaitClocks) {
-      *dead = 1;
-      return false;
-    }
-  }
-}
-
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(umma::smem_u32(bar))
-               : "memory");
-}
-
-__device__ __forceinline__ void expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(umma::smem_u32(bar)), "r"(bytes)
-               : "memory");
-}
-
-// The same into both CTAs of the cluster, at the same offsets, each signalling its own barrier.
+// A bulk copy into both CTAs of the cluster, at the same offsets, each signalling its own barrier.
 __device__ __forceinline__ void bulk_load_both(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::
@@ -422,35 +384,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
         const uint8_t* cp = cs + (size_t)(t.plane + (pass == 1)) * cplane;
         for (int k = 0; k < kb; k++, it++) {
           const int s = it % kStages;
-          if (it >= kStages && !bounded_wait(&empty[s], ((it / kStages) & 1) ^ 1, dead)) break;
-          expect_tx(&full[s], kTileBytes + 2 * b_bytes);
+          if (it >= kStages && !umma::bounded_wait(&empty[s], ((it / kStages) & 1) ^ 1, dead)) break;
+          umma::expect_tx(&full[s], kTileBytes + 2 * b_bytes);
           const uint32_t dst = stage0 + (uint32_t)s * kStageBytes;
-          bulk_load(dst, xp + (size_t)k * kTileBytes, kTileBytes, &full[s]);
+          umma::bulk_load(dst, xp + (size_t)k * kTileBytes, kTileBytes, &full[s]);
           bulk_load_both(dst + kTileBytes + rank * b_bytes, cp + (size_t)k * b_bytes, b_bytes, &full[s]);
         }
       }
     }
-    // after a failed wait: the copies in flight land before the block exits (bounded)
-    if (*dead) {
-      const long long t0 = clock64();
-      for (int s = 0; s < kStages && it > (uint32_t)s; s++) {
-        const uint32_t last = it - 1 - ((it - 1 - (uint32_t)s) % kStages);
-        while (!try_wait_bar(&full[s], (last / kStages) & 1) && clock64() - t0 < kWaitClocks / 4) {
-        }
-      }
-    }
+    if (*dead) umma::drain_copies(full, kStages, it);
   } else if (warp == 1 && lane == 0) {  // MMA issuer
     uint32_t it = 0, n = 0;
     for (int64_t u = first; u < n_units && !*dead; u += step, n++) {
       const Unit t = unit_of(D, a, u, nmt2);
       const int hw = D.hw[t.o], nk = D.kb[1 - t.o] * (t.abs ? 3 : 1), b = n & 1;
       const uint32_t idesc = umma::idesc_bf16(128, 2 * hw);
-      if (n >= 2 && !bounded_wait(&tempty[b], ((n >> 1) & 1) ^ 1, dead)) break;
+      if (n >= 2 && !umma::bounded_wait(&tempty[b], ((n >> 1) & 1) ^ 1, dead)) break;
       umma::fence_after();
       bool ok = true;
       for (int k = 0; k < nk && ok; k++, it++) {
         const int s = it % kStages;
-        ok = bounded_wait(&full[s], (it / kStages) & 1, dead);
+        ok = umma::bounded_wait(&full[s], (it / kStages) & 1, dead);
         if (!ok) break;
         umma::fence_after();
         const uint32_t sa = stage0 + (uint32_t)s * kStageBytes, sb = sa + kTileBytes;
@@ -464,9 +418,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
     }
     if (*dead) {  // after a failed wait: the MMAs in flight finish (bounded) before the release
       umma::commit(&fin);
-      const long long t0 = clock64();
-      while (!try_wait_bar(&fin, 0) && clock64() - t0 < kWaitClocks / 4) {
-      }
+      umma::drain_wait(&fin, 0);
     }
   } else if (warp >= 4) {  // epilogue
     const int qd = warp & 3;
@@ -474,7 +426,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
     for (int64_t u = first; u < n_units && !*dead; u += step, n++) {
       const Unit t = unit_of(D, a, u, nmt2);
       const int b = n & 1, nw = 2 * D.hw[t.o], ldy = D.ldy[t.o];
-      const bool ok = bounded_wait(&tfull[b], (n >> 1) & 1, dead);
+      const bool ok = umma::bounded_wait(&tfull[b], (n >> 1) & 1, dead);
       if (!__all_sync(0xffffffffu, ok)) break;
       umma::fence_after();
       const int64_t wl = (int64_t)t.mt * 256 + (int)rank * 128 + qd * 32 + lane;
@@ -526,38 +478,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
   umma::fence_after();
   if (warp == 2) umma::tmem_dealloc(tb, 512);
   if (a.stamp && tid == 0) atomicMax(a.stamp + 1, now_ns());
-}
-
-// RN(x) 2^e for a 128-bit integer x, correctly rounded (ties to even) when the result is normal.
-__device__ __noinline__ double scale_slow(double m, int e) { return ldexp(m, e); }
-
-__device__ __forceinline__ double i128_to_double(unsigned long long hi, unsigned long long lo, int e) {
-  const unsigned long long sign = hi & 0x8000000000000000ULL;
-  if (sign) {
-    lo = ~lo + 1;
-    hi = ~hi + (lo == 0);
-  }
-  if ((hi | lo) == 0) return 0.0;
-  if (hi == 0) {
-    hi = lo;
-    lo = 0;
-    e -= 64;
-  }
-  const int lz = __clzll(hi);
-  if (lz) {
-    hi = (hi << lz) | (lo >> (64 - lz));
-    lo <<= lz;
-  }
-  // value = hi.lo 2^(e + 64 - lz), hi in [2^63, 2^64): 53 bits kept, 11 (and lo) rounded
-  unsigned long long m = hi >> 11;
-  const unsigned rem = (unsigned)hi & 0x7ffu;
-  if (rem > 0x400u || (rem == 0x400u && (lo != 0 || (m & 1)))) m++;
-  const int be = e + 64 - lz + 11 + 52 + 1023;  // biased exponent of m = 1.xxx 2^52
-  if (be < 1 || be > 2045) {
-    const double s = scale_slow((double)m, e + 64 - lz + 11);
-    return sign ? -s : s;
-  }
-  return __longlong_as_double((long long)(sign | (((unsigned long long)(be - 1) << 52) + m)));
 }
 
 // Reconstruction of v and u from the residue bytes, with Psi~ = r_up . v and its magnitude sum:

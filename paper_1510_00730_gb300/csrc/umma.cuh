@@ -117,5 +117,58 @@ __device__ __forceinline__ void commit(uint64_t* bar) {
                : "memory");
 }
 
+// ---- pipelines of bulk copies and MMAs ----
+// Every wait is bounded, in SM clocks (a read of the global timer takes longer than a pipeline
+// stage); *dead is set by the first wait of the block that runs out and ends the others.
+constexpr long long kWaitClocks = 8000000000LL;  // about 4 s
+
+__device__ __forceinline__ bool try_wait_bar(uint64_t* bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+               : "=r"(done)
+               : "r"(smem_u32(bar)), "r"(parity)
+               : "memory");
+  return done != 0;
+}
+
+__device__ __forceinline__ bool bounded_wait(uint64_t* bar, uint32_t parity, volatile int* dead) {
+  if (try_wait_bar(bar, parity)) return true;
+  const long long t0 = clock64();
+  for (;;) {
+    if (try_wait_bar(bar, parity)) return true;
+    if (*dead) return false;
+    if (clock64() - t0 > kWaitClocks) {
+      *dead = 1;
+      return false;
+    }
+  }
+}
+
+// After a wait has run out: waits (bounded) for a barrier that copies or MMAs in flight arrive on,
+__device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
+  const long long t0 = clock64();
+  while (!try_wait_bar(bar, parity) && clock64() - t0 < kWaitClocks / 4) {
+  }
+}
+
+// and for the copies of the last stages of a ring after `issued` fills.
+__device__ __forceinline__ void drain_copies(uint64_t* full, int stages, uint32_t issued) {
+  for (int s = 0; s < stages && issued > (uint32_t)s; s++) {
+    const uint32_t last = issued - 1 - ((issued - 1 - (uint32_t)s) % stages);
+    drain_wait(&full[s], (last / stages) & 1);
+  }
+}
+
+__device__ __forceinline__ void expect_tx(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+
+// A bulk copy of contiguous global memory (16-byte aligned, as its size) into shared memory.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+
 }  // namespace umma
 }  // namespace mdet

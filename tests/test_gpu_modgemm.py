@@ -2,7 +2,7 @@
 against the sparse FP64 sums and against the oracle.
 
 Expansions dense enough take the residue products; set_tuning(spmm_blocks > 0) selects
-the sparse sums on the same context. The kernels launched tell the two apart (7 and 6 per
+the sparse sums on the same context. The kernels launched tell the two apart (8 and 6 per
 evaluation without the fallback).
 """
 from __future__ import annotations
@@ -56,7 +56,7 @@ def test_residue_products_match_oracle_and_sparse_sums(nu, nd, prec):
     assert rep["ok"], rep
     ctx.set_fallback(0.0)
     table = _eval(ctx, wl.R)
-    assert ctx.last_kernels == 7
+    assert ctx.last_kernels == 8
     ctx.set_tuning(spmm_blocks=SPARSE_GRID)
     sparse = _eval(ctx, wl.R)
     assert ctx.last_kernels == 6
@@ -119,4 +119,4 @@ def test_dense_rows_take_smaller_moduli():
     ctx = pkg.Context.from_workload(wl, device=0)
     rep = compare(_eval(ctx, wl.R), oracle.evaluate(wl), **TOL[pkg.PRECISION_FP64])
     assert rep["ok"], rep
-    assert ctx.last_kernels == 12
+    assert ctx.last_kernels == 13

@@ -1,0 +1,69 @@
+"""The digit products of the orbitals (csrc/mdet_mo_digits.cu) at the edges of their tiles (16-AO
+slices, 32-MO chunks, 16-electron blocks, 128-row tiles), both precisions, against the oracle, and
+against the CUDA-core products (mo_impl 1) for positions that are not finite."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import oracle
+import paper_1510_00730_gb300 as pkg
+from paper_1510_00730_gb300 import synth
+from tests.parity import compare
+
+pytestmark = pytest.mark.gpu
+
+PRECISIONS = [pytest.param(pkg.PRECISION_FP64, id="fp64"), pytest.param(pkg.PRECISION_MIXED, id="mixed")]
+TOL = {pkg.PRECISION_FP64: dict(tol_psi=1e-10, tol_der=1e-8), pkg.PRECISION_MIXED: dict(tol_psi=1e-9, tol_der=1e-6)}
+KEYS = ("log_abs_psi", "sign", "grad", "lap", "e_local", "status")
+
+
+def _eval(ctx, R):
+    out = ctx.evaluate(torch.from_numpy(np.ascontiguousarray(R)).to("cuda:0"))
+    torch.cuda.synchronize()
+    return {k: out[k].cpu().numpy() for k in KEYS}
+
+
+def _workload(shells, n_mo, n_walk, n_up=3, n_dn=2, seed=9):
+    return synth.make_workload("orb", seed, n_up, n_dn, n_up + n_dn, shells, (0.05, 500.0), n_mo, 60, 3, n_walk,
+                               n_unique=(12, 10))
+
+
+# (shells per l) -> AOs: 16, 17, 48, 112, 113, 160; MOs around the 16- and 32-wide chunks
+CASES = [((7, 3, 0), 10, 1), ((8, 3, 0), 17, 5), ((12, 6, 3), 33, 26), ((12, 10, 5, 4), 96, 3), ((13, 10, 5, 4), 97, 31),
+         ((20, 20, 5, 5), 129, 7), ((20, 20, 5, 5), 31, 52)]
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("shells,n_mo,n_walk", CASES)
+def test_tile_edges(shells, n_mo, n_walk, prec):
+    wl = _workload(shells, n_mo, n_walk)
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    if prec == pkg.PRECISION_MIXED:
+        ctx.set_fallback(1e-7)  # below the test tolerance, as the parity tests of this path
+    rep = compare(_eval(ctx, wl.R), oracle.evaluate(wl), **TOL[prec])
+    assert rep["ok"], rep
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+def test_positions_that_are_not_finite(prec):
+    """A NaN or infinite coordinate: that walker's outputs are as with the CUDA-core products, and
+    the other walkers' log|Psi| (summed in a fixed order) is untouched."""
+    wl = _workload((20, 20, 5, 5), 70, 40)
+    R = wl.R.copy()
+    R[4, 1, 2] = np.nan
+    R[21, 3, 0] = np.inf
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    ctx.set_fallback(0.0)
+    clean, got = _eval(ctx, wl.R), _eval(ctx, R)
+    ctx.set_tuning(mo_impl=1)
+    plain = _eval(ctx, R)
+    assert np.array_equal(got["status"], plain["status"])
+    for k in KEYS[:-1]:
+        assert np.array_equal(np.isfinite(got[k]), np.isfinite(plain[k])), k
+    ok = np.ones(40, bool)
+    ok[[4, 21]] = False
+    tol = 22 * 2.0 ** -50 * np.maximum(oracle.evaluate(wl)["kappa"], 1.0)  # the sparse sums' atomics, in any order
+    assert np.all(np.abs(got["log_abs_psi"] - clean["log_abs_psi"])[ok] <= (tol + 1e-14)[ok])
