@@ -7,12 +7,12 @@
 //   (element (r, k) at p[r * rs + k * ks], zero outside the matrix), so that the
 //   transposed operands of the backward pass need no copies;
 //   operands rounded to BF16 (nearest even) as they are staged, FP32 accumulation.
-// Tile: 128 rows of A (the TMEM lanes) x up to 256 rows of B (TMEM columns), K in
-// chunks of 64. Per chunk the 128 threads stage both operands into shared memory as
-// K-major core matrices of 8 rows x 16 bytes (no swizzle; 8-row groups 1 KB apart,
-// core matrices along K 128 B apart), one thread issues four MMAs of K = 16 and
-// commits them to an mbarrier, and all threads wait for it before the next chunk
-// overwrites the tiles. Then each warp reads its 32 TMEM lanes back with tcgen05.ld
+// Tile: 128 rows of A (the TMEM lanes) x up to 128 rows of B (TMEM columns), K in chunks of 64
+// through a ring of three shared-memory stages in the 128-byte swizzle. 256 threads stage a chunk
+// (8 elements per thread and item: two 16-byte loads where an operand is contiguous along K and
+// aligned, scalar loads with consecutive lanes in consecutive rows where it is contiguous along its
+// rows), one thread issues four MMAs of K = 16 and commits them to the stage's mbarrier, and the
+// next chunk's loads run beside them. Then each warp reads its 32 TMEM lanes back with tcgen05.ld
 // and applies the epilogue:
 //   kEpiTanhBias  out = tanh(D + bias[n])          (hidden layers)
 //   kEpiBias      out = D + bias[n]                (output layer)
@@ -35,59 +35,86 @@ namespace mdet {
 namespace {
 
 constexpr int kGM = 128;      // rows of A per CTA: the MMA's M (TMEM lanes)
-constexpr int kGN = 256;      // rows of B per CTA: the largest N of one MMA
+constexpr int kGN = 128;      // rows of B per CTA: the MMA's N; two CTAs per SM share its tensor memory
 constexpr int kGK = 64;       // K per staged chunk: four MMAs of K = 16
-constexpr int kThreads = 128;
-constexpr int kTmemCols = 256;
+constexpr int kThreads = 256;
+constexpr int kStages = 3;
+constexpr int kTmemCols = 128;
 constexpr int kWaitLimit = 1 << 24;
 constexpr int kTileA = kGM * kGK * 2;  // bytes of the staged A chunk
 constexpr int kTileB = kGN * kGK * 2;
-// 100 KB of dynamic shared memory per CTA (the tiles take 48 KB) keeps at most two CTAs
-// on an SM, whose 2 x 256 tensor-memory columns fit its 512
-constexpr size_t kSmem = 100 * 1024;
-static_assert(kTileA + kTileB <= (int)kSmem, "tiles exceed the dynamic shared memory");
+constexpr size_t kSmem = (size_t)kStages * (kTileA + kTileB);
 
+// Eight elements (r, k) .. (r, k + 7) of o as BF16, zero outside the matrix.
 __device__ __forceinline__ float op_get(const GemmOperand& o, int64_t r, int64_t k) {
   if (r >= o.rows || k >= o.cols) return 0.0f;
   const int64_t i = r * o.rs + k * o.ks;
   return o.bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(o.p)[i]) : static_cast<const float*>(o.p)[i];
 }
-
-// rows [r0, r0 + nr) and k [k0, k0 + 64) of o, as BF16, into the K-major tile s:
-// element (r, k) at (r / 8) * 1024 + (k / 8) * 128 + (r % 8) * 16 + (k % 8) * 2
-__device__ __forceinline__ void stage(const GemmOperand& o, int64_t r0, int nr, int64_t k0, uint8_t* s) {
-  for (int r = threadIdx.x; r < nr; r += kThreads) {
-#pragma unroll 2
-    for (int g = 0; g < kGK / 8; g++) {
-      uint32_t w[4];
+__device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
+  uint32_t w[4];
 #pragma unroll
-      for (int h = 0; h < 4; h++) {
-        const int64_t k = k0 + 8 * g + 2 * h;
-        const __nv_bfloat162 b = __floats2bfloat162_rn(op_get(o, r0 + r, k), op_get(o, r0 + r, k + 1));
-        w[h] = *reinterpret_cast<const uint32_t*>(&b);  // even k in the low half
+  for (int h = 0; h < 4; h++) {
+    const __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * h], v[2 * h + 1]);
+    w[h] = *reinterpret_cast<const uint32_t*>(&b);  // even k in the low half
+  }
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
+// Whether rows of 8 elements along K can be loaded as 16-byte words: unit stride along K, and the
+// base and the row stride multiples of 16 bytes.
+__device__ __forceinline__ bool vector_rows(const GemmOperand& o) {
+  const int per = o.bf16 ? 8 : 4;
+  return o.ks == 1 && o.rs % per == 0 && (reinterpret_cast<uintptr_t>(o.p) & 15) == 0;
+}
+
+// rows [r0, r0 + 128) and k [k0, k0 + 64) of o, as BF16, into the tile s: 16-byte chunk g of row r at
+// 128 r + 16 (g ^ (r mod 8)). Item (row, chunk): chunks fastest where K is contiguous (a row's 8
+// chunks are 256 consecutive bytes in FP32), rows fastest where the rows are.
+__device__ __forceinline__ void stage(const GemmOperand& o, bool vec, int64_t r0, int nr, int64_t k0, uint8_t* s) {
+  const bool along_k = o.ks == 1;
+  const int n = nr * (kGK / 8);
+#pragma unroll
+  for (int q = 0; q < 128 * (kGK / 8) / kThreads; q++) {
+    const int t = threadIdx.x + q * kThreads;
+    if (t >= n) break;
+    const int r = along_k ? t >> 3 : t % nr, g = along_k ? t & 7 : t / nr;
+    const int64_t R = r0 + r, k = k0 + 8 * g;
+    uint4 w;
+    if (vec && R < o.rows && k + 8 <= o.cols) {
+      if (o.bf16) {
+        w = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(o.p) + R * o.rs + k);
+      } else {
+        const float4* p = reinterpret_cast<const float4*>(static_cast<const float*>(o.p) + R * o.rs + k);
+        const float4 a = p[0], b = p[1];
+        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+        w = pack8(v);
       }
-      *reinterpret_cast<uint4*>(s + (r >> 3) * 1024 + g * 128 + (r & 7) * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+    } else {
+      float v[8];
+#pragma unroll
+      for (int h = 0; h < 8; h++) v[h] = op_get(o, R, k + h);
+      w = pack8(v);
     }
+    *reinterpret_cast<uint4*>(s + r * 128 + ((g ^ (r & 7)) << 4)) = w;
   }
 }
 
 __global__ void __launch_bounds__(kThreads) k_gemm_bf16(GemmOperand A, GemmOperand B, int64_t k_per_cta,
                                                         GemmEpilogue E) {
   extern __shared__ __align__(1024) uint8_t smg[];
-  uint8_t* sA = smg;
-  uint8_t* sB = smg + kTileA;
-  __shared__ __align__(8) uint64_t bar;
+  __shared__ __align__(8) uint64_t bar[kStages];
   __shared__ uint32_t tbase;
   __shared__ int stop_s;
   volatile int* stop = &stop_s;
-  const int tid = threadIdx.x, warp = tid >> 5;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int64_t m0 = (int64_t)blockIdx.x * kGM, n0 = (int64_t)blockIdx.y * kGN;
   const int64_t kb = (int64_t)blockIdx.z * k_per_cta, ke = A.cols < kb + k_per_cta ? A.cols : kb + k_per_cta;
   const int nt = (int)(B.rows - n0 < kGN ? B.rows - n0 : kGN);  // rows of B in this tile
   const int nmma = (nt + 15) / 16 * 16;                     // the MMA's N (a multiple of 16)
   if (warp == 0) umma::tmem_alloc(&tbase, kTmemCols);
   if (tid == 0) {
-    umma::mbar_init(&bar, 1);
+    for (int b = 0; b < kStages; b++) umma::mbar_init(&bar[b], 1);
     *stop = 0;
   }
   umma::fence_before();
@@ -95,62 +122,88 @@ __global__ void __launch_bounds__(kThreads) k_gemm_bf16(GemmOperand A, GemmOpera
   umma::fence_after();
   const uint32_t tb = tbase;
   const uint32_t idesc = umma::idesc_bf16(kGM, nmma);
-  const uint32_t a_s = umma::smem_u32(sA), b_s = umma::smem_u32(sB);
-  uint32_t phase = 0;
-  bool any = false;  // at least one chunk accumulated
-  for (int64_t k0 = kb; k0 < ke; k0 += kGK) {
-    stage(A, m0, kGM, k0, sA);
-    stage(B, n0, nmma, k0, sB);
+  const bool va = vector_rows(A), vb = vector_rows(B);
+  int c = 0;  // chunks issued
+  for (int64_t k0 = kb; k0 < ke; k0 += kGK, c++) {
+    const int b = c % kStages;
+    uint8_t* sA = smg + b * (kTileA + kTileB);
+    uint8_t* sB = sA + kTileA;
+    // the MMAs that read this stage last
+    if (c >= kStages && !umma::mbar_wait(&bar[b], ((c / kStages) & 1) ^ 1, kWaitLimit)) *stop = 1;
+    stage(A, va, m0, kGM, k0, sA);
+    stage(B, vb, n0, nmma, k0, sB);
     umma::fence_smem_async();
     umma::fence_before();
-    __syncthreads();
+    __syncthreads();  // also shows every thread the same stop flag
     umma::fence_after();
+    if (*stop) break;
     if (tid == 0) {
+      const uint32_t a_s = umma::smem_u32(sA), b_s = umma::smem_u32(sB);
 #pragma unroll
       for (int ks = 0; ks < kGK / 16; ks++)
-        umma::mma_smem_a(tb, umma::desc(a_s + ks * 256, 128, 1024), umma::desc(b_s + ks * 256, 128, 1024), idesc,
-                         (any || ks > 0) ? 1u : 0u);
-      umma::commit(&bar);
+        umma::mma_smem_a(tb, umma::desc_sw128(a_s + ks * 32), umma::desc_sw128(b_s + ks * 32), idesc,
+                         (c > 0 || ks > 0) ? 1u : 0u);
+      umma::commit(&bar[b]);
     }
-    any = true;
-    if (!umma::mbar_wait(&bar, phase, kWaitLimit)) *stop = 1;
-    phase ^= 1u;
-    umma::fence_after();
-    __syncthreads();  // the tiles are free again, and every thread sees the same stop flag
-    if (*stop) break;
   }
-  // epilogue: warp w holds rows m0 + 32 w + lane in TMEM lanes 32 w + lane
-  const int64_t m = m0 + tid;
-  const bool row_ok = any && m < A.rows;
-  const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-  for (int c0 = 0; c0 < nmma; c0 += 16) {
+  // every MMA precedes the last commit
+  if (c > 0 && !umma::mbar_wait(&bar[(c - 1) % kStages], ((c - 1) / kStages) & 1, kWaitLimit)) *stop = 1;
+  umma::fence_after();
+  __syncthreads();
+  // epilogue: warp w holds rows m0 + 32 (w mod 4) + lane in TMEM lanes 32 (w mod 4) + lane, and takes every
+  // other group of 16 columns
+  const int64_t m = m0 + 32 * (warp & 3) + lane;
+  const bool row_ok = c > 0 && m < A.rows;
+  const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+  // 16-byte accesses of the output (and of h) where rows are contiguous and aligned
+  const bool vec = E.ldn == 1 && E.ldm % 4 == 0 && (reinterpret_cast<uintptr_t>(E.out) & 15) == 0 &&
+                   (E.kind != kEpiDtanh || (E.ldh % 4 == 0 && (reinterpret_cast<uintptr_t>(E.h) & 15) == 0));
+  for (int c0 = 16 * (warp >> 2); c0 < nmma; c0 += 32) {
     uint32_t v[16];
     umma::tmem_ld16(tb + lane_base + (uint32_t)c0, v);  // the whole warp, converged
     if (!row_ok) continue;
-#pragma unroll
-    for (int j = 0; j < 16; j++) {
+    const bool dead = *stop;
+    auto value = [&](int j, float h) -> float {
       const int64_t n = n0 + c0 + j;
-      if (c0 + j >= nt) break;
-      const float d = *stop ? __int_as_float(0x7fc00000) : __uint_as_float(v[j]);
-      float* o = E.out + m * E.ldm + n * E.ldn;
+      const float d = dead ? __int_as_float(0x7fc00000) : __uint_as_float(v[j]);
       switch (E.kind) {
-        case kEpiTanhBias: *o = tanhf(d + E.bias[n]); break;
-        case kEpiBias: *o = d + E.bias[n]; break;
-        case kEpiStore: *o = d; break;
-        case kEpiDtanh: {
-          const float h = E.h[m * E.ldh + n];
-          *o = d * (1.0f - h * h);
-          break;
-        }
-        default: atomicAdd(o, d);
+        case kEpiTanhBias: return tanhf(d + E.bias[n]);
+        case kEpiBias: return d + E.bias[n];
+        case kEpiDtanh: return d * (1.0f - h * h);
+        default: return d;
+      }
+    };
+#pragma unroll
+    for (int j = 0; j < 16; j += 4) {
+      float* o = E.out + m * E.ldm + (n0 + c0 + j) * E.ldn;
+      if (vec && c0 + j + 4 <= nt) {
+        float4 h = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (E.kind == kEpiDtanh) h = *reinterpret_cast<const float4*>(E.h + m * E.ldh + n0 + c0 + j);
+        const float4 x = make_float4(value(j, h.x), value(j + 1, h.y), value(j + 2, h.z), value(j + 3, h.w));
+        if (E.kind == kEpiAtomic)
+          atomicAdd(reinterpret_cast<float4*>(o), x);
+        else
+          *reinterpret_cast<float4*>(o) = x;
+        continue;
+      }
+#pragma unroll
+      for (int z = 0; z < 4; z++) {
+        if (c0 + j + z >= nt) break;
+        const float x = value(j + z, E.kind == kEpiDtanh ? E.h[m * E.ldh + n0 + c0 + j + z] : 0.0f);
+        if (E.kind == kEpiAtomic)
+          atomicAdd(o + z * E.ldn, x);
+        else
+          o[z * E.ldn] = x;
       }
     }
   }
   umma::fence_before();
   __syncthreads();
-  if (*stop && tid == 0) {  // a wait ran out: let the MMAs in flight finish (bounded) before the release
-    umma::commit(&bar);
-    umma::mbar_wait(&bar, phase, kWaitLimit);
+  umma::fence_after();
+  if (*stop && tid == 0) {  // after a wait ran out: the MMAs in flight finish (bounded) before the release
+    umma::commit(&bar[0]);
+    umma::drain_wait(&bar[0], 0);
+    umma::drain_wait(&bar[0], 1);
   }
   __syncthreads();
   if (warp == 0) umma::tmem_dealloc(tb, kTmemCols);
@@ -164,7 +217,8 @@ cudaError_t launch_gemm_bf16(const GemmOperand& A, const GemmOperand& B, int64_t
   const int64_t kc = std::max<int64_t>(kGK, (k_per_cta + kGK - 1) / kGK * kGK);
   const dim3 grid((unsigned)((A.rows + kGM - 1) / kGM), (unsigned)((B.rows + kGN - 1) / kGN),
                   (unsigned)((A.cols + kc - 1) / kc));
-  cudaError_t e = cudaFuncSetAttribute(k_gemm_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem);
+  static SmemOptIn opt;
+  cudaError_t e = opt.ensure(k_gemm_bf16, kSmem);
   if (e != cudaSuccess) return e;
   k_gemm_bf16<<<grid, kThreads, kSmem, st>>>(A, B, kc, E);
   return cudaGetLastError();

@@ -243,29 +243,30 @@ struct Head {
 // with respect to the raw outputs (mean over walkers):
 //   NLL = sum_c d_c^2 / (2 sigma_e^2) + 3 sum_e s_e,  d_c = R1_c - R0_c - mu_c,
 //   dNLL/dmu_c = -d_c / sigma_e^2,  dNLL/ds_e = 3 - sum_c (d_c^2 + d_c mu_c) / sigma_e^2.
+// One thread per walker and electron.
 __global__ void k_nll(Head hd, int64_t n_walk, const double* __restrict__ R0, const double* __restrict__ R1,
                       const float* __restrict__ out, float* __restrict__ dout, double* __restrict__ loss) {
-  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int N = hd.N, no = 4 * N;
   double l = 0.0;
-  if (w < n_walk) {
-    const int N = hd.N, no = 4 * N;
+  if (t < n_walk * N) {
+    const int64_t w = t / N;
+    const int e = (int)(t - w * N);
     const float invB = 1.0f / (float)n_walk;
-    for (int e = 0; e < N; e++) {
-      const float ts = tanhf(out[w * no + 3 * N + e]);
-      const float s = (float)hd.s0 + (float)hd.s_span * ts;
-      const float sig = expf(s), iv = expf(-2.0f * s);
-      float d2 = 0.0f, dmu = 0.0f;
-      for (int c = 0; c < 3; c++) {
-        const float tm = tanhf(out[w * no + 3 * e + c]);
-        const float mu = sig * (float)hd.mu_max * tm;
-        const float d = (float)(R1[w * 3 * N + 3 * e + c] - R0[w * 3 * N + 3 * e + c]) - mu;
-        d2 += d * d;
-        dmu += d * mu;
-        dout[w * no + 3 * e + c] = invB * (-d * iv) * sig * (float)hd.mu_max * (1.0f - tm * tm);
-      }
-      l += 0.5 * d2 * iv + 3.0 * s;
-      dout[w * no + 3 * N + e] = invB * (3.0f - (d2 + dmu) * iv) * (float)hd.s_span * (1.0f - ts * ts);
+    const float ts = tanhf(out[w * no + 3 * N + e]);
+    const float s = (float)hd.s0 + (float)hd.s_span * ts;
+    const float sig = expf(s), iv = expf(-2.0f * s);
+    float d2 = 0.0f, dmu = 0.0f;
+    for (int c = 0; c < 3; c++) {
+      const float tm = tanhf(out[w * no + 3 * e + c]);
+      const float mu = sig * (float)hd.mu_max * tm;
+      const float d = (float)(R1[w * 3 * N + 3 * e + c] - R0[w * 3 * N + 3 * e + c]) - mu;
+      d2 += d * d;
+      dmu += d * mu;
+      dout[w * no + 3 * e + c] = invB * (-d * iv) * sig * (float)hd.mu_max * (1.0f - tm * tm);
     }
+    l = 0.5 * d2 * iv + 3.0 * s;
+    dout[w * no + 3 * N + e] = invB * (3.0f - (d2 + dmu) * iv) * (float)hd.s_span * (1.0f - ts * ts);
   }
 #pragma unroll
   for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
@@ -654,10 +655,11 @@ mdet_status mdet_mlp_backward(mdet_mlp* m, int64_t n_walk, const float* dout, vo
   if (e == cudaSuccess)
     e = launch_gemm_bf16(GemmOperand{m->d2, H, 1, n_walk, H, 0}, GemmOperand{pb + m->oW2, H, 1, H, H, 1}, H,
                          GemmEpilogue{kEpiDtanh, m->d1, H, 1, nullptr, m->h1, H}, st);
-  // weight gradients, summed over the walkers (the GEMMs' K), 1,024 walkers per CTA:
+  // weight gradients, summed over the walkers (the GEMMs' K), 256 walkers per CTA (with 1,024 a batch
+  // of 8,192 gave 16 CTAs, and the three products took 600 us):
   // gW3[k][j] = sum_w h2[w][k] dout[w][j], gW2[k][j] = sum_w h1[w][k] d2[w][j],
   // gW1[i][j] = sum_w x[w][i] d1[w][j] (computed as its transpose: rows j, columns i)
-  const int64_t kpc = 1024;
+  const int64_t kpc = 256;
   if (e == cudaSuccess)
     e = launch_gemm_bf16(GemmOperand{m->h2, 1, H, H, n_walk, 0}, GemmOperand{dout, 1, no, no, n_walk, 0}, kpc,
                          GemmEpilogue{kEpiAtomic, m->g + m->oW3, no, 1, nullptr, nullptr, 0}, st);
@@ -670,7 +672,7 @@ mdet_status mdet_mlp_backward(mdet_mlp* m, int64_t n_walk, const float* dout, vo
   if (e != cudaSuccess) return cuda_status(e);
   // bias gradients from the unrounded deltas
   const ColSumJobs jobs{{{dout, (int)no, m->g + m->ob3}, {m->d2, (int)H, m->g + m->ob2}, {m->d1, (int)H, m->g + m->ob1}}};
-  const int64_t per = 256;
+  const int64_t per = 64;
   const dim3 grid(blocks(std::max(no, H), 128), (unsigned)((n_walk + per - 1) / per), 3);
   k_bias_grad<<<grid, 128, 0, st>>>(jobs, n_walk, per);
   return cuda_status(cudaGetLastError());
@@ -697,7 +699,7 @@ mdet_status mdet_mlp_nll_grad(const mdet_mlp* m, int64_t n_walk, const double* R
   if (!m || n_walk < 1 || !R0 || !R1 || !out || !dout || !loss) return MDET_E_ARG;
   if (cudaSetDevice(m->device) != cudaSuccess) return MDET_E_CUDA;
   if (cudaMemsetAsync(loss, 0, sizeof(double), (cudaStream_t)stream) != cudaSuccess) return MDET_E_CUDA;
-  k_nll<<<blocks(n_walk, 128), 128, 0, (cudaStream_t)stream>>>(head(m), n_walk, R0, R1, out, dout, loss);
+  k_nll<<<blocks(n_walk * m->n_elec, 128), 128, 0, (cudaStream_t)stream>>>(head(m), n_walk, R0, R1, out, dout, loss);
   return cuda_status(cudaGetLastError());
 }
 
