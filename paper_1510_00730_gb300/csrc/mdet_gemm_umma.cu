@@ -45,12 +45,6 @@ constexpr int kTileA = kGM * kGK * 2;  // bytes of the staged A chunk
 constexpr int kTileB = kGN * kGK * 2;
 constexpr size_t kSmem = (size_t)kStages * (kTileA + kTileB);
 
-// Eight elements (r, k) .. (r, k + 7) of o as BF16, zero outside the matrix.
-__device__ __forceinline__ float op_get(const GemmOperand& o, int64_t r, int64_t k) {
-  if (r >= o.rows || k >= o.cols) return 0.0f;
-  const int64_t i = r * o.rs + k * o.ks;
-  return o.bf16 ? __bfloat162float(static_cast<const __nv_bfloat16*>(o.p)[i]) : static_cast<const float*>(o.p)[i];
-}
 __device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
   uint32_t w[4];
 #pragma unroll
@@ -61,43 +55,84 @@ __device__ __forceinline__ uint4 pack8(const float (&v)[8]) {
   return make_uint4(w[0], w[1], w[2], w[3]);
 }
 
+__device__ __forceinline__ float to_f32(float x) { return x; }
+__device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
+
 // Whether rows of 8 elements along K can be loaded as 16-byte words: unit stride along K, and the
-// base and the row stride multiples of 16 bytes.
+// base and the row stride multiples of 16 bytes, and no row ending inside 8 elements.
 __device__ __forceinline__ bool vector_rows(const GemmOperand& o) {
   const int per = o.bf16 ? 8 : 4;
-  return o.ks == 1 && o.rs % per == 0 && (reinterpret_cast<uintptr_t>(o.p) & 15) == 0;
+  return o.ks == 1 && o.rs % per == 0 && o.cols % 8 == 0 && (reinterpret_cast<uintptr_t>(o.p) & 15) == 0;
 }
 
-// rows [r0, r0 + 128) and k [k0, k0 + 64) of o, as BF16, into the tile s: 16-byte chunk g of row r at
-// 128 r + 16 (g ^ (r mod 8)). Item (row, chunk): chunks fastest where K is contiguous (a row's 8
-// chunks are 256 consecutive bytes in FP32), rows fastest where the rows are.
-__device__ __forceinline__ void stage(const GemmOperand& o, bool vec, int64_t r0, int nr, int64_t k0, uint8_t* s) {
+// rows [r0, r0 + nr) and k [k0, k0 + 64) of o, as BF16 (zero outside the matrix), into the tile s:
+// 16-byte chunk g of row r at 128 r + 16 (g ^ (r mod 8)). Item (row, chunk): chunks fastest where K is
+// contiguous (a row's 8 chunks are 256 consecutive bytes in FP32), rows fastest where the rows are.
+// The loads of two items are issued before either is converted.
+template <class T>
+__device__ __forceinline__ void stage_t(const GemmOperand& o, bool vec, int64_t r0, int nr, int64_t k0, uint8_t* s) {
+  const T* base = static_cast<const T*>(o.p);
   const bool along_k = o.ks == 1;
   const int n = nr * (kGK / 8);
+  constexpr int kItems = 128 * (kGK / 8) / kThreads, kBatch = 2;
 #pragma unroll
-  for (int q = 0; q < 128 * (kGK / 8) / kThreads; q++) {
-    const int t = threadIdx.x + q * kThreads;
-    if (t >= n) break;
-    const int r = along_k ? t >> 3 : t % nr, g = along_k ? t & 7 : t / nr;
-    const int64_t R = r0 + r, k = k0 + 8 * g;
-    uint4 w;
-    if (vec && R < o.rows && k + 8 <= o.cols) {
-      if (o.bf16) {
-        w = *reinterpret_cast<const uint4*>(static_cast<const __nv_bfloat16*>(o.p) + R * o.rs + k);
-      } else {
-        const float4* p = reinterpret_cast<const float4*>(static_cast<const float*>(o.p) + R * o.rs + k);
-        const float4 a = p[0], b = p[1];
-        const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
-        w = pack8(v);
+  for (int q0 = 0; q0 < kItems; q0 += kBatch) {
+    uint4 w[kBatch];
+    uint8_t* at[kBatch];
+    if (vec) {
+      uint4 a[kBatch][sizeof(T) / 2];
+#pragma unroll
+      for (int q = 0; q < kBatch; q++) {
+        const int t = threadIdx.x + (q0 + q) * kThreads, r = t >> 3, g = t & 7;
+        const int64_t R = r0 + r, k = k0 + 8 * g;
+        const bool in = t < n && R < o.rows && k < o.cols;  // (cols is a multiple of 8 here)
+        at[q] = t < n ? s + r * 128 + ((g ^ (r & 7)) << 4) : nullptr;
+        const uint4* p = reinterpret_cast<const uint4*>(base + R * o.rs + k);
+#pragma unroll
+        for (int h = 0; h < (int)sizeof(T) / 2; h++) a[q][h] = in ? p[h] : make_uint4(0u, 0u, 0u, 0u);
+      }
+#pragma unroll
+      for (int q = 0; q < kBatch; q++) {
+        if constexpr (sizeof(T) == 2) {
+          w[q] = a[q][0];
+        } else {
+          const float v[8] = {__uint_as_float(a[q][0].x), __uint_as_float(a[q][0].y), __uint_as_float(a[q][0].z),
+                              __uint_as_float(a[q][0].w), __uint_as_float(a[q][1].x), __uint_as_float(a[q][1].y),
+                              __uint_as_float(a[q][1].z), __uint_as_float(a[q][1].w)};
+          w[q] = pack8(v);
+        }
       }
     } else {
-      float v[8];
+      T v[kBatch][8];
 #pragma unroll
-      for (int h = 0; h < 8; h++) v[h] = op_get(o, R, k + h);
-      w = pack8(v);
+      for (int q = 0; q < kBatch; q++) {
+        const int t = threadIdx.x + (q0 + q) * kThreads;
+        const int r = along_k ? t >> 3 : t % nr, g = along_k ? t & 7 : t / nr;
+        const int64_t R = r0 + r, k = k0 + 8 * g;
+        at[q] = t < n ? s + r * 128 + ((g ^ (r & 7)) << 4) : nullptr;
+        const T* p = base + R * o.rs + k * o.ks;
+#pragma unroll
+        for (int h = 0; h < 8; h++) v[q][h] = t < n && R < o.rows && k + h < o.cols ? p[h * o.ks] : T(0.0f);
+      }
+#pragma unroll
+      for (int q = 0; q < kBatch; q++) {
+        float f[8];
+#pragma unroll
+        for (int h = 0; h < 8; h++) f[h] = to_f32(v[q][h]);
+        w[q] = pack8(f);
+      }
     }
-    *reinterpret_cast<uint4*>(s + r * 128 + ((g ^ (r & 7)) << 4)) = w;
+#pragma unroll
+    for (int q = 0; q < kBatch; q++)
+      if (at[q]) *reinterpret_cast<uint4*>(at[q]) = w[q];
   }
+}
+
+__device__ __forceinline__ void stage(const GemmOperand& o, bool vec, int64_t r0, int nr, int64_t k0, uint8_t* s) {
+  if (o.bf16)
+    stage_t<__nv_bfloat16>(o, vec, r0, nr, k0, s);
+  else
+    stage_t<float>(o, vec, r0, nr, k0, s);
 }
 
 __global__ void __launch_bounds__(kThreads) k_gemm_bf16(GemmOperand A, GemmOperand B, int64_t k_per_cta,
