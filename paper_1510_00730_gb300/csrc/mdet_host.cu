@@ -357,7 +357,7 @@ void pick_items(const mdet_ctx* c, DevProblem& P, int64_t n_walk) {
 
 void free_arrays(DevScratch& S) {
   void* ptrs[] = {S.phi, S.Ainv, S.ld0, S.sg0, S.g, S.kap, S.est, S.T, S.Tdf, S.r, S.rdf, S.vu, S.psit, S.psia, S.wstat,
-                  S.xmax, S.dx, S.dy, S.dyabs, S.derr, S.xd, S.xer,
+                  S.xmax, S.dx, S.dy, S.dyabs, S.derr, S.xd, S.xer, S.W,
                   S.fb, S.fb_list, S.fb_acc, S.queue, S.R_stage, S.out_stage};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -735,6 +735,12 @@ mdet_status alloc_eval_arrays(mdet_ctx* c, DevScratch& S, int64_t W, bool df_tab
   if ((s = dalloc(c, &S.psit, (size_t)wp))) return s;
   if ((s = dalloc(c, &S.psia, (size_t)wp))) return s;
   if ((s = dalloc(c, &S.wstat, (size_t)W))) return s;
+  const bool main_scratch = df_tables || c->precision == MDET_PRECISION_FP64;  // not a re-evaluation's
+  if (main_scratch && scatter_group_walkers(P, W, df_tables) > 0 &&
+      cudaMalloc((void**)&S.W, sizeof(double) * W * N * M) != cudaSuccess) {  // no room: the epilogue's own scatter
+    cudaGetLastError();
+    S.W = nullptr;
+  }
   if (mo_digits_supported(P, df_tables)) {  // digits of the AO values, for blocks of walkers
     const int64_t row_bytes = (int64_t)mo_digits_row_bytes(P, df_tables), per = 5 * N * row_bytes;
     S.xd_walk = std::min(W, std::max<int64_t>(1, (int64_t)kDigitBytes / per));
@@ -1355,7 +1361,7 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
     *n = std::min<int64_t>(t1 * kWalkerPad, n_walk) - *off;
   };
   const bool dense = use_dense(c) && c->S.xmax;
-  int contract_kernels = 0, orbital_kernels = 0;
+  int contract_kernels = 0, orbital_kernels = 0, scatter_kernels = 0;
   // stage i (MDET_STAGE_*) of chunk k on stream ks, bracketed by its two profiling events
   auto stage = [&](int k, int i, cudaStream_t ks, int persistent) -> mdet_status {
     int64_t off, n;
@@ -1390,6 +1396,7 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
         break;
       }
       default:
+        if (S.W && scatter_group_walkers(P, n, mixed) > 0) scatter_kernels++;
         CUDA_TRY(c, launch_final(P, S, n, Rk, log_abs_psi + off, sign + off, grad + off * N * 3, lap + off * N,
                                  e_local ? e_local + off : nullptr, status ? status + off : nullptr, mixed, ks));
     }
@@ -1438,12 +1445,12 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
   c->prof_chunks = nch;
   // stability fallback over the whole batch, after every chunk has finished: mixed precision
   // escalates to FP64 first, FP64 goes to full LU directly
-  // kernels: 3 per chunk (reference, ratios, epilogue), its orbitals' (2 per walker block of the digit
+  // kernels: 3 per chunk (reference, ratios, epilogue; 4 with the epilogue's separate scatter), its orbitals' (2 per walker block of the digit
   // products, else 1) and its contraction's (1 for the sparse sums, 2 in double-float, 3 per walker
   // block of the residue products); the full-LU
   // fallback 5 (list, dets, scale, rows, out); the mixed refinement adds its list, gather,
   // FP64 orbitals and scatter, and either the mark or the 5 FP64 table kernels
-  c->last_kernels = 3 * nch + orbital_kernels + contract_kernels;
+  c->last_kernels = 3 * nch + orbital_kernels + contract_kernels + scatter_kernels;
   if (prof_all) CUDA_TRY(c, cudaEventRecord(c->ev_refine[0], st));
   if (mixed && c->E.fb && P.fallback_tol > 0.0) {
     const bool table = escalation_on(c);

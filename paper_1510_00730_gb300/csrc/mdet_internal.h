@@ -164,6 +164,7 @@ struct DevScratch {
   int* derr = nullptr;
   int64_t dblk = 0;
   // digits and row exponents of the AO values of xd_walk walkers (null: no room for them)
+  double* W = nullptr;  // [W][n_elec][n_mo] aggregated cofactors, of k_scatter (mixed: unnormalised pairs)
   uint8_t* xd = nullptr;
   int* xer = nullptr;
   int64_t xd_walk = 0;
@@ -287,6 +288,8 @@ cudaError_t launch_selftest_df(int64_t n, const double* x, double* y_df, double*
                                cudaStream_t st);
 cudaError_t launch_selftest_inv_r(int64_t n, const double* x, double* y_nr, double* y_ref, cudaStream_t st);
 size_t final_smem_bytes(const DevProblem& P, bool mixed);
+// Walkers per group of the epilogue's separate scatter kernel, 0 where the epilogue scatters itself.
+int scatter_group_walkers(const DevProblem& P, int64_t n_walk, bool mixed);
 // wide: 512 threads per walker instead of 128 (FP64 only; lower latency for a few walkers)
 cudaError_t launch_final(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R,
                          double* log_abs_psi, int8_t* sign, double* grad, double* lap, double* e_local,

@@ -34,6 +34,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 
 #include "df32.cuh"
 #include "mdet_device.cuh"
@@ -672,6 +673,172 @@ __device__ __forceinline__ void scatter_cof_df(const Exc& e, long long wb, const
 }
 
 // ---------------------------------------------------------------------------
+// K6a (many walkers): W of one spin for a group of L walkers. Lanes are walkers (32 / L
+// determinants per warp), so that the table entries load coalesced, no lane waits on another's
+// determinant, and the accumulators in shared memory, [slot][walker], are hit without bank
+// conflicts; the per-walker scatter of k_final spends most of its time on conflicting shared-memory
+// atomics. A warp takes its own stretch of each degree's list, so warps rarely meet in a slot. W goes
+// to global memory walker-major, where k_final reads it. 8,192 walkers, 750k products, 3,015
+// determinants per spin, k_final before and both kernels after: 4.62 -> 2.94 ms in double-float
+// (issue-bound), 10.1 -> 6.4 ms in FP64 (bound by the FP64 pipe).
+//
+// Double-float: the same accumulation as k_final's scatter (hi by TwoSum, its error and the term's
+// low word into lo), the pair replaced by a 64-bit compare-and-swap, all slots of a determinant at
+// once; one that lost its race is retried.
+__device__ __forceinline__ unsigned long long w_add(unsigned long long old, df32 x) {
+  const float hi = __uint_as_float((unsigned)old), lo = __uint_as_float((unsigned)(old >> 32));
+  float s, e;
+  two_sum(hi, x.hi, s, e);
+  const float l = __fadd_rn(lo, __fadd_rn(e, x.lo));
+  return (unsigned long long)__float_as_uint(s) | ((unsigned long long)__float_as_uint(l) << 32);
+}
+
+template <int K>
+__device__ __forceinline__ void scatter_group(const Exc& e, long long wb, const float2* __restrict__ T, int64_t wp, int M,
+                                              uint8_t* Wsm, int ld, int) {
+  df32 m[4][4], cof[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; a++)
+#pragma unroll
+    for (int b = 0; b < 4; b++) {
+      const float2 v = (a < K && b < K) ? __ldg(T + (size_t)(e.h[a] * M + e.p[b]) * wp) : make_float2(0.f, 0.f);
+      m[a][b] = df32(v.x, v.y);
+    }
+  small_cof_dot<K>(m, cof);
+  const df32 wd = df_from_bits(wb);
+  unsigned long long* W = reinterpret_cast<unsigned long long*>(Wsm);
+  unsigned long long old[K * K];
+#pragma unroll
+  for (int q = 0; q < K * K; q++) old[q] = W[(e.h[q / K] * M + e.p[q % K]) * ld];
+#pragma unroll
+  for (int q = 0; q < K * K; q++) {
+    const df32 x = cof[q / K][q % K] * wd;
+    unsigned long long* at = W + (e.h[q / K] * M + e.p[q % K]) * ld;
+    const unsigned long long got = atomicCAS(at, old[q], w_add(old[q], x));
+    if (got != old[q]) {
+      unsigned long long cur = got, was;
+      do {
+        was = cur;
+        cur = atomicCAS(at, was, w_add(was, x));
+      } while (cur != was);
+    }
+  }
+}
+
+// FP64: the cofactors weighted through their 2 x 2 minors or rows (fewer products on the FP64 pipe
+// than weighting each), accumulated in three FP32 words off that pipe (acc3_add), `plane` floats apart.
+template <int K>
+__device__ __forceinline__ void scatter_group(const Exc& e, long long wb, const double* __restrict__ T, int64_t wp, int M,
+                                              uint8_t* Wsm, int ld, int plane) {
+  double m[K][K], cof[K][K];
+#pragma unroll
+  for (int a = 0; a < K; a++)
+#pragma unroll
+    for (int b = 0; b < K; b++) m[a][b] = __ldg(T + (size_t)(e.h[a] * M + e.p[b]) * wp);
+  const double w = __longlong_as_double(wb);
+  if constexpr (K == 1) {
+    cof[0][0] = w;
+  } else if constexpr (K == 2) {
+    cof[0][0] = w * m[1][1];
+    cof[0][1] = -w * m[1][0];
+    cof[1][0] = -w * m[0][1];
+    cof[1][1] = w * m[0][0];
+  } else if constexpr (K == 3) {
+    double r0[3], r1[3];  // w times rows 0 and 1
+#pragma unroll
+    for (int b = 0; b < 3; b++) {
+      r0[b] = w * m[0][b];
+      r1[b] = w * m[1][b];
+    }
+#pragma unroll
+    for (int b = 0; b < 3; b++) {
+      const int x = (b + 1) % 3, y = (b + 2) % 3;  // cyclic minors carry their own sign
+      cof[0][b] = r1[x] * m[2][y] - r1[y] * m[2][x];
+      cof[1][b] = m[2][x] * r0[y] - m[2][y] * r0[x];
+      cof[2][b] = r0[x] * m[1][y] - r0[y] * m[1][x];
+    }
+  } else {
+    double top[4][4], bot[4][4];  // w times the 2 x 2 minors of rows (0,1) and (2,3), columns x < y
+#pragma unroll
+    for (int x = 0; x < 4; x++)
+#pragma unroll
+      for (int y = x + 1; y < 4; y++) {
+        top[x][y] = w * (m[0][x] * m[1][y] - m[0][y] * m[1][x]);
+        bot[x][y] = w * (m[2][x] * m[3][y] - m[2][y] * m[3][x]);
+      }
+#pragma unroll
+    for (int a = 0; a < 4; a++) {
+      const int rho = a < 2 ? 1 - a : 5 - a;  // the remaining row of the removed row's pair
+#pragma unroll
+      for (int b = 0; b < 4; b++) {
+        const int c0 = b == 0 ? 1 : 0, c1 = b <= 1 ? 2 : 1, c2 = b == 3 ? 2 : 3;
+        const double d12 = a < 2 ? bot[c1][c2] : top[c1][c2], d02 = a < 2 ? bot[c0][c2] : top[c0][c2],
+                     d01 = a < 2 ? bot[c0][c1] : top[c0][c1];
+        const double d = m[rho][c0] * d12 - m[rho][c1] * d02 + m[rho][c2] * d01;
+        cof[a][b] = ((a + b) & 1) ? -d : d;
+      }
+    }
+  }
+  float* W = reinterpret_cast<float*>(Wsm);
+#pragma unroll
+  for (int q = 0; q < K * K; q++) {
+    float* at = W + (e.h[q / K] * M + e.p[q % K]) * ld;
+    acc3_add(at, at + plane, at + 2 * plane, cof[q / K][q % K]);
+  }
+}
+
+template <class V, int L>  // V: float2 (double-float pairs) or double
+__global__ void __launch_bounds__(512) k_scatter(DevProblem P, DevScratch S, int64_t n_walk) {
+  // pairs: [n M][L + 1] of 8 bytes; FP64: three planes [n M][L + 1] of FP32
+  extern __shared__ __align__(16) uint8_t Wsm[];
+  constexpr bool kPairs = sizeof(V) == sizeof(float2) && !std::is_same<V, double>::value;
+  constexpr int ld = L + 1, kSub = 32 / L, kWarps = 16;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int wl = lane % L, sub = lane / L;
+  const int sp = blockIdx.y, M = P.n_mo, nu = P.n_up, n = sp ? P.n_dn : nu;
+  const int nu_det = P.n_det_sp[0], ntot = nu_det + P.n_det_sp[1];
+  const int64_t w0 = (int64_t)blockIdx.x * L, w = min(w0 + wl, n_walk - 1);
+  const int slots = n * M, plane = slots * ld;
+  for (int t = threadIdx.x; t < plane * (kPairs ? 2 : 3); t += blockDim.x) reinterpret_cast<float*>(Wsm)[t] = 0.0f;
+  __syncthreads();
+  const V* T = (kPairs ? reinterpret_cast<const V*>(S.Tdf) : reinterpret_cast<const V*>(S.T)) +
+               (size_t)(sp ? nu * M : 0) * S.wp + w;
+  uint8_t* Wl = Wsm + wl * (kPairs ? 8 : 4);
+  const double* wt = S.vu + w * ntot + (sp ? nu_det : 0);
+  for (int k = 1; k <= kMaxExc; k++) {
+    const int s0 = P.deg_start[sp][k], n_k = P.deg_start[sp][k + 1] - s0;
+    // this lane's stretch: 16 warps x kSub parts of the degree's list
+    const int part = warp * kSub + sub, parts = kWarps * kSub;
+    const int b = s0 + (int)((int64_t)n_k * part / parts), e = s0 + (int)((int64_t)n_k * (part + 1) / parts);
+    for (int t = b; t < e; t++) {
+      const Exc x = P.exc[sp][t];
+      long long wb = __double_as_longlong(wt[t]);
+      if ((wb & 0x7fffffffffffffffLL) == 0) continue;
+      if (x.eps < 0) wb ^= (long long)(1ULL << 63);
+      switch (k) {
+        case 1: scatter_group<1>(x, wb, T, S.wp, M, Wl, ld, plane); break;
+        case 2: scatter_group<2>(x, wb, T, S.wp, M, Wl, ld, plane); break;
+        case 3: scatter_group<3>(x, wb, T, S.wp, M, Wl, ld, plane); break;
+        default: scatter_group<4>(x, wb, T, S.wp, M, Wl, ld, plane); break;
+      }
+    }
+  }
+  __syncthreads();
+  for (int l = warp; l < L && w0 + l < n_walk; l += kWarps) {
+    V* out = reinterpret_cast<V*>(S.W) + (w0 + l) * (int64_t)P.n_elec * M + (sp ? nu * M : 0);
+    for (int s = lane; s < slots; s += 32) {
+      if constexpr (kPairs) {
+        const unsigned long long v = reinterpret_cast<const unsigned long long*>(Wsm)[s * ld + l];
+        out[s] = make_float2(__uint_as_float((unsigned)v), __uint_as_float((unsigned)(v >> 32)));
+      } else {
+        const float* v = reinterpret_cast<const float*>(Wsm) + s * ld + l;
+        out[s] = ((double)v[0] + (double)v[plane]) + (double)v[2 * plane];
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // K6: per walker: W scatter over every determinant, Q = A^T W, Pm = T Q^T,
 // G_{i mu} = g Psi~ + sum_m d_mu phi[i][m] Q[i][m] - sum_b d_mu phi[i][o_b] Pm[b][i],
 // then grad, Laplacian, log|Psi|, sign and E_L. grid n_walk, block 128.
@@ -718,8 +885,9 @@ __global__ void __launch_bounds__(NT, MIXED ? 5 : 1) k_final(DevProblem P, DevSc
   for (int t = threadIdx.x; t < NM; t += blockDim.x) {
     if (MIXED) {
       Tdf[(t / M) * Mt + t % M] = S.Tdf[(size_t)t * wp + w];
-      Whi[t] = 0.0f;
-      Wlo[t] = 0.0f;
+      const float2 w0 = S.W ? reinterpret_cast<const float2*>(S.W)[w * NM + t] : make_float2(0.0f, 0.0f);  // already summed (k_scatter)?
+      Whi[t] = w0.x;
+      Wlo[t] = w0.y;
     } else {
       Ts[t] = S.T[(size_t)t * wp + w];
       Whi[t] = 0.0f;
@@ -743,7 +911,7 @@ __global__ void __launch_bounds__(NT, MIXED ? 5 : 1) k_final(DevProblem P, DevSc
     // ... with a prime stride that does not divide L (a permutation), so the lanes of a
     // warp hold determinants far apart in key order, which rarely share a (hole,
     // particle) slot of W, and every thread gets an even share of the group.
-    for (int grp = 0; grp < 2 * kMaxExc; grp++) {
+    for (int grp = 0; grp < (S.W ? 0 : 2 * kMaxExc); grp++) {
       const int sp = grp / kMaxExc, k = grp % kMaxExc + 1;
       const int base = sp ? nu_det : 0;
       const int s0 = P.deg_start[sp][k], L = P.deg_start[sp][k + 1] - s0;
@@ -774,7 +942,7 @@ __global__ void __launch_bounds__(NT, MIXED ? 5 : 1) k_final(DevProblem P, DevSc
     // each thread walks its own contiguous block (sequential loads of records and weights;
     // the FP64 pipe, not the balance, bounds this variant)
     const int per = (ntot + nth - 1) / nth;
-    const int n_mine = max(0, min(per, ntot - tid * per));
+    const int n_mine = S.W ? 0 : max(0, min(per, ntot - tid * per));
     for (int j = 0; j < n_mine; j++) {
       const int t = tid * per + j;
       const int sp = t < nu_det ? 0 : 1;
@@ -881,7 +1049,9 @@ __global__ void __launch_bounds__(NT, MIXED ? 5 : 1) k_final(DevProblem P, DevSc
   } else {
     // W's three words summed into FP64, through Q's space (free until Q is formed), then back
     // over the words
-    for (int t = threadIdx.x; t < NM; t += blockDim.x) Qs[t] = ((double)Whi[t] + (double)Wlo[t]) + (double)W3[t];
+    for (int t = threadIdx.x; t < NM; t += blockDim.x)
+      Qs[t] = S.W ? reinterpret_cast<const double*>(S.W)[w * NM + t]
+                  : ((double)Whi[t] + (double)Wlo[t]) + (double)W3[t];
     __syncthreads();
     double* Wd = Ws;
     for (int t = threadIdx.x; t < NM; t += blockDim.x) Wd[t] = Qs[t];
@@ -1207,6 +1377,7 @@ DevScratch scratch_view(const DevScratch& S, const DevProblem& P, int64_t off) {
   if (S.rdf) V.rdf = S.rdf + off;
   V.psit = S.psit + off;
   V.psia = S.psia + off;
+  if (S.W) V.W = S.W + off * N * M;
   return V;
 }
 
@@ -1217,6 +1388,50 @@ cudaError_t launch_spmm_rows_f64(const DevProblem& P, const double* r_dn, const 
   dim3 grid((unsigned)((nchunks + 7) / 8), (unsigned)((n_walk + 127) / 128));
   k_spmm_f64<<<grid, 256, 0, st>>>(P.csr_row, P.csr_col, P.csr_val, P.nnz, chunk, r_dn, v, ld, r_up, psit);
   return cudaGetLastError();
+}
+
+// Walkers per group of k_scatter (0: k_final's own scatter): of the groups whose accumulators fit
+// an SM, the one with the least work on the busiest SM (one block per SM at a time; smaller groups
+// leave a shorter last round, but their warps' lanes, on different determinants, meet in banks and
+// slots: groups of 16 take 1.28 times as long per walker in double-float, and groups of 8 three times;
+// in FP64, whose pipe bounds it, groups of 8 take 1.05). The blocks have to cover four fifths of the
+// SMs (900 determinants per spin, FP64 / pairs: 500 walkers 231 us against 292 / 195 against 154, 1,000
+// walkers 430 against 532 / 249 against 295), and below a few hundred distinct determinants the scatter
+// is too short to be worth a launch.
+int scatter_group_walkers(const DevProblem& P, int64_t n_walk, bool mixed) {
+  const int64_t slot_bytes = (int64_t)P.n_up * P.n_mo * (mixed ? 8 : 12), n_sm = std::max(P.n_sm, 1);
+  if (P.n_det_sp[0] + P.n_det_sp[1] < 512) return 0;
+  int best = 0;
+  double best_cost = 0;
+  for (int L : {32, 16, 8}) {
+    const int64_t blocks = 2 * ((n_walk + L - 1) / L);
+    if (slot_bytes * (L + 1) > 220 * 1024 || blocks * 5 < n_sm * 4 || (mixed && L == 8)) continue;
+    const double cost = (double)((blocks + n_sm - 1) / n_sm * L) * (L == 32 ? 1.0 : (mixed ? 1.28 : (L == 8 ? 1.05 : 1.0)));
+    if (!best || cost < best_cost) {
+      best = L;
+      best_cost = cost;
+    }
+  }
+  return best;
+}
+
+template <class V, int L>
+static cudaError_t launch_scatter_l(const DevProblem& P, const DevScratch& S, int64_t n_walk, cudaStream_t st) {
+  static SmemOptIn opt;
+  const size_t smem = (size_t)P.n_up * P.n_mo * (L + 1) * (std::is_same<V, double>::value ? 12 : 8);
+  cudaError_t e = opt.ensure(k_scatter<V, L>, smem);
+  if (e != cudaSuccess) return e;
+  k_scatter<V, L><<<dim3((unsigned)((n_walk + L - 1) / L), 2), 512, smem, st>>>(P, S, n_walk);
+  return cudaGetLastError();
+}
+
+template <class V>
+static cudaError_t launch_scatter(const DevProblem& P, const DevScratch& S, int64_t n_walk, int L, cudaStream_t st) {
+  switch (L) {
+    case 32: return launch_scatter_l<V, 32>(P, S, n_walk, st);
+    case 16: return launch_scatter_l<V, 16>(P, S, n_walk, st);
+    default: return launch_scatter_l<V, 8>(P, S, n_walk, st);
+  }
 }
 
 size_t final_smem_bytes(const DevProblem& P, bool mixed) {
@@ -1231,6 +1446,13 @@ size_t final_smem_bytes(const DevProblem& P, bool mixed) {
 cudaError_t launch_final(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R,
                          double* log_abs_psi, int8_t* sign, double* grad, double* lap, double* e_local,
                          uint32_t* status, bool mixed, cudaStream_t st, bool wide) {
+  DevScratch Sf = S;
+  const int L = S.W ? scatter_group_walkers(P, n_walk, mixed) : 0;
+  if (L == 0) Sf.W = nullptr;
+  if (L) {
+    const cudaError_t es = mixed ? launch_scatter<float2>(P, S, n_walk, L, st) : launch_scatter<double>(P, S, n_walk, L, st);
+    if (es != cudaSuccess) return es;
+  }
   const size_t smem = final_smem_bytes(P, mixed);
   // wide: 512 threads per walker (FP64 only), for a few walkers whose latency matters
   const int variant = mixed ? 1 : (wide ? 2 : 0);
@@ -1239,7 +1461,7 @@ cudaError_t launch_final(const DevProblem& P, const DevScratch& S, int64_t n_wal
   static SmemOptIn opt[3];  // dynamic shared memory per variant (static arrays come on top)
   cudaError_t e = opt[variant].ensure(kern, smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)n_walk, nt, smem, st>>>(P, S, R, log_abs_psi, sign, grad, lap, e_local, status);
+  kern<<<(unsigned)n_walk, nt, smem, st>>>(P, Sf, R, log_abs_psi, sign, grad, lap, e_local, status);
   return cudaGetLastError();
 }
 
