@@ -172,7 +172,10 @@ __device__ __forceinline__ long long block_max_ll(long long v, long long* red) {
 // d = mantissa 2^(e - L) in place and in a contiguous copy for the gathers (exact, by the
 // exponent bits; below 2^-1022 of the largest they are zero), and cleared accumulators.
 // acc layout per slot: [0] L_up ln 2, [1] L_dn ln 2, [2] Psi, [3..3+4N) G[i][mu].
-__global__ void __launch_bounds__(kFbScaleThreads) k_fb_scale(DevProblem P, DevScratch S) {
+// rw (optional): the scaled values walker-minor too, [ntot][ldw], with the largest high FP64 word of
+// each spin in xmax[2][ldw], the inputs of the residue products.
+__global__ void __launch_bounds__(kFbScaleThreads) k_fb_scale(DevProblem P, DevScratch S, double* __restrict__ rw,
+                                                              uint32_t* __restrict__ xmax, int64_t ldw) {
   const int slot = blockIdx.x;
   const int count = min(S.fb_list[0], P.fallback_cap);
   if (slot >= count) return;
@@ -204,7 +207,10 @@ __global__ void __launch_bounds__(kFbScaleThreads) k_fb_scale(DevProblem P, DevS
     }
     r[0] = d;
     dv[t] = d;
+    if (rw) rw[(size_t)t * ldw + slot] = d;
   }
+  // the largest scaled value of a spin is a mantissa in [0.5, 1): biased exponent 1022
+  if (rw && threadIdx.x < 2) xmax[threadIdx.x * ldw + slot] = 1022u << 20;
   for (int q = threadIdx.x; q < 1 + 4 * N; q += blockDim.x) acc[2 + q] = 0.0;
   if (threadIdx.x == 0) {
     acc[0] = (double)Lu * 0.69314718055994530942;
@@ -265,6 +271,55 @@ __global__ void __launch_bounds__(256) k_fb_rows(DevProblem P, DevScratch S) {
     for (int q = threadIdx.x; q < 1 + 4 * N; q += blockDim.x)
       if (G[q] != 0.0) atomicAdd(&acc[2 + q], G[q]);
     __syncthreads();
+  }
+}
+
+// The same sums from v, u (walker-major vu) and Psi of the residue products: per flagged walker, the
+// determinants' derivatives weighted by v d and u d, a warp per determinant and lanes over its 4 n
+// derivatives, items of kFbSumDets determinants of one spin. Reads each record once (its bound).
+constexpr int kFbSumDets = 512;
+
+__global__ void __launch_bounds__(256) k_fb_sum(DevProblem P, DevScratch S, const double* __restrict__ psit) {
+  const int count = min(S.fb_list[0], P.fallback_cap);
+  const int nu = P.n_up, nd = P.n_dn, nmax = max(nu, nd);
+  const int nu_det = P.n_det_sp[0], nd_det = P.n_det_sp[1], ntot = nu_det + nd_det;
+  const int stride = 2 + 4 * nmax;
+  const int n_u = (nu_det + kFbSumDets - 1) / kFbSumDets, n_it = n_u + (nd_det + kFbSumDets - 1) / kFbSumDets;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double G[8][4 * kFbMax];
+  for (int64_t item = blockIdx.x; item < (int64_t)count * n_it; item += gridDim.x) {
+    const int slot = (int)(item / n_it), it = (int)(item - (int64_t)slot * n_it);
+    const bool up = it < n_u;
+    const int n = up ? nu : nd, base = up ? 0 : nu_det, t0 = (up ? it : it - n_u) * kFbSumDets;
+    const int t1 = min(t0 + kFbSumDets, up ? nu_det : nd_det);
+    const double* rec = S.fb + ((size_t)slot * ntot + base) * stride;
+    const double* v = S.vu + (size_t)slot * ntot + base;
+    double a[(4 * kFbMax + 31) / 32];
+#pragma unroll
+    for (int j = 0; j < (4 * kFbMax + 31) / 32; j++) a[j] = 0.0;
+    for (int t = t0 + warp; t < t1; t += 8) {
+      const double* r = rec + (size_t)t * stride;
+      const double vd = v[t] * r[0];
+      if (vd == 0.0) continue;
+#pragma unroll
+      for (int j = 0; j < (4 * kFbMax + 31) / 32; j++) {
+        const int q = lane + 32 * j;
+        if (q < 4 * n) a[j] = fma(vd, r[2 + q], a[j]);
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < (4 * kFbMax + 31) / 32; j++)
+      if (lane + 32 * j < 4 * n) G[warp][lane + 32 * j] = a[j];
+    __syncthreads();
+    double* acc = S.fb_acc + (size_t)slot * (3 + 4 * 2 * kFbMax);
+    for (int q = threadIdx.x; q < 4 * n; q += blockDim.x) {
+      double s = 0.0;
+#pragma unroll
+      for (int p = 0; p < 8; p++) s += G[p][q];
+      atomicAdd(&acc[3 + (up ? 0 : 4 * nu) + q], s);
+    }
+    if (it == 0 && threadIdx.x == 0) acc[2] = psit[slot];
   }
 }
 
@@ -424,13 +479,33 @@ cudaError_t launch_fallback(const DevProblem& P, const DevScratch& S, int64_t n_
   dim3 g1((ntot + tpb - 1) / tpb, P.fallback_cap);
   k_fb_dets<<<g1, tpb, smem, st>>>(P, S);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_fb_scale<<<P.fallback_cap, kFbScaleThreads, 0, st>>>(P, S);
+  // many flagged walkers (FP64 at its own tolerance: hundreds): their contraction as residue products
+  // too, 0.4 ms instead of 3.6 for 410 walkers and 750k products
+  const int64_t ldw = (P.fallback_cap + kWalkerPad - 1) / kWalkerPad * kWalkerPad;
+  const bool dense = S.fb_r && S.xmax && !S.live;
+  k_fb_scale<<<P.fallback_cap, kFbScaleThreads, 0, st>>>(P, S, dense ? S.fb_r : nullptr, S.fb_xmax, ldw);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   static int n_sm = 0;
   if (!n_sm) {
     int dev = 0;
     cudaGetDevice(&dev);
     if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm <= 0) n_sm = 132;
+  }
+  if (dense) {
+    DevScratch F = S;  // the listed walkers' determinant values in place of ratios
+    F.r = S.fb_r;
+    F.xmax = S.fb_xmax;
+    F.wp = ldw;
+    F.live = S.fb_list;  // (a count beyond the cap: the cap bounds the launch)
+    F.psit = S.fb_psi;
+    const int64_t n_fb = std::min<int64_t>(P.fallback_cap, S.wp);
+    if ((e = launch_contract_dense(P, F, n_fb, st, nullptr, nullptr)) != cudaSuccess) return e;
+    const int64_t sums = (int64_t)P.fallback_cap * ((P.n_det_sp[0] + kFbSumDets - 1) / kFbSumDets +
+                                                    (P.n_det_sp[1] + kFbSumDets - 1) / kFbSumDets);
+    k_fb_sum<<<(unsigned)std::min<int64_t>(sums, 8 * n_sm), 256, 0, st>>>(P, S, S.fb_psi);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    k_fb_out<<<P.fallback_cap, 64, 0, st>>>(P, S, R, log_abs_psi, sign, grad, lap, e_local, status);
+    return cudaGetLastError();
   }
   const int64_t items = (int64_t)P.fallback_cap * ((ntot + kFbRowsPerItem - 1) / kFbRowsPerItem);
   k_fb_rows<<<(unsigned)std::min<int64_t>(items, 4 * n_sm), 256, 0, st>>>(P, S);

@@ -357,7 +357,7 @@ void pick_items(const mdet_ctx* c, DevProblem& P, int64_t n_walk) {
 
 void free_arrays(DevScratch& S) {
   void* ptrs[] = {S.phi, S.Ainv, S.ld0, S.sg0, S.g, S.kap, S.est, S.T, S.Tdf, S.r, S.rdf, S.vu, S.psit, S.psia, S.wstat,
-                  S.xmax, S.dx, S.dy, S.dyabs, S.derr, S.xd, S.xer, S.W,
+                  S.xmax, S.dx, S.dy, S.dyabs, S.derr, S.xd, S.xer, S.W, S.fb_r, S.fb_xmax, S.fb_psi,
                   S.fb, S.fb_list, S.fb_acc, S.queue, S.R_stage, S.out_stage};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -790,6 +790,19 @@ mdet_status alloc_fallback(mdet_ctx* c, DevScratch& S) {
   mdet_status s;
   if ((s = dalloc(c, &S.fb, (size_t)P.fallback_cap * ndt * (3 + 4 * nmax)))) return s;
   if ((s = dalloc(c, &S.fb_list, (size_t)P.fallback_cap + 1))) return s;
+  if (S.xmax && c->precision == MDET_PRECISION_FP64) {
+    const int64_t ldw = (P.fallback_cap + kWalkerPad - 1) / kWalkerPad * kWalkerPad;
+    if (cudaMalloc((void**)&S.fb_r, sizeof(double) * ndt * ldw) != cudaSuccess ||
+        cudaMalloc((void**)&S.fb_xmax, sizeof(uint32_t) * 2 * ldw) != cudaSuccess ||
+        cudaMalloc((void**)&S.fb_psi, sizeof(double) * ldw) != cudaSuccess) {  // no room: the sparse sums
+      cudaGetLastError();
+      if (S.fb_r) cudaFree(S.fb_r);
+      S.fb_r = nullptr;
+    } else {
+      CUDA_TRY(c, cudaMemset(S.fb_r, 0, sizeof(double) * ndt * ldw));
+      CUDA_TRY(c, cudaMemset(S.fb_xmax, 0, sizeof(uint32_t) * 2 * ldw));
+    }
+  }
   return dalloc(c, &S.fb_acc, (size_t)P.fallback_cap * (3 + 8 * MDET_FALLBACK_MAX_SPIN));
 }
 
@@ -1458,8 +1471,11 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
     if (es != MDET_OK) return es;
     c->last_kernels += 3 + 5 + (table ? mo_kernels(P, c->E, P.fallback_cap, false) + (c->E.xmax ? 6 : 4) : 1 + 1);
   } else {
-    CUDA_TRY(c, launch_fallback(P, c->S, n_walk, R, log_abs_psi, sign, grad, lap, e_local, status, st));
-    if (P.fallback_tol > 0.0 && c->S.fb && P.n_up <= MDET_FALLBACK_MAX_SPIN) c->last_kernels += 5;
+    DevScratch Sb = c->S;
+    if (!dense) Sb.xmax = nullptr;
+    CUDA_TRY(c, launch_fallback(P, Sb, n_walk, R, log_abs_psi, sign, grad, lap, e_local, status, st));
+    if (P.fallback_tol > 0.0 && c->S.fb && P.n_up <= MDET_FALLBACK_MAX_SPIN)
+      c->last_kernels += dense && c->S.fb_r ? 8 : 5;
   }
   if (prof_all) {
     CUDA_TRY(c, cudaEventRecord(c->ev_refine[1], st));

@@ -170,6 +170,11 @@ struct DevScratch {
   int64_t xd_walk = 0;
   uint32_t* wstat = nullptr;  // [W] status bits
   double* fb = nullptr;       // fallback: [cap][n_det_up + n_det_dn][2 + 4 max(n_up, n_dn)], then [cap][ndt] values
+  // FP64 path with residue products: the listed walkers' determinant values walker-minor, their largest
+  // magnitudes and Psi sums
+  double* fb_r = nullptr;
+  uint32_t* fb_xmax = nullptr;
+  double* fb_psi = nullptr;
   int* fb_list = nullptr;     // fallback: [1 + cap] count, then walker indices
   double* fb_acc = nullptr;   // fallback: [cap][3 + 8 MDET_FALLBACK_MAX_SPIN] scales, Psi, G
   unsigned long long* queue = nullptr;  // [6 * walker chunks] per chunk: the work counters of its two

@@ -855,7 +855,7 @@ __global__ void __launch_bounds__(512) k_scatter(DevProblem P, DevScratch S, int
 // smem, MIXED: W[N][M] as hi/lo FP32 arrays, Q[N][M], A blocks, Pm (all pairs),
 //       Tdf[N][M].
 template <bool MIXED, int NT>
-__global__ void __launch_bounds__(NT, MIXED ? 5 : 1) k_final(DevProblem P, DevScratch S, const double* __restrict__ R,
+__global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 1)) : 1) k_final(DevProblem P, DevScratch S, const double* __restrict__ R,
                                                double* __restrict__ log_abs_psi, int8_t* __restrict__ sign,
                                                double* __restrict__ grad, double* __restrict__ lap,
                                                double* __restrict__ e_local, uint32_t* __restrict__ status) {
@@ -1454,12 +1454,14 @@ cudaError_t launch_final(const DevProblem& P, const DevScratch& S, int64_t n_wal
     if (es != cudaSuccess) return es;
   }
   const size_t smem = final_smem_bytes(P, mixed);
-  // wide: 512 threads per walker (FP64 only), for a few walkers whose latency matters
-  const int variant = mixed ? 1 : (wide ? 2 : 0);
-  auto kern = variant == 1 ? k_final<true, 128> : (variant == 2 ? k_final<false, 512> : k_final<false, 128>);
-  const int nt = variant == 2 ? 512 : 128;
-  static SmemOptIn opt[3];  // dynamic shared memory per variant (static arrays come on top)
-  cudaError_t e = opt[variant].ensure(kern, smem);
+  // threads per walker: 512 for a few walkers (fewer than SMs, or `wide`), whose latency matters; 256
+  // where the walker's tables let fewer than five blocks on an SM (34 electrons, 103 MOs, 94 KB of
+  // pairs: 1.23 ms for 2,161 walkers with 128); else 128
+  const int nt = wide || n_walk < P.n_sm ? 512 : (smem > 45 * 1024 ? 256 : 128);
+  auto kern = mixed ? (nt == 512 ? k_final<true, 512> : (nt == 256 ? k_final<true, 256> : k_final<true, 128>))
+                    : (nt == 512 ? k_final<false, 512> : (nt == 256 ? k_final<false, 256> : k_final<false, 128>));
+  static SmemOptIn opt[2][3];  // dynamic shared memory per variant (static arrays come on top)
+  cudaError_t e = opt[mixed][nt == 512 ? 2 : nt / 128 - 1].ensure(kern, smem);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)n_walk, nt, smem, st>>>(P, Sf, R, log_abs_psi, sign, grad, lap, e_local, status);
   return cudaGetLastError();

@@ -119,4 +119,24 @@ def test_dense_rows_take_smaller_moduli():
     ctx = pkg.Context.from_workload(wl, device=0)
     rep = compare(_eval(ctx, wl.R), oracle.evaluate(wl), **TOL[pkg.PRECISION_FP64])
     assert rep["ok"], rep
-    assert ctx.last_kernels == 13
+    assert ctx.last_kernels == 8 + 8  # the residue products, and the full-LU fallback with its own
+
+
+@pytest.mark.parametrize("n_walk", [5, 300])
+def test_full_lu_contraction(n_walk):
+    """Every walker through full LU (a tolerance below any estimate): its contraction as residue
+    products, against the oracle and against the sparse sums."""
+    wl = _workload(130, 70, n_walk)
+    ctx = pkg.Context.from_workload(wl, device=0)
+    ctx.set_fallback(1e-30, 512)
+    got = _eval(ctx, wl.R)
+    assert ctx.last_kernels == 8 + 8 and np.all(got["status"] & pkg.WS_FALLBACK)
+    ref = oracle.evaluate(wl)
+    rep = compare(got, ref, **TOL[pkg.PRECISION_FP64])
+    assert rep["ok"], rep
+    ctx.set_tuning(spmm_blocks=SPARSE_GRID)
+    sparse = _eval(ctx, wl.R)
+    assert ctx.last_kernels == 6 + 5
+    tol = 200 * 2.0 ** -53 * np.maximum(ref["kappa"], 1.0) + 4 * np.spacing(np.abs(ref["log_abs_psi"]))
+    assert np.all(np.abs(got["log_abs_psi"] - sparse["log_abs_psi"]) <= tol)
+    assert np.array_equal(got["sign"], sparse["sign"]) and np.array_equal(got["status"], sparse["status"])
