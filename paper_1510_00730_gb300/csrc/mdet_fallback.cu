@@ -275,8 +275,9 @@ __global__ void __launch_bounds__(256) k_fb_rows(DevProblem P, DevScratch S) {
 }
 
 // The same sums from v, u (walker-major vu) and Psi of the residue products: per flagged walker, the
-// determinants' derivatives weighted by v d and u d, a warp per determinant and lanes over its 4 n
-// derivatives, items of kFbSumDets determinants of one spin. Reads each record once (its bound).
+// determinants' derivatives weighted by v d and u d, in items of kFbSumDets determinants of one spin.
+// A warp takes 8 determinants at a time, whose 32 n derivatives are n full rows of lanes: element
+// 32 j + lane always belongs to the same derivative, so each lane keeps n sums.
 constexpr int kFbSumDets = 512;
 
 __global__ void __launch_bounds__(256) k_fb_sum(DevProblem P, DevScratch S, const double* __restrict__ psit) {
@@ -286,40 +287,39 @@ __global__ void __launch_bounds__(256) k_fb_sum(DevProblem P, DevScratch S, cons
   const int stride = 2 + 4 * nmax;
   const int n_u = (nu_det + kFbSumDets - 1) / kFbSumDets, n_it = n_u + (nd_det + kFbSumDets - 1) / kFbSumDets;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  __shared__ double G[8][4 * kFbMax];
+  __shared__ double G[4 * kFbMax];
   for (int64_t item = blockIdx.x; item < (int64_t)count * n_it; item += gridDim.x) {
     const int slot = (int)(item / n_it), it = (int)(item - (int64_t)slot * n_it);
     const bool up = it < n_u;
-    const int n = up ? nu : nd, base = up ? 0 : nu_det, t0 = (up ? it : it - n_u) * kFbSumDets;
+    const int n = up ? nu : nd, n4 = 4 * n, base = up ? 0 : nu_det, t0 = (up ? it : it - n_u) * kFbSumDets;
     const int t1 = min(t0 + kFbSumDets, up ? nu_det : nd_det);
     const double* rec = S.fb + ((size_t)slot * ntot + base) * stride;
     const double* v = S.vu + (size_t)slot * ntot + base;
-    double a[(4 * kFbMax + 31) / 32];
+    for (int q = threadIdx.x; q < n4; q += blockDim.x) G[q] = 0.0;
+    __syncthreads();
+    double a[kFbMax];
 #pragma unroll
-    for (int j = 0; j < (4 * kFbMax + 31) / 32; j++) a[j] = 0.0;
-    for (int t = t0 + warp; t < t1; t += 8) {
-      const double* r = rec + (size_t)t * stride;
-      const double vd = v[t] * r[0];
-      if (vd == 0.0) continue;
+    for (int j = 0; j < kFbMax; j++) a[j] = 0.0;
+    for (int t = t0 + 8 * warp; t < t1; t += 64) {
+      // the weights v d of the warp's determinants, in lanes 0-7
+      const int td = t + (lane & 7);
+      const double vd = td < t1 ? v[td] * rec[(size_t)td * stride] : 0.0;
 #pragma unroll
-      for (int j = 0; j < (4 * kFbMax + 31) / 32; j++) {
-        const int q = lane + 32 * j;
-        if (q < 4 * n) a[j] = fma(vd, r[2 + q], a[j]);
+      for (int j = 0; j < kFbMax; j++) {
+        if (j >= n) break;
+        const int x = 32 * j + lane, d = x / n4, q = x - d * n4;
+        const double w = __shfl_sync(0xffffffffu, vd, d);
+        if (w != 0.0) a[j] = fma(w, rec[(size_t)(t + d) * stride + 2 + q], a[j]);
       }
     }
-    __syncthreads();
 #pragma unroll
-    for (int j = 0; j < (4 * kFbMax + 31) / 32; j++)
-      if (lane + 32 * j < 4 * n) G[warp][lane + 32 * j] = a[j];
+    for (int j = 0; j < kFbMax; j++)
+      if (j < n) atomicAdd(&G[(32 * j + lane) % n4], a[j]);
     __syncthreads();
     double* acc = S.fb_acc + (size_t)slot * (3 + 4 * 2 * kFbMax);
-    for (int q = threadIdx.x; q < 4 * n; q += blockDim.x) {
-      double s = 0.0;
-#pragma unroll
-      for (int p = 0; p < 8; p++) s += G[p][q];
-      atomicAdd(&acc[3 + (up ? 0 : 4 * nu) + q], s);
-    }
+    for (int q = threadIdx.x; q < n4; q += blockDim.x) atomicAdd(&acc[3 + (up ? 0 : 4 * nu) + q], G[q]);
     if (it == 0 && threadIdx.x == 0) acc[2] = psit[slot];
+    __syncthreads();
   }
 }
 
