@@ -70,10 +70,10 @@ struct DenseContract {
   uint16_t* planes[2];   // BF16 residue planes of C and C^T; the two magnitude planes of C
   const int* es[2];      // [n_det_sp[o]] exponents of the rows of C and of C^T
   ModConst m[kMaxModuli];
-  uint32_t M4[kMaxModuli][4];  // reconstruction weights modulo 2^128
-  uint32_t F[kMaxModuli];      // 2^32 ((P / p)^-1 mod p) / p
-  uint32_t init4[4], P4[4];
-  long long finit;
+  // reconstruction weights modulo 2^128 in 16-bit limbs, and (limb 8) 2^16 ((P / p)^-1 mod p) / p, the
+  // two moduli of a pair in the halves of a word; the limbs of P; the initial sums
+  uint32_t M2[kMaxModuli / 2][9];
+  uint32_t P8[8], init9[9];
 };
 
 // Read-only problem description resident on the device.

@@ -21,8 +21,8 @@
 //    the actual residues when the moduli are chosen) keeps every partial sum of the FP32
 //    accumulator an exact integer. The accumulators are reduced mod p_q to one byte.
 //  - Reconstruction: X = sum_q y_q M_q - k P with M_q = (P / p_q) ((P / p_q)^-1 mod p_q),
-//    P = prod p_q > 2^124.6 and k = rint(sum_q y_q ((P / p_q)^-1 mod p_q) / p_q), in 128-bit
-//    wrap-around integers: X is exact, and v_i = RN(X) 2^(es_i + xe_w - 123).
+//    P = prod p_q > 2^124.6 and k = rint(sum_q y_q ((P / p_q)^-1 mod p_q) / p_q) (|X| / P < 0.36, and
+//    16-bit fractions put the sum within 0.05), in 128-bit wrap-around integers: X is exact, and v_i = RN(X) 2^(es_i + xe_w - 123).
 //  - The magnitude sum behind Psi~ (sum_j |c_ij| |r_j|, for the error estimate) rides along as
 //    one more product: both magnitudes as a BF16 pair h + l (2^-17 relative), h h + h l + l h
 //    in one FP32 accumulator.
@@ -44,6 +44,8 @@ namespace {
 constexpr int kCBits = 61, kRBits = 62;  // fixed-point fractions of C rows and of a walker's ratios
 constexpr int kTileBytes = 128 * 64 * 2;  // 128 walkers x 64 determinants of one plane
 constexpr int kMinP = 16, kMaxP = 256;
+constexpr uint32_t kMaxQuotient = 4096;  // above |sum_q y_q ((P / p_q)^-1 mod p_q) / p_q| <= 128 kMaxModuli
+static_assert(128 * kMaxModuli < (int)kMaxQuotient, "quotient offset");
 
 __device__ __forceinline__ long long c_fixed(double c, int es) { return __double2ll_rn(scalbn(c, kCBits - es)); }
 
@@ -482,11 +484,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
 
 // Reconstruction of v and u from the residue bytes, with Psi~ = r_up . v and its magnitude sum:
 // a warp per walker and product, four consecutive determinants per lane (one 4-byte load per
-// modulus, all issued before the arithmetic). Every walker's Psi~ is summed in one warp, in a
-// fixed order. Stores go through shared memory so that a warp writes 256 consecutive bytes.
-__global__ void __launch_bounds__(256) k_mod_crt(const __grid_constant__ DenseContract D, DevProblem P, DevScratch S,
+// modulus, all issued before the arithmetic). Bound by instruction issue and the loads' latency at 24
+// warps an SM, not by its 25 bytes a determinant. The weighted sums run in 16-bit limbs with dp2a, two
+// moduli at a time, and each weight is fetched once for four determinants: 0.82 ms at 8192 walkers of
+// 750000 determinants in FP64 or mixed, against 1.22 ms with 32-bit limbs in 64-bit multiply-adds and
+// 1.15 ms with two determinants per lane (the constant loads then bound it). Q, the pairs of moduli,
+// is a template argument for the usual counts: unrolled to the largest it takes 0.88 ms. Every
+// walker's Psi~ is summed in one warp, in a fixed order. Stores go through shared memory so that a
+// warp writes 256 consecutive bytes.
+template <int Q>
+__global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ DenseContract D, DevProblem P, DevScratch S,
                                                  int64_t w0, int64_t n_walk, int nmt, int n_abs) {
-  __shared__ double tile[8][128];
+  __shared__ double2 tile[8][64];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int o = warp >> 2;  // warps 0-3: v of four walkers, 4-7: u of the same
   const int64_t wl = (int64_t)blockIdx.x * 4 + (warp & 3), w = w0 + wl;
@@ -527,58 +536,61 @@ __global__ void __launch_bounds__(256) k_mod_crt(const __grid_constant__ DenseCo
     for (int base = 0; base < n; base += 128) {
       const int i0 = base + 4 * lane;
       if (i0 < ldy) {
-        unsigned long long s[4][4];
-        long long kf[4];
+        // sums over the moduli of residue byte x weight in 16-bit limbs (and the quotient's, limb 8): the
+        // bytes of two moduli against their two weights with one dp2a per determinant and limb
+        uint32_t a[4][9];
 #pragma unroll
-        for (int z = 0; z < 4; z++) {
-          kf[z] = D.finit;
+        for (int l = 0; l < 9; l++) a[0][l] = a[1][l] = a[2][l] = a[3][l] = D.init9[l];
+        uint32_t yw[2 * Q];  // all the loads first
 #pragma unroll
-          for (int j = 0; j < 4; j++) s[z][j] = D.init4[j];
-        }
-        uint32_t yw[kMaxModuli];  // all the loads first
+        for (int q = 0; q < 2 * Q; q++)
+          yw[q] = q < D.nm ? __ldg(reinterpret_cast<const uint32_t*>(y + q * yplane + i0)) : 0u;
 #pragma unroll
-        for (int q = 0; q < kMaxModuli; q++)
-          if (q < D.nm) yw[q] = __ldg(reinterpret_cast<const uint32_t*>(y + q * yplane + i0));
+        for (int q = 0; q < 2 * Q; q += 2) {
+          const uint32_t y01 = __byte_perm(yw[q], yw[q + 1], 0x5140), y23 = __byte_perm(yw[q], yw[q + 1], 0x7362);
 #pragma unroll
-        for (int q = 0; q < kMaxModuli; q++) {
-          if (q >= D.nm) break;
-          const uint32_t yb = yw[q];
-          const uint32_t m0 = D.M4[q][0], m1 = D.M4[q][1], m2 = D.M4[q][2], m3 = D.M4[q][3], F = D.F[q];
-#pragma unroll
-          for (int z = 0; z < 4; z++) {
-            const uint32_t b = (yb >> (8 * z)) & 0xffu;
-            s[z][0] += (unsigned long long)b * m0;
-            s[z][1] += (unsigned long long)b * m1;
-            s[z][2] += (unsigned long long)b * m2;
-            s[z][3] += (uint32_t)(b * m3);
-            kf[z] += (long long)((unsigned long long)b * F);
+          for (int l = 0; l < 9; l++) {
+            const uint32_t m = D.M2[q / 2][l];
+            a[0][l] = __dp2a_lo(m, y01, a[0][l]);
+            a[1][l] = __dp2a_hi(m, y01, a[1][l]);
+            a[2][l] = __dp2a_lo(m, y23, a[2][l]);
+            a[3][l] = __dp2a_hi(m, y23, a[3][l]);
           }
         }
+        double v[4];
 #pragma unroll
         for (int z = 0; z < 4; z++) {
-          const unsigned long long t1 = s[z][1] + (s[z][0] >> 32), t2 = s[z][2] + (t1 >> 32), t3 = s[z][3] + (t2 >> 32);
-          unsigned __int128 X = ((unsigned __int128)((t3 << 32) | (uint32_t)t2) << 64) | ((t1 << 32) | (uint32_t)s[z][0]);
-          const long long k = (kf[z] + 0x80000000LL) >> 32;
-          const unsigned __int128 Pm = ((unsigned __int128)(((unsigned long long)D.P4[3] << 32) | D.P4[2]) << 64) |
-                                       (((unsigned long long)D.P4[1] << 32) | D.P4[0]);
-          X -= (unsigned __int128)(__int128)k * Pm;
+          const uint32_t k = kMaxQuotient - (uint32_t)((int)(a[z][8] + (1u << 15)) >> 16);  // > 0
+          uint32_t w[4], carry = 0;
+#pragma unroll
+          for (int l = 0; l < 8; l += 2) {  // X + (k - kMaxQuotient) P, the constant in the initial limbs
+            const uint32_t c0 = a[z][l] + k * D.P8[l] + carry, c1 = a[z][l + 1] + k * D.P8[l + 1] + (c0 >> 16);
+            w[l / 2] = __byte_perm(c0, c1, 0x5410);
+            carry = c1 >> 16;
+          }
           const int i = i0 + z;
-          tile[warp][4 * lane + z] =
-              i < n ? i128_to_double((unsigned long long)(X >> 64), (unsigned long long)X, e0 + D.es[o][i]) : 0.0;
+          v[z] = i < n ? i128_to_double(((unsigned long long)w[3] << 32) | w[2],
+                                        ((unsigned long long)w[1] << 32) | w[0], e0 + D.es[o][i])
+                       : 0.0;
         }
+        tile[warp][2 * lane] = make_double2(v[0], v[1]);
+        tile[warp][2 * lane + 1] = make_double2(v[2], v[3]);
       }
       __syncwarp();
 #pragma unroll
       for (int j = 0; j < 4; j++) {
         const int i = base + 32 * j + lane;
         if (i < n) {
-          const double v = tile[warp][32 * j + lane];
+          const double v = reinterpret_cast<const double*>(tile[warp])[32 * j + lane];
           out[i] = v;
           if (!o) {
             const double ri = S.r[(size_t)i * wp + w];
             psi = fma(ri, v, psi);
-            if (n_abs)
-              pa = fmaf(abs_f32_of(ri), ldexpf(S.dyabs[(size_t)wl * ldy + i], D.es[0][i] + xb - 1022), pa);
+            if (n_abs) {
+              const int es = D.es[0][i];
+              const float m = S.dyabs[(size_t)wl * ldy + i];
+              pa = fmaf(abs_f32_of(ri), es >= -126 && es <= 127 ? m * __int_as_float((es + 127) << 23) : ldexpf(m, es), pa);
+            }
           }
         }
       }
@@ -593,7 +605,9 @@ __global__ void __launch_bounds__(256) k_mod_crt(const __grid_constant__ DenseCo
   }
   if (lane == 0) {
     S.psit[w] = psi;
-    if (!S.live) S.psia[w] = pa;  // a re-evaluation keeps the sum of the evaluation that flagged it
+    // a re-evaluation keeps the sum of the evaluation that flagged it. The columns' power of two, at least
+    // 2, is left to the end; the FP64 sum above carries none
+    if (!S.live) S.psia[w] = xb >= 0x7ff || failed ? pa : ldexpf(pa, xb - 1022);
   }
 }
 
@@ -644,17 +658,21 @@ bool choose_moduli(const uint32_t* rowmax, DenseContract* D) {
     int inv = 1;
     while (inv * om % p != 1 % p) inv++;
     const u128 M = others * (u128)inv;
-    for (int j = 0; j < 4; j++) D->M4[q][j] = (uint32_t)(M >> (32 * j));
-    D->F[q] = (uint32_t)std::llrint(4294967296.0 * inv / p);
+    const uint32_t F = (uint32_t)std::llrint(65536.0 * inv / p);
+    for (int l = 0; l < 9; l++) {
+      const uint32_t limb = l < 8 ? (uint32_t)(M >> (16 * l)) & 0xffffu : F;
+      D->M2[q / 2][l] |= limb << (16 * (q % 2));
+    }
     init -= (u128)128 * M;  // the bytes are residues + 128
-    fi -= 128LL * (long long)D->F[q];
+    fi -= 128LL * (long long)F;
     D->m[q] = mod_const(p);
   }
-  for (int j = 0; j < 4; j++) {
-    D->P4[j] = (uint32_t)(Pm >> (32 * j));
-    D->init4[j] = (uint32_t)(init >> (32 * j));
+  init -= (u128)kMaxQuotient * Pm;
+  for (int l = 0; l < 8; l++) {
+    D->P8[l] = (uint32_t)(Pm >> (16 * l)) & 0xffffu;
+    D->init9[l] = (uint32_t)(init >> (16 * l)) & 0xffffu;
   }
-  D->finit = fi;
+  D->init9[8] = (uint32_t)fi;
   return true;
 }
 
@@ -717,7 +735,8 @@ cudaError_t launch_contract_dense(const DevProblem& P, const DevScratch& S, int6
     const int64_t units = (int64_t)(nmt / 2) * ((int64_t)(D.nm + n_abs) * D.nt[0] + (int64_t)D.nm * D.nt[1]);
     const int64_t pairs = std::min<int64_t>(units, std::max(P.n_sm / 2, 1));
     k_mod_gemm<<<(unsigned)(2 * pairs), 256, smem, st>>>(D, a);
-    k_mod_crt<<<(unsigned)((nb + 3) / 4), 256, 0, st>>>(D, P, S, w0, n_walk, nmt, n_abs);
+    auto* crt = D.nm <= 16 ? k_mod_crt<8> : D.nm <= 18 ? k_mod_crt<9> : k_mod_crt<kMaxModuli / 2>;
+    crt<<<(unsigned)((nb + 3) / 4), 256, 0, st>>>(D, P, S, w0, n_walk, nmt, n_abs);
     if (n_kernels) *n_kernels += 3;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
