@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(128) k_mo_f64(DevProblem P, double* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// K2+K3: reference inverse and tables. grid n_walk, block 64: warp s factorises
+// K2+K3: reference inverse and tables. grid n_walk, block 64 or 256: warp s < 2 factorises
 // spin s by Gauss-Jordan elimination with partial pivoting on [S | I] (rows
 // stay in their lanes; the pivot order is a permutation whose parity enters
 // the sign of the determinant). Then every thread computes T and g.
@@ -99,9 +99,19 @@ __global__ void __launch_bounds__(128) k_mo_f64(DevProblem P, double* __restrict
 // stay FP64, while A is rounded to double-float pairs (written to Ainv as pairs),
 // and T = A Phi and g are formed in double-float on the FP32 pipe (written to Tdf
 // and, as pairs, to g); the FP64 table is not written.
+// Bound by latency: a step of the elimination depends on the one before, and 2 warps a block fill
+// an SM only if its shared memory is small. Sized by the electrons instead of for 32 a spin (32 KB:
+// 7 blocks an SM), with the pivot search over the lanes and n active columns: 0.54 -> 0.28 ms at
+// 8192 walkers of 9 + 8 electrons (pairs; FP64 0.47 -> 0.35), 0.70 -> 0.37 ms at 2161 of 17 + 17.
+// Up to kRefFewBlocks walkers an SM the blocks are all resident at once and one of them runs alone
+// in time: 256 threads then share the tables (256 walkers of 17 + 17: 0.16 -> 0.06 ms); beyond
+// that the two warps' elimination would leave the other six waiting in too many slots.
+constexpr int kRefThreadsFew = 256, kRefFewBlocks = 4;
 template <bool MIXED>
-__global__ void __launch_bounds__(64) k_ref(DevProblem P, DevScratch S) {
-  __shared__ double aug[2][kMaxSpin][2 * kMaxSpin];
+__global__ void __launch_bounds__(kRefThreadsFew, 4) k_ref(DevProblem P, DevScratch S) {
+  extern __shared__ double ref_smem[];  // ref_smem_bytes(P): [2][n][2 n + 1], n the larger spin
+  const int nx = max(P.n_up, P.n_dn), pitch = 2 * nx + 1;
+  auto aug = [&](int sp, int i, int c) -> double& { return ref_smem[(sp * nx + i) * pitch + c]; };
   __shared__ int rowof[2][kMaxSpin];  // pivot row of column a: the row of R that holds row a of A
   __shared__ int bad[2];
   __shared__ uint32_t stf[2];
@@ -109,24 +119,32 @@ __global__ void __launch_bounds__(64) k_ref(DevProblem P, DevScratch S) {
   if (S.live && w >= *S.live) return;
   const int N = P.n_elec, M = P.n_mo;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  {
+  if (warp < 2) {
     // Gauss-Jordan elimination on [S | I] with partial pivoting, lanes owning columns: for
     // column j the pivot row p_j is the unused row of largest |S[i][j]|, row p_j is scaled
     // by 1/pivot and column j is eliminated from every other row. Rows stay in place, so
-    // at the end the left half is the permutation L[p_j][j] = 1, the right half R = L S^-1,
+    // at the end the left half would be the permutation L[p_j][j] = 1 (finished columns are
+    // left as they are), the right half R = L S^-1,
     // row a of A = S^-1 is row p_a of R, and det S = sgn(j -> p_j) * prod of the pivots.
-    // Pivot magnitudes are compared in FP32 from the FP64 bits, and |prod of pivots| is
-    // carried as mantissa * 2^exponent with one log at the end, so the FP64 pipe only sees
-    // the elimination itself (n FMAs per lane and column step), one reciprocal per pivot
+    // At step j only n columns are neither finished nor still those of the identity: the left
+    // ones after j and the right ones of the pivot rows so far. Lane l has the left column l
+    // until step l and the right column p_l from then on, so that a step is one pass of the
+    // FP64 pipe over n rows at any n. The rows go by in groups of four, loads before stores:
+    // one by one the two loads, the FMA and the store of a row are a chain.
+    // Pivot magnitudes are compared in FP32 from the FP64 bits (a row per lane, the first of
+    // the largest), and |prod of pivots| is carried as mantissa * 2^exponent with one log at the
+    // end, so the FP64 pipe only sees the elimination itself, one reciprocal per pivot
     // and one product per pivot.
     const int sp = warp;
     const int n = sp ? P.n_dn : P.n_up, e0 = sp ? P.n_up : 0;
     const int* occ = P.ref_occ + sp * kMaxSpin;
-    for (int c = lane; c < 2 * n; c += 32)
+    for (int c = lane; c < 2 * n; c += 32) {
+      const int m = c < n ? occ[c] : 0;
+#pragma unroll 4
       for (int i = 0; i < n; i++) {
         double v = (c - n == i) ? 1.0 : 0.0;
         if (c < n) {
-          const size_t ix = ((w * 5 + 0) * N + e0 + i) * M + occ[c];
+          const size_t ix = ((w * 5 + 0) * N + e0 + i) * M + m;
           if (MIXED) {
             const float2 f = reinterpret_cast<const float2*>(S.phi)[ix];
             v = df_to_double_int(df32(f.x, f.y));
@@ -134,45 +152,41 @@ __global__ void __launch_bounds__(64) k_ref(DevProblem P, DevScratch S) {
             v = S.phi[ix];
           }
         }
-        aug[sp][i][c] = v;
+        aug(sp, i, c) = v;
       }
+    }
     __syncwarp();
     // |S|_1: the largest column sum (FP32 magnitudes suffice for a conditioning estimate)
     float cs = 0.0f;
     for (int c = lane; c < n; c += 32) {
       float s = 0.0f;
-      for (int i = 0; i < n; i++) s += abs_f32_of(aug[sp][i][c]);
+      for (int i = 0; i < n; i++) s += abs_f32_of(aug(sp, i, c));
       cs = fmaxf(cs, s);
     }
 #pragma unroll
     for (int off = 16; off; off >>= 1) cs = fmaxf(cs, __shfl_xor_sync(0xffffffffu, cs, off));
     const float normS = cs;
-    uint32_t used = 0u;
-    double pm = 1.0;  // |prod of pivots| = pm 2^pe, pm in [0.5, 1)
+    bool used = lane >= n;  // row `lane` has been a pivot row
+    int col = lane;         // this lane's column
+    double pm = 1.0;        // |prod of pivots| = pm 2^pe, pm in [0.5, 1)
     int pe = 0, negs = 0, singular = 0;
     float pmax = 0.0f, pmin = FLT_MAX;
     for (int j = 0; j < n; j++) {
-      int p = -1;
-      if (lane == (j & 31)) {
-        float best = 0.0f;
-        for (int i = 0; i < n; i++) {  // integer and FP32 tests only
-          const long long xb = __double_as_longlong(aug[sp][i][j]);
-          const float v = abs_f32_of(aug[sp][i][j]);
-          if (!((used >> i) & 1u) && (v > best || (p < 0 && (xb << 1) != 0))) {
-            best = v;
-            p = i;
-          }
-        }
-        if (p >= 0 && ((__double_as_longlong(aug[sp][p][j]) >> 52) & 0x7ff) == 0x7ff) p = -1;  // Inf or NaN
-      }
-      p = __shfl_sync(0xffffffffu, p, j & 31);
-      if (p < 0) {  // no nonzero pivot (or a NaN input): singular reference
+      const double cand = used ? 0.0 : aug(sp, lane, j);
+      const unsigned key = (__double_as_longlong(cand) << 1) != 0 ? __float_as_uint(abs_f32_of(cand)) + 1u : 0u;
+      const unsigned kmax = __reduce_max_sync(0xffffffffu, key);
+      const int p = __ffs(__ballot_sync(0xffffffffu, key == kmax)) - 1;
+      const double piv = __shfl_sync(0xffffffffu, cand, p);
+      // no nonzero pivot, or Inf or NaN: singular reference
+      if (kmax == 0u || ((__double_as_longlong(piv) >> 52) & 0x7ff) == 0x7ff) {
         singular = 1;
         break;
       }
-      used |= 1u << p;
-      if (lane == 0) rowof[sp][j] = p;
-      const double piv = aug[sp][p][j];
+      if (lane == p) used = true;
+      if (lane == j) {
+        rowof[sp][j] = p;
+        col = n + p;
+      }
       {
         const long long b = __double_as_longlong(piv);
         negs += (int)((unsigned long long)b >> 63);
@@ -189,17 +203,21 @@ __global__ void __launch_bounds__(64) k_ref(DevProblem P, DevScratch S) {
         pmin = fminf(pmin, a);
       }
       const double inv = 1.0 / piv;
-      __syncwarp();
-      for (int c = lane; c < 2 * n; c += 32) {
-        if (c == j) continue;
-        const double apc = aug[sp][p][c] * inv;
-        aug[sp][p][c] = apc;
-        for (int i = 0; i < n; i++)
-          if (i != p) aug[sp][i][c] = fma(-aug[sp][i][j], apc, aug[sp][i][c]);
+      if (lane < n) {
+        const double apc = aug(sp, p, col) * inv;
+        for (int i0 = 0; i0 < n; i0 += 4) {
+          double f[4], x[4];
+#pragma unroll
+          for (int k = 0; k < 4; k++) {
+            const int i = min(i0 + k, n - 1);
+            f[k] = aug(sp, i, j);
+            x[k] = aug(sp, i, col);
+          }
+#pragma unroll
+          for (int k = 0; k < 4; k++)
+            if (i0 + k < n) aug(sp, i0 + k, col) = i0 + k == p ? apc : fma(-f[k], apc, x[k]);
+        }
       }
-      __syncwarp();
-      if (lane == (j & 31))
-        for (int i = 0; i < n; i++) aug[sp][i][j] = (i == p) ? 1.0 : 0.0;
       __syncwarp();
     }
     // sign: pivots' signs times the parity of j -> p_j (inversions counted by lane j)
@@ -215,7 +233,7 @@ __global__ void __launch_bounds__(64) k_ref(DevProblem P, DevScratch S) {
     if (!singular)
       for (int c = lane; c < n; c += 32) {
         float s = 0.0f;
-        for (int i = 0; i < n; i++) s += abs_f32_of(aug[sp][i][n + c]);
+        for (int i = 0; i < n; i++) s += abs_f32_of(aug(sp, i, n + c));
         ca = fmaxf(ca, s);
       }
 #pragma unroll
@@ -247,16 +265,16 @@ __global__ void __launch_bounds__(64) k_ref(DevProblem P, DevScratch S) {
     // which the elimination no longer needs
     const int t = threadIdx.x, sp = t >> 5, lane = t & 31;
     const int n = sp ? nd : nu;
-    if (lane < n && !bad[sp]) {
-      float2* dst = reinterpret_cast<float2*>(&aug[sp][lane][0]);
+    if (sp < 2 && lane < n && !bad[sp]) {
+      float2* dst = reinterpret_cast<float2*>(&aug(sp, lane, 0));
       for (int i = 0; i < n; i++) {
-        const df32 d = df_from_bits(__double_as_longlong(aug[sp][lane][n + i]));
+        const df32 d = df_from_bits(__double_as_longlong(aug(sp, lane, n + i)));
         dst[i] = make_float2(d.hi, d.lo);
       }
     }
     __syncthreads();
     auto Adf = [&](int sp, int a, int i) {
-      const float2 v = reinterpret_cast<const float2*>(&aug[sp][rowof[sp][a]][0])[i];
+      const float2 v = reinterpret_cast<const float2*>(&aug(sp, rowof[sp][a], 0))[i];
       return df32(v.x, v.y);
     };
     const float2* phi2 = reinterpret_cast<const float2*>(S.phi);
@@ -299,7 +317,7 @@ __global__ void __launch_bounds__(64) k_ref(DevProblem P, DevScratch S) {
   }
   // A to global, T = A Phi (walker-minor), g
   // A[a][i] of spin sp
-  auto Aat = [&](int sp, int a, int i) { return aug[sp][rowof[sp][a]][(sp ? nd : nu) + i]; };
+  auto Aat = [&](int sp, int a, int i) { return aug(sp, rowof[sp][a], (sp ? nd : nu) + i); };
   double* Ag = S.Ainv + w * (nu * nu + nd * nd);
   for (int t = threadIdx.x; t < nu * nu + nd * nd; t += blockDim.x) {
     const int sp = t < nu * nu ? 0 : 1;
@@ -1276,10 +1294,13 @@ cudaError_t launch_mo_f64(const DevProblem& P, const DevScratch& S, int64_t n_wa
 
 cudaError_t launch_ref_tables(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool mixed,
                               cudaStream_t st) {
+  const int nx = std::max(P.n_up, P.n_dn);
+  const size_t smem = (size_t)2 * nx * (2 * nx + 1) * sizeof(double);  // 33 KB at most
+  const unsigned nt = n_walk <= (int64_t)kRefFewBlocks * P.n_sm ? kRefThreadsFew : 64;
   if (mixed)
-    k_ref<true><<<(unsigned)n_walk, 64, 0, st>>>(P, S);
+    k_ref<true><<<(unsigned)n_walk, nt, smem, st>>>(P, S);
   else
-    k_ref<false><<<(unsigned)n_walk, 64, 0, st>>>(P, S);
+    k_ref<false><<<(unsigned)n_walk, nt, smem, st>>>(P, S);
   return cudaGetLastError();
 }
 
