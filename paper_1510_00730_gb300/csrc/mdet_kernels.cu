@@ -856,6 +856,23 @@ __global__ void __launch_bounds__(512) k_scatter(DevProblem P, DevScratch S, int
   }
 }
 
+// kSumLanes lanes to one sum over the MOs in k_final, their partial sums added in a fixed order. Two:
+// at 4096 walkers of 17 electrons and 100 MOs (pairs, 256 threads) the the last round of one lane to a sum
+// leaves most threads idle (10% slower), and with four or eight the additions across lanes cost as much.
+constexpr int kSumLanes = 2;
+static __device__ __forceinline__ df32 lanes_sum(df32 v) {
+#pragma unroll
+  for (int off = kSumLanes / 2; off; off >>= 1)
+    v = v + df32(__shfl_xor_sync(0xffffffffu, v.hi, off), __shfl_xor_sync(0xffffffffu, v.lo, off));
+  return v;
+}
+template <class T>
+static __device__ __forceinline__ T lanes_sum(T v) {
+#pragma unroll
+  for (int off = kSumLanes / 2; off; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+
 // ---------------------------------------------------------------------------
 // K6: per walker: W scatter over every determinant, Q = A^T W, Pm = T Q^T,
 // G_{i mu} = g Psi~ + sum_m d_mu phi[i][m] Q[i][m] - sum_b d_mu phi[i][o_b] Pm[b][i],
@@ -867,13 +884,19 @@ __global__ void __launch_bounds__(512) k_scatter(DevProblem P, DevScratch S, int
 // a compensated pair of FP32 shared atomics: the atomic returns the old value,
 // so TwoSum(old, x) recovers the rounding error of the addition it performed,
 // which goes into the low word. Q, Pm and G are double-float too (orbitals,
-// A and g arrive as pairs), so the FP64 pipe is left to the contraction; the
+// A and g arrive as pairs; full double-float sums: a compensated dot product would save a tenth of the
+// kernel and its errors are up to 1.3 times as large), so the FP64 pipe is left to the contraction; the
 // sums G are converted to FP64 with integer instructions.
 // smem, FP64: T[N][M], W[3][N][M] (FP32), Q[N][M], A blocks, Pm.
 // smem, MIXED: W[N][M] as hi/lo FP32 arrays, Q[N][M], A blocks, Pm (all pairs),
 //       Tdf[N][M].
-template <bool MIXED, int NT>
-__global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 1)) : 1) k_final(DevProblem P, DevScratch S, const double* __restrict__ R,
+// SCAT: the scatter runs here; otherwise k_scatter has left the sums in S.W, and without the
+// cofactor code 64 registers are enough. That variant is bound by latency between its barriers at the
+// four or five walkers an SM that 45 KB of shared memory allow, so it takes 256 threads: 0.57 ->
+// 0.43 ms at 8192 walkers of 17 electrons and 100 MOs in pairs, 1.09 -> 0.82 in FP64 (128 threads, one
+// kernel for both); 512 threads take 0.62 and 0.98.
+template <bool MIXED, int NT, bool SCAT>
+__global__ void __launch_bounds__(NT, SCAT ? (MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 1)) : 1) : 4) k_final(DevProblem P, DevScratch S, const double* __restrict__ R,
                                                double* __restrict__ log_abs_psi, int8_t* __restrict__ sign,
                                                double* __restrict__ grad, double* __restrict__ lap,
                                                double* __restrict__ e_local, uint32_t* __restrict__ status) {
@@ -882,12 +905,12 @@ __global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 
   const int NM = N * M;
   const int64_t w = blockIdx.x, wp = S.wp;
   if (S.live && w >= *S.live) return;
-  // MIXED keeps T and Q as pairs with rows padded to Mt = M + 1 entries, so that
+  // MIXED keeps T and Q as pairs with rows padded to an odd number Mt of entries, so that
   // threads reading the same column of different rows hit different banks
-  const int Mt = MIXED ? M + 1 : M;
+  const int Mt = MIXED ? M | 1 : M;
   double* Ts = MIXED ? nullptr : sm;    // [N][M] (FP64 only)
   double* Ws = MIXED ? sm : sm + NM;    // [N][M] (MIXED: hi words, then lo words; FP64: three FP32 words)
-  double* Qs = Ws + (MIXED ? NM : (3 * NM + 1) / 2);  // [N][Mt]
+  double* Qs = Ws + (MIXED || !SCAT ? NM : (3 * NM + 1) / 2);  // [N][Mt]
   double* As = Qs + N * Mt;             // [nu*nu + nd*nd]
   double* Pm = As + nu * nu + nd * nd;  // [nu*nu + nd*nd]  Pm[b][i] per spin
   float2* Tdf = reinterpret_cast<float2*>(Pm + nu * nu + nd * nd);  // [N][Mt] (MIXED)
@@ -900,14 +923,19 @@ __global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 
   __shared__ float Ga[kMaxSpin * 2][4];
   __shared__ float G2[kMaxSpin * 2][4];
   __shared__ float rmsG[4], estw[2][4];
-  for (int t = threadIdx.x; t < NM; t += blockDim.x) {
+#pragma unroll 4
+  for (int t = threadIdx.x; t < NM; t += NT) {
     if (MIXED) {
-      Tdf[(t / M) * Mt + t % M] = S.Tdf[(size_t)t * wp + w];
-      const float2 w0 = S.W ? reinterpret_cast<const float2*>(S.W)[w * NM + t] : make_float2(0.0f, 0.0f);  // already summed (k_scatter)?
+      Tdf[(t / M) * Mt + t % M] = __ldg(S.Tdf + (size_t)t * wp + w);
+      const float2 w0 = SCAT ? make_float2(0.0f, 0.0f) : __ldg(reinterpret_cast<const float2*>(S.W) + w * NM + t);
       Whi[t] = w0.x;
       Wlo[t] = w0.y;
     } else {
-      Ts[t] = S.T[(size_t)t * wp + w];
+      Ts[t] = __ldg(S.T + (size_t)t * wp + w);
+      if (!SCAT) {
+        Ws[t] = __ldg(reinterpret_cast<const double*>(S.W) + w * NM + t);
+        continue;
+      }
       Whi[t] = 0.0f;
       Wlo[t] = 0.0f;
       W3[t] = 0.0f;
@@ -920,16 +948,17 @@ __global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 
       As[t] = S.Ainv[w * (nu * nu + nd * nd) + t];
   }
   __syncthreads();
-  const int nu_det = P.n_det_sp[0], ntot = nu_det + P.n_det_sp[1];
-  const int tid = threadIdx.x, nth = blockDim.x;
-  if constexpr (MIXED) {
+  [[maybe_unused]] const int nu_det = P.n_det_sp[0], ntot = nu_det + P.n_det_sp[1];
+  [[maybe_unused]] const int tid = threadIdx.x, nth = blockDim.x;
+  if constexpr (!SCAT) {
+  } else if constexpr (MIXED) {
     // The determinants of one spin and excitation degree k at a time (the context orders
     // each spin's list by degree), so every lane of a warp runs the same k x k cofactor
     // code; within the group, determinant (q * stride) mod L for q = thread, thread + NT,
     // ... with a prime stride that does not divide L (a permutation), so the lanes of a
     // warp hold determinants far apart in key order, which rarely share a (hole,
     // particle) slot of W, and every thread gets an even share of the group.
-    for (int grp = 0; grp < (S.W ? 0 : 2 * kMaxExc); grp++) {
+    for (int grp = 0; grp < 2 * kMaxExc; grp++) {
       const int sp = grp / kMaxExc, k = grp % kMaxExc + 1;
       const int base = sp ? nu_det : 0;
       const int s0 = P.deg_start[sp][k], L = P.deg_start[sp][k + 1] - s0;
@@ -960,7 +989,7 @@ __global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 
     // each thread walks its own contiguous block (sequential loads of records and weights;
     // the FP64 pipe, not the balance, bounds this variant)
     const int per = (ntot + nth - 1) / nth;
-    const int n_mine = S.W ? 0 : max(0, min(per, ntot - tid * per));
+    const int n_mine = max(0, min(per, ntot - tid * per));
     for (int j = 0; j < n_mine; j++) {
       const int t = tid * per + j;
       const int sp = t < nu_det ? 0 : 1;
@@ -991,6 +1020,8 @@ __global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 
   const double psit = S.psit[w];
   const double ld = S.ld0[w * 2] + S.ld0[w * 2 + 1];
   const double sg = S.sg0[w * 2] * S.sg0[w * 2 + 1];
+  // (sum, lane) items of Pm and of G, in whole warps
+  const int nP = ((nu * nu + nd * nd) * kSumLanes + 31) / 32 * 32, nG = (N * 4 * kSumLanes + 31) / 32 * 32;
   if constexpr (MIXED) {
     // W normalised into (hi, lo) pairs in place
     for (int t = threadIdx.x; t < NM; t += blockDim.x) {
@@ -1010,6 +1041,7 @@ __global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 
       const int n = sp ? nd : nu, e0 = sp ? nu : 0, i = row - e0;
       const float2* A = A2 + (sp ? nu * nu : 0);
       df32 acc(0.0f, 0.0f);
+#pragma unroll 4
       for (int a = 0; a < n; a++) {
         const float2 av = A[a * n + i];
         const int wi = (e0 + a) * M + m;
@@ -1019,61 +1051,80 @@ __global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 
     }
     __syncthreads();
     // Pm[b][i] = sum_m T[b][m] Q[i][m]
-    for (int t = threadIdx.x; t < nu * nu + nd * nd; t += blockDim.x) {
-      const int sp = t < nu * nu ? 0 : 1;
-      const int n = sp ? nd : nu, e0 = sp ? nu : 0;
-      const int tt = sp ? t - nu * nu : t;
-      const int b = tt / n, i = tt - b * n;
-      const float2* Tr = Tdf + (e0 + b) * Mt;
-      const float2* Qr = Q2 + (e0 + i) * Mt;
+    for (int q = threadIdx.x; q < nP; q += NT) {
+      const int t = q / kSumLanes, gl = q % kSumLanes;
+      const bool on = t < nu * nu + nd * nd;
       df32 acc(0.0f, 0.0f);
-      for (int m = 0; m < M; m++) acc = acc + df32(Tr[m].x, Tr[m].y) * df32(Qr[m].x, Qr[m].y);
-      P2[t] = make_float2(acc.hi, acc.lo);
+      if (on) {
+        const int sp = t < nu * nu ? 0 : 1;
+        const int n = sp ? nd : nu, e0 = sp ? nu : 0;
+        const int tt = sp ? t - nu * nu : t;
+        const int b = tt / n, i = tt - b * n;
+        const float2* Tr = Tdf + (e0 + b) * Mt;
+        const float2* Qr = Q2 + (e0 + i) * Mt;
+#pragma unroll 4
+        for (int m = gl; m < M; m += kSumLanes) acc = acc + df32(Tr[m].x, Tr[m].y) * df32(Qr[m].x, Qr[m].y);
+      }
+      acc = lanes_sum(acc);
+      if (on && gl == 0) P2[t] = make_float2(acc.hi, acc.lo);
     }
     __syncthreads();
     const df32 psit_df = df_from_bits(__double_as_longlong(psit));
     const float2* phi2 = reinterpret_cast<const float2*>(S.phi);
     const float2* g2 = reinterpret_cast<const float2*>(S.g);
-    for (int t = threadIdx.x; t < N * 4; t += blockDim.x) {
+    for (int q = threadIdx.x; q < nG; q += NT) {
+      const int t = q / kSumLanes, gl = q % kSumLanes;
       const int e = t >> 2, mu = t & 3;
-      const int sp = e < nu ? 0 : 1;
-      const int n = sp ? nd : nu, e0 = sp ? nu : 0, i = e - e0;
-      const int* occ = P.ref_occ + sp * kMaxSpin;
-      const float2* dphi = phi2 + ((w * 5 + 1 + mu) * N + e) * M;
-      const float2* Qr = Q2 + e * Mt;
-      const float2 gv = g2[(w * N + e) * 4 + mu];
-      df32 acc = df32(gv.x, gv.y) * psit_df;
+      df32 acc(0.0f, 0.0f);
       // magnitudes of the terms, for the error estimate (FP32 is plenty for an estimate)
-      float aab = fabsf(acc.hi), aa2 = aab * aab;
-      for (int m = 0; m < M; m++) {
-        const float2 dv = dphi[m];
-        acc = acc + df32(dv.x, dv.y) * df32(Qr[m].x, Qr[m].y);
-        const float tm = fabsf(dv.x * Qr[m].x);
-        aab += tm;
-        aa2 = fmaf(tm, tm, aa2);
+      float aab = 0.0f, aa2 = 0.0f;
+      if (e < N) {
+        const int sp = e < nu ? 0 : 1;
+        const int n = sp ? nd : nu, e0 = sp ? nu : 0, i = e - e0;
+        const int* occ = P.ref_occ + sp * kMaxSpin;
+        const float2* dphi = phi2 + ((w * 5 + 1 + mu) * N + e) * M;
+        const float2* Qr = Q2 + e * Mt;
+        if (gl == 0) {
+          const float2 gv = g2[(w * N + e) * 4 + mu];
+          acc = df32(gv.x, gv.y) * psit_df;
+          aab = fabsf(acc.hi);
+          aa2 = aab * aab;
+        }
+#pragma unroll 4
+        for (int m = gl; m < M; m += kSumLanes) {
+          const float2 dv = __ldg(dphi + m);
+          acc = acc + df32(dv.x, dv.y) * df32(Qr[m].x, Qr[m].y);
+          const float tm = fabsf(dv.x * Qr[m].x);
+          aab += tm;
+          aa2 = fmaf(tm, tm, aa2);
+        }
+        const float2* Pb = P2 + (sp ? nu * nu : 0);
+        for (int b = gl; b < n; b += kSumLanes) {
+          const float2 dv = __ldg(dphi + occ[b]), pv = Pb[b * n + i];
+          acc = acc - df32(dv.x, dv.y) * df32(pv.x, pv.y);
+          const float tm = fabsf(dv.x * pv.x);
+          aab += tm;
+          aa2 = fmaf(tm, tm, aa2);
+        }
       }
-      const float2* Pb = P2 + (sp ? nu * nu : 0);
-      for (int b = 0; b < n; b++) {
-        const float2 dv = dphi[occ[b]], pv = Pb[b * n + i];
-        acc = acc - df32(dv.x, dv.y) * df32(pv.x, pv.y);
-        const float tm = fabsf(dv.x * pv.x);
-        aab += tm;
-        aa2 = fmaf(tm, tm, aa2);
+      acc = lanes_sum(acc);
+      aab = lanes_sum(aab);
+      aa2 = lanes_sum(aa2);
+      if (e < N && gl == 0) {
+        Gs[e][mu] = df_to_double_int(acc);
+        Ga[e][mu] = aab;
+        G2[e][mu] = sqrtf(aa2);
       }
-      Gs[e][mu] = df_to_double_int(acc);
-      Ga[e][mu] = aab;
-      G2[e][mu] = sqrtf(aa2);
     }
   } else {
-    // W's three words summed into FP64, through Q's space (free until Q is formed), then back
-    // over the words
-    for (int t = threadIdx.x; t < NM; t += blockDim.x)
-      Qs[t] = S.W ? reinterpret_cast<const double*>(S.W)[w * NM + t]
-                  : ((double)Whi[t] + (double)Wlo[t]) + (double)W3[t];
-    __syncthreads();
     double* Wd = Ws;
-    for (int t = threadIdx.x; t < NM; t += blockDim.x) Wd[t] = Qs[t];
-    __syncthreads();
+    if (SCAT) {  // W's three words summed into FP64, through Q's space (free until Q is formed), then
+                 // back over the words
+      for (int t = threadIdx.x; t < NM; t += blockDim.x) Qs[t] = ((double)Whi[t] + (double)Wlo[t]) + (double)W3[t];
+      __syncthreads();
+      for (int t = threadIdx.x; t < NM; t += blockDim.x) Wd[t] = Qs[t];
+      __syncthreads();
+    }
     // Q[i][m] = sum_a A[a][i] W[a][m] (per spin block)
     for (int t = threadIdx.x; t < NM; t += blockDim.x) {
       const int row = t / M, m = t - row * M;
@@ -1087,44 +1138,66 @@ __global__ void __launch_bounds__(NT, MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 
     }
     __syncthreads();
     // Pm[b][i] = sum_m T[b][m] Q[i][m]
-    for (int t = threadIdx.x; t < nu * nu + nd * nd; t += blockDim.x) {
-      const int sp = t < nu * nu ? 0 : 1;
-      const int n = sp ? nd : nu, e0 = sp ? nu : 0;
-      const int tt = sp ? t - nu * nu : t;
-      const int b = tt / n, i = tt - b * n;
-      const double* Tr = Ts + (e0 + b) * M;
-      const double* Qr = Qs + (e0 + i) * M;
+    for (int q = threadIdx.x; q < nP; q += NT) {
+      const int t = q / kSumLanes, gl = q % kSumLanes;
+      const bool on = t < nu * nu + nd * nd;
       double acc = 0.0;
-      for (int m = 0; m < M; m++) acc = fma(Tr[m], Qr[m], acc);
-      Pm[t] = acc;
+      if (on) {
+        const int sp = t < nu * nu ? 0 : 1;
+        const int n = sp ? nd : nu, e0 = sp ? nu : 0;
+        const int tt = sp ? t - nu * nu : t;
+        const int b = tt / n, i = tt - b * n;
+        const double* Tr = Ts + (e0 + b) * M;
+        const double* Qr = Qs + (e0 + i) * M;
+#pragma unroll 4
+        for (int m = gl; m < M; m += kSumLanes) acc = fma(Tr[m], Qr[m], acc);
+      }
+      acc = lanes_sum(acc);
+      if (on && gl == 0) Pm[t] = acc;
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < N * 4; t += blockDim.x) {
+    for (int q = threadIdx.x; q < nG; q += NT) {
+      const int t = q / kSumLanes, gl = q % kSumLanes;
       const int e = t >> 2, mu = t & 3;
-      const int sp = e < nu ? 0 : 1;
-      const int n = sp ? nd : nu, e0 = sp ? nu : 0, i = e - e0;
-      const int* occ = P.ref_occ + sp * kMaxSpin;
-      const double* dphi = S.phi + ((w * 5 + 1 + mu) * N + e) * M;
-      const double* Qr = Qs + e * M;
-      double acc = S.g[(w * N + e) * 4 + mu] * psit;
+      double acc = 0.0;
       // magnitudes of the terms, for the error estimate (FP32 is plenty for an estimate)
-      float aab = fabsf((float)acc), aa2 = aab * aab;
-      for (int m = 0; m < M; m++) {
-        acc = fma(dphi[m], Qr[m], acc);
-        const float tm = fabsf((float)dphi[m] * (float)Qr[m]);
-        aab += tm;
-        aa2 = fmaf(tm, tm, aa2);
+      float aab = 0.0f, aa2 = 0.0f;
+      if (e < N) {
+        const int sp = e < nu ? 0 : 1;
+        const int n = sp ? nd : nu, e0 = sp ? nu : 0, i = e - e0;
+        const int* occ = P.ref_occ + sp * kMaxSpin;
+        const double* dphi = S.phi + ((w * 5 + 1 + mu) * N + e) * M;
+        const double* Qr = Qs + e * M;
+        if (gl == 0) {
+          acc = S.g[(w * N + e) * 4 + mu] * psit;
+          aab = fabsf((float)acc);
+          aa2 = aab * aab;
+        }
+#pragma unroll 4
+        for (int m = gl; m < M; m += kSumLanes) {
+          const double dv = __ldg(dphi + m);
+          acc = fma(dv, Qr[m], acc);
+          const float tm = fabsf((float)dv * (float)Qr[m]);
+          aab += tm;
+          aa2 = fmaf(tm, tm, aa2);
+        }
+        const double* Pb = Pm + (sp ? nu * nu : 0);
+        for (int b = gl; b < n; b += kSumLanes) {
+          const double dv = __ldg(dphi + occ[b]);
+          acc = fma(-dv, Pb[b * n + i], acc);
+          const float tm = fabsf((float)dv * (float)Pb[b * n + i]);
+          aab += tm;
+          aa2 = fmaf(tm, tm, aa2);
+        }
       }
-      const double* Pb = Pm + (sp ? nu * nu : 0);
-      for (int b = 0; b < n; b++) {
-        acc = fma(-dphi[occ[b]], Pb[b * n + i], acc);
-        const float tm = fabsf((float)dphi[occ[b]] * (float)Pb[b * n + i]);
-        aab += tm;
-        aa2 = fmaf(tm, tm, aa2);
+      acc = lanes_sum(acc);
+      aab = lanes_sum(aab);
+      aa2 = lanes_sum(aa2);
+      if (e < N && gl == 0) {
+        Gs[e][mu] = acc;
+        Ga[e][mu] = aab;
+        G2[e][mu] = sqrtf(aa2);
       }
-      Gs[e][mu] = acc;
-      Ga[e][mu] = aab;
-      G2[e][mu] = sqrtf(aa2);
     }
   }
   __syncthreads();
@@ -1457,7 +1530,7 @@ static cudaError_t launch_scatter(const DevProblem& P, const DevScratch& S, int6
 
 size_t final_smem_bytes(const DevProblem& P, bool mixed) {
   const size_t NM = (size_t)P.n_elec * P.n_mo;
-  const size_t NMt = (size_t)P.n_elec * (P.n_mo + 1);  // rows padded by one pair (MIXED)
+  const size_t NMt = (size_t)P.n_elec * (P.n_mo + 1);  // rows padded by up to one pair (MIXED)
   const size_t AB = 2 * (size_t)(P.n_up * P.n_up + P.n_dn * P.n_dn);
   // FP64: T, W (three FP32 words), Q, A blocks and Pm; MIXED: W (hi and lo words), Q and T
   // pairs, A blocks and Pm
@@ -1467,24 +1540,26 @@ size_t final_smem_bytes(const DevProblem& P, bool mixed) {
 cudaError_t launch_final(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R,
                          double* log_abs_psi, int8_t* sign, double* grad, double* lap, double* e_local,
                          uint32_t* status, bool mixed, cudaStream_t st, bool wide) {
-  DevScratch Sf = S;
   const int L = S.W ? scatter_group_walkers(P, n_walk, mixed) : 0;
-  if (L == 0) Sf.W = nullptr;
   if (L) {
     const cudaError_t es = mixed ? launch_scatter<float2>(P, S, n_walk, L, st) : launch_scatter<double>(P, S, n_walk, L, st);
     if (es != cudaSuccess) return es;
   }
-  const size_t smem = final_smem_bytes(P, mixed);
-  // threads per walker: 512 for a few walkers (fewer than SMs, or `wide`), whose latency matters; 256
+  size_t smem = final_smem_bytes(P, mixed);
+  // threads per walker: 256 after k_scatter; else 512 for a few walkers (fewer than SMs, or `wide`), whose latency matters; 256
   // where the walker's tables let fewer than five blocks on an SM (34 electrons, 103 MOs, 94 KB of
-  // pairs: 1.23 ms for 2,161 walkers with 128); else 128
-  const int nt = wide || n_walk < P.n_sm ? 512 : (smem > 45 * 1024 ? 256 : 128);
-  auto kern = mixed ? (nt == 512 ? k_final<true, 512> : (nt == 256 ? k_final<true, 256> : k_final<true, 128>))
-                    : (nt == 512 ? k_final<false, 512> : (nt == 256 ? k_final<false, 256> : k_final<false, 128>));
-  static SmemOptIn opt[2][3];  // dynamic shared memory per variant (static arrays come on top)
-  cudaError_t e = opt[mixed][nt == 512 ? 2 : nt / 128 - 1].ensure(kern, smem);
+  // pairs: 1.23 ms for 2,161 walkers with 128, 0.74 with 256); else 128
+  const int big = smem > 45 * 1024;
+  const int v = L ? 3 : (wide || n_walk < P.n_sm ? 2 : big);
+  static const int threads[4] = {128, 256, 512, 256};
+  static decltype(&k_final<true, 128, true>) const kernels[2][4] = {
+      {k_final<false, 128, true>, k_final<false, 256, true>, k_final<false, 512, true>, k_final<false, 256, false>},
+      {k_final<true, 128, true>, k_final<true, 256, true>, k_final<true, 512, true>, k_final<true, 256, false>}};
+  if (L && !mixed) smem -= sizeof(double) * (size_t)((P.n_elec * P.n_mo + 1) / 2);  // one word a sum
+  static SmemOptIn opt[2][4];  // dynamic shared memory per variant (static arrays come on top)
+  cudaError_t e = opt[mixed][v].ensure(kernels[mixed][v], smem);
   if (e != cudaSuccess) return e;
-  kern<<<(unsigned)n_walk, nt, smem, st>>>(P, Sf, R, log_abs_psi, sign, grad, lap, e_local, status);
+  kernels[mixed][v]<<<(unsigned)n_walk, threads[v], smem, st>>>(P, S, R, log_abs_psi, sign, grad, lap, e_local, status);
   return cudaGetLastError();
 }
 
