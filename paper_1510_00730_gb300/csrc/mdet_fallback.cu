@@ -5,7 +5,8 @@
 // in FP64, followed by their own contraction and epilogue (Eqs. 2, 5-8).
 //
 //   k_fb_list    compacts the flagged walkers into a device list (no host sync)
-//   k_fb_dets    one thread per (determinant, flagged walker): in-place
+//   k_fb_dets    one thread per (determinant, flagged walker), from 12 electrons per spin up four
+//                (k_fb_dets_quad): in-place
 //                Gauss-Jordan inversion with partial pivoting of the Slater
 //                matrix, D as a signed mantissa times 2^e, and (d_{i mu} D)/D = sum_a d_mu phi_{o_a}(r_i) (S^-1)_{a i}
 //   k_fb_scale   per flagged walker: common power-of-two scale of its determinant values
@@ -150,6 +151,162 @@ __global__ void __launch_bounds__(64) k_fb_dets(DevProblem P, DevScratch S) {
       for (int a = 0; a < n; a++) acc = fma(dph[cols[a]], A[a * n + i], acc);
       rec[2 + i * 4 + mu] = acc;
     }
+}
+
+// The same inversion by four lanes to a determinant, eight determinants to a warp, the columns dealt
+// to the lanes. A thread's whole matrix in shared memory leaves room for 96 threads an SM at 17
+// electrons, three warps that wait for their own loads and FMAs; four times the lanes on the same
+// memory keep the FP64 pipe busy (the reciprocal of a pivot, which every lane forms, is a seventh of a
+// step's work there). Every element goes through the operations of k_fb_dets in their order. At 17 + 17
+// electrons, 590 determinants and 10 walkers 0.46 -> 0.25 ms. Below 12 electrons, where a thread's
+// matrix is small, the thread is as fast for few walkers and twice as fast for many (9 + 8 electrons:
+// 0.11 against 0.13 ms for 10 walkers and 1800 determinants, 5.2 against 12.8 ms for 410 and 6000).
+constexpr int kQuadDets = 8, kQuadMinSpin = 12;
+
+__global__ void __launch_bounds__(32) k_fb_dets_quad(DevProblem P, DevScratch S, int ds) {
+  extern __shared__ double fsm[];
+  __shared__ uint8_t cols_s[kQuadDets][kFbMax], piv_s[kQuadDets][kFbMax];
+  const int qd = threadIdx.x >> 2, ql = threadIdx.x & 3;
+  uint8_t *cols = cols_s[qd], *piv = piv_s[qd];
+  double* A = fsm + qd * ds;  // n x n, row-major, stride n
+  const int count = min(S.fb_list[0], P.fallback_cap);
+  const int nu = P.n_up, nd = P.n_dn, N = nu + nd, M = P.n_mo, nmax = max(nu, nd);
+  const int nu_det = P.n_det_sp[0], ntot = nu_det + P.n_det_sp[1];
+  const int stride = 2 + 4 * nmax;
+  const int t = blockIdx.x * kQuadDets + qd;
+  const int sp = t < nu_det ? 0 : 1;
+  const int n = t < ntot ? (sp ? nd : nu) : 0, e0 = sp ? nu : 0;  // 0: no determinant, along for the barriers
+  Exc e{};
+  if (n) e = P.exc[sp][sp ? t - nu_det : t];
+  if (n && ql == 0) {
+    const int* occ = P.ref_occ + sp * kMaxSpin;
+    for (int a = 0; a < n; a++) cols[a] = (uint8_t)occ[a];
+    for (int q = 0; q < e.k; q++) cols[e.h[q]] = e.p[q];
+  }
+  __syncwarp();
+  for (int slot = blockIdx.y; slot < count; slot += gridDim.y) {
+    const double* ph = S.phi + (size_t)S.fb_list[1 + slot] * 5 * N * M;
+    for (int a = ql; a < n; a += 4) {
+      const int c = cols[a];
+#pragma unroll 4
+      for (int i = 0; i < n; i++) A[i * n + a] = ph[(size_t)(e0 + i) * M + c];
+    }
+    __syncwarp();
+    double pm = 1.0;
+    int pe = 0, neg = e.eps < 0;
+    bool singular = false;
+    for (int k = 0; k < nmax; k++) {
+      bool act = k < n && !singular;
+      unsigned long long best = 0ULL;
+      int p = 127;
+      if (act)
+        for (int i = k + ql; i < n; i += 4) {
+          const unsigned long long v = (unsigned long long)__double_as_longlong(A[i * n + k]) & 0x7fffffffffffffffULL;
+          if (p == 127 || v > best) {
+            best = v;
+            p = i;
+          }
+        }
+#pragma unroll
+      for (int off = 2; off; off >>= 1) {  // the first row of the largest magnitude
+        const unsigned long long ob = __shfl_xor_sync(0xffffffffu, best, off);
+        const int op = __shfl_xor_sync(0xffffffffu, p, off);
+        if (ob > best || (ob == best && op < p)) {
+          best = ob;
+          p = op;
+        }
+      }
+      if (act && (best == 0ULL || best >= 0x7ff0000000000000ULL)) {  // no nonzero pivot, or Inf / NaN: singular
+        singular = true;
+        act = false;
+      }
+      __syncwarp();
+      if (act) {
+        if (ql == 0) piv[k] = (uint8_t)p;
+        if (p != k) {
+          neg ^= 1;
+          for (int j = ql; j < n; j += 4) {
+            const double tmp = A[k * n + j];
+            A[k * n + j] = A[p * n + j];
+            A[p * n + j] = tmp;
+          }
+        }
+      }
+      __syncwarp();
+      const double d = act ? A[k * n + k] : 1.0;
+      if (act) {
+        const long long b = __double_as_longlong(d);
+        neg ^= (int)((unsigned long long)b >> 63);
+        int ex = (int)((b >> 52) & 0x7ff);
+        long long bn = b;
+        if (ex == 0) {  // a subnormal pivot: scaled by 2^64 into the normal range (exact)
+          bn = __double_as_longlong(d * 0x1p64);
+          ex = (int)((bn >> 52) & 0x7ff) - 64;
+        }
+        pm *= __longlong_as_double((bn & 0x000fffffffffffffLL) | 0x3fe0000000000000LL);
+        pe += ex - 1022;
+        const long long bm = __double_as_longlong(pm);  // back into [0.5, 1)
+        pe += (int)((bm >> 52) & 0x7ff) - 1022;
+        pm = __longlong_as_double((bm & 0x000fffffffffffffLL) | 0x3fe0000000000000LL);
+      }
+      const double inv = 1.0 / d;
+      __syncwarp();  // every lane has the pivot
+      if (act)
+        for (int j = ql; j < n; j += 4) A[k * n + j] = (j == k ? 1.0 : A[k * n + j]) * inv;
+      for (int i0 = 0; i0 < nmax; i0 += 4) {
+        double f[4];
+#pragma unroll
+        for (int r = 0; r < 4; r++) f[r] = act && i0 + r < n && i0 + r != k ? A[(i0 + r) * n + k] : 0.0;
+        __syncwarp();  // every lane has these rows of column k
+        if (act)
+          for (int j = ql; j < n; j += 4) {
+            const double rk = A[k * n + j];
+            double x[4];
+#pragma unroll
+            for (int r = 0; r < 4; r++) x[r] = j != k && i0 + r < n ? A[(i0 + r) * n + j] : 0.0;
+#pragma unroll
+            for (int r = 0; r < 4; r++)
+              if ((__double_as_longlong(f[r]) << 1) != 0) A[(i0 + r) * n + j] = fma(-f[r], rk, x[r]);
+          }
+      }
+      __syncwarp();
+    }
+    if (n) {
+      double* rec = S.fb + ((size_t)slot * ntot + t) * stride;
+      if (singular) {
+        if (ql == 0) {
+          rec[0] = -INFINITY;
+          rec[1] = 0.0;
+        }
+        for (int q = ql; q < 4 * n; q += 4) rec[2 + q] = 0.0;
+      } else {
+        // (P S)^-1 = S^-1 P^-1: undo the row interchanges on the columns, last first (rows dealt to the lanes)
+        for (int k = n - 1; k >= 0; k--)
+          if (piv[k] != k)
+            for (int i = ql; i < n; i += 4) {
+              const double tmp = A[i * n + k];
+              A[i * n + k] = A[i * n + piv[k]];
+              A[i * n + piv[k]] = tmp;
+            }
+        if (ql == 0) {
+          rec[0] = __longlong_as_double((long long)pe);  // the exponent, an integer in the bits
+          rec[1] = __longlong_as_double(__double_as_longlong(pm) | ((long long)neg << 63));  // D / 2^pe
+        }
+      }
+    }
+    __syncwarp();
+    if (n && !singular) {
+      double* rec = S.fb + ((size_t)slot * ntot + t) * stride;
+      for (int i = 0; i < n; i++) {
+        const double* dph = ph + ((size_t)(1 + ql) * N + e0 + i) * M;
+        double acc = 0.0;
+#pragma unroll 4
+        for (int a = 0; a < n; a++) acc = fma(dph[cols[a]], A[a * n + i], acc);
+        rec[2 + i * 4 + ql] = acc;
+      }
+    }
+    __syncwarp();
+  }
 }
 
 // threads per flagged walker of k_fb_scale (its exponentials and two block reductions over every
@@ -470,14 +627,20 @@ cudaError_t launch_fallback(const DevProblem& P, const DevScratch& S, int64_t n_
   if (e != cudaSuccess) return e;
   const int nmax = P.n_up > P.n_dn ? P.n_up : P.n_dn;
   const int ntot = P.n_det_sp[0] + P.n_det_sp[1];
-  // one thread per determinant, its Slater matrix in shared memory: 32-thread blocks from 12
-  // electrons per spin up, so that three blocks (96 threads) fit an SM at 17 instead of one of 64
-  const int tpb = nmax >= 12 ? 32 : 64;
-  const size_t smem = sizeof(double) * tpb * nmax * nmax;
-  static SmemOptIn opt;
-  if ((e = opt.ensure(k_fb_dets, smem)) != cudaSuccess) return e;
-  dim3 g1((ntot + tpb - 1) / tpb, P.fallback_cap);
-  k_fb_dets<<<g1, tpb, smem, st>>>(P, S);
+  static SmemOptIn opt, opt4;
+  if (nmax >= kQuadMinSpin) {
+    const int ds = (nmax * nmax + 11) / 16 * 16 + 4;  // 4 modulo 16: four determinants' columns on 16 banks
+    const size_t smem = sizeof(double) * kQuadDets * ds;
+    if ((e = opt4.ensure(k_fb_dets_quad, smem)) != cudaSuccess) return e;
+    dim3 g((ntot + kQuadDets - 1) / kQuadDets, std::min(P.fallback_cap, 64));
+    k_fb_dets_quad<<<g, 32, smem, st>>>(P, S, ds);
+  } else {
+    constexpr int tpb = 64;
+    const size_t smem = sizeof(double) * tpb * nmax * nmax;
+    if ((e = opt.ensure(k_fb_dets, smem)) != cudaSuccess) return e;
+    dim3 g1((ntot + tpb - 1) / tpb, P.fallback_cap);
+    k_fb_dets<<<g1, tpb, smem, st>>>(P, S);
+  }
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // many flagged walkers (FP64 at its own tolerance: hundreds): their contraction as residue products
   // too, 0.4 ms instead of 3.6 for 410 walkers and 750k products
