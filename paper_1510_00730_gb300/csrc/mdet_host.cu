@@ -437,7 +437,7 @@ mdet_status spin_tables(mdet_ctx* c, int sp, int n_int, const std::vector<uint64
 }
 
 // The digits of B as operand tiles of the tcgen05 orbital product: per chunk of 32 MOs and slice of
-// 16 AOs, [digit][AO / 8 mod 2][MO][AO mod 8]. Mixed precision: the 7 digits `dig` of B_dig; FP64: 8
+// 16 AOs, [AO / 8 mod 2][digit][MO][AO mod 8], so that the digits' MOs are rows of one operand. Mixed precision: the 7 digits `dig` of B_dig; FP64: 8
 // digits of B_am 2^(62 - fexp_m) (balanced base 256, the bytes of that integer + 0x80...80 less 128).
 // *out is null when some order's sum could exceed 2^24, where the product's FP32 accumulators would
 // no longer be exact (the AO digits are at most 256, the first of 7, else 128).
@@ -455,9 +455,9 @@ mdet_status upload_digit_tiles(mdet_ctx* c, const std::vector<double>& B, const 
       const uint64_t v = D == 8 ? (uint64_t)std::llrint(std::ldexp(B[(size_t)mu * M + m], 62 - fexp[m])) +
                                       0x8080808080808080ULL
                                 : 0;
-      uint16_t* t = &tiles[(size_t)D * Kp * m0 + (size_t)(mu / 16) * D * 16 * cw + (size_t)((mu % 16) / 8) * cw * 8 +
-                           (size_t)(m - m0) * 8 + mu % 8];
-      for (int j = 0; j < D; j++, t += 16 * cw) {
+      uint16_t* t = &tiles[(size_t)D * Kp * m0 + (size_t)(mu / 16) * D * 16 * cw +
+                           (size_t)((mu % 16) / 8) * D * cw * 8 + (size_t)(m - m0) * 8 + mu % 8];
+      for (int j = 0; j < D; j++, t += 8 * cw) {
         float d;
         uint32_t bits;
         if (D == 8) {

@@ -329,7 +329,6 @@ __global__ void __launch_bounds__(384, 1) k_mo_orders(DevProblem P, const uint16
     for (int64_t tile = blockIdx.x; tile < tiles && !*dead; tile += gridDim.x)
       for (int c = 0; c < n_chunk && !*dead; c++, n++) {
         const int cw = min(kChunk, Np - c * kChunk), b = n & 1;
-        const uint32_t idesc = umma::idesc_bf16(128, cw);
         if (n >= 2 && !umma::bounded_wait(&tempty[b], ((n >> 1) & 1) ^ 1, dead)) break;
         umma::fence_after();
         bool ok = true;
@@ -340,11 +339,10 @@ __global__ void __launch_bounds__(384, 1) k_mo_orders(DevProblem P, const uint16
           umma::fence_after();
           const uint32_t sa = stage0 + (uint32_t)s * kStageBytes, sb = sa + kABytes;
 #pragma unroll
-          for (int i = 0; i < D; i++)
-#pragma unroll
-            for (int j = 0; j < D - i; j++)
-              umma::mma_smem_a(tb + 256u * b + (uint32_t)((i + j) * cw), umma::desc(sa + i * kSliceBytes, 2048, 128),
-                               umma::desc(sb + (uint32_t)(j * cw * 32), (uint32_t)cw * 16, 128), idesc, k != 0 || i != 0);
+          for (int i = 0; i < D; i++)  // X's digit i + 1 against B's digits 1 .. D - i: orders i + 2 .. D + 1
+            umma::mma_smem_a(tb + 256u * b + (uint32_t)(i * cw), umma::desc(sa + i * kSliceBytes, 2048, 128),
+                             umma::desc(sb, (uint32_t)(D * cw * 16), 128), umma::idesc_bf16(128, (D - i) * cw),
+                             k != 0 || i != 0);
           umma::commit(&empty[s]);
         }
         if (ok) umma::commit(&tfull[b]);
