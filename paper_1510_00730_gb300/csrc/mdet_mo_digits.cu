@@ -18,15 +18,20 @@
 //  k_mo_ao      AO values (FP64, or double-float on the FP32 pipe), row exponents and digits.
 //               Three blocks of 256 threads per SM; bound by the AO arithmetic (FP64: the FP64
 //               pipe) and by the digit stores, 14 or 16 bytes per AO value.
-//  k_mo_orders  the digit products. The rows are the MMA's M = 128, a chunk of 32 MOs its N; the
+//  k_mo_orders  the digit products. The rows are the MMA's M = 128, a chunk of 32 MOs of all of B's
+//               digits its N: a digit of X against the digits 1 .. D + 1 - i of B is one MMA into
+//               neighbouring orders, so X is read D times a slice and not D (D + 1) / 2 times. The
 //               D orders' accumulators (32 columns each) are double-buffered in tensor memory, so
-//               the epilogue of one chunk overlaps the products of the next. Bound by the reads
-//               of the A operand from shared memory (N = 32 uses a quarter of the MMA rate).
+//               the epilogue of one chunk overlaps the products of the next; 16 warps take it, 8
+//               MOs of a row to a lane with their chains side by side. Bound by that epilogue and
+//               by the reads of X's digits from L2, once a chunk (the tensor cores are busy a third
+//               of the time).
 // FP64 orbitals of small bases and of re-evaluated walkers take k_mo_ao with plain FP64 rows instead of digits, and
 //  k_mo_dot     the FP64 dot products, one thread per row and MO.
-// 8,192 walkers of 17 electrons, 110 AOs, 80 MOs: 1.51 ms as pairs (3.60 as one kernel that kept
-// the digits in shared memory and the MO planes in tensor memory, a single 256-thread block per
-// SM) and 2.5 ms in FP64 (16.0 with dot products on the FP64 pipe).
+// 8,192 walkers of 17 electrons, 110 AOs, 80 MOs: k_mo_ao 0.73 and k_mo_orders 0.42 ms as pairs (3.60
+// as one kernel that kept the digits in shared memory and the MO planes in tensor memory, a single
+// 256-thread block per SM), 1.69 and 0.49 ms in FP64 (16.0 with dot products on the FP64 pipe). With
+// an MMA per digit pair and eight warps that took one MO after the other, k_mo_orders 0.76 and 0.95.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -43,6 +48,7 @@ namespace {
 constexpr int kNE = 16;                       // electrons per block of k_mo_ao
 constexpr int kSliceBytes = 2 * 128 * 16;     // one plane of 128 rows x 16 AOs
 constexpr int kChunk = 32;                    // MOs per accumulator set
+constexpr int kEpiWarps = 16, kOrderThreads = 128 + 32 * kEpiWarps;
 constexpr int64_t kMinDigitWork = 2048;       // AOs x MOs from which FP64 orbitals take digits
 constexpr int kBadRow = 1 << 20;              // row exponent of a row with a value that is not finite
 
@@ -77,7 +83,21 @@ __device__ __forceinline__ void digit_pairs(double x0, double x1, int er, uint32
 
 // Pairs: digit by digit on the scaled value, the remainder kept as a pair (exact).
 __device__ __forceinline__ void digit_pairs(df32 x0, df32 x1, int er, uint32_t (&w)[7]) {
-  float vh[2] = {ldexpf(x0.hi, -er), ldexpf(x1.hi, -er)}, vl[2] = {ldexpf(x0.lo, -er), ldexpf(x1.lo, -er)};
+  float vh[2] = {x0.hi, x1.hi}, vl[2] = {x0.lo, x1.lo};
+  if (er >= -127 && er <= 126) {  // 2^-er as a normal number: one rounding, as ldexpf
+    const float s = __uint_as_float((uint32_t)(127 - er) << 23);
+#pragma unroll
+    for (int y = 0; y < 2; y++) {
+      vh[y] = __fmul_rn(vh[y], s);
+      vl[y] = __fmul_rn(vl[y], s);
+    }
+  } else {
+#pragma unroll
+    for (int y = 0; y < 2; y++) {
+      vh[y] = ldexpf(vh[y], -er);
+      vl[y] = ldexpf(vl[y], -er);
+    }
+  }
 #pragma unroll
   for (int i = 0; i < 7; i++) {
     uint32_t b[2];
@@ -230,7 +250,7 @@ __global__ void __launch_bounds__(256) k_mo_dot(const double* __restrict__ X, co
 }
 
 // Phi = 2^e sum_t 2^(-8 (t + 2)) G_t from the orders' exact sums. FP64: in integers, rounded once.
-__device__ __forceinline__ void put_value(double* out, const uint32_t (&v)[8][8], int j, int e) {
+__device__ __forceinline__ double value_of(double, const uint32_t (&v)[8][8], int j, int e) {
   long long sh = 0, sl = 0;
 #pragma unroll
   for (int t = 0; t < 8; t++) {
@@ -241,11 +261,11 @@ __device__ __forceinline__ void put_value(double* out, const uint32_t (&v)[8][8]
       sl += G * (1 << (8 * (7 - t)));
   }
   const __int128 V = (__int128)sh * (1LL << 32) + sl;
-  *out = i128_to_double((unsigned long long)(V >> 64), (unsigned long long)V, e - 72);
+  return i128_to_double((unsigned long long)(V >> 64), (unsigned long long)V, e - 72);
 }
 
 // Pairs: summed in double-float, the leading order first.
-__device__ __forceinline__ void put_value(float2* out, const uint32_t (&v)[7][8], int j, int e) {
+__device__ __forceinline__ float2 value_of(float2, const uint32_t (&v)[7][8], int j, int e) {
   df32 acc(0.0f, 0.0f);
 #pragma unroll
   for (int t = 0; t < 7; t++) {
@@ -254,11 +274,19 @@ __device__ __forceinline__ void put_value(float2* out, const uint32_t (&v)[7][8]
     fast_two_sum(s, __fadd_rn(acc.lo, r), hi, lo);
     acc = df32(hi, lo);
   }
-  *out = make_float2(ldexpf(acc.hi, e), ldexpf(acc.lo, e));
+  if (e >= -126 && e <= 127) {  // 2^e as a normal number: one rounding, as ldexpf
+    const float s = __uint_as_float((uint32_t)(e + 127) << 23);
+    return make_float2(__fmul_rn(acc.hi, s), __fmul_rn(acc.lo, s));
+  }
+  return make_float2(ldexpf(acc.hi, e), ldexpf(acc.lo, e));
 }
 
-__device__ __forceinline__ void put_nan(double* out) { *out = __longlong_as_double(0x7ff8000000000000LL); }
-__device__ __forceinline__ void put_nan(float2* out) { *out = make_float2(__int_as_float(0x7fc00000), 0.0f); }
+__device__ __forceinline__ double nan_of(double) { return __longlong_as_double(0x7ff8000000000000LL); }
+__device__ __forceinline__ float2 nan_of(float2) { return make_float2(__int_as_float(0x7fc00000), 0.0f); }
+__device__ __forceinline__ void put_two(double* p, double a, double b) { *reinterpret_cast<double2*>(p) = make_double2(a, b); }
+__device__ __forceinline__ void put_two(float2* p, float2 a, float2 b) {
+  *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+}
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -269,11 +297,11 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
 
 // The digit products of 128-row tiles: per tile and chunk of MOs, all pairs of every 16-AO slice
 // into the orders' accumulators. Warps: 0 the producer (one bulk copy each for the slice's
-// planes of X and of B), 1 the MMA issuer, 2 tensor memory, 4-11 the epilogue (two warps per
-// lane quarter). Every wait is bounded in time; after one runs out the rest of the CTA's orbitals
+// planes of X and of B), 1 the MMA issuer, 2 tensor memory, the others the epilogue (four warps
+// per lane quarter). Every wait is bounded in time; after one runs out the rest of the CTA's orbitals
 // are NaN, which the epilogue of the evaluation flags.
 template <class T, class Out>
-__global__ void __launch_bounds__(384, 1) k_mo_orders(DevProblem P, const uint16_t* __restrict__ b_tiles,
+__global__ void __launch_bounds__(kOrderThreads, 1) k_mo_orders(DevProblem P, const uint16_t* __restrict__ b_tiles,
                                                       const uint8_t* __restrict__ xd, const int* __restrict__ xer,
                                                       Out* __restrict__ phi, int64_t n_rows,
                                                       const int* __restrict__ live, int64_t w0) {
@@ -296,7 +324,7 @@ __global__ void __launch_bounds__(384, 1) k_mo_orders(DevProblem P, const uint16
     }
     for (int b = 0; b < 2; b++) {
       umma::mbar_init(&tfull[b], 1);
-      umma::mbar_init(&tempty[b], 8);
+      umma::mbar_init(&tempty[b], kEpiWarps);
     }
     umma::mbar_init(&fin, 1);
     dead_s = 0;
@@ -352,7 +380,7 @@ __global__ void __launch_bounds__(384, 1) k_mo_orders(DevProblem P, const uint16
       umma::drain_wait(&fin, 0);
     }
   } else if (warp >= 4) {
-    const int qd = warp & 3, half = (warp - 4) >> 2;
+    const int qd = warp & 3, part = (warp - 4) >> 2;
     uint32_t n = 0;
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
       const int64_t row = tile * 128 + 32 * qd + lane;
@@ -363,24 +391,48 @@ __global__ void __launch_bounds__(384, 1) k_mo_orders(DevProblem P, const uint16
         const bool ok = __all_sync(0xffffffffu, umma::bounded_wait(&tfull[b], (n >> 1) & 1, dead));
         umma::fence_after();
         const uint32_t ta = tb + ((uint32_t)(32 * qd) << 16) + 256u * b;
-        for (int g = half; g < cw / 8; g += 2) {
-          uint32_t v[D][8];
+        for (int g = part; g < cw / 8; g += kEpiWarps / 4) {
+          const int m0 = c * kChunk + 8 * g;
+          const int fl = lane < 8 && m0 + lane < M ? __ldg(P.B_exp + m0 + lane) : kBadRow;
+          uint32_t v[D][8] = {};
           if (ok) {
 #pragma unroll
             for (int t = 0; t < D; t++) tmem_ld8(ta + (uint32_t)(t * cw + 8 * g), v[t]);
             asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
           }
-          const int m0 = c * kChunk + 8 * g;
+          // pairs: the eight values side by side (each is a chain over the orders)
+          constexpr int kSide = std::is_same<Out, double>::value ? 2 : 8;
           Out* dst = phi + row * M + m0;
+          const bool wide = M % 2 == 0 && m0 + 8 <= M;  // two values to a store
 #pragma unroll
-          for (int j = 0; j < 8; j++) {
-            if (!valid || m0 + j >= M) continue;
-            const int f = P.B_exp[m0 + j];
-            if (!ok || er == kBadRow || f == kBadRow) {
-              put_nan(dst + j);
-              continue;
+          for (int j0 = 0; j0 < 8; j0 += kSide) {
+            Out o[kSide];
+#pragma unroll
+            for (int j = 0; j < kSide; j++) {
+              const int f = __shfl_sync(0xffffffffu, fl, j0 + j);
+              const bool bad = !ok || er == kBadRow || f == kBadRow;
+              const Out x = value_of(Out(), v, j0 + j, bad ? 0 : er + AoType<T>::kLead + f);
+              o[j] = bad ? nan_of(Out()) : x;
             }
-            put_value(dst + j, v, j, er + AoType<T>::kLead + f);
+            if (valid && wide) {
+#pragma unroll
+              for (int j = 0; j < kSide; j += 2) put_two(dst + j0 + j, o[j], o[j + 1]);
+            } else if (kSide == 8 && valid && m0 + 8 <= M) {  // M odd: an odd row starts half a store later
+              if (row & 1) {
+                dst[0] = o[0];
+#pragma unroll
+                for (int j = 1; j < 7; j += 2) put_two(dst + j, o[j % kSide], o[(j + 1) % kSide]);
+                dst[7] = o[7 % kSide];
+              } else {
+#pragma unroll
+                for (int j = 0; j < 8; j += 2) put_two(dst + j, o[j % kSide], o[(j + 1) % kSide]);
+              }
+            } else if (valid) {
+#pragma unroll
+              for (int j = 0; j < kSide; j++)
+                if (m0 + j0 + j < M) dst[j0 + j] = o[j];
+            }
+            __syncwarp();
           }
         }
         umma::fence_before();
@@ -436,7 +488,7 @@ static cudaError_t launch_mo_digits_t(const DevProblem& P, const DevScratch& S, 
       continue;
     }
     k_mo_ao<T, false><<<g1, 256, smem1, st>>>(P, R, w0, nb * N, S.xd, S.xer, P.tc_kp, S.live);
-    k_mo_orders<T, Out><<<g2, 384, smem2, st>>>(P, b_tiles, S.xd, S.xer,
+    k_mo_orders<T, Out><<<g2, kOrderThreads, smem2, st>>>(P, b_tiles, S.xd, S.xer,
                                                 reinterpret_cast<Out*>(S.phi + w0 * 5 * N * P.n_mo), rows, S.live, w0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
