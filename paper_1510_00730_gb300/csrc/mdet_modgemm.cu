@@ -492,13 +492,20 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
 // is a template argument for the usual counts: unrolled to the largest it takes 0.88 ms. Every
 // walker's Psi~ is summed in one warp, in a fixed order. Stores go through shared memory so that a
 // warp writes 256 consecutive bytes.
+// Few walkers (a re-evaluation, or too few for the warps of three blocks an SM): four warps to a walker
+// and product, so that each walks a quarter of the determinants: 67 of 256 slots
+// with 900 + 900 determinants 44 -> 14 us, 87 with 3000 + 3000 120 -> 34, 1000 walkers of 900 + 900 46 -> 40.
+constexpr int kCrtFewWalkers = 8;
 template <int Q>
 __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ DenseContract D, DevProblem P, DevScratch S,
-                                                 int64_t w0, int64_t n_walk, int nmt, int n_abs) {
+                                                  int64_t w0, int64_t n_walk, int nmt, int n_abs, int parts) {
   __shared__ double2 tile[8][64];
+  __shared__ double psi_s[4];
+  __shared__ float pa_s[4];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int o = warp >> 2;  // warps 0-3: v of four walkers, 4-7: u of the same
-  const int64_t wl = (int64_t)blockIdx.x * 4 + (warp & 3), w = w0 + wl;
+  const int o = warp >> 2;  // warps 0-3: v, 4-7: u, of four walkers or (parts = 4) of four parts of one walker
+  const int part = parts == 4 ? warp & 3 : 0;
+  const int64_t wl = parts == 4 ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * 4 + (warp & 3), w = w0 + wl;
   if (w >= n_walk || (S.live && w >= *S.live)) return;
   const int nu = P.n_det_sp[0], nd = P.n_det_sp[1];
   const int64_t wp = S.wp;
@@ -513,7 +520,7 @@ __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ Dens
     const int* gi = o ? P.csc_row : P.csr_col;
     const double* val = o ? P.csc_val : P.csr_val;
     const double* x = S.r + (size_t)(o ? 0 : nu) * wp + w;
-    for (int i = lane; i < n; i += 32) {
+    for (int i = 32 * part + lane; i < n; i += 32 * parts) {
       double acc = 0.0;
       float aa = 0.0f;
       for (int k = ptr[i]; k < ptr[i + 1]; k++) {
@@ -533,7 +540,7 @@ __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ Dens
     const int e0 = xb - 1022 - kCBits - kRBits;
     const uint8_t* y = S.dy + (o ? (size_t)D.nm * nmt * 128 * D.ldy[0] : 0) + (size_t)wl * ldy;
     const size_t yplane = (size_t)nmt * 128 * ldy;
-    for (int base = 0; base < n; base += 128) {
+    for (int base = 128 * part; base < n; base += 128 * parts) {
       const int i0 = base + 4 * lane;
       if (i0 < ldy) {
         // sums over the moduli of residue byte x weight in 16-bit limbs (and the quotient's, limb 8): the
@@ -597,11 +604,21 @@ __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ Dens
       __syncwarp();
     }
   }
-  if (o) return;
+  if (o && parts == 1) return;
 #pragma unroll
   for (int off = 16; off; off >>= 1) {
     psi += __shfl_xor_sync(0xffffffffu, psi, off);
     pa += __shfl_xor_sync(0xffffffffu, pa, off);
+  }
+  if (parts == 4) {  // (a whole block: none of its warps has returned)
+    if (!o && lane == 0) {
+      psi_s[part] = psi;
+      pa_s[part] = pa;
+    }
+    __syncthreads();
+    if (warp) return;
+    psi = ((psi_s[0] + psi_s[1]) + psi_s[2]) + psi_s[3];
+    pa = ((pa_s[0] + pa_s[1]) + pa_s[2]) + pa_s[3];
   }
   if (lane == 0) {
     S.psit[w] = psi;
@@ -736,7 +753,8 @@ cudaError_t launch_contract_dense(const DevProblem& P, const DevScratch& S, int6
     const int64_t pairs = std::min<int64_t>(units, std::max(P.n_sm / 2, 1));
     k_mod_gemm<<<(unsigned)(2 * pairs), 256, smem, st>>>(D, a);
     auto* crt = D.nm <= 16 ? k_mod_crt<8> : D.nm <= 18 ? k_mod_crt<9> : k_mod_crt<kMaxModuli / 2>;
-    crt<<<(unsigned)((nb + 3) / 4), 256, 0, st>>>(D, P, S, w0, n_walk, nmt, n_abs);
+    const int parts = S.live || nb <= (int64_t)kCrtFewWalkers * P.n_sm ? 4 : 1;
+    crt<<<(unsigned)(parts == 4 ? nb : (nb + 3) / 4), 256, 0, st>>>(D, P, S, w0, n_walk, nmt, n_abs, parts);
     if (n_kernels) *n_kernels += 3;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -67,7 +67,7 @@ def test_residue_products_match_oracle_and_sparse_sums(nu, nd, prec):
     assert np.array_equal(table["sign"], sparse["sign"]) and np.array_equal(table["status"], sparse["status"])
 
 
-@pytest.mark.parametrize("n_walk", [1, 31, 255, 257, 513])
+@pytest.mark.parametrize("n_walk", [1, 31, 255, 257, 513, 1301])
 def test_ragged_walkers(n_walk):
     wl = _workload(130, 70, n_walk, seed=6 + n_walk)
     ctx = pkg.Context.from_workload(wl, device=0)
