@@ -106,6 +106,14 @@ static __device__ __forceinline__ df32 operator+(df32 x, df32 y) {
   return {zh, zl};
 }
 
+// x + y for a float y: the sum above with y.lo = 0, to the bit, without the operations that add zero
+static __device__ __forceinline__ df32 add_float(df32 x, float y) {
+  float sh, sl, vh, vl;
+  two_sum(x.hi, y, sh, sl);
+  fast_two_sum(sh, __fadd_rn(sl, x.lo), vh, vl);
+  return {vh, vl};
+}
+
 static __device__ __forceinline__ df32 operator-(df32 x) { return {-x.hi, -x.lo}; }
 
 static __device__ __forceinline__ df32 operator-(df32 x, df32 y) { return x + (-y); }
@@ -177,18 +185,19 @@ static __device__ __forceinline__ df32 df_exp_nonpos(df32 t) {
   if (!(t.hi > -87.0f)) return df32(0.0f, 0.0f);
   const float kf = rintf(__fmul_rn(t.hi, 1.44269504f));
   // r = t - k ln2, each piece of k ln2 exact in double-float
-  df32 r = t + df32(__fmul_rn(-kf, kLn2a), 0.0f);
+  df32 r = add_float(t, __fmul_rn(-kf, kLn2a));
   {
     const float p = __fmul_rn(-kf, kLn2b);
     const float e = __fmaf_rn(-kf, kLn2b, -p);
     r = r + df32(p, e);
   }
-  r = r + df32(__fmul_rn(-kf, kLn2c), 0.0f);
+  r = add_float(r, __fmul_rn(-kf, kLn2c));
   df32 p(kInvFact[13][0], kInvFact[13][1]);
 #pragma unroll
-  for (int n = 12; n >= 0; n--) p = p * r + df32(kInvFact[n][0], kInvFact[n][1]);
-  const int k = (int)kf;
-  return df32(ldexpf(p.hi, k), ldexpf(p.lo, k));
+  for (int n = 12; n >= 2; n--) p = p * r + df32(kInvFact[n][0], kInvFact[n][1]);
+  p = add_float(add_float(p * r, 1.0f) * r, 1.0f);
+  const float s = __uint_as_float((unsigned)((int)kf + 127) << 23);  // 2^k, -126 <= k <= 0: rounds as ldexpf
+  return df32(__fmul_rn(p.hi, s), __fmul_rn(p.lo, s));
 }
 
 }  // namespace mdet

@@ -367,10 +367,86 @@ static __device__ __forceinline__ void ao_shell_values(const DevProblem& P, int 
 // The same AO values in double-float arithmetic on the FP32 pipe (mixed
 // path): coordinates, exponents and coefficients arrive as (hi, lo) pairs and
 // exp is df_exp_nonpos. Same formulas, component order and store() contract.
-static __device__ __forceinline__ df32 df_ipow(df32 x, int n) {
-  df32 r(1);
-  for (int i = 0; i < n; i++) r = r * x;
-  return r;
+// The powers of a shell's functions are compile-time constants, and a factor of exactly one, a power
+// of two or a term of exactly zero costs nothing; the operations that remain, and their order, are
+// those of the general expressions in ao_shell_values, so the values are too, to the bit.
+template <bool ONE>
+struct DfFactor {  // a value, or exactly one
+  df32 v;
+};
+template <bool A, bool B>
+static __device__ __forceinline__ DfFactor<A && B> operator*(DfFactor<A> x, DfFactor<B> y) {
+  if constexpr (A)
+    return {y.v};
+  else if constexpr (B)
+    return {x.v};
+  else
+    return {x.v * y.v};
+}
+template <int N>
+static __device__ __forceinline__ DfFactor<N == 0> df_power(df32 x) {
+  if constexpr (N == 0)
+    return {df32(1)};
+  else if constexpr (N == 1)
+    return {x};
+  else
+    return {df_power<N - 1>(x).v * x};
+}
+template <int K>
+static __device__ __forceinline__ df32 df_times(df32 v) {  // K v
+  if constexpr (K == 1)
+    return v;
+  else if constexpr (K == 2 || K == 4)
+    return {__fmul_rn((float)K, v.hi), __fmul_rn((float)K, v.lo)};
+  else
+    return df32(K) * v;
+}
+template <int K, bool ONE>
+static __device__ __forceinline__ df32 df_times(DfFactor<ONE> f, df32 v) {  // (K f) v
+  if constexpr (ONE)
+    return df_times<K>(v);
+  else
+    return df_times<K>(f.v) * v;
+}
+
+// x^A y^B z^C: f0, f1 the radial sums, lapf the radial part of the Laplacian
+template <int A, int B, int C, class Store>
+static __device__ __forceinline__ void ao_function_df(df32 x, df32 y, df32 z, df32 f0, df32 f1, df32 lapf, int q,
+                                                      Store store) {
+  const auto xa = df_power<A>(x);
+  const auto yb = df_power<B>(y);
+  const auto zc = df_power<C>(z);
+  const auto yz = yb * zc;
+  const auto P0 = xa * yz;
+  const df32 P0f1 = df_times<2>(df_times<1>(P0, f1));
+  store(0, q, df_times<1>(P0, f0));
+  df32 dx = x * P0f1, dy = y * P0f1, dz = z * P0f1;
+  if constexpr (A > 0) dx = df_times<A>(df_power<A - 1>(x) * yz, f0) + dx;
+  if constexpr (B > 0) dy = df_times<B>(xa * df_power<B - 1>(y) * zc, f0) + dy;
+  if constexpr (C > 0) dz = df_times<C>(xa * yb * df_power<C - 1>(z), f0) + dz;
+  store(1, q, dx);
+  store(2, q, dy);
+  store(3, q, dz);
+  const df32 radial = df_times<1>(P0, lapf);
+  constexpr int kTerms = (A >= 2) + (B >= 2) + (C >= 2);
+  static_assert(kTerms <= 1, "s to f functions square one coordinate at most");
+  if constexpr (kTerms == 0)
+    store(4, q, radial);
+  else if constexpr (A >= 2)
+    store(4, q, df_times<A * (A - 1)>(df_power<A - 2>(x) * yz, f0) + radial);
+  else if constexpr (B >= 2)
+    store(4, q, df_times<B * (B - 1)>(xa * df_power<B - 2>(y) * zc, f0) + radial);
+  else
+    store(4, q, df_times<C * (C - 1)>(xa * yb * df_power<C - 2>(z), f0) + radial);
+}
+// the functions of a shell of degree L, x^A first
+template <int L, int A, int B, class Store>
+static __device__ __forceinline__ void ao_shell_df(df32 x, df32 y, df32 z, df32 f0, df32 f1, df32 lapf, int q, Store store) {
+  ao_function_df<A, B, L - A - B>(x, y, z, f0, f1, lapf, q, store);
+  if constexpr (B > 0)
+    ao_shell_df<L, A, B - 1>(x, y, z, f0, f1, lapf, q + 1, store);
+  else if constexpr (A > 0)
+    ao_shell_df<L, A - 1, L - A + 1>(x, y, z, f0, f1, lapf, q + 1, store);
 }
 
 template <class Store>
@@ -388,33 +464,24 @@ static __device__ __forceinline__ void ao_shell_values_df(const DevProblem& P, i
     const df32 al(a2.x, a2.y), cf(c2.x, c2.y);
     const df32 ex = cf * df_exp_nonpos(-(al * s2));
     const df32 ae = al * ex;
-    f0 = f0 + ex;
-    f1 = f1 - ae;
-    f2 = f2 + al * ae;
-  }
-  const df32 lapf = df32(4 * l + 6) * f1 + df32(4) * (s2 * f2);
-  const df32 two(2);
-  int q = 0;
-  for (int a = l; a >= 0; a--)
-    for (int b = l - a; b >= 0; b--, q++) {
-      const int cc = l - a - b;
-      const df32 xa = df_ipow(x, a), yb = df_ipow(y, b), zc = df_ipow(z, cc);
-      const df32 yz = yb * zc;
-      const df32 P0 = xa * yz;
-      const df32 Px = a ? df32(a) * (df_ipow(x, a - 1) * yz) : df32(0);
-      const df32 Py = b ? df32(b) * (xa * df_ipow(y, b - 1) * zc) : df32(0);
-      const df32 Pz = cc ? df32(cc) * (xa * yb * df_ipow(z, cc - 1)) : df32(0);
-      df32 lapP(0);
-      if (a >= 2) lapP = lapP + df32(a * (a - 1)) * (df_ipow(x, a - 2) * yz);
-      if (b >= 2) lapP = lapP + df32(b * (b - 1)) * (xa * df_ipow(y, b - 2) * zc);
-      if (cc >= 2) lapP = lapP + df32(cc * (cc - 1)) * (xa * yb * df_ipow(z, cc - 2));
-      const df32 P0f1 = two * (P0 * f1);
-      store(0, q, P0 * f0);
-      store(1, q, Px * f0 + x * P0f1);
-      store(2, q, Py * f0 + y * P0f1);
-      store(3, q, Pz * f0 + z * P0f1);
-      store(4, q, lapP * f0 + P0 * lapf);
+    if (p == 0) {
+      f0 = ex;
+      f1 = -ae;
+      f2 = al * ae;
+    } else {
+      f0 = f0 + ex;
+      f1 = f1 - ae;
+      f2 = f2 + al * ae;
     }
+  }
+  const df32 lapf = df32(4 * l + 6) * f1 + df_times<4>(s2 * f2);
+  static_assert(kMaxL == 3, "one case for each degree");
+  switch (l) {
+    case 0: ao_shell_df<0, 0, 0>(x, y, z, f0, f1, lapf, 0, store); break;
+    case 1: ao_shell_df<1, 1, 0>(x, y, z, f0, f1, lapf, 0, store); break;
+    case 2: ao_shell_df<2, 2, 0>(x, y, z, f0, f1, lapf, 0, store); break;
+    default: ao_shell_df<3, 3, 0>(x, y, z, f0, f1, lapf, 0, store); break;
+  }
 }
 
 }  // namespace mdet

@@ -104,7 +104,8 @@ __device__ __forceinline__ void digit_pairs(df32 x0, df32 x1, int er, uint32_t (
 #pragma unroll
     for (int y = 0; y < 2; y++) {
       const float h = __fmul_rn(vh[y], 256.0f), l = __fmul_rn(vl[y], 256.0f), d = rintf(h);
-      two_sum(__fsub_rn(h, d), l, vh[y], vl[y]);
+      // h - d is zero or at least an ulp of h, twice |l|
+      fast_two_sum(__fsub_rn(h, d), l, vh[y], vl[y]);
       b[y] = __float_as_uint(d);  // |d| <= 256: exact in BF16
     }
     w[i] = __byte_perm(b[0], b[1], 0x7632);
