@@ -28,10 +28,11 @@
 //               of the time).
 // FP64 orbitals of small bases and of re-evaluated walkers take k_mo_ao with plain FP64 rows instead of digits, and
 //  k_mo_dot     the FP64 dot products, one thread per row and MO.
-// 8,192 walkers of 17 electrons, 110 AOs, 80 MOs: k_mo_ao 0.73 and k_mo_orders 0.42 ms as pairs (3.60
+// 8,192 walkers of 17 electrons, 110 AOs, 80 MOs: k_mo_ao 0.50 and k_mo_orders 0.42 ms as pairs (3.60
 // as one kernel that kept the digits in shared memory and the MO planes in tensor memory, a single
-// 256-thread block per SM), 1.69 and 0.49 ms in FP64 (16.0 with dot products on the FP64 pipe). With
-// an MMA per digit pair and eight warps that took one MO after the other, k_mo_orders 0.76 and 0.95.
+// 256-thread block per SM), 0.96 and 0.49 ms in FP64 (16.0 with dot products on the FP64 pipe). With
+// an MMA per digit pair and eight warps that took one MO after the other, k_mo_orders 0.76 and 0.95;
+// with the powers of the AO functions as run-time loops, k_mo_ao 0.73 and 1.69.
 #include <algorithm>
 #include <cstdint>
 #include <type_traits>
@@ -185,8 +186,10 @@ __global__ void __launch_bounds__(256) k_mo_ao(DevProblem P, const double* __res
     auto put = [&](int c, int q, T v) {
       *reinterpret_cast<uint2*>(smx + (c * kNE + e) * stride + (ao0 + q) * 8) = AoType<T>::bits(v);
     };
-    if constexpr (std::is_same<T, double>::value)
+    if constexpr (RAW)  // (the order of operations of the CUDA-core kernel)
       ao_shell_values(P, s, pos[e], put);
+    else if constexpr (std::is_same<T, double>::value)
+      ao_shell_values_short(P, s, pos[e], put);
     else
       ao_shell_values_df(P, s, pos[e], put);
   }
