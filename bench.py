@@ -27,11 +27,27 @@ METRIC = "walker-steps/s (Ψ,∇Ψ,∇²Ψ), 17e⁻, N_det=750k: mixed vs FP64 a
 UNIT = "walker-steps/s"
 CPU_SAMPLE_WALKERS = 96     # bounded oracle sample for the CPU baseline (~10-30 s of CPU work)
 CPU_SINGLE_CORE_WALKERS = 8  # the same oracle on one core, for the per-core figure
-# dram__bytes_read.sum + dram__bytes_write.sum of the average k_spmm_seg launch on the 750k workload
-# with 8,192 walkers, from one ncu capture of the current kernel per (precision, walker chunks):
-# mixed in three chunks of 6, 21 and 5 tiles (the six launches of one evaluation), FP64 in one; null
-# for a configuration that was not captured
-SPMM_TRAFFIC_750K = {("mixed", 3): 182.7e6, ("fp64", 1): 602.1e6}
+# dram__bytes_read.sum + dram__bytes_write.sum of one k_mod_gemm launch on the 750k workload with 8,192
+# walkers, from one ncu capture per precision; null for a configuration that was not captured
+GEMM_TRAFFIC_750K = {}
+# The CI contraction as residue products (k_mod_gemm) keeps 124.6 bits in moduli of at most 8: at least
+# 16 planes of each order's C. The magnitude sum of the error estimate is not counted.
+MIN_RESIDUE_PLANES = 16
+
+
+def contraction_dense(n_det, n_up, n_dn):
+    """The library's rule for the residue products: dense enough that the tensor cores' dense products
+    take less time than the sparse FP64 sums."""
+    return n_det >= 4096 and n_det > 0.012 * n_up * n_dn
+
+
+def bf16_peak():
+    """(TFLOP/s, source): the measured cuBLAS BF16 burst rate of this GPU model."""
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
+            return float(json.load(f)["bf16_tflops"]), "measured: cuBLAS BF16 burst rate"
+    except (OSError, KeyError, ValueError):
+        return 1900.0, "fallback: one earlier cuBLAS BF16 measurement"
 
 
 def _env_int(k, d):
@@ -360,28 +376,38 @@ def run_ours(args):
     h2d = W * N * 3 * 8
     d2h = W * (8 + 1 + 3 * N * 8 + N * 8 + 8 + 4)
 
-    # roofline of the dominant kernel: the FP64 sparse contraction k_spmm_seg, 2 launches per
-    # step and walker chunk (v = C r_dn, u = C^T r_up), each 2 FLOP per nonzero per walker;
-    # the average launch covers W / chunks walkers
+    # roofline of the CI contraction: residue products on the BF16 tensor cores (one launch, both
+    # orders), or the FP64 sparse sums (one launch for both orders and walker chunk, each 2 FLOP per
+    # nonzero per walker)
     kern = main["kern"]
-    flops_launch = 2.0 * st["n_det"] * W / main_chunks
-    launch_ms = kern["contract_timed"] / (2 * main_chunks)
-    achieved = flops_launch / (launch_ms / 1e3) / 1e12
-    traffic = args.traffic
-    if traffic is None and args.workload == "chlorine_like_750k" and W == 8192:
-        traffic = SPMM_TRAFFIC_750K.get((primary, main_chunks))
     peak, peak_ms, peak_clocks = fp64_peak(local, _gpu_index(local))
-    roofline = {"kernel": "k_spmm_seg", "bound": "alu", "achieved": achieved, "peak": peak,
-                "unit": "TFLOP/s", "frac": achieved / peak, "traffic": traffic,
-                "traffic_unit": "bytes per launch (ncu dram read + write)",
-                "peak_source": "measured in this run: FP64 FMA probe (mdet_measure_fp64_rate, 8 independent "
-                               "accumulators per thread fed from L1-resident tables, 16 warps per SM, fastest of "
-                               "12 launches of %.1f ms)" % peak_ms,
-                "peak_clocks": peak_clocks, "peak_nominal": 1.25,
-                "flops_per_launch": flops_launch, "launch_ms": launch_ms,
-                "launch_ms_source": "mean over the timed steps of each launch's device duration, from its first "
-                                    "block's start to its last warp's exit on the GPU global timer (written by the "
-                                    "kernel; CUDA events in the pipelined streams lengthen the step by about 10 %)"}
+    timed = ("mean over the timed steps of each launch's device duration, from its first block's start to its "
+             "last warp's exit on the GPU global timer (written by the kernel)")
+    traffic = args.traffic
+    if contraction_dense(st["n_det"], st["n_det_up"], st["n_det_dn"]):
+        if traffic is None and args.workload == "chlorine_like_750k" and W == 8192:
+            traffic = GEMM_TRAFFIC_750K.get(primary)
+        flops_launch = 2.0 * 2.0 * MIN_RESIDUE_PLANES * st["n_det_up"] * st["n_det_dn"] * W / main_chunks
+        launch_ms = kern["contract_timed"] / main_chunks
+        tpeak, tsource = bf16_peak()
+        achieved = flops_launch / (launch_ms / 1e3) / 1e12
+        roofline = {"kernel": "k_mod_gemm", "bound": "tensor", "achieved": achieved, "peak": tpeak,
+                    "unit": "TFLOP/s", "frac": achieved / tpeak, "peak_source": tsource, "peak_nominal": 2250.0,
+                    "flops_note": "BF16 operations of %d residue planes (the least any expansion has), without the "
+                                  "magnitude sums" % MIN_RESIDUE_PLANES}
+    else:
+        flops_launch = 4.0 * st["n_det"] * W / main_chunks
+        launch_ms = kern["contract_timed"] / main_chunks
+        achieved = flops_launch / (launch_ms / 1e3) / 1e12
+        roofline = {"kernel": "k_spmm_seg", "bound": "alu", "achieved": achieved, "peak": peak,
+                    "unit": "TFLOP/s", "frac": achieved / peak,
+                    "peak_source": "measured in this run: FP64 FMA probe (mdet_measure_fp64_rate, 8 independent "
+                                   "accumulators per thread fed from L1-resident tables, 16 warps per SM, fastest of "
+                                   "12 launches of %.1f ms)" % peak_ms,
+                    "peak_clocks": peak_clocks, "peak_nominal": 1.25}
+    roofline.update(traffic=traffic, traffic_unit="bytes per launch (ncu dram read + write)",
+                    flops_per_launch=flops_launch, launch_ms=launch_ms, launch_ms_source=timed,
+                    fp64_peak_tflops=peak)
 
     line = {"metric": METRIC, "value": main["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": main["ms"], "higher_is_better": True, "scaling": "weak",
@@ -477,8 +503,8 @@ def measure_batched(precision, steps, warmup, streams=8, tune_ms=60.0, fallback_
     ms = statistics.mean(a.elapsed_time(b) for a, b in ev)
     W = sum(wl.n_walk for wl in wls)
     # time of each expansion alone (no batching), for the gain of sharing the GPU, and the roofline
-    # of its FP64 contraction (4 FLOP per product and walker; launch times from the kernels' own
-    # timer stamps, profiling mode 2, which adds no event to the streams)
+    # of the FP64 contraction of those on the sparse sums (4 FLOP per product and walker; launch times
+    # from the kernels' own timer stamps, profiling mode 2, which adds no event to the streams)
     solo = 0.0
     contract_tf = []
     for c, R, wl in zip(ctxs, Rs, wls):
@@ -493,9 +519,13 @@ def measure_batched(precision, steps, warmup, streams=8, tune_ms=60.0, fallback_
         solo += a.elapsed_time(b)
         cms = c.profile()["contract"]
         c.set_profiling(False)
-        contract_tf.append((4.0 * wl.n_det * wl.n_walk / (cms * 1e-3) / 1e12 if cms > 0 else float("nan"),
-                            4.0 * wl.n_det * wl.n_walk, cms))
+        cst = c.stats()
+        if not contraction_dense(cst["n_det"], cst["n_det_up"], cst["n_det_dn"]):
+            contract_tf.append((4.0 * wl.n_det * wl.n_walk / (cms * 1e-3) / 1e12 if cms > 0 else float("nan"),
+                                4.0 * wl.n_det * wl.n_walk, cms))
     peak, _, _ = fp64_peak(dev.index, _gpu_index(dev.index))
+    if not contract_tf:  # every expansion took the residue products
+        contract_tf.append((float("nan"), 0.0, float("nan")))
     tf = np.array([t[0] for t in contract_tf])
     flops = np.array([t[1] for t in contract_tf])
     weighted = float(flops.sum() / (sum(t[2] for t in contract_tf) * 1e-3) / 1e12)
@@ -514,8 +544,8 @@ def measure_batched(precision, steps, warmup, streams=8, tune_ms=60.0, fallback_
                 "achieved": {"min": float(np.nanmin(tf)), "median": float(np.nanmedian(tf)),
                              "max": float(np.nanmax(tf)), "all_expansions": weighted},
                 "frac_median": float(np.nanmedian(tf)) / peak, "frac_all_expansions": weighted / peak,
-                "note": "each expansion evaluated alone; all_expansions = total contraction FLOPs over total "
-                        "contraction time"},
+                "note": "each expansion of the sparse sums (%d of %d) evaluated alone; all_expansions = their total "
+                        "contraction FLOPs over their total contraction time" % (len(contract_tf), len(ctxs))},
             "tuning_histogram": {k: dict(zip(*np.unique([t[k] for t in tunes], return_counts=True)))
                                  for k in ("spmm_chunk", "mo_ec", "walker_chunks")},
             "clocks": clk.summary(),

@@ -298,8 +298,9 @@ mdet_status mdet_get_fallback(const mdet_ctx* ctx, double* tol, int* max_walkers
  * higher priority, the FP64 contractions one after another on a persistent grid
  * that leaves part of every SM free. So the contraction of chunk k overlaps the
  * orbitals and tables of chunk k+1 and the epilogue of chunk k-1. 0 selects the
- * automatic choice (3 chunks with the FP64 contraction, at least 100,000
- * products and 3,072 walkers; otherwise 1), 1 disables the overlap. Values
+ * automatic choice (3 chunks with the sparse FP64 contraction, at least 100,000
+ * products and 3,072 walkers; otherwise, and always with the contraction as
+ * residue products on the tensor cores, 1), 1 disables the overlap. Values
  * above 8 are clamped, and so are values above the number of 256-walker tiles.
  * The FP64 path always runs as one chunk on the caller's stream.
  */
@@ -312,20 +313,26 @@ mdet_status mdet_get_last_launches(const mdet_ctx* ctx, int32_t* n_chunks, int32
 
 /*
  * Tile shapes of the evaluation kernels (tuning knobs with no counterpart in
- * the paper): spmm_chunk nonzeros of C per warp in the contraction (64..8192),
+ * the paper): spmm_chunk nonzeros of C per warp in the sparse contraction
+ * (64..8192; the default, 512, is lowered to 16 for small expansions),
  * mo_ec electrons per thread block in the orbital kernels (4, 6 or 8),
- * walker_chunks as in mdet_set_walker_chunks, spmm_blocks the grid of the FP64
- * contraction (0: one warp per work item with one chunk, 4 blocks per SM with
- * several; otherwise a persistent grid of at most that many 128-thread blocks
- * whose warps draw work items from a counter), mo_impl the mixed-precision
- * orbital product (2, the default: exact BF16 digit products on the tcgen05
- * tensor cores with TMEM accumulators, accurate to about 2^-55 of the row and
- * column maxima, for at most 112 AOs and 128 MOs, beyond which it falls back to
- * 1; 1: the compensated FP32 dot product on the CUDA cores, accurate relative to
- * each term; 0: the same digit products on warp-level mma.sync),
- * contract_impl the CI contraction of the mixed path (0, the default: FP64;
- * 1: double-float pairs on the FP32 pipe with a compensated dot product, an
- * option outside the FP64 contraction of the method's precision plan).
+ * walker_chunks as in mdet_set_walker_chunks, spmm_blocks the form of the
+ * contraction (0: where C is dense enough, more than 1.2 % of at least 4,096
+ * products, exact residue products on the tcgen05 tensor cores with one rounding
+ * at the end, if the device has room for C's planes; elsewhere sparse FP64 sums,
+ * one warp per work item with one chunk, 4 blocks per SM with several; any other
+ * value: the sparse sums on a persistent grid of at most that many 128-thread
+ * blocks whose warps draw work items from a counter), mo_impl the orbital product
+ * (2, the default: exact BF16 digit products on the tcgen05 tensor cores with
+ * TMEM accumulators, in mixed precision accurate to about 2^-55 of the row and
+ * column maxima and in FP64 to 2^-63; for small bases and the re-evaluation of
+ * flagged walkers FP64 dot products; where the digits' sums could exceed 2^24 it
+ * falls back to 1; 1: on the CUDA cores, the compensated FP32 dot product, accurate
+ * relative to each term, or the FP64 product; 0: mixed precision, the same digit
+ * products on warp-level mma.sync),
+ * contract_impl the CI contraction of the mixed path (0, the default: exact or
+ * FP64 as above; 1: double-float pairs on the FP32 pipe with a compensated dot
+ * product, an option outside the FP64 contraction of the method's precision plan).
  * Defaults: spmm_chunk 512, mo_ec 4 (mixed) or 6 (FP64), walker_chunks 0,
  * spmm_blocks 0, mo_impl 2, contract_impl 0.
  * best_ms and trials are filled by mdet_autotune (the fastest step time seen
@@ -397,7 +404,8 @@ void mdet_batch_destroy(mdet_batch* b);
  * tenth. Mode 2 therefore records no event: the contraction kernels write the
  * GPU's global timer (ns) at their first block's start and their last warp's
  * exit into words of the context's scratch, and mdet_get_profile returns the
- * sum of those launch durations as the contraction entry (the other entries
+ * sum of those launch durations as the contraction entry (with the residue
+ * products, from the first to the last matrix product; the other entries
  * stay zero). 0 (the default) records nothing. MDET_E_ARG for another mode.
  * mdet_get_profile waits for the last evaluation's stream (mode 2) or events.
  */
@@ -406,7 +414,7 @@ enum {
   MDET_STAGE_REFERENCE = 1, /* reference LU, inverse, tables (Sec. 2.2, Sec. 5) */
   MDET_STAGE_RATIOS = 2,    /* determinant ratios (Sec. 2.2) */
   MDET_STAGE_ZERO = 3,      /* clearing of the contraction accumulators */
-  MDET_STAGE_CONTRACT = 4,  /* sparse bilinear contraction (Sec. 2.4) */
+  MDET_STAGE_CONTRACT = 4,  /* bilinear contraction (Sec. 2.4) */
   MDET_STAGE_FINAL = 5,     /* derivative aggregation and epilogue (Sec. 2.3) */
   MDET_N_STAGES = 6
 };

@@ -1,14 +1,18 @@
 // FP64 kernels of one evaluation (Sec. 2.2-2.4), in launch order:
-//   k_mo_f64         orbitals and their derivatives at every electron (Sec. 2)
+//   k_mo_f64         orbitals and their derivatives at every electron (Sec. 2) on the CUDA cores
+//                    (the default is the digit products of mdet_mo_digits.cu)
 //   k_ref            LU with partial pivoting of each reference Slater matrix,
 //                    its inverse A, log|D_ref|, the table T = A Phi and the
 //                    single-determinant derivatives g (Sec. 2.2; Sec. 5 Table method)
 //   k_ratio_f64      D_I / D_ref = eps_I det T[h_I, p_I] for every distinct
 //                    spin determinant (k x k, k <= 4)
-//   k_spmm_wm        v = C r_dn (plus Psi~ = r_up . v) and u = C^T r_up (Sec. 2.4),
-//                    8 walkers per lane, walker-major output (k_spmm_df: the
-//                    double-float option of the mixed path; k_spmm_f64: the
-//                    walker-minor form used by the allocation-free entry point)
+//   k_spmm_seg       v = C r_dn (plus Psi~ = r_up . v) and u = C^T r_up (Sec. 2.4) as sparse
+//                    sums, walker-major output (dense expansions: mdet_modgemm.cu;
+//                    k_spmm_df: the double-float option of the mixed path;
+//                    k_spmm_f64: the walker-minor form used by the allocation-free
+//                    entry point)
+//   k_scatter        the cofactor sums W of the derivative aggregation, lanes over walkers
+//                    (many walkers; k_final scatters by itself otherwise)
 //   k_final          derivative aggregation and the per-walker epilogue (Eqs. 5-8)
 // k_ref and k_final take a MIXED flag: the mixed-precision variants (and the
 // mixed orbital and ratio kernels of mdet_kernels_mixed.cu) run the

@@ -1,7 +1,7 @@
 // Inline-PTX helpers for the 5th-generation tensor cores (tcgen05, sm_100a /
 // sm_103a): shared-memory matrix descriptors, the instruction descriptor of
-// kind::f16 with BF16 operands, bounded mbarrier waits, tensor-memory loads and
-// stores, and the MMA forms used by the orbital product and the perceptron.
+// kind::f16 with BF16 operands, bounded mbarrier waits, bulk copies, tensor-memory loads
+// and the MMA used by the orbital product, the residue products and the perceptron.
 //
 // Operand layout (orbital product and perceptron): K-major, no swizzle. A core matrix is 8 rows of
 // 16 bytes (8 BF16 along K); `lbo` is the byte distance between core matrices
@@ -76,12 +76,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t base, uint32_t ncols) {
   asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(base), "r"(ncols) : "memory");
 }
 
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t (&v)[8]) {
-  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(taddr), "r"(v[0]),
-               "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-               : "memory");
-}
-
 // 16 consecutive 32-bit columns of the warp's 32 lanes (lane i of the warp gets lane
 // base + i), waited for.
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
@@ -92,15 +86,6 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
       : "r"(taddr)
       : "memory");
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// D (+)= A B^T with A in tensor memory (lane = row, two BF16 per column, even k low)
-// and B described in shared memory; acc = 0 overwrites D.
-__device__ __forceinline__ void mma_tmem_a(uint32_t d, uint32_t a, uint64_t bdesc, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}" ::"r"(d),
-      "r"(a), "l"(bdesc), "r"(idesc), "r"(acc)
-      : "memory");
 }
 
 // D (+)= A B^T with both operands described in shared memory.
