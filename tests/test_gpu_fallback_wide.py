@@ -1,5 +1,6 @@
-"""The full-LU fallback from 12 electrons per spin up (four lanes to a determinant): sizes around the
-groups of four rows and columns, unequal spins, determinant counts that leave a ragged last group."""
+"""The full-LU fallback at the electron numbers where its kernels change (matrix in registers up to 8 a
+spin, in shared memory up to 11, four lanes to a determinant from 12): sizes around the groups of four
+rows and columns, unequal spins, determinant counts that leave a ragged last group."""
 from __future__ import annotations
 
 import numpy as np
@@ -16,7 +17,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("prec", [pytest.param(pkg.PRECISION_FP64, id="fp64"), pytest.param(pkg.PRECISION_MIXED, id="mixed")])
-@pytest.mark.parametrize("n_up,n_dn", [(11, 11), (12, 9), (13, 12), (15, 14), (16, 16), (17, 1), (17, 16)])
+@pytest.mark.parametrize("n_up,n_dn", [(2, 2), (3, 2), (4, 4), (5, 4), (7, 6), (8, 8), (9, 8), (10, 10), (11, 11), (12, 9), (13, 12), (15, 14), (16, 16), (17, 1), (17, 16)])
 def test_every_walker_by_full_lu(n_up, n_dn, prec):
     wl = synth.make_workload("wide", 5 + n_up, n_up, n_dn, n_up + n_dn, (9, 6, 2), (0.05, 500.0), n_up + 6, 90, 4, 7,
                              n_unique=(13, 10))
