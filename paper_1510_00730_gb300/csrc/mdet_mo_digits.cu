@@ -46,7 +46,9 @@ namespace mdet {
 
 namespace {
 
-constexpr int kNE = 16;                       // electrons per block of k_mo_ao
+// electrons per block of k_mo_ao: 16 keep two shells to a warp; with fewer such blocks than SMs 8 (512
+// electrons as pairs 15 -> 10 us, 2056 in FP64 25 -> 22; 4 and 2 electrons 10 and 10, 33 and 42)
+constexpr int kNE = 16, kNEFew = 8;
 constexpr int kSliceBytes = 2 * 128 * 16;     // one plane of 128 rows x 16 AOs
 constexpr int kChunk = 32;                    // MOs per accumulator set
 constexpr int kEpiWarps = 16, kOrderThreads = 128 + 32 * kEpiWarps;
@@ -146,23 +148,23 @@ struct AoType<df32> {
 // is (5 w + c) N + e, the row of the orbital array; its digits go to
 // [row / 128][AO / 16][digit][AO / 8 mod 2][row mod 128][AO mod 8].
 // RAW: the FP64 values themselves, as rows of K.
-template <class T, bool RAW>
+template <class T, bool RAW, int NE>
 __global__ void __launch_bounds__(256) k_mo_ao(DevProblem P, const double* __restrict__ R, int64_t w0, int64_t n_el,
                                                uint8_t* __restrict__ xd, int* __restrict__ xer, int Kp,
                                                const int* __restrict__ live) {
   constexpr int D = AoType<T>::D, kABytes = D * kSliceBytes;
   extern __shared__ __align__(16) uint8_t smx[];
-  __shared__ int rexp[5 * kNE];
-  __shared__ int rowbase[kNE];
-  __shared__ T pos[kNE][3];
+  __shared__ int rexp[5 * NE];
+  __shared__ int rowbase[NE];
+  __shared__ T pos[NE][3];
   const int K = P.n_ao, N = P.n_elec;
   const int stride = Kp * 8 + 16;
-  const int64_t g0 = (int64_t)blockIdx.x * kNE;  // first electron, counted from walker w0
+  const int64_t g0 = (int64_t)blockIdx.x * NE;  // first electron, counted from walker w0
   if (live) n_el = min(n_el, max((int64_t)0, (*live - w0) * N));
   if (g0 >= n_el) return;
-  const int ne = (int)min((int64_t)kNE, n_el - g0);
+  const int ne = (int)min((int64_t)NE, n_el - g0);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid < kNE) {
+  if (tid < NE) {
     const int64_t g = g0 + tid, w = g / N;
     rowbase[tid] = (int)(w * 4 * N + g);  // 5 w N + e
   }
@@ -174,17 +176,17 @@ __global__ void __launch_bounds__(256) k_mo_ao(DevProblem P, const double* __res
       pos[tid / 3][tid % 3] = df_from_double(x);
   }
   // AO padding
-  for (int t = tid; t < 5 * kNE * (Kp - K); t += 256) {
+  for (int t = tid; t < 5 * NE * (Kp - K); t += 256) {
     const int row = t / (Kp - K);
     *reinterpret_cast<double*>(smx + row * stride + (K + t - row * (Kp - K)) * 8) = 0.0;
   }
   __syncthreads();
-  for (int t = tid; t < kNE * P.n_shell; t += 256) {
-    const int e = t % kNE, s = t / kNE;
+  for (int t = tid; t < NE * P.n_shell; t += 256) {
+    const int e = t % NE, s = t / NE;
     if (e >= ne) continue;
     const int ao0 = P.shell_ao0[s];
     auto put = [&](int c, int q, T v) {
-      *reinterpret_cast<uint2*>(smx + (c * kNE + e) * stride + (ao0 + q) * 8) = AoType<T>::bits(v);
+      *reinterpret_cast<uint2*>(smx + (c * NE + e) * stride + (ao0 + q) * 8) = AoType<T>::bits(v);
     };
     if constexpr (RAW)  // (the order of operations of the CUDA-core kernel)
       ao_shell_values(P, s, pos[e], put);
@@ -196,31 +198,31 @@ __global__ void __launch_bounds__(256) k_mo_ao(DevProblem P, const double* __res
   __syncthreads();
   if constexpr (RAW) {
     double* out = reinterpret_cast<double*>(xd);
-    for (int t = tid; t < 5 * kNE * K; t += 256) {
+    for (int t = tid; t < 5 * NE * K; t += 256) {
       const int r = t / K, k = t - r * K;
-      if (r % kNE < ne)
-        out[((int64_t)rowbase[r % kNE] + (int64_t)(r / kNE) * N) * K + k] =
+      if (r % NE < ne)
+        out[((int64_t)rowbase[r % NE] + (int64_t)(r / NE) * N) * K + k] =
             *reinterpret_cast<const double*>(smx + r * stride + k * 8);
     }
     return;
   }
   // row exponents: |x| < 2^e over the row
-  for (int r = warp; r < 5 * kNE; r += 8) {
-    if (r % kNE >= ne) continue;
+  for (int r = warp; r < 5 * NE; r += 8) {
+    if (r % NE >= ne) continue;
     unsigned k = 0;
     for (int a = lane; a < K; a += 32) k = max(k, AoType<T>::key(*reinterpret_cast<const uint2*>(smx + r * stride + a * 8)));
     k = __reduce_max_sync(0xffffffffu, k);
     if (lane == 0) {
       const int e = AoType<T>::row_exp(k);
       rexp[r] = e;
-      xer[rowbase[r % kNE] + r / kNE * N] = e;
+      xer[rowbase[r % NE] + r / NE * N] = e;
     }
   }
   __syncthreads();
   // digits of 8 consecutive AOs of one row: 16 bytes per plane, consecutive lanes in consecutive rows
   const int n_k8 = Kp / 8;
-  for (int t = tid; t < 5 * kNE * n_k8; t += 256) {
-    const int k8 = t / (5 * kNE), r = t - k8 * 5 * kNE, e = r % kNE;
+  for (int t = tid; t < 5 * NE * n_k8; t += 256) {
+    const int k8 = t / (5 * NE), r = t - k8 * 5 * NE, e = r % NE;
     if (e >= ne) continue;
     const int er = rexp[r];  // (a bad row's products are not used)
     const uint8_t* src = smx + r * stride + k8 * 64;
@@ -230,7 +232,7 @@ __global__ void __launch_bounds__(256) k_mo_ao(DevProblem P, const double* __res
       const uint4 b = *reinterpret_cast<const uint4*>(src + z * 8);
       digit_pairs(AoType<T>::value(make_uint2(b.x, b.y)), AoType<T>::value(make_uint2(b.z, b.w)), er, w[z >> 1]);
     }
-    const int64_t row = (int64_t)rowbase[e] + (int64_t)(r / kNE) * N;
+    const int64_t row = (int64_t)rowbase[e] + (int64_t)(r / NE) * N;
     uint8_t* dst = xd + ((row >> 7) * (Kp / 16) + (k8 >> 1)) * kABytes + (k8 & 1) * 2048 + (row & 127) * 16;
 #pragma unroll
     for (int i = 0; i < D; i++)
@@ -468,30 +470,34 @@ bool use_mo_digits(const DevProblem& P, const DevScratch& S, int64_t n_walk, boo
 template <class T, class Out>
 static cudaError_t launch_mo_digits_t(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R,
                                       const uint16_t* b_tiles, cudaStream_t st) {
-  static SmemOptIn opt[3];
-  const size_t smem1 = (size_t)5 * kNE * (P.tc_kp * 8 + 16);
+  static SmemOptIn opt[5];
   const size_t smem2 = (size_t)AoType<T>::kStages * AoType<T>::D * (kSliceBytes + 2 * kChunk * 16);
   // FP64 dot products on the FP64 pipe, to the bit those of the CUDA-core kernel: for small bases,
   // where they cost little (2,048: a 45 x 45 basis), and for the few walkers of a re-evaluation,
   // whose ill-conditioned references amplify any change of rounding
   const bool raw = std::is_same<T, double>::value && ((int64_t)P.n_ao * P.n_mo < kMinDigitWork || S.live || !b_tiles);
-  cudaError_t e = raw ? opt[2].ensure(k_mo_ao<double, true>, smem1) : opt[0].ensure(k_mo_ao<T, false>, smem1);
+  const bool few = (n_walk * P.n_elec + kNE - 1) / kNE < P.n_sm;
+  const int ne = few ? kNEFew : kNE;
+  const size_t smem1 = (size_t)5 * ne * (P.tc_kp * 8 + 16);
+  auto* ao = raw ? (few ? k_mo_ao<double, true, kNEFew> : k_mo_ao<double, true, kNE>)
+                 : (few ? k_mo_ao<T, false, kNEFew> : k_mo_ao<T, false, kNE>);
+  cudaError_t e = opt[few ? 3 + raw : 2 * raw].ensure(ao, smem1);
   if (e == cudaSuccess && !raw) e = opt[1].ensure(k_mo_orders<T, Out>, smem2);
   if (e != cudaSuccess) return e;
   const int64_t N = P.n_elec;
   for (int64_t w0 = 0; w0 < n_walk; w0 += S.xd_walk) {
     const int64_t nb = std::min<int64_t>(S.xd_walk, n_walk - w0), rows = nb * 5 * N;
-    const unsigned g1 = (unsigned)((nb * N + kNE - 1) / kNE);
+    const unsigned g1 = (unsigned)((nb * N + ne - 1) / ne);
     const unsigned g2 = (unsigned)std::min<int64_t>((rows + 127) / 128, std::max(P.n_sm, 1));
     if (raw) {
-      k_mo_ao<double, true><<<g1, 256, smem1, st>>>(P, R, w0, nb * N, S.xd, S.xer, P.tc_kp, S.live);
+      ao<<<g1, 256, smem1, st>>>(P, R, w0, nb * N, S.xd, S.xer, P.tc_kp, S.live);
       k_mo_dot<<<(unsigned)((rows * P.n_mo + 255) / 256), 256, 0, st>>>(
           reinterpret_cast<const double*>(S.xd), P.B, P.n_ao, P.n_mo, S.phi + w0 * 5 * N * P.n_mo, rows, 5 * P.n_elec,
           S.live, w0);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       continue;
     }
-    k_mo_ao<T, false><<<g1, 256, smem1, st>>>(P, R, w0, nb * N, S.xd, S.xer, P.tc_kp, S.live);
+    ao<<<g1, 256, smem1, st>>>(P, R, w0, nb * N, S.xd, S.xer, P.tc_kp, S.live);
     k_mo_orders<T, Out><<<g2, kOrderThreads, smem2, st>>>(P, b_tiles, S.xd, S.xer,
                                                 reinterpret_cast<Out*>(S.phi + w0 * 5 * N * P.n_mo), rows, S.live, w0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
