@@ -486,15 +486,16 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
 // a warp per walker and product, four consecutive determinants per lane (one 4-byte load per
 // modulus, all issued before the arithmetic). Bound by instruction issue and the loads' latency at 24
 // warps an SM, not by its 25 bytes a determinant. The weighted sums run in 16-bit limbs with dp2a, two
-// moduli at a time, and each weight is fetched once for four determinants: 0.82 ms at 8192 walkers of
-// 750000 determinants in FP64 or mixed, against 1.22 ms with 32-bit limbs in 64-bit multiply-adds and
-// 1.15 ms with two determinants per lane (the constant loads then bound it). Q, the pairs of moduli,
-// is a template argument for the usual counts: unrolled to the largest it takes 0.88 ms. Every
+// moduli at a time, and each weight is fetched once for four determinants: an evaluation's two launches
+// (8192 walkers of 750000 determinants, and those it re-evaluates) 0.82 ms, of which the first is
+// 0.70, against 1.22 with 32-bit limbs in 64-bit multiply-adds and 1.15 with two determinants per
+// lane (the constant loads then bound it). Q, the pairs of moduli, is a template argument for the
+// usual counts: unrolled to the largest 0.88. Every
 // walker's Psi~ is summed in one warp, in a fixed order. Stores go through shared memory so that a
 // warp writes 256 consecutive bytes.
 // Few walkers (a re-evaluation, or too few for the warps of three blocks an SM): four warps to a walker
-// and product, so that each walks a quarter of the determinants: 67 of 256 slots
-// with 900 + 900 determinants 44 -> 14 us, 87 with 3000 + 3000 120 -> 34, 1000 walkers of 900 + 900 46 -> 40.
+// and product, so that each walks a quarter of the determinants: 67 of 256 slots with 900 + 900
+// determinants 44 -> 14 us, 87 with 3000 + 3000 120 -> 34, 1000 walkers of 900 + 900 46 -> 40.
 constexpr int kCrtFewWalkers = 8;
 template <int Q>
 __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ DenseContract D, DevProblem P, DevScratch S,
