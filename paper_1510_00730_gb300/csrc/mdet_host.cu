@@ -753,7 +753,9 @@ mdet_status alloc_eval_arrays(mdet_ctx* c, DevScratch& S, int64_t W, bool df_tab
       S.xer = nullptr;
     }
   }
-  if (c->dense_ok) {  // the workspace of the residue products, for blocks of walkers that it holds
+  // the workspace of the residue products, for blocks of walkers that it holds (a re-evaluation takes the
+  // sparse sums: see refine)
+  if (c->dense_ok && main_scratch) {
     size_t x, y, ya;
     dense_bytes(c->dense, &x, &y, &ya);
     const int64_t fit = (int64_t)(kDenseWorkBytes / (x + y + ya)) / kWalkerPad * kWalkerPad;
@@ -889,12 +891,12 @@ mdet_status refine(mdet_ctx* c, bool table, int64_t n_walk, const double* R, dou
   CUDA_TRY(c, launch_ref_tables(P, E, cap, false, st));
   CUDA_TRY(c, launch_ratios_f64(Pe, E, cap, st));  // clears the cut segments of Pe's items
   // few walkers: short work items keep the contraction's chains short, and the epilogue
-  // spreads each walker's determinants over 512 threads
+  // spreads each walker's determinants over 512 threads. Sparse sums also where the evaluation took
+  // residue products: these walkers are the ill-conditioned ones, which amplify any change of rounding
+  // (up to 7e-9 of grad Psi / Psi against 1e-11 to 1e-9 between two runs), and for the 60 to 140 of an
+  // evaluation the sparse sums take about as long.
   Pe.spmm_blocks = 0;
-  if (E.xmax)
-    CUDA_TRY(c, launch_contract_dense(Pe, E, cap, st, nullptr, nullptr));
-  else
-    CUDA_TRY(c, launch_contract_f64(Pe, E, cap, st));
+  CUDA_TRY(c, launch_contract_f64(Pe, E, cap, st));
   CUDA_TRY(c, launch_final(P, E, cap, c->e_R, o.log_abs_psi, o.sign, o.grad, o.lap, o.e_local, o.status, false, st,
                            true));
   CUDA_TRY(c, launch_fallback(P, E, cap, c->e_R, o.log_abs_psi, o.sign, o.grad, o.lap, o.e_local, o.status, st));
@@ -1462,14 +1464,14 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
   // products, else 1) and its contraction's (1 for the sparse sums, 2 in double-float, 3 per walker
   // block of the residue products); the full-LU
   // fallback 5 (list, dets, scale, rows, out); the mixed refinement adds its list, gather,
-  // FP64 orbitals and scatter, and either the mark or the 5 FP64 table kernels
+  // FP64 orbitals and scatter, and either the mark or the 4 FP64 table kernels
   c->last_kernels = 3 * nch + orbital_kernels + contract_kernels + scatter_kernels;
   if (prof_all) CUDA_TRY(c, cudaEventRecord(c->ev_refine[0], st));
   if (mixed && c->E.fb && P.fallback_tol > 0.0) {
     const bool table = escalation_on(c);
     mdet_status es = refine(c, table, n_walk, R, log_abs_psi, sign, grad, lap, e_local, status, st);
     if (es != MDET_OK) return es;
-    c->last_kernels += 3 + 5 + (table ? mo_kernels(P, c->E, P.fallback_cap, false) + (c->E.xmax ? 6 : 4) : 1 + 1);
+    c->last_kernels += 3 + 5 + (table ? mo_kernels(P, c->E, P.fallback_cap, false) + 4 : 1 + 1);
   } else {
     DevScratch Sb = c->S;
     if (!dense) Sb.xmax = nullptr;

@@ -140,3 +140,28 @@ def test_full_lu_contraction(n_walk):
     tol = 200 * 2.0 ** -53 * np.maximum(ref["kappa"], 1.0) + 4 * np.spacing(np.abs(ref["log_abs_psi"]))
     assert np.all(np.abs(got["log_abs_psi"] - sparse["log_abs_psi"]) <= tol)
     assert np.array_equal(got["sign"], sparse["sign"]) and np.array_equal(got["status"], sparse["status"])
+
+
+def test_reevaluated_walkers_take_the_sparse_sums():
+    """A mixed context re-evaluates its flagged walkers by the FP64 tables and the sparse sums, also where
+    the evaluation itself takes the residue products: the kernels launched tell, and the walkers agree with
+    an FP64 context on the sparse sums up to the order in which Psi~ is added."""
+    wl = _workload(130, 70, 200)
+    ctx = pkg.Context.from_workload(wl, device=0, precision=pkg.PRECISION_MIXED)
+    ctx.set_escalation(pkg.Context.ESCALATE_ALWAYS)
+    ctx.set_fallback(1e9)
+    _eval(ctx, wl.R)
+    _, est = ctx.error_estimates(200)
+    ctx.set_fallback(float(np.median(est[:, 0])), 256)  # half the walkers; the FP64 estimates are 64 times smaller
+    got = _eval(ctx, wl.R)
+    # 8 of the evaluation; list, gather, two for the orbitals, reference, ratios, sums, epilogue, 5 of full LU, scatter
+    assert ctx.last_kernels == 8 + 14
+    esc = (got["status"] & pkg.WS_ESCALATED != 0) & (got["status"] & pkg.WS_FALLBACK == 0)
+    assert esc.sum() > 50
+    f64 = pkg.Context.from_workload(wl, device=0)
+    f64.set_fallback(0.0)
+    f64.set_tuning(spmm_blocks=SPARSE_GRID, mo_impl=1)
+    want = _eval(f64, wl.R)
+    tol = 200 * 2.0 ** -53 * np.maximum(oracle.evaluate(wl)["kappa"], 1.0) + 4 * np.spacing(np.abs(want["log_abs_psi"]))
+    assert np.all(np.abs(got["log_abs_psi"] - want["log_abs_psi"])[esc] <= tol[esc])
+    assert np.array_equal(got["sign"][esc], want["sign"][esc])
