@@ -247,6 +247,17 @@ mdet_status mdet_get_ratios(mdet_ctx* ctx, int64_t n_walk, double* r_up, double*
 #define MDET_FALLBACK_MAX_SPIN 17
 mdet_status mdet_set_fallback(mdet_ctx* ctx, double tol, int max_walkers);
 /*
+ * Device memory of the optional workspaces: digit_bytes for the AO values and
+ * digits of the orbital product (default 1.25 GiB), product_bytes for the residues
+ * of the contraction as residue products (default 4 GiB); 0 keeps the default. An
+ * evaluation whose walkers need more goes through a workspace in blocks of the
+ * walkers that fit (at least one, and 256), with the same results. Frees the
+ * scratch, which the next evaluation allocates again, so it is not to be called
+ * while a captured batch of the context is in use. Errors: MDET_E_ARG for a null
+ * context or a negative size.
+ */
+mdet_status mdet_set_workspace(mdet_ctx* ctx, int64_t digit_bytes, int64_t product_bytes);
+/*
  * Norm-based truncation of a CI expansion (Sec. 3). Host call, no context.
  * The expansion is given as products (det_up[k], det_dn[k], coef[k]), k < n_det,
  * in the layout of mdet_set_ci_expansion (host pointers). The squared norm

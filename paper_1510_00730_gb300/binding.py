@@ -87,6 +87,7 @@ def load_library(build_if_missing: bool = True):
     L.mdet_get_last_launches.argtypes = [vp, vp, vp]
     L.mdet_set_escalation.argtypes = [vp, i32]
     L.mdet_set_fallback.argtypes = [vp, C.c_double, i32]
+    L.mdet_set_workspace.argtypes = [vp, i64, i64]
     L.mdet_get_fallback.argtypes = [vp, vp, vp]
     L.mdet_get_error_estimates.argtypes = [vp, i64, vp, vp]
     L.mdet_selftest_df32.argtypes = [i32, i64, vp, vp, vp, vp]
@@ -107,7 +108,7 @@ def load_library(build_if_missing: bool = True):
                  "mdet_evaluate_host", "mdet_get_ratios", "mdet_get_stats", "mdet_get_spin_dets",
                  "mdet_get_ci_matrix", "mdet_omega_sort", "mdet_truncate_norm", "mdet_sm_chain", "mdet_set_ci_expansion_device", "mdet_set_profiling", "mdet_get_profile",
                  "mdet_psi_tilde_noalloc", "mdet_set_walker_chunks", "mdet_get_last_launches", "mdet_set_escalation", "mdet_selftest_df32", "mdet_selftest_inv_r", "mdet_get_tuning",
-                 "mdet_set_tuning", "mdet_autotune", "mdet_batch_evaluate", "mdet_batch_create", "mdet_batch_launch", "mdet_set_fallback", "mdet_get_fallback",
+                 "mdet_set_tuning", "mdet_autotune", "mdet_batch_evaluate", "mdet_batch_create", "mdet_batch_launch", "mdet_set_fallback", "mdet_set_workspace", "mdet_get_fallback",
                  "mdet_get_error_estimates", "mdet_measure_fp64_rate", "mdet_get_timeline"):
         getattr(L, name).restype = i32
     # VMC moves and the learned proposal (include/mdet_vmc.h)
@@ -458,6 +459,10 @@ class Context:
         if max_walkers is None:
             max_walkers = self.fallback[1]
         self._check(self._L.mdet_set_fallback(self._h, float(tol), int(max_walkers)), "mdet_set_fallback")
+
+    def set_workspace(self, digit_bytes=0, product_bytes=0):
+        """Device memory of the optional workspaces (mdet_set_workspace; 0: the defaults)."""
+        self._check(self._L.mdet_set_workspace(self._h, int(digit_bytes), int(product_bytes)), "mdet_set_workspace")
 
     @property
     def fallback(self):

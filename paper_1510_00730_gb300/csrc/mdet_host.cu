@@ -76,6 +76,7 @@ struct mdet_ctx {
   int spmm_blocks = 0;
   int mo_impl = 2;  // mixed orbitals: exact digit products on the tcgen05 tensor cores
   int mo_ec = 4;
+  int64_t digit_bytes = 0, product_bytes = 0;  // workspaces (mdet_set_workspace; 0: the defaults)
   int contract_impl = 0;  // FP64 contraction (the double-float one is an option of the mixed path)
   mdet_tuning last_tune{};
   cudaStream_t fstream = nullptr, cstream = nullptr;
@@ -114,11 +115,10 @@ constexpr int64_t kItemWarps = 4096;
 // the global-timer stamps (start complemented, end) of each
 constexpr int kQueueWords = 6;
 
-// residue planes of C above this size, and workspace of the residue products per context
-constexpr size_t kDenseMaxBytes = (size_t)8 << 30, kDenseWorkBytes = (size_t)4 << 30;
-
-// workspace of the orbitals' AO digits
-constexpr size_t kDigitBytes = (size_t)5 << 28;
+// residue planes of C above this size; default workspaces of the residue products and of the
+// orbitals' AO digits (mdet_set_workspace)
+constexpr size_t kDenseMaxBytes = (size_t)8 << 30;
+constexpr int64_t kDenseWorkBytes = (int64_t)4 << 30, kDigitBytes = (int64_t)5 << 28;
 
 // weights of the first, each middle and the last walker chunk of the pipelined evaluation. The
 // first chunk's orbitals and tables run before any contraction, and the last chunk's epilogue
@@ -743,7 +743,7 @@ mdet_status alloc_eval_arrays(mdet_ctx* c, DevScratch& S, int64_t W, bool df_tab
   }
   if (mo_digits_supported(P, df_tables)) {  // digits of the AO values, for blocks of walkers
     const int64_t row_bytes = (int64_t)mo_digits_row_bytes(P, df_tables), per = 5 * N * row_bytes;
-    S.xd_walk = std::min(W, std::max<int64_t>(1, (int64_t)kDigitBytes / per));
+    S.xd_walk = std::min(W, std::max<int64_t>(1, (c->digit_bytes > 0 ? c->digit_bytes : kDigitBytes) / per));
     const int64_t rows = (S.xd_walk * 5 * N + 127) / 128 * 128;
     if (cudaMalloc((void**)&S.xd, rows * row_bytes) != cudaSuccess ||
         cudaMalloc((void**)&S.xer, sizeof(int) * rows) != cudaSuccess) {  // no room: the CUDA-core products
@@ -758,7 +758,8 @@ mdet_status alloc_eval_arrays(mdet_ctx* c, DevScratch& S, int64_t W, bool df_tab
   if (c->dense_ok && main_scratch) {
     size_t x, y, ya;
     dense_bytes(c->dense, &x, &y, &ya);
-    const int64_t fit = (int64_t)(kDenseWorkBytes / (x + y + ya)) / kWalkerPad * kWalkerPad;
+    const int64_t work = c->product_bytes > 0 ? c->product_bytes : kDenseWorkBytes;
+    const int64_t fit = work / (int64_t)(x + y + ya) / kWalkerPad * kWalkerPad;
     S.dblk = std::min(wp, std::max<int64_t>(fit, kWalkerPad));
     bool ok = cudaMalloc((void**)&S.xmax, sizeof(uint32_t) * 2 * wp) == cudaSuccess &&
               cudaMalloc((void**)&S.dx, x * S.dblk) == cudaSuccess &&
@@ -1568,6 +1569,15 @@ mdet_status mdet_set_fallback(mdet_ctx* c, double tol, int max_walkers) {
   c->P.fallback_tol = tol;
   c->P.fallback_cap = max_walkers;
   if (resize) free_scratch(c);  // the fallback scratch is sized by the cap
+  return MDET_OK;
+}
+
+mdet_status mdet_set_workspace(mdet_ctx* c, int64_t digit_bytes, int64_t product_bytes) {
+  if (!c || digit_bytes < 0 || product_bytes < 0) return MDET_E_ARG;
+  c->digit_bytes = digit_bytes;
+  c->product_bytes = product_bytes;
+  if (c->device >= 0) CUDA_TRY(c, cudaSetDevice(c->device));
+  free_scratch(c);
   return MDET_OK;
 }
 

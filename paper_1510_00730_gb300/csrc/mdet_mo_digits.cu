@@ -423,8 +423,8 @@ __global__ void __launch_bounds__(kOrderThreads, 1) k_mo_orders(DevProblem P, co
             if (valid && wide) {
 #pragma unroll
               for (int j = 0; j < kSide; j += 2) put_two(dst + j0 + j, o[j], o[j + 1]);
-            } else if (kSide == 8 && valid && m0 + 8 <= M) {  // M odd: an odd row starts half a store later
-              if (row & 1) {
+            } else if (kSide == 8 && valid && m0 + 8 <= M) {  // M odd: every other row starts half a store later
+              if (reinterpret_cast<uintptr_t>(dst) & 15) {  // (which ones depends on the block of walkers)
                 dst[0] = o[0];
 #pragma unroll
                 for (int j = 1; j < 7; j += 2) put_two(dst + j, o[j % kSide], o[(j + 1) % kSide]);

@@ -165,3 +165,20 @@ def test_reevaluated_walkers_take_the_sparse_sums():
     tol = 200 * 2.0 ** -53 * np.maximum(oracle.evaluate(wl)["kappa"], 1.0) + 4 * np.spacing(np.abs(want["log_abs_psi"]))
     assert np.all(np.abs(got["log_abs_psi"] - want["log_abs_psi"])[esc] <= tol[esc])
     assert np.array_equal(got["sign"][esc], want["sign"][esc])
+
+
+@pytest.mark.parametrize("prec", [pkg.PRECISION_FP64, pkg.PRECISION_MIXED])
+@pytest.mark.parametrize("n_walk", [513, 700])
+def test_blocks_of_walkers(n_walk, prec):
+    """The residue products in blocks of 256 walkers (a workspace that holds no more), the last one ragged,
+    are those of one block to the bit."""
+    wl = _workload(130, 70, n_walk)
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    ctx.set_fallback(0.0)
+    whole = _eval(ctx, wl.R)
+    assert ctx.last_kernels == 8
+    ctx.set_workspace(product_bytes=1)
+    got = _eval(ctx, wl.R)
+    assert ctx.last_kernels == 8 + 2 * 3
+    for k in ("log_abs_psi", "sign"):  # each walker's Psi~ is summed in a fixed order
+        assert np.array_equal(got[k], whole[k]), k

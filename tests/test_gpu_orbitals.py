@@ -67,3 +67,22 @@ def test_positions_that_are_not_finite(prec):
     ok[[4, 21]] = False
     tol = 22 * 2.0 ** -50 * np.maximum(oracle.evaluate(wl)["kappa"], 1.0)  # the sparse sums' atomics, in any order
     assert np.all(np.abs(got["log_abs_psi"] - clean["log_abs_psi"])[ok] <= (tol + 1e-14)[ok])
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("digit_bytes", [1, 400_000])
+@pytest.mark.parametrize("n_mo", [31, 33])
+def test_blocks_of_walkers(n_mo, digit_bytes, prec):
+    """The orbitals in blocks of walkers (one at a time, and an odd few) with odd numbers of electrons and
+    MOs, so that every other block's array starts half a 16-byte store later; 160 AOs, whose FP64 orbitals
+    take digits."""
+    wl = _workload((20, 20, 5, 5), n_mo, 23)
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    if prec == pkg.PRECISION_MIXED:
+        ctx.set_fallback(1e-7)  # as in test_tile_edges
+    whole = _eval(ctx, wl.R)
+    ctx.set_workspace(digit_bytes=digit_bytes)
+    got = _eval(ctx, wl.R)
+    rep = compare(got, oracle.evaluate(wl), **TOL[prec])
+    assert rep["ok"], rep
+    assert np.array_equal(got["status"], whole["status"]) and np.array_equal(got["sign"], whole["sign"])
