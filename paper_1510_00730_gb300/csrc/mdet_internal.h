@@ -65,7 +65,7 @@ struct ModConst {
 struct DenseContract {
   int nm;                // moduli
   int kb[2];             // 64-wide K blocks over the distinct determinants of each spin
-  int nt[2], hw[2];      // determinant tiles of 2 hw rows of product o (0: v, 1: u)
+  int nt[2], nw[2];      // determinant tiles of nw rows of product o (0: v, 1: u)
   int ldy[2];            // row stride of the residue bytes of product o
   uint16_t* planes[2];   // BF16 residue planes of C and C^T; the two magnitude planes of C
   const int* es[2];      // [n_det_sp[o]] exponents of the rows of C and of C^T

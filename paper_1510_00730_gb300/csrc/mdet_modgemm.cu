@@ -6,8 +6,8 @@
 // TFLOP/s, and they bound the whole evaluation. As a dense product of residues the same sums
 // run on the BF16 tensor cores, which are 1,500 times as fast, so a filled-in C of a few per
 // cent of nonzeros is still far cheaper: 750,000 products over 3,015 x 3,015 distinct
-// determinants and 8,192 walkers take 20.5 ms as FP64 sums, and 5.1 ms here (residues 0.43,
-// products 3.44 at 1.66 PFLOP/s, 0.86 of the measured BF16 burst rate, reconstruction 1.2).
+// determinants and 8,192 walkers take 20.5 ms as FP64 sums, and 4.0 ms here (residues 0.43,
+// products 2.86, reconstruction 0.70).
 //
 // Method (multi-modular integer products, the Chinese remainder theorem).
 //  - Fixed point: row i of C as chat_ij = rint(c_ij 2^(61 - es_i)) with sum_j |c_ij| < 2^es_i,
@@ -127,20 +127,20 @@ __global__ void __launch_bounds__(256) k_mod_rowsum(const int* __restrict__ ptr,
 }
 
 // The residue planes of C in one order (rows = the product's outputs, gathered index = K), and
-// with n_abs the two magnitude planes. Blocks of hw rows x 64 K in the 128-byte swizzle of the
+// with n_abs the two magnitude planes. Blocks of nw rows x 64 K in the 128-byte swizzle of the
 // MMA's shared-memory operands (row r at 128 r, its 16-byte chunk j at chunk j ^ (r mod 8)),
-// [plane][tile][half][K block][row][64]; zeroed before.
+// [plane][tile][K block][row][64]; zeroed before.
 __global__ void __launch_bounds__(256) k_mod_planes(const __grid_constant__ DenseContract D, int o,
                                                     const int* __restrict__ row, const int* __restrict__ col,
                                                     const double* __restrict__ val, int64_t nnz, int n_abs) {
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nnz) return;
-  const int i = row[k], j = col[k], hw = D.hw[o], kb = D.kb[1 - o];
+  const int i = row[k], j = col[k], nw = D.nw[o], kb = D.kb[1 - o];
   const int es = D.es[o][i];
   const long long c = c_fixed(val[k], es);
-  const int h = i / hw, rr = i - h * hw;  // half tiles are consecutive blocks of hw rows
-  const size_t plane = (size_t)D.nt[o] * 2 * kb * hw * 64;
-  const size_t at = ((size_t)h * kb + j / 64) * hw * 64 + (size_t)rr * 64 + (((j % 64) / 8) ^ (rr & 7)) * 8 + j % 8;
+  const int t = i / nw, rr = i - t * nw;
+  const size_t plane = (size_t)D.nt[o] * kb * nw * 64;
+  const size_t at = ((size_t)t * kb + j / 64) * nw * 64 + (size_t)rr * 64 + (((j % 64) / 8) ^ (rr & 7)) * 8 + j % 8;
   for (int q = 0; q < D.nm; q++)
     D.planes[o][q * plane + at] = (uint16_t)(__float_as_uint((float)balanced_mod(c, (int)D.m[q].p)) >> 16);
   if (n_abs) {
@@ -230,25 +230,26 @@ __global__ void __launch_bounds__(256) k_mod_residues(const __grid_constant__ De
 }
 
 // ---------------------------------------------------------------------------
-// The residue products. A work unit is one 256 walker x NW determinant tile (NW = 2 hw <= 256)
-// of one plane: D[w][i] = sum_k Xplane[w][k] Cplane[i][k]. A cluster of two CTAs takes it, 128
-// walkers each (MMAs of M = 128, N = NW, K = 16); the determinant rows serve both, so each CTA
-// fetches one half of them and multicasts it into both shared memories: 32 KB of L2 reads per SM
-// and 64 K instead of 48.
-// Warps: 0 the producer (bulk copies of pre-tiled blocks into a 4-stage ring), 1 the MMA issuer,
-// 2 tensor memory, 4-7 the epilogue of the previous unit from the other of two 256-column
-// accumulators: reduction mod p to one byte, 16 bytes per store. A stage is refilled when both
-// CTAs' MMAs have read it (their commits arrive on both CTAs' barriers).
+// The residue products. A work unit is one 256 walker x nw determinant tile (nw <= 256) of one plane:
+// D[w][i] = sum_k Xplane[w][k] Cplane[i][k]. One CTA takes it as two halves of 128 walkers (MMAs of
+// M = 128, N = nw, K = 16) on the same determinant rows: 64 KB of L2 reads for two 128 x 256 x 64
+// products. A 128 x 256 tile of its own for each half would read 96 KB, which L2 cannot deliver to
+// 152 SMs at the tensor cores' rate.
+// Warps: 0 the producer (bulk copies of pre-tiled blocks into a ring of 3 stages of 64 K), 1 the MMA
+// issuer, 2 tensor memory, 4-11 the epilogue: reduction mod p to one byte, 16 bytes per store.
+// The two halves' accumulators fill tensor memory (2 x 256 columns). The epilogue of a half moves its
+// 128 columns a warp into registers and frees them before it computes, so that the next unit's products
+// wait for that read only. The issuing thread adds stage and K offsets to two descriptors: with the
+// descriptors built, and stages counted modulo 3, for every MMA (and registers spilled, which a
+// launch bound of 640 threads forces) it fell behind the tensor cores, 3.56 ms instead of 2.86 (8,192
+// walkers, 3,015 x 3,015 determinants), and taking the first and last two K blocks half by half, which
+// would hide more of the read, holds stages back and measured 3.25.
 // Units are ordered plane by plane, so that one plane of C and of the ratios stays in L2.
-// cta_group::2 pairs measured 10 % faster alone, but their collective tensor-memory allocation
-// never returned on some SM pairs while other streams' kernels held part of the SMs; CTAs that
-// only share copies have no such dependence. The barrier operations keep their default (CTA)
-// scope: cluster-scope acquires and releases put a fence into every pipeline stage and halved
-// the rate, and the data they guard is written and read by the asynchronous proxy only.
 // Every wait is bounded in time; when one runs out the CTA sets *err and finishes without
 // further copies or MMAs, and the reconstruction writes NaN.
-constexpr int kStages = 4;
-constexpr int kStageBytes = 3 * kTileBytes;
+constexpr int kStages = 3;
+constexpr int kStageBytes = 4 * kTileBytes;  // two tiles of walkers, up to 256 rows of C
+constexpr int kEpiWarps = 8, kGemmThreads = 128 + 32 * kEpiWarps;
 
 struct GemmArgs {
   const uint16_t* X;
@@ -266,34 +267,6 @@ __device__ __forceinline__ unsigned long long now_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
-}
-
-__device__ __forceinline__ uint32_t cta_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-
-// A bulk copy into both CTAs of the cluster, at the same offsets, each signalling its own barrier.
-__device__ __forceinline__ void bulk_load_both(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], %2, [%3], %4;" ::
-          "r"(dst),
-      "l"(src), "r"(bytes), "r"(umma::smem_u32(bar)), "h"((uint16_t)3)
-      : "memory");
-}
-
-// Arrives on both CTAs' barrier at this offset once every MMA this thread issued has completed.
-__device__ __forceinline__ void commit_both(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          umma::smem_u32(bar)),
-      "h"((uint16_t)3)
-      : "memory");
-}
-
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.aligned;\nbarrier.cluster.wait.aligned;" ::: "memory");
 }
 
 __device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t (&v)[16]) {
@@ -334,7 +307,7 @@ __device__ __forceinline__ Unit unit_of(const DenseContract& D, const GemmArgs& 
   return r;
 }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
+__global__ void __launch_bounds__(kGemmThreads, 1)
     k_mod_gemm(const __grid_constant__ DenseContract D, const __grid_constant__ GemmArgs a) {
   extern __shared__ __align__(1024) uint8_t stage_mem[];
   __shared__ __align__(8) uint64_t full[kStages], empty[kStages], tfull[2], tempty[2], fin;
@@ -342,141 +315,149 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(256, 1)
   __shared__ int dead_s;
   volatile int* dead = &dead_s;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const uint32_t rank = cta_rank();
   if (a.stamp && tid == 0) atomicMax(a.stamp, ~now_ns());
   if (warp == 2) umma::tmem_alloc(&tbase, 512);
   if (tid == 0) {
     for (int s = 0; s < kStages; s++) {
       umma::mbar_init(&full[s], 1);
-      umma::mbar_init(&empty[s], 2);
+      umma::mbar_init(&empty[s], 1);
     }
-    for (int b = 0; b < 2; b++) {
-      umma::mbar_init(&tfull[b], 1);
-      umma::mbar_init(&tempty[b], 4);
+    for (int h = 0; h < 2; h++) {
+      umma::mbar_init(&tfull[h], 1);
+      umma::mbar_init(&tempty[h], kEpiWarps);
     }
     umma::mbar_init(&fin, 1);
     dead_s = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   umma::fence_before();
   __syncthreads();
-  cluster_sync();
   umma::fence_after();
   const uint32_t tb = tbase;
   const int64_t w_live = a.live ? max((int64_t)0, (int64_t)*a.live - a.w0) : (int64_t)a.nmt * 128;
   const int nmt2 = (int)min((int64_t)(a.nmt / 2), (w_live + 255) / 256);
   const int64_t n_units = (int64_t)(a.n_abs + D.nm) * nmt2 * D.nt[0] + (int64_t)D.nm * nmt2 * D.nt[1];
-  const int64_t first = blockIdx.x >> 1, step = gridDim.x >> 1;
+  const int64_t first = blockIdx.x, step = gridDim.x;
   const uint32_t stage0 = umma::smem_u32(stage_mem);
 
-  if (warp == 0 && lane == 0) {  // producer: this CTA's walkers, and its half of the determinant rows for both
+  if (warp == 0 && lane == 0) {  // producer
     uint32_t it = 0;
     for (int64_t u = first; u < n_units && !*dead; u += step) {
       const Unit t = unit_of(D, a, u, nmt2);
-      const int sp = 1 - t.o, kb = D.kb[sp], hw = D.hw[t.o];
-      const uint32_t b_bytes = (uint32_t)hw * 128;  // half of the determinant rows
-      const size_t xplane = (size_t)a.nmt * kb * kTileBytes, cplane = (size_t)D.nt[t.o] * 2 * kb * b_bytes;
+      const int sp = 1 - t.o, kb = D.kb[sp];
+      const uint32_t b_bytes = (uint32_t)D.nw[t.o] * 128;
+      const size_t xtile = (size_t)kb * kTileBytes, xplane = (size_t)a.nmt * xtile,
+                   cplane = (size_t)D.nt[t.o] * kb * b_bytes;
       const uint8_t* xs = reinterpret_cast<const uint8_t*>(a.X) +
-                          (sp ? (size_t)D.nm * a.nmt * D.kb[0] * kTileBytes : 0) +
-                          ((size_t)(t.mt * 2 + (int)rank) * kb) * kTileBytes;
-      const uint8_t* cs =
-          reinterpret_cast<const uint8_t*>(D.planes[t.o]) + ((size_t)(t.nt * 2 + (int)rank) * kb) * b_bytes;
+                          (sp ? (size_t)D.nm * a.nmt * D.kb[0] * kTileBytes : 0) + (size_t)t.mt * 2 * xtile;
+      const uint8_t* cs = reinterpret_cast<const uint8_t*>(D.planes[t.o]) + (size_t)t.nt * kb * b_bytes;
       for (int pass = 0; pass < (t.abs ? 3 : 1); pass++) {  // magnitudes: h h, h l, l h
         const uint8_t* xp = xs + (size_t)(t.plane + (pass == 2)) * xplane;
         const uint8_t* cp = cs + (size_t)(t.plane + (pass == 1)) * cplane;
         for (int k = 0; k < kb; k++, it++) {
           const int s = it % kStages;
           if (it >= kStages && !umma::bounded_wait(&empty[s], ((it / kStages) & 1) ^ 1, dead)) break;
-          umma::expect_tx(&full[s], kTileBytes + 2 * b_bytes);
+          umma::expect_tx(&full[s], 2 * kTileBytes + b_bytes);
           const uint32_t dst = stage0 + (uint32_t)s * kStageBytes;
           umma::bulk_load(dst, xp + (size_t)k * kTileBytes, kTileBytes, &full[s]);
-          bulk_load_both(dst + kTileBytes + rank * b_bytes, cp + (size_t)k * b_bytes, b_bytes, &full[s]);
+          umma::bulk_load(dst + kTileBytes, xp + xtile + (size_t)k * kTileBytes, kTileBytes, &full[s]);
+          umma::bulk_load(dst + 2 * kTileBytes, cp + (size_t)k * b_bytes, b_bytes, &full[s]);
         }
       }
     }
     if (*dead) umma::drain_copies(full, kStages, it);
   } else if (warp == 1 && lane == 0) {  // MMA issuer
-    uint32_t it = 0, n = 0;
-    for (int64_t u = first; u < n_units && !*dead; u += step, n++) {
+    // the descriptors of stage 0's operands; tile and K offsets are added to their address fields
+    const uint64_t da = umma::desc_sw128(stage0), db = umma::desc_sw128(stage0 + 2 * kTileBytes);
+    uint32_t s = 0, ph = 0, n = 0;  // the next K block's stage and phase
+    bool ok = true;
+    for (int64_t u = first; u < n_units && ok && !*dead; u += step, n++) {
       const Unit t = unit_of(D, a, u, nmt2);
-      const int hw = D.hw[t.o], nk = D.kb[1 - t.o] * (t.abs ? 3 : 1), b = n & 1;
-      const uint32_t idesc = umma::idesc_bf16(128, 2 * hw);
-      if (n >= 2 && !umma::bounded_wait(&tempty[b], ((n >> 1) & 1) ^ 1, dead)) break;
-      umma::fence_after();
-      bool ok = true;
-      for (int k = 0; k < nk && ok; k++, it++) {
-        const int s = it % kStages;
-        ok = umma::bounded_wait(&full[s], (it / kStages) & 1, dead);
-        if (!ok) break;
-        umma::fence_after();
-        const uint32_t sa = stage0 + (uint32_t)s * kStageBytes, sb = sa + kTileBytes;
+      const int nk = D.kb[1 - t.o] * (t.abs ? 3 : 1);
+      const uint32_t idesc = umma::idesc_bf16(128, D.nw[t.o]);
+      for (int k = 0; k < nk && ok; k++) {
+        const uint64_t off = (uint64_t)(s * (kStageBytes / 16));
+        ok = umma::bounded_wait(&full[s], ph, dead);
 #pragma unroll
-        for (int ks = 0; ks < 4; ks++)
-          umma::mma_smem_a(tb + 256u * b, umma::desc_sw128(sa + ks * 32), umma::desc_sw128(sb + ks * 32), idesc,
-                           (k | ks) != 0);
-        commit_both(&empty[s]);
+        for (int h = 0; h < 2; h++) {
+          if (k == 0 && n >= 1 && ok) ok = umma::bounded_wait(&tempty[h], (n & 1) ^ 1, dead);
+          if (!ok) break;
+          umma::fence_after();
+#pragma unroll
+          for (int ks = 0; ks < 4; ks++)
+            umma::mma_smem_a(tb + 256u * h, da + off + h * (kTileBytes / 16) + 2 * ks, db + off + 2 * ks, idesc,
+                             (k | ks) != 0);
+          if (h == 1) umma::commit(&empty[s]);
+          if (k + 1 == nk) umma::commit(&tfull[h]);
+        }
+        if (++s == kStages) {
+          s = 0;
+          ph ^= 1;
+        }
       }
-      if (ok) umma::commit(&tfull[b]);
     }
     if (*dead) {  // after a failed wait: the MMAs in flight finish (bounded) before the release
       umma::commit(&fin);
       umma::drain_wait(&fin, 0);
     }
-  } else if (warp >= 4) {  // epilogue
-    const int qd = warp & 3;
+  } else if (warp >= 4) {  // epilogue: a quarter of the lanes and half of the columns per warp
+    const int qd = warp & 3, part = (warp - 4) >> 2;
     uint32_t n = 0;
-    for (int64_t u = first; u < n_units && !*dead; u += step, n++) {
+    bool ok = true;
+    for (int64_t u = first; u < n_units && ok && !*dead; u += step, n++) {
       const Unit t = unit_of(D, a, u, nmt2);
-      const int b = n & 1, nw = 2 * D.hw[t.o], ldy = D.ldy[t.o];
-      const bool ok = umma::bounded_wait(&tfull[b], (n >> 1) & 1, dead);
-      if (!__all_sync(0xffffffffu, ok)) break;
-      umma::fence_after();
-      const int64_t wl = (int64_t)t.mt * 256 + (int)rank * 128 + qd * 32 + lane;
-      const uint32_t ta = tb + ((uint32_t)(32 * qd) << 16) + 256u * b;
-      uint32_t v[16];
-      if (t.abs) {
-        float* dst = a.Yabs + wl * ldy + t.nt * nw;
-        for (int c = 0; c < nw; c += 16) {
-          umma::tmem_ld16(ta + c, v);
+      const int nw = D.nw[t.o], ldy = D.ldy[t.o];
+      const int c0 = part * (nw / 2), nc = nw / 2;  // up to 128 columns, a multiple of 16
+      for (int h = 0; h < 2; h++) {
+        ok = __all_sync(0xffffffffu, umma::bounded_wait(&tfull[h], n & 1, dead));
+        if (!ok) break;
+        umma::fence_after();
+        const int64_t wl = (int64_t)t.mt * 256 + h * 128 + qd * 32 + lane;
+        const uint32_t ta = tb + ((uint32_t)(32 * qd) << 16) + 256u * h + (uint32_t)c0;
+        uint32_t v[8][16];
 #pragma unroll
-          for (int j = 0; j < 4; j++)
-            *reinterpret_cast<uint4*>(dst + c + 4 * j) = make_uint4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-        }
-      } else {
-        const float p = D.m[t.plane].p, ip = D.m[t.plane].invp;
-        uint8_t* dst = a.Y + (t.o ? (size_t)D.nm * a.nmt * 128 * D.ldy[0] : 0) +
-                       ((size_t)t.plane * a.nmt * 128 + wl) * ldy + t.nt * nw;
-        auto bytes = [&](const uint32_t* x) {  // residues of four accumulators, as signed bytes + 128
-          uint32_t w[4];
+        for (int g = 0; g < 8; g++)
+          if (16 * g < nc) tmem_ld16_issue(ta + 16 * g, v[g]);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        umma::fence_before();  // the accumulators are free once they are in registers
+        __syncwarp();
+        if (lane == 0) umma::mbar_arrive(&tempty[h]);
+        if (t.abs) {
+          float* dst = a.Yabs + wl * ldy + t.nt * nw + c0;
 #pragma unroll
-          for (int j = 0; j < 4; j++) {
-            const float f = __uint_as_float(x[j]);
-            const float k = __fadd_rn(__fmaf_rn(f, ip, 12582912.0f), -12582912.0f);
-            w[j] = __float_as_uint(__fadd_rn(__fmaf_rn(-k, p, f), 12583040.0f));  // 1.5 * 2^23 + 128
+          for (int g = 0; g < 8; g++) {
+            if (16 * g >= nc) break;
+#pragma unroll
+            for (int j = 0; j < 16; j += 4)
+              *reinterpret_cast<uint4*>(dst + 16 * g + j) = make_uint4(v[g][j], v[g][j + 1], v[g][j + 2], v[g][j + 3]);
           }
-          return __byte_perm(__byte_perm(w[0], w[1], 0x0040), __byte_perm(w[2], w[3], 0x0040), 0x5410);
-        };
-        uint32_t v2[16];
-        tmem_ld16_issue(ta, v);
-        for (int c = 0; c < nw; c += 32) {  // nw is a multiple of 32
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          tmem_ld16_issue(ta + c + 16, v2);
-          *reinterpret_cast<uint4*>(dst + c) = make_uint4(bytes(v), bytes(v + 4), bytes(v + 8), bytes(v + 12));
-          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (c + 32 < nw) tmem_ld16_issue(ta + c + 32, v);
-          *reinterpret_cast<uint4*>(dst + c + 16) = make_uint4(bytes(v2), bytes(v2 + 4), bytes(v2 + 8), bytes(v2 + 12));
+        } else {
+          const float p = D.m[t.plane].p, ip = D.m[t.plane].invp;
+          uint8_t* dst = a.Y + (t.o ? (size_t)D.nm * a.nmt * 128 * D.ldy[0] : 0) +
+                         ((size_t)t.plane * a.nmt * 128 + wl) * ldy + t.nt * nw + c0;
+          auto bytes = [&](const uint32_t* x) {  // residues of four accumulators, as signed bytes + 128
+            uint32_t w[4];
+#pragma unroll
+            for (int j = 0; j < 4; j++) {
+              const float f = __uint_as_float(x[j]);
+              const float k = __fadd_rn(__fmaf_rn(f, ip, 12582912.0f), -12582912.0f);
+              w[j] = __float_as_uint(__fadd_rn(__fmaf_rn(-k, p, f), 12583040.0f));  // 1.5 * 2^23 + 128
+            }
+            return __byte_perm(__byte_perm(w[0], w[1], 0x0040), __byte_perm(w[2], w[3], 0x0040), 0x5410);
+          };
+#pragma unroll
+          for (int g = 0; g < 8; g++) {
+            if (16 * g >= nc) break;
+            *reinterpret_cast<uint4*>(dst + 16 * g) =
+                make_uint4(bytes(v[g]), bytes(v[g] + 4), bytes(v[g] + 8), bytes(v[g] + 12));
+          }
         }
       }
-      umma::fence_before();
-      __syncwarp();
-      if (lane == 0) umma::mbar_arrive(&tempty[b]);
     }
   }
   __syncwarp();
   umma::fence_before();
   __syncthreads();
   if (tid == 0 && *dead) *a.err = 1;
-  cluster_sync();  // neither CTA exits while the other's copies or commits may still reach it
   umma::fence_after();
   if (warp == 2) umma::tmem_dealloc(tb, 512);
   if (a.stamp && tid == 0) atomicMax(a.stamp + 1, now_ns());
@@ -704,7 +685,7 @@ cudaError_t launch_dense_rowsum(const DevProblem& P, const int* const es[2], uin
   return cudaGetLastError();
 }
 
-size_t dense_plane_elems(const DenseContract& D, int o) { return (size_t)D.nt[o] * 2 * D.kb[1 - o] * D.hw[o] * 64; }
+size_t dense_plane_elems(const DenseContract& D, int o) { return (size_t)D.nt[o] * D.kb[1 - o] * D.nw[o] * 64; }
 
 cudaError_t launch_dense_planes(const DevProblem& P, const DenseContract& D, cudaStream_t st) {
   for (int o = 0; o < 2; o++) {
@@ -723,8 +704,8 @@ void dense_shape(int n_up, int n_dn, DenseContract* D) {
   for (int o = 0; o < 2; o++) {
     D->kb[o] = (n[o] + 63) / 64;
     D->nt[o] = (n[o] + 255) / 256;
-    D->hw[o] = ((n[o] + D->nt[o] - 1) / D->nt[o] + 31) / 32 * 16;  // NW = 2 hw, a multiple of 32
-    D->ldy[o] = D->nt[o] * 2 * D->hw[o];
+    D->nw[o] = ((n[o] + D->nt[o] - 1) / D->nt[o] + 31) / 32 * 32;
+    D->ldy[o] = D->nt[o] * D->nw[o];
   }
 }
 
@@ -751,8 +732,7 @@ cudaError_t launch_contract_dense(const DevProblem& P, const DevScratch& S, int6
                                                                  P.n_det_sp[1], S.dx, nmt, n_abs, S.derr, S.live);
     GemmArgs a{S.dx, S.dy, S.dyabs, nmt, n_abs, w0, S.live, S.derr, stamp};
     const int64_t units = (int64_t)(nmt / 2) * ((int64_t)(D.nm + n_abs) * D.nt[0] + (int64_t)D.nm * D.nt[1]);
-    const int64_t pairs = std::min<int64_t>(units, std::max(P.n_sm / 2, 1));
-    k_mod_gemm<<<(unsigned)(2 * pairs), 256, smem, st>>>(D, a);
+    k_mod_gemm<<<(unsigned)std::min<int64_t>(units, std::max(P.n_sm, 1)), kGemmThreads, smem, st>>>(D, a);
     auto* crt = D.nm <= 16 ? k_mod_crt<8> : D.nm <= 18 ? k_mod_crt<9> : k_mod_crt<kMaxModuli / 2>;
     const int parts = S.live || nb <= (int64_t)kCrtFewWalkers * P.n_sm ? 4 : 1;
     crt<<<(unsigned)(parts == 4 ? nb : (nb + 3) / 4), 256, 0, st>>>(D, P, S, w0, n_walk, nmt, n_abs, parts);

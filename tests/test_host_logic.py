@@ -246,3 +246,11 @@ def test_uneven_batch_generator_ranges():
         assert 256 <= wl.n_walk <= 4096
     nd = np.log10([wl.n_det for wl in wls])
     assert nd.min() < 3.6 and nd.max() > 5.4   # spans the decades
+
+
+def test_no_multicast_loads():
+    """Every rank of a multi-GPU run executes these kernels: no bulk copy in them is a cluster multicast."""
+    csrc = os.path.join(ROOT, "paper_1510_00730_gb300", "csrc")
+    for fn in sorted(os.listdir(csrc)):
+        txt = open(os.path.join(csrc, fn)).read()
+        assert not re.search(r"cp\.async\.bulk[\w.:]*multicast", txt), fn
