@@ -609,6 +609,16 @@ mdet_status upload_problem(mdet_ctx* c) {
     UP(dig, P.B_dig);
     UP(fexp, P.B_exp);
     P.B_tiles = P.B_tiles8 = nullptr;
+    P.B_mag = P.B_top = nullptr;
+    if (mo_repairs(P, P.phi_df)) {
+      std::vector<float> mag((size_t)c->n_mo * P.tc_kp, 0.0f), top((size_t)c->n_ao * c->n_mo, 0.0f);
+      for (int m = 0; m < c->n_mo; m++)
+        for (int mu = 0; mu < c->n_ao && fexp[m] != mo_bad_exponent(); mu++)
+          mag[(size_t)m * P.tc_kp + mu] = top[(size_t)mu * c->n_mo + m] =
+              (float)std::ldexp(std::fabs(B[(size_t)mu * c->n_mo + m]), -fexp[m]);
+      UP(mag, P.B_mag);
+      UP(top, P.B_top);
+    }
     if ((s = upload_digit_tiles(c, B, dig, fexp, P.phi_df ? &P.B_tiles : &P.B_tiles8)) != MDET_OK) return s;
   }
   auto split = [](const std::vector<double>& v) {
@@ -908,7 +918,7 @@ mdet_status refine(mdet_ctx* c, bool table, int64_t n_walk, const double* R, dou
 
 // Kernels of the orbitals of one evaluation (or chunk) on scratch S.
 int mo_kernels(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df) {
-  return use_mo_digits(P, S, n_walk, df) ? 2 * (int)((n_walk + S.xd_walk - 1) / S.xd_walk) : 1;
+  return use_mo_digits(P, S, n_walk, df) ? mo_digits_kernels(P, S, n_walk, df) : 1;
 }
 
 // Whether an evaluation's contraction runs as residue products: its expansion has them, its
@@ -1461,8 +1471,8 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
   c->prof_chunks = nch;
   // stability fallback over the whole batch, after every chunk has finished: mixed precision
   // escalates to FP64 first, FP64 goes to full LU directly
-  // kernels: 3 per chunk (reference, ratios, epilogue; 4 with the epilogue's separate scatter), its orbitals' (2 per walker block of the digit
-  // products, else 1) and its contraction's (1 for the sparse sums, 2 in double-float, 3 per walker
+  // kernels: 3 per chunk (reference, ratios, epilogue; 4 with the epilogue's separate scatter), its orbitals' (2 or 3 per walker block of the
+  // digit products, else 1) and its contraction's (1 for the sparse sums, 2 in double-float, 3 per walker
   // block of the residue products); the full-LU
   // fallback 5 (list, dets, scale, rows, out); the mixed refinement adds its list, gather,
   // FP64 orbitals and scatter, and either the mark or the 4 FP64 table kernels

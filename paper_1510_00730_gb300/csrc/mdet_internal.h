@@ -105,6 +105,8 @@ struct DevProblem {
   const int* B_exp;       // [n_mo] column exponents of B_dig
   // 7 and 8 digits of B in the operand tiles of mdet_mo_digits.cu (null where the order sums are not exact)
   const uint16_t *B_tiles, *B_tiles8;
+  // |B| 2^-B_exp for mdet_mo_digits.cu's repairs (null where it makes none), [n_mo][tc_kp] and [n_ao][n_mo]
+  const float *B_mag, *B_top;
   int tc_kp, tc_mp, tc_sx;  // K padded to 16, M padded to 8, shared row stride of the AO digits
   double fallback_tol;    // estimated relative error above which a walker is re-evaluated by full LU (<= 0: off)
   int fallback_cap;       // walkers re-evaluated per evaluation at most
@@ -214,7 +216,7 @@ cudaError_t launch_gemm_bf16(const GemmOperand& A, const GemmOperand& B, int64_t
                              cudaStream_t st);
 
 // The orbitals by digit products on the tcgen05 tensor cores (mdet_mo_digits.cu), FP64 or (df)
-// double-float pairs; two kernels per block of S.xd_walk walkers. row_bytes: digits of one row of
+// double-float pairs; two or three kernels per block of S.xd_walk walkers. row_bytes: digits of one row of
 // the product (5 n_elec rows per walker); bad_exponent: B_exp of an MO whose coefficients are not
 // all finite.
 bool mo_digits_supported(const DevProblem& P, bool df);
@@ -222,6 +224,9 @@ size_t mo_digits_row_bytes(const DevProblem& P, bool df);
 int mo_bad_exponent();
 cudaError_t launch_mo_digits(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R, bool df,
                              cudaStream_t st);
+// whether their inaccurate elements are formed again (a third kernel), and the kernels in all
+bool mo_repairs(const DevProblem& P, bool df);
+int mo_digits_kernels(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df);
 // Whether an evaluation of n_walk walkers takes them (mo_impl 2, a workspace, and enough work).
 bool use_mo_digits(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df);
 cudaError_t launch_ref_tables(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool mixed,

@@ -26,6 +26,8 @@
 //               MOs of a row to a lane with their chains side by side. Bound by that epilogue and
 //               by the reads of X's digits from L2, once a chunk (the tensor cores are busy a third
 //               of the time).
+//  k_mo_repair  the elements that the cuts leave less accurate than a dot product would be (see there),
+//               in FP64, and in pairs beyond kPlainAos AOs or kPlainMos MOs.
 // FP64 orbitals of small bases and of re-evaluated walkers take k_mo_ao with plain FP64 rows instead of digits, and
 //  k_mo_dot     the FP64 dot products, one thread per row and MO.
 // 8,192 walkers of 17 electrons, 110 AOs, 80 MOs: k_mo_ao 0.50 and k_mo_orders 0.42 ms as pairs (3.60
@@ -53,7 +55,19 @@ constexpr int kSliceBytes = 2 * 128 * 16;     // one plane of 128 rows x 16 AOs
 constexpr int kChunk = 32;                    // MOs per accumulator set
 constexpr int kEpiWarps = 16, kOrderThreads = 128 + 32 * kEpiWarps;
 constexpr int64_t kMinDigitWork = 2048;       // AOs x MOs from which FP64 orbitals take digits
-constexpr int kBadRow = 1 << 20;              // row exponent of a row with a value that is not finite
+constexpr int kBadRow = 2047;                 // row exponent of a row with a value that is not finite
+constexpr int kRepairBits = 6;                // 2^-6 of row and column maximum: see k_mo_repair
+// pairs: bases up to this size take the digit products as they are (their cuts, 2^-57 of row and column
+// maxima, are that path's accuracy as documented); the compensated dot product served larger ones
+constexpr int kPlainAos = 112, kPlainMos = 128;
+
+// A row's word in xer: its exponent and the AO of its largest value.
+__device__ __forceinline__ int row_word(int e, int ao) { return (int)((unsigned)e << 9 | (unsigned)ao); }
+__device__ __forceinline__ int word_ao(int x) { return x & 511; }
+__device__ __forceinline__ int word_exp(int x) { return x >> 9; }
+
+// shared memory of a warp of k_mo_repair: five AO rows and a list of elements
+__host__ __device__ inline int repair_warp_bytes(int Kp, int M) { return 5 * (Kp * 8 + 16) + (10 * M + 15) / 16 * 16; }
 
 // x 2^(62 - er) rounded to an integer, |x| < 2^er
 __device__ __forceinline__ long long fixed_point(double x, int er) {
@@ -127,6 +141,7 @@ struct AoType<double> {
   static __device__ __forceinline__ uint2 bits(double x) {
     return make_uint2((unsigned)__double2loint(x), (unsigned)__double2hiint(x));
   }
+  static __device__ __forceinline__ int value_exp(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1022; }
   static __device__ __forceinline__ int row_exp(unsigned k) {
     return k >= 0x7ff00000u ? kBadRow : (k == 0 ? 0 : (int)max(k >> 20, 1u) - 1022);
   }
@@ -137,6 +152,7 @@ struct AoType<df32> {
   static __device__ __forceinline__ unsigned key(uint2 b) { return b.x & 0x7fffffffu; }
   static __device__ __forceinline__ df32 value(uint2 b) { return df32(__uint_as_float(b.x), __uint_as_float(b.y)); }
   static __device__ __forceinline__ uint2 bits(df32 x) { return make_uint2(__float_as_uint(x.hi), __float_as_uint(x.lo)); }
+  static __device__ __forceinline__ int value_exp(float2 x) { return (int)((__float_as_uint(x.x) >> 23) & 0xff) - 126; }
   static __device__ __forceinline__ int row_exp(unsigned k) {
     return k >= 0x7f800000u ? kBadRow : (k == 0 ? 0 : (int)max(k >> 23, 1u) - 126);
   }
@@ -210,12 +226,21 @@ __global__ void __launch_bounds__(256) k_mo_ao(DevProblem P, const double* __res
   for (int r = warp; r < 5 * NE; r += 8) {
     if (r % NE >= ne) continue;
     unsigned k = 0;
-    for (int a = lane; a < K; a += 32) k = max(k, AoType<T>::key(*reinterpret_cast<const uint2*>(smx + r * stride + a * 8)));
-    k = __reduce_max_sync(0xffffffffu, k);
+    int at = 0;  // the AO of the lane's largest key
+    for (int a = lane; a < K; a += 32) {
+      const unsigned key = AoType<T>::key(*reinterpret_cast<const uint2*>(smx + r * stride + a * 8));
+      if (key > k) {
+        k = key;
+        at = a;
+      }
+    }
+    const unsigned top = __reduce_max_sync(0xffffffffu, k);
+    if (P.B_top)  // for k_mo_repair
+      at = __shfl_sync(0xffffffffu, at, __ffs(__ballot_sync(0xffffffffu, k == top)) - 1);
     if (lane == 0) {
-      const int e = AoType<T>::row_exp(k);
+      const int e = AoType<T>::row_exp(top);
       rexp[r] = e;
-      xer[rowbase[r % NE] + r / NE * N] = e;
+      xer[rowbase[r % NE] + r / NE * N] = row_word(e, at);
     }
   }
   __syncthreads();
@@ -391,7 +416,7 @@ __global__ void __launch_bounds__(kOrderThreads, 1) k_mo_orders(DevProblem P, co
     for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
       const int64_t row = tile * 128 + 32 * qd + lane;
       const bool valid = row < n_rows;
-      const int er = valid ? xer[row] : 0;
+      const int er = valid ? word_exp(xer[row]) : 0;
       for (int c = 0; c < n_chunk; c++, n++) {
         const int cw = min(kChunk, Np - c * kChunk), b = n & 1;
         const bool ok = __all_sync(0xffffffffu, umma::bounded_wait(&tfull[b], (n >> 1) & 1, dead));
@@ -454,28 +479,189 @@ __global__ void __launch_bounds__(kOrderThreads, 1) k_mo_orders(DevProblem P, co
   if (warp == 2) umma::tmem_dealloc(tb, 512);
 }
 
+// Where the cuts cost accuracy. An element's error here is relative to 2^(e_r + f_m), whatever its own size: 2^-59.2
+// of it in FP64 (rms; 110 and 141 AOs, simulated on the synthetic walkers), while that of an FP64 dot
+// product is 2^-52.7 of the element's sum of magnitudes S = sum_k |x_k b_km|. They meet where S is 2^-6.5
+// of 2^(e_r + f_m): an MO with next to nothing on the AO that dominates the row, for instance one without
+// tight s functions at an electron near the nucleus. (Pairs: 2^-55 and 2^-48, the same line.) An element
+// below 2^-6 by cancellation only, as 3.6 % of the synthetic ones are, is more accurate as it stands.
+// So a warp takes the five rows of an electron: elements below 2^-6 (read from phi) whose S is not
+// bounded from below by its term on the row's largest AO (0.44 % are left) go into a list, eight
+// lanes each form a better bound from the first two digits of the row and the magnitudes of B (none of the
+// synthetic ones is below 2^-6), and where that is below 2^-6 too, the warp forms the electron's AO values
+// again and the elements' dot products, relative to each term. Bound by the latency of those loads,
+// which mostly go to DRAM: 8,192 walkers of 17 electrons and 80 MOs, FP64, 0.50 ms with every small
+// element in the list, 0.18 with these (and no less with the 0.02 % that the two largest AOs leave).
+template <class T, class Out>
+__global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 4 : 3) k_mo_repair(DevProblem P, const double* __restrict__ R, int64_t w0, int64_t n_el,
+                                                   const uint8_t* __restrict__ xd, const int* __restrict__ xer,
+                                                   Out* __restrict__ phi) {
+  constexpr int kABytes = AoType<T>::D * kSliceBytes;
+  constexpr bool kDouble = std::is_same<T, double>::value;
+  constexpr unsigned kAll = 0xffffffffu;
+  extern __shared__ __align__(16) uint8_t smr[];
+  const int K = P.n_ao, M = P.n_mo, N = P.n_elec, Kp = P.tc_kp, stride = Kp * 8 + 16;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, lane8 = lane & 7, quad = lane >> 3;
+  const int64_t g = (int64_t)blockIdx.x * 8 + warp;  // electron, counted from walker w0
+  if (g >= n_el) return;
+  uint8_t* rows = smr + warp * repair_warp_bytes(Kp, M);                // [5] rows of AO values
+  uint16_t* list = reinterpret_cast<uint16_t*>(rows + 5 * stride);      // elements: quantity 256 + MO
+  const int64_t row0 = 4 * N * (g / N) + g;                             // row of quantity 0, the others N apart
+  const int xer_l = lane < 5 ? xer[row0 + (int64_t)lane * N] : 0;
+  int n = 0;
+#pragma unroll 2
+  for (int m0 = 0; m0 < M; m0 += 32) {
+    const int m = m0 + lane, f = m < M ? __ldg(P.B_exp + m) : kBadRow;
+    int e[5];
+#pragma unroll
+    for (int c = 0; c < 5; c++)
+      e[c] = f != kBadRow ? AoType<T>::value_exp(phi[(row0 + (int64_t)c * N) * M + m]) : 0;
+#pragma unroll
+    for (int c = 0; c < 5; c++) {
+      const int x = __shfl_sync(kAll, xer_l, c), er = word_exp(x);
+      bool small = f != kBadRow && er != kBadRow && e[c] <= er + f - kRepairBits;
+      // (the row's largest value is at least half of 2^er)
+      if (small) small = __ldg(P.B_top + (size_t)word_ao(x) * M + m) < 2.0f / (1 << kRepairBits);
+      const unsigned who = __ballot_sync(kAll, small);
+      if (small) list[n + __popc(who & ((1u << lane) - 1u))] = (uint16_t)(c << 8 | m);
+      n += __popc(who);
+    }
+  }
+  __syncwarp();
+  int n2 = 0;
+  for (int i0 = 0; i0 < n; i0 += 4) {
+    const int i = i0 + quad;
+    float sum = 0.0f;
+    int at = 0;
+    if (i < n) {
+      at = list[i];
+      const int64_t row = row0 + (int64_t)(at >> 8) * N;
+      const uint8_t* src = xd + (row >> 7) * (Kp / 16) * kABytes + (row & 127) * 16;  // its first digits
+      const float* b = P.B_mag + (size_t)(at & 255) * Kp;
+#pragma unroll 2
+      for (int k8 = lane8; k8 < Kp / 8; k8 += 8) {
+        const uint4* p = reinterpret_cast<const uint4*>(src + (size_t)(k8 >> 1) * kABytes + (k8 & 1) * 2048);
+        const uint4 d1 = __ldg(p), d2 = __ldg(p + kSliceBytes / 16);
+        const float4 b0 = __ldg(reinterpret_cast<const float4*>(b + 8 * k8)),
+                     b1 = __ldg(reinterpret_cast<const float4*>(b + 8 * k8 + 4));
+        auto one = [&](uint32_t w1, uint32_t w2, float bk) {  // |256 d_1 + d_2| less what follows
+          sum = fmaf(fmaxf(fabsf(fmaf(256.0f, __uint_as_float(w1), __uint_as_float(w2))) - 1.0f, 0.0f), bk, sum);
+        };
+        auto two = [&](uint32_t w1, uint32_t w2, float lo, float hi) {
+          one(w1 << 16, w2 << 16, lo);
+          one(w1 & 0xffff0000u, w2 & 0xffff0000u, hi);
+        };
+        two(d1.x, d2.x, b0.x, b0.y);
+        two(d1.y, d2.y, b0.z, b0.w);
+        two(d1.z, d2.z, b1.x, b1.y);
+        two(d1.w, d2.w, b1.z, b1.w);
+      }
+    }
+#pragma unroll
+    for (int off = 4; off; off >>= 1) sum += __shfl_xor_sync(kAll, sum, off);
+    // the second digit weighs 2^-16, and 4 times that in FP64; the list is compacted in place
+    const bool again = i < n && lane8 == 0 && !(sum * (kDouble ? 0x1p-14f : 0x1p-16f) >= 1.0f / (1 << kRepairBits));
+    const unsigned who = __ballot_sync(kAll, again);
+    if (again) list[n2 + __popc(who & ((1u << lane) - 1u))] = (uint16_t)at;
+    n2 += __popc(who);
+    __syncwarp();
+  }
+  if (n2 == 0) return;
+  T pos[3];
+#pragma unroll
+  for (int d = 0; d < 3; d++) {
+    const double x = R[(w0 * N + g) * 3 + d];
+    if constexpr (kDouble)
+      pos[d] = x;
+    else
+      pos[d] = df_from_double(x);
+  }
+  for (int s = lane; s < P.n_shell; s += 32) {
+    const int ao0 = P.shell_ao0[s];
+    auto put = [&](int c, int q, T v) {
+      *reinterpret_cast<uint2*>(rows + c * stride + (ao0 + q) * 8) = AoType<T>::bits(v);
+    };
+    if constexpr (kDouble)
+      ao_shell_values_short(P, s, pos, put);
+    else
+      ao_shell_values_df(P, s, pos, put);
+  }
+  __syncwarp();
+  for (int i0 = 0; i0 < n2; i0 += 4) {
+    const int i = i0 + quad;
+    const bool on = i < n2;
+    const int at = on ? list[i] : 0, m = at & 255;
+    const uint8_t* x = rows + (at >> 8) * stride;
+    Out* dst = phi + (row0 + (int64_t)(at >> 8) * N) * M + m;
+    if constexpr (kDouble) {
+      double acc = 0.0;
+      if (on)
+        for (int k = lane8; k < K; k += 8)
+          acc = fma(*reinterpret_cast<const double*>(x + k * 8), __ldg(P.B + (size_t)k * M + m), acc);
+#pragma unroll
+      for (int off = 4; off; off >>= 1) acc += __shfl_xor_sync(kAll, acc, off);
+      if (on && lane8 == 0) *dst = acc;
+    } else {  // the compensated dot product of the CUDA-core kernel, and the lanes' sums by TwoSum
+      float sh = 0.0f, sl = 0.0f;
+      if (on)
+        for (int k = lane8; k < K; k += 8) {
+          const float2 a = *reinterpret_cast<const float2*>(x + k * 8);
+          const float bh = __ldg(P.B_hi + (size_t)k * M + m), bl = __ldg(P.B_lo + (size_t)k * M + m);
+          const float p = __fmul_rn(a.x, bh), pe = __fmaf_rn(a.x, bh, -p);
+          const float cross = __fmaf_rn(a.x, bl, __fmul_rn(a.y, bh));
+          float t, e;
+          two_sum(sh, p, t, e);
+          sh = t;
+          sl = __fadd_rn(sl, __fadd_rn(e, __fadd_rn(pe, cross)));
+        }
+#pragma unroll
+      for (int off = 4; off; off >>= 1) {
+        const float oh = __shfl_xor_sync(kAll, sh, off), ol = __shfl_xor_sync(kAll, sl, off);
+        float t, e;
+        two_sum(sh, oh, t, e);
+        sh = t;
+        sl = __fadd_rn(__fadd_rn(sl, ol), e);
+      }
+      float hi, lo;
+      two_sum(sh, sl, hi, lo);
+      if (on && lane8 == 0) *dst = make_float2(hi, lo);
+    }
+  }
+}
+
 }  // namespace
 
 size_t mo_digits_row_bytes(const DevProblem& P, bool df) { return (size_t)(df ? AoType<df32>::D : AoType<double>::D) * 2 * P.tc_kp; }
 int mo_bad_exponent() { return kBadRow; }
 
 bool mo_digits_supported(const DevProblem& P, bool df) {
-  return (!df || P.B_tiles) && (size_t)5 * kNE * (P.tc_kp * 8 + 16) <= 200 * 1024;
+  return (!df || P.B_tiles) && (size_t)5 * kNE * (P.tc_kp * 8 + 16) <= 200 * 1024 && P.n_ao <= 511;
 }
 
 bool use_mo_digits(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df) {
   return P.mo_impl == 2 && S.xd && mo_digits_supported(P, df);
 }
 
+bool mo_repairs(const DevProblem& P, bool df) { return !df || P.n_ao > kPlainAos || P.n_mo > kPlainMos; }
+
+// FP64 dot products on the FP64 pipe, to the bit those of the CUDA-core kernel: for small bases,
+// where they cost little (2,048: a 45 x 45 basis), and for the few walkers of a re-evaluation,
+// whose ill-conditioned references amplify any change of rounding
+static bool plain_rows(const DevProblem& P, const DevScratch& S, bool df) {
+  return !df && ((int64_t)P.n_ao * P.n_mo < kMinDigitWork || S.live || !P.B_tiles8);
+}
+
+int mo_digits_kernels(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df) {
+  return (int)((n_walk + S.xd_walk - 1) / S.xd_walk) * (!plain_rows(P, S, df) && mo_repairs(P, df) ? 3 : 2);
+}
+
 template <class T, class Out>
 static cudaError_t launch_mo_digits_t(const DevProblem& P, const DevScratch& S, int64_t n_walk, const double* R,
                                       const uint16_t* b_tiles, cudaStream_t st) {
-  static SmemOptIn opt[5];
+  static SmemOptIn opt[6];
+  constexpr bool kDf = !std::is_same<T, double>::value;
   const size_t smem2 = (size_t)AoType<T>::kStages * AoType<T>::D * (kSliceBytes + 2 * kChunk * 16);
-  // FP64 dot products on the FP64 pipe, to the bit those of the CUDA-core kernel: for small bases,
-  // where they cost little (2,048: a 45 x 45 basis), and for the few walkers of a re-evaluation,
-  // whose ill-conditioned references amplify any change of rounding
-  const bool raw = std::is_same<T, double>::value && ((int64_t)P.n_ao * P.n_mo < kMinDigitWork || S.live || !b_tiles);
+  const bool raw = plain_rows(P, S, kDf), repair = !raw && mo_repairs(P, kDf);
   const bool few = (n_walk * P.n_elec + kNE - 1) / kNE < P.n_sm;
   const int ne = few ? kNEFew : kNE;
   const size_t smem1 = (size_t)5 * ne * (P.tc_kp * 8 + 16);
@@ -483,6 +669,8 @@ static cudaError_t launch_mo_digits_t(const DevProblem& P, const DevScratch& S, 
                  : (few ? k_mo_ao<T, false, kNEFew> : k_mo_ao<T, false, kNE>);
   cudaError_t e = opt[few ? 3 + raw : 2 * raw].ensure(ao, smem1);
   if (e == cudaSuccess && !raw) e = opt[1].ensure(k_mo_orders<T, Out>, smem2);
+  const size_t smem3 = (size_t)8 * repair_warp_bytes(P.tc_kp, P.n_mo);
+  if (e == cudaSuccess && repair) e = opt[5].ensure(k_mo_repair<T, Out>, smem3);
   if (e != cudaSuccess) return e;
   const int64_t N = P.n_elec;
   for (int64_t w0 = 0; w0 < n_walk; w0 += S.xd_walk) {
@@ -500,6 +688,9 @@ static cudaError_t launch_mo_digits_t(const DevProblem& P, const DevScratch& S, 
     ao<<<g1, 256, smem1, st>>>(P, R, w0, nb * N, S.xd, S.xer, P.tc_kp, S.live);
     k_mo_orders<T, Out><<<g2, kOrderThreads, smem2, st>>>(P, b_tiles, S.xd, S.xer,
                                                 reinterpret_cast<Out*>(S.phi + w0 * 5 * N * P.n_mo), rows, S.live, w0);
+    if (repair)
+      k_mo_repair<T, Out><<<(unsigned)((nb * N + 7) / 8), 256, smem3, st>>>(
+          P, R, w0, nb * N, S.xd, S.xer, reinterpret_cast<Out*>(S.phi + w0 * 5 * N * P.n_mo));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -3,6 +3,8 @@ slices, 32-MO chunks, 16-electron blocks, 128-row tiles), both precisions, again
 against the CUDA-core products (mo_impl 1) for positions that are not finite."""
 from __future__ import annotations
 
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -86,3 +88,32 @@ def test_blocks_of_walkers(n_mo, digit_bytes, prec):
     rep = compare(got, oracle.evaluate(wl), **TOL[prec])
     assert rep["ok"], rep
     assert np.array_equal(got["status"], whole["status"]) and np.array_equal(got["sign"], whole["sign"])
+
+
+@pytest.mark.parametrize("prec,shells,n_mo", [(pkg.PRECISION_FP64, (20, 20, 5, 0), 31), (pkg.PRECISION_FP64, (20, 20, 5, 5), 96),
+                                              (pkg.PRECISION_MIXED, (20, 20, 5, 5), 31), (pkg.PRECISION_MIXED, (20, 20, 5, 5), 129)])
+@pytest.mark.parametrize("some", [False, True])
+def test_mos_without_the_dominant_aos(prec, shells, n_mo, some):
+    """Electrons near the nucleus, where tight s functions set the largest value of every row, in MOs (all, or
+    every other one) that have none of them: the digits, cut relative to that value, would lose most of
+    their decimal places. Every orbital is to be as accurate as a dot product over its own terms (mo_impl 1),
+    within a rounding per AO, so that the outputs agree within 4 K times the estimated error of one
+    rounding per orbital."""
+    wl = _workload(shells, n_mo, 40)
+    mo = wl.mo_coef.copy()
+    assert np.all(wl.shell_l[:shells[0]] == 0) and np.all(wl.shell_nprim == 3)
+    mo[np.ix_(np.arange(shells[0]), np.arange(0, n_mo, 2 if some else 1))] = 0.0
+    alpha = wl.alpha.copy()
+    alpha[:3 * shells[0]] *= 1e6  # s functions of exponents up to 5e8, the others up to 500
+    wl = dataclasses.replace(wl, mo_coef=mo, alpha=alpha, R=wl.R * 1e-4)
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    ctx.set_fallback(1e30)  # estimates on, nothing flagged
+    got = _eval(ctx, wl.R)
+    ctx.set_tuning(mo_impl=1)
+    want = _eval(ctx, wl.R)
+    _, est = ctx.error_estimates(len(wl.R))
+    for k in ("grad", "lap"):
+        d = np.abs(got[k] - want[k]).reshape(len(wl.R), -1).max(1)
+        scale = np.sqrt((want[k] ** 2).reshape(len(wl.R), -1).mean(1))
+        assert np.all(d <= 4 * wl.n_ao * est[:, 0] * scale), (k, (d / scale / est[:, 0]).max())
+    assert np.array_equal(got["sign"], want["sign"])
