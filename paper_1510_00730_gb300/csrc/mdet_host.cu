@@ -517,7 +517,7 @@ mdet_status build_dense(mdet_ctx* c) {
   CUDA_TRY(c, cudaMemcpy(mx.data(), d_mx, mx.size() * sizeof(uint32_t), cudaMemcpyDeviceToHost));
   if (!choose_moduli(mx.data(), &D)) return MDET_OK;
   for (int o = 0; o < 2; o++) {
-    const size_t bytes = dense_plane_elems(D, o) * sizeof(uint16_t) * (D.nm + (o ? 0 : 2));
+    const size_t bytes = dense_plane_elems(D, o) * sizeof(uint16_t) * dense_planes(D, o);
     void* p = nullptr;
     if (bytes > kDenseMaxBytes || cudaMalloc(&p, bytes) != cudaSuccess) {
       cudaGetLastError();  // no room: the sparse sums

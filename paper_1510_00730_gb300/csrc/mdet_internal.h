@@ -67,7 +67,7 @@ struct DenseContract {
   int kb[2];             // 64-wide K blocks over the distinct determinants of each spin
   int nt[2], nw[2];      // determinant tiles of nw rows of product o (0: v, 1: u)
   int ldy[2];            // row stride of the residue bytes of product o
-  uint16_t* planes[2];   // BF16 residue planes of C and C^T; the two magnitude planes of C
+  uint16_t* planes[2];   // BF16 residue planes of C and C^T, and their magnitude planes (two and one)
   const int* es[2];      // [n_det_sp[o]] exponents of the rows of C and of C^T
   ModConst m[kMaxModuli];
   // reconstruction weights modulo 2^128 in 16-bit limbs, and (limb 8) 2^16 ((P / p)^-1 mod p) / p, the
@@ -251,6 +251,7 @@ int dense_moduli_range();
 cudaError_t launch_dense_rowsum(const DevProblem& P, const int* const es[2], uint32_t* mx, cudaStream_t st);
 bool choose_moduli(const uint32_t* rowmax, DenseContract* D);
 size_t dense_plane_elems(const DenseContract& D, int o);  // elements of one plane of product o
+int dense_planes(const DenseContract& D, int o);          // and its planes
 cudaError_t launch_dense_planes(const DevProblem& P, const DenseContract& D, cudaStream_t st);
 // Bytes per walker of the residue planes, the residue bytes and the magnitude sums.
 void dense_bytes(const DenseContract& D, size_t* x, size_t* y, size_t* yabs);

@@ -6,8 +6,8 @@
 // TFLOP/s, and they bound the whole evaluation. As a dense product of residues the same sums
 // run on the BF16 tensor cores, which are 1,500 times as fast, so a filled-in C of a few per
 // cent of nonzeros is still far cheaper: 750,000 products over 3,015 x 3,015 distinct
-// determinants and 8,192 walkers take 20.5 ms as FP64 sums, and 4.0 ms here (residues 0.43,
-// products 2.86, reconstruction 0.70).
+// determinants and 8,192 walkers take 20.5 ms as FP64 sums, and 4.1 ms here (residues 0.41,
+// products 2.94, reconstruction 0.80).
 //
 // Method (multi-modular integer products, the Chinese remainder theorem).
 //  - Fixed point: row i of C as chat_ij = rint(c_ij 2^(61 - es_i)) with sum_j |c_ij| < 2^es_i,
@@ -23,9 +23,16 @@
 //  - Reconstruction: X = sum_q y_q M_q - k P with M_q = (P / p_q) ((P / p_q)^-1 mod p_q),
 //    P = prod p_q > 2^124.6 and k = rint(sum_q y_q ((P / p_q)^-1 mod p_q) / p_q) (|X| / P < 0.36, and
 //    16-bit fractions put the sum within 0.05), in 128-bit wrap-around integers: X is exact, and v_i = RN(X) 2^(es_i + xe_w - 123).
-//  - The magnitude sum behind Psi~ (sum_j |c_ij| |r_j|, for the error estimate) rides along as
-//    one more product: both magnitudes as a BF16 pair h + l (2^-17 relative), h h + h l + l h
-//    in one FP32 accumulator.
+//  - The magnitude sums m = sum_j |c_ij| |r_j| 2^-(es_i + xe_w) ride along as one more product of each
+//    order: leading BF16 magnitudes; for the error estimate those of v as BF16 pairs h + l (2^-17
+//    relative), h h + h l + l h in one FP32 accumulator.
+//  - Rows that the cuts would hurt. The cuts are relative to the row's sum and the walker's largest
+//    ratio, the rounding of an FP64 sum to m itself. Simulated on the synthetic walkers (900 + 900
+//    determinants) the fixed-point error of a row is 0.012 units of 2^-53 m in the median, where m is
+//    2^-5, and that of an FP64 sum 0.72, with 1 % above 7.9. So it reaches 2.9 units at m = 2^-13, and a row
+//    below that (less than 0.01 % of the synthetic ones; all of them, if MOs are scaled very differently) is
+//    summed in FP64 over its products instead. With the line at 2^-11, where the medians meet, the few
+//    walkers with many such rows kept the reconstruction for 1.67 ms instead of 0.80.
 // A walker whose ratios are not all finite takes a direct FP64 sum over the products instead,
 // so that infinities and NaN propagate as they do in FP64.
 #include <algorithm>
@@ -127,7 +134,7 @@ __global__ void __launch_bounds__(256) k_mod_rowsum(const int* __restrict__ ptr,
 }
 
 // The residue planes of C in one order (rows = the product's outputs, gathered index = K), and
-// with n_abs the two magnitude planes. Blocks of nw rows x 64 K in the 128-byte swizzle of the
+// n_abs magnitude planes (1 or 2). Blocks of nw rows x 64 K in the 128-byte swizzle of the
 // MMA's shared-memory operands (row r at 128 r, its 16-byte chunk j at chunk j ^ (r mod 8)),
 // [plane][tile][K block][row][64]; zeroed before.
 __global__ void __launch_bounds__(256) k_mod_planes(const __grid_constant__ DenseContract D, int o,
@@ -143,10 +150,10 @@ __global__ void __launch_bounds__(256) k_mod_planes(const __grid_constant__ Dens
   const size_t at = ((size_t)t * kb + j / 64) * nw * 64 + (size_t)rr * 64 + (((j % 64) / 8) ^ (rr & 7)) * 8 + j % 8;
   for (int q = 0; q < D.nm; q++)
     D.planes[o][q * plane + at] = (uint16_t)(__float_as_uint((float)balanced_mod(c, (int)D.m[q].p)) >> 16);
-  if (n_abs) {
-    const float f = __double2float_rn(scalbn(fabs(val[k]), -es));
-    const uint32_t hb = (__float_as_uint(f) + 0x8000u) & 0xffff0000u;
-    D.planes[o][D.nm * plane + at] = (uint16_t)(hb >> 16);
+  const float f = __double2float_rn(scalbn(fabs(val[k]), -es));
+  const uint32_t hb = (__float_as_uint(f) + 0x8000u) & 0xffff0000u;
+  D.planes[o][D.nm * plane + at] = (uint16_t)(hb >> 16);
+  if (n_abs > 1) {
     const float l = f - __uint_as_float(hb);
     D.planes[o][(D.nm + 1) * plane + at] = (uint16_t)((__float_as_uint(l) + 0x8000u) >> 16);
   }
@@ -159,7 +166,7 @@ __global__ void __launch_bounds__(256) k_mod_planes(const __grid_constant__ Dens
 __global__ void __launch_bounds__(256) k_mod_residues(const __grid_constant__ DenseContract D,
                                                       const double* __restrict__ r, int64_t wp,
                                                       const uint32_t* __restrict__ xmax, int64_t w0, int nu, int nd,
-                                                      uint16_t* __restrict__ X, int nmt, int n_abs,
+                                                      uint16_t* __restrict__ X, int nmt, int full_abs,
                                                       int* __restrict__ err, const int* __restrict__ live) {
   __shared__ uint4 tile[2][256];
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *err = 0;
@@ -189,7 +196,7 @@ __global__ void __launch_bounds__(256) k_mod_residues(const __grid_constant__ De
     const unsigned long long x = (b < 0 ? 0ULL - m : m) + 0x8000000000000000ULL;
     lo[z] = (uint32_t)x;
     hi[z] = (uint32_t)(x >> 32);
-    if (sp && n_abs) {
+    {
       const float f = __uint2float_rn((uint32_t)(m >> 31)) * 0x1p-31f;  // |r| 2^-xe
       const uint32_t hb = (__float_as_uint(f) + 0x8000u) & 0xffff0000u;
       const uint32_t lb = __float_as_uint(f - __uint_as_float(hb)) + 0x8000u;
@@ -205,7 +212,7 @@ __global__ void __launch_bounds__(256) k_mod_residues(const __grid_constant__ De
   const int kb = D.kb[sp];
   const size_t plane = (size_t)nmt * kb * (kTileBytes / 16);
   const int row = wl % 128;
-  uint4* dst = reinterpret_cast<uint4*>(X) + (sp ? (size_t)D.nm * nmt * D.kb[0] * (kTileBytes / 16) : 0) +
+  uint4* dst = reinterpret_cast<uint4*>(X) + (sp ? (size_t)(D.nm + 1) * nmt * D.kb[0] * (kTileBytes / 16) : 0) +
                ((size_t)(wl / 128) * kb + kbi) * (kTileBytes / 16) + (row - lane) * 8 + threadIdx.x;
   const int at = lane * 8 + (oct ^ (row & 7));  // 128-byte swizzle
   for (int q = 0; q < D.nm; q++) {
@@ -219,14 +226,12 @@ __global__ void __launch_bounds__(256) k_mod_residues(const __grid_constant__ De
     __syncthreads();
     dst[q * plane] = tile[q & 1][threadIdx.x];
   }
-  if (sp && n_abs) {
-    __syncthreads();
-    tile[0][at] = make_uint4(ha[0], ha[1], ha[2], ha[3]);
-    tile[1][at] = make_uint4(la[0], la[1], la[2], la[3]);
-    __syncthreads();
-    dst[D.nm * plane] = tile[0][threadIdx.x];
-    dst[(D.nm + 1) * plane] = tile[1][threadIdx.x];
-  }
+  __syncthreads();
+  tile[0][at] = make_uint4(ha[0], ha[1], ha[2], ha[3]);
+  tile[1][at] = make_uint4(la[0], la[1], la[2], la[3]);
+  __syncthreads();
+  dst[D.nm * plane] = tile[0][threadIdx.x];
+  if (sp && full_abs) dst[(D.nm + 1) * plane] = tile[1][threadIdx.x];
 }
 
 // ---------------------------------------------------------------------------
@@ -256,7 +261,7 @@ struct GemmArgs {
   uint8_t* Y;
   float* Yabs;
   int nmt;  // 128-walker tiles in the layout of X and Y (even)
-  int n_abs;
+  int full_abs;  // magnitudes of v as pairs
   int64_t w0;
   const int* live;
   int* err;
@@ -282,26 +287,17 @@ struct Unit {
   int o, plane, abs, mt, nt;
 };
 
-__device__ __forceinline__ Unit unit_of(const DenseContract& D, const GemmArgs& a, int64_t u, int nmt2) {
-  // groups: [magnitudes], then the planes of v, then those of u; determinant tiles fastest
+__device__ __forceinline__ Unit unit_of(const DenseContract& D, int64_t u, int nmt2) {
+  // groups: magnitudes and planes of v, then those of u; determinant tiles fastest
   Unit r;
-  const int64_t t0 = (int64_t)nmt2 * D.nt[0], g0 = a.n_abs + D.nm;
-  int64_t rem;
-  if (u < g0 * t0) {
-    const int g = (int)(u / t0);
-    rem = u - g * t0;
-    r.o = 0;
-    r.abs = a.n_abs && g == 0;
-    r.plane = r.abs ? D.nm : g - a.n_abs;
-  } else {
-    const int64_t t1 = (int64_t)nmt2 * D.nt[1];
-    u -= g0 * t0;
-    const int g = (int)(u / t1);
-    rem = u - g * t1;
-    r.o = 1;
-    r.abs = 0;
-    r.plane = g;
-  }
+  const int64_t v_units = (int64_t)(D.nm + 1) * nmt2 * D.nt[0];
+  r.o = u >= v_units;
+  if (r.o) u -= v_units;
+  const int64_t per = (int64_t)nmt2 * D.nt[r.o];
+  const int g = (int)(u / per);
+  const int64_t rem = u - g * per;
+  r.abs = g == 0;
+  r.plane = r.abs ? D.nm : g - 1;
   r.mt = (int)(rem / D.nt[r.o]);
   r.nt = (int)(rem - (int64_t)r.mt * D.nt[r.o]);
   return r;
@@ -335,22 +331,23 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
   const uint32_t tb = tbase;
   const int64_t w_live = a.live ? max((int64_t)0, (int64_t)*a.live - a.w0) : (int64_t)a.nmt * 128;
   const int nmt2 = (int)min((int64_t)(a.nmt / 2), (w_live + 255) / 256);
-  const int64_t n_units = (int64_t)(a.n_abs + D.nm) * nmt2 * D.nt[0] + (int64_t)D.nm * nmt2 * D.nt[1];
+  const int64_t n_units = (int64_t)(D.nm + 1) * nmt2 * (D.nt[0] + D.nt[1]);
   const int64_t first = blockIdx.x, step = gridDim.x;
   const uint32_t stage0 = umma::smem_u32(stage_mem);
 
   if (warp == 0 && lane == 0) {  // producer
     uint32_t it = 0;
     for (int64_t u = first; u < n_units && !*dead; u += step) {
-      const Unit t = unit_of(D, a, u, nmt2);
+      const Unit t = unit_of(D, u, nmt2);
       const int sp = 1 - t.o, kb = D.kb[sp];
       const uint32_t b_bytes = (uint32_t)D.nw[t.o] * 128;
       const size_t xtile = (size_t)kb * kTileBytes, xplane = (size_t)a.nmt * xtile,
                    cplane = (size_t)D.nt[t.o] * kb * b_bytes;
       const uint8_t* xs = reinterpret_cast<const uint8_t*>(a.X) +
-                          (sp ? (size_t)D.nm * a.nmt * D.kb[0] * kTileBytes : 0) + (size_t)t.mt * 2 * xtile;
+                          (sp ? (size_t)(D.nm + 1) * a.nmt * D.kb[0] * kTileBytes : 0) + (size_t)t.mt * 2 * xtile;
       const uint8_t* cs = reinterpret_cast<const uint8_t*>(D.planes[t.o]) + (size_t)t.nt * kb * b_bytes;
-      for (int pass = 0; pass < (t.abs ? 3 : 1); pass++) {  // magnitudes: h h, h l, l h
+      const int passes = t.abs && t.o == 0 && a.full_abs ? 3 : 1;  // magnitudes: h h, h l, l h
+      for (int pass = 0; pass < passes; pass++) {
         const uint8_t* xp = xs + (size_t)(t.plane + (pass == 2)) * xplane;
         const uint8_t* cp = cs + (size_t)(t.plane + (pass == 1)) * cplane;
         for (int k = 0; k < kb; k++, it++) {
@@ -371,8 +368,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     uint32_t s = 0, ph = 0, n = 0;  // the next K block's stage and phase
     bool ok = true;
     for (int64_t u = first; u < n_units && ok && !*dead; u += step, n++) {
-      const Unit t = unit_of(D, a, u, nmt2);
-      const int nk = D.kb[1 - t.o] * (t.abs ? 3 : 1);
+      const Unit t = unit_of(D, u, nmt2);
+      const int nk = D.kb[1 - t.o] * (t.abs && t.o == 0 && a.full_abs ? 3 : 1);
       const uint32_t idesc = umma::idesc_bf16(128, D.nw[t.o]);
       for (int k = 0; k < nk && ok; k++) {
         const uint64_t off = (uint64_t)(s * (kStageBytes / 16));
@@ -404,7 +401,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
     uint32_t n = 0;
     bool ok = true;
     for (int64_t u = first; u < n_units && ok && !*dead; u += step, n++) {
-      const Unit t = unit_of(D, a, u, nmt2);
+      const Unit t = unit_of(D, u, nmt2);
       const int nw = D.nw[t.o], ldy = D.ldy[t.o];
       const int c0 = part * (nw / 2), nc = nw / 2;  // up to 128 columns, a multiple of 16
       for (int h = 0; h < 2; h++) {
@@ -422,7 +419,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
         __syncwarp();
         if (lane == 0) umma::mbar_arrive(&tempty[h]);
         if (t.abs) {
-          float* dst = a.Yabs + wl * ldy + t.nt * nw + c0;
+          float* dst = a.Yabs + (t.o ? (size_t)a.nmt * 128 * D.ldy[0] : 0) + wl * ldy + t.nt * nw + c0;
 #pragma unroll
           for (int g = 0; g < 8; g++) {
             if (16 * g >= nc) break;
@@ -471,16 +468,59 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 // (8192 walkers of 750000 determinants, and those it re-evaluates) 0.82 ms, of which the first is
 // 0.70, against 1.22 with 32-bit limbs in 64-bit multiply-adds and 1.15 with two determinants per
 // lane (the constant loads then bound it). Q, the pairs of moduli, is a template argument for the
-// usual counts: unrolled to the largest 0.88. Every
+// usual counts: unrolled to the largest 0.88. (Before the choice of wide rows, which takes 0.1 ms.) Every
 // walker's Psi~ is summed in one warp, in a fixed order. Stores go through shared memory so that a
 // warp writes 256 consecutive bytes.
 // Few walkers (a re-evaluation, or too few for the warps of three blocks an SM): four warps to a walker
 // and product, so that each walks a quarter of the determinants: 67 of 256 slots with 900 + 900
 // determinants 44 -> 14 us, 87 with 3000 + 3000 120 -> 34, 1000 walkers of 900 + 900 46 -> 40.
 constexpr int kCrtFewWalkers = 8;
+constexpr float kWideRow = 0x1p-13f;
+
+// The sums over one segment of C (a row, or a column): eight lanes to a segment (lane8), acc = sum c x in
+// FP64 and aa = sum |c| |x|, in all eight.
+__device__ __forceinline__ void segment_sum(int b, int e, const int* __restrict__ gi, const double* __restrict__ val,
+                                            const double* __restrict__ x, int64_t wp, int lane8, double& acc, float& aa) {
+  acc = 0.0;
+  aa = 0.0f;
+#pragma unroll 4
+  for (int k = b + lane8; k < e; k += 8) {
+    const double c = __ldg(val + k), xv = x[(size_t)__ldg(gi + k) * wp];
+    acc = fma(c, xv, acc);
+    aa = fmaf(abs_f32_of(c), abs_f32_of(xv), aa);
+  }
+#pragma unroll
+  for (int off = 4; off; off >>= 1) {
+    acc += __shfl_xor_sync(0xffffffffu, acc, off);
+    aa += __shfl_xor_sync(0xffffffffu, aa, off);
+  }
+}
+
+// Rows of one stretch of 128 formed in FP64 instead, four at a time: bit l of mask z is row base + 4 l + z,
+// whose value goes into the stretch's tile.
+__device__ __noinline__ void wide_rows(const int* __restrict__ ptr, const int* __restrict__ gi,
+                                       const double* __restrict__ val, const double* __restrict__ x, int64_t wp, int base,
+                                       uint4 masks, double* tile) {
+  const int lane = threadIdx.x & 31, lane8 = lane & 7, quad = lane >> 3;
+  for (int z = 0; z < 4; z++) {
+    unsigned m = z == 0 ? masks.x : (z == 1 ? masks.y : (z == 2 ? masks.z : masks.w));
+    while (m) {
+      int mine = -1;
+      for (int q = 0; q < 4 && m; q++, m &= m - 1)
+        if (q == quad) mine = 4 * (__ffs(m) - 1) + z;
+      const int b = mine >= 0 ? __ldg(ptr + base + mine) : 0, e = mine >= 0 ? __ldg(ptr + base + mine + 1) : 0;
+      double acc;
+      float aa;
+      segment_sum(b, e, gi, val, x, wp, lane8, acc, aa);
+      if (mine >= 0 && lane8 == 0) tile[mine] = acc;
+    }
+  }
+  __syncwarp();
+}
+
 template <int Q>
 __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ DenseContract D, DevProblem P, DevScratch S,
-                                                  int64_t w0, int64_t n_walk, int nmt, int n_abs, int parts) {
+                                                  int64_t w0, int64_t n_walk, int nmt, int full_abs, int parts) {
   __shared__ double2 tile[8][64];
   __shared__ double psi_s[4];
   __shared__ float pa_s[4];
@@ -497,34 +537,36 @@ __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ Dens
   double* out = S.vu + w * ((int64_t)nu + nd) + (o ? nu : 0);
   double psi = 0.0;
   float pa = 0.0f;
+  const int* ptr = o ? P.csc_ptr : P.csr_ptr;
+  const int* gi = o ? P.csc_row : P.csr_col;
+  const double* val = o ? P.csc_val : P.csr_val;
+  const double* x = S.r + (size_t)(o ? 0 : nu) * wp + w;
   if (xb >= 0x7ff || failed) {  // ratios that are not finite: the FP64 sum itself
-    const int* ptr = o ? P.csc_ptr : P.csr_ptr;
-    const int* gi = o ? P.csc_row : P.csr_col;
-    const double* val = o ? P.csc_val : P.csr_val;
-    const double* x = S.r + (size_t)(o ? 0 : nu) * wp + w;
-    for (int i = 32 * part + lane; i < n; i += 32 * parts) {
-      double acc = 0.0;
-      float aa = 0.0f;
-      for (int k = ptr[i]; k < ptr[i + 1]; k++) {
-        const double xv = x[(size_t)gi[k] * wp];
-        acc = fma(val[k], xv, acc);
-        aa = fmaf(abs_f32_of(val[k]), abs_f32_of(xv), aa);
-      }
+    for (int i0 = 4 * part; i0 < n; i0 += 4 * parts) {
+      const int i = i0 + (lane >> 3), b = i < n ? ptr[i] : 0, e = i < n ? ptr[i + 1] : 0;
+      double acc;
+      float aa;
+      segment_sum(b, e, gi, val, x, wp, lane & 7, acc, aa);
       if (failed) acc = __longlong_as_double(0x7ff8000000000000LL);
-      out[i] = acc;
-      if (!o) {
-        const double ri = S.r[(size_t)i * wp + w];
-        psi = fma(ri, acc, psi);
-        pa = fmaf(abs_f32_of(ri), aa, pa);
+      if (i < n && (lane & 7) == 0) {
+        out[i] = acc;
+        if (!o) {
+          const double ri = S.r[(size_t)i * wp + w];
+          psi = fma(ri, acc, psi);
+          pa = fmaf(abs_f32_of(ri), aa, pa);
+        }
       }
     }
   } else {
     const int e0 = xb - 1022 - kCBits - kRBits;
     const uint8_t* y = S.dy + (o ? (size_t)D.nm * nmt * 128 * D.ldy[0] : 0) + (size_t)wl * ldy;
     const size_t yplane = (size_t)nmt * 128 * ldy;
+    const float* yabs = S.dyabs + (o ? (size_t)nmt * 128 * D.ldy[0] : 0) + (size_t)wl * ldy;
     for (int base = 128 * part; base < n; base += 128 * parts) {
       const int i0 = base + 4 * lane;
+      float4 mag = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
       if (i0 < ldy) {
+        mag = __ldg(reinterpret_cast<const float4*>(yabs + i0));
         // sums over the moduli of residue byte x weight in 16-bit limbs (and the quotient's, limb 8): the
         // bytes of two moduli against their two weights with one dp2a per determinant and limb
         uint32_t a[4][9];
@@ -566,6 +608,12 @@ __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ Dens
         tile[warp][2 * lane + 1] = make_double2(v[2], v[3]);
       }
       __syncwarp();
+      const uint4 wide = make_uint4(__ballot_sync(0xffffffffu, i0 < n && mag.x < kWideRow),
+                                    __ballot_sync(0xffffffffu, i0 + 1 < n && mag.y < kWideRow),
+                                    __ballot_sync(0xffffffffu, i0 + 2 < n && mag.z < kWideRow),
+                                    __ballot_sync(0xffffffffu, i0 + 3 < n && mag.w < kWideRow));
+      if (wide.x | wide.y | wide.z | wide.w)
+        wide_rows(ptr, gi, val, x, wp, base, wide, reinterpret_cast<double*>(tile[warp]));
 #pragma unroll
       for (int j = 0; j < 4; j++) {
         const int i = base + 32 * j + lane;
@@ -575,9 +623,9 @@ __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ Dens
           if (!o) {
             const double ri = S.r[(size_t)i * wp + w];
             psi = fma(ri, v, psi);
-            if (n_abs) {
+            if (full_abs) {
               const int es = D.es[0][i];
-              const float m = S.dyabs[(size_t)wl * ldy + i];
+              const float m = yabs[i];
               pa = fmaf(abs_f32_of(ri), es >= -126 && es <= 127 ? m * __int_as_float((es + 127) << 23) : ldexpf(m, es), pa);
             }
           }
@@ -685,16 +733,18 @@ cudaError_t launch_dense_rowsum(const DevProblem& P, const int* const es[2], uin
   return cudaGetLastError();
 }
 
+int dense_planes(const DenseContract& D, int o) { return D.nm + (o ? 1 : 2); }
+
 size_t dense_plane_elems(const DenseContract& D, int o) { return (size_t)D.nt[o] * D.kb[1 - o] * D.nw[o] * 64; }
 
 cudaError_t launch_dense_planes(const DevProblem& P, const DenseContract& D, cudaStream_t st) {
   for (int o = 0; o < 2; o++) {
-    const size_t bytes = dense_plane_elems(D, o) * 2 * (D.nm + (o ? 0 : 2));
+    const size_t bytes = dense_plane_elems(D, o) * sizeof(uint16_t) * dense_planes(D, o);
     cudaError_t e = cudaMemsetAsync(D.planes[o], 0, bytes, st);
     if (e != cudaSuccess) return e;
     k_mod_planes<<<(unsigned)((P.nnz + 255) / 256), 256, 0, st>>>(D, o, o ? P.csc_col : P.csr_row,
                                                                  o ? P.csc_row : P.csr_col, o ? P.csc_val : P.csr_val,
-                                                                 P.nnz, o ? 0 : 1);
+                                                                 P.nnz, dense_planes(D, o) - D.nm);
   }
   return cudaGetLastError();
 }
@@ -710,9 +760,9 @@ void dense_shape(int n_up, int n_dn, DenseContract* D) {
 }
 
 void dense_bytes(const DenseContract& D, size_t* x, size_t* y, size_t* yabs) {
-  *x = (size_t)(D.nm * (D.kb[0] + D.kb[1]) + 2 * D.kb[1]) * 64 * 2;
+  *x = (size_t)(dense_planes(D, 1) * D.kb[0] + dense_planes(D, 0) * D.kb[1]) * 64 * sizeof(uint16_t);
   *y = (size_t)D.nm * (D.ldy[0] + D.ldy[1]);
-  *yabs = (size_t)D.ldy[0] * sizeof(float);
+  *yabs = (size_t)(D.ldy[0] + D.ldy[1]) * sizeof(float);
 }
 
 cudaError_t launch_contract_dense(const DevProblem& P, const DevScratch& S, int64_t n_walk, cudaStream_t st,
@@ -723,19 +773,20 @@ cudaError_t launch_contract_dense(const DevProblem& P, const DevScratch& S, int6
   cudaError_t e = opt.ensure(k_mod_gemm, smem);
   if (e != cudaSuccess) return e;
   if (stamp && (e = cudaMemsetAsync(stamp, 0, 4 * sizeof(unsigned long long), st)) != cudaSuccess) return e;
-  // the magnitude sum feeds the error estimate only, and a re-evaluation keeps the one it has
-  const int n_abs = !S.live && P.fallback_tol > 0.0 && P.n_up <= MDET_FALLBACK_MAX_SPIN;
+  // the error estimate wants the magnitude sums of v more accurately than the choice of rows does (full LU's
+  // contraction has none)
+  const int full_abs = !S.live && P.fallback_tol > 0.0 && P.n_up <= MDET_FALLBACK_MAX_SPIN;
   for (int64_t w0 = 0; w0 < n_walk; w0 += S.dblk) {
     const int64_t nb = std::min<int64_t>(S.dblk, n_walk - w0);
     const int nmt = (int)((nb + 255) / 256) * 2;
     k_mod_residues<<<dim3(D.kb[0] + D.kb[1], nmt * 4), 256, 0, st>>>(D, S.r, S.wp, S.xmax, w0, P.n_det_sp[0],
-                                                                 P.n_det_sp[1], S.dx, nmt, n_abs, S.derr, S.live);
-    GemmArgs a{S.dx, S.dy, S.dyabs, nmt, n_abs, w0, S.live, S.derr, stamp};
-    const int64_t units = (int64_t)(nmt / 2) * ((int64_t)(D.nm + n_abs) * D.nt[0] + (int64_t)D.nm * D.nt[1]);
+                                                                 P.n_det_sp[1], S.dx, nmt, full_abs, S.derr, S.live);
+    GemmArgs a{S.dx, S.dy, S.dyabs, nmt, full_abs, w0, S.live, S.derr, stamp};
+    const int64_t units = (int64_t)(nmt / 2) * (D.nm + 1) * (D.nt[0] + D.nt[1]);
     k_mod_gemm<<<(unsigned)std::min<int64_t>(units, std::max(P.n_sm, 1)), kGemmThreads, smem, st>>>(D, a);
     auto* crt = D.nm <= 16 ? k_mod_crt<8> : D.nm <= 18 ? k_mod_crt<9> : k_mod_crt<kMaxModuli / 2>;
     const int parts = S.live || nb <= (int64_t)kCrtFewWalkers * P.n_sm ? 4 : 1;
-    crt<<<(unsigned)(parts == 4 ? nb : (nb + 3) / 4), 256, 0, st>>>(D, P, S, w0, n_walk, nmt, n_abs, parts);
+    crt<<<(unsigned)(parts == 4 ? nb : (nb + 3) / 4), 256, 0, st>>>(D, P, S, w0, n_walk, nmt, full_abs, parts);
     if (n_kernels) *n_kernels += 3;
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

@@ -7,6 +7,8 @@ evaluation without the fallback).
 """
 from __future__ import annotations
 
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -182,3 +184,35 @@ def test_blocks_of_walkers(n_walk, prec):
     assert ctx.last_kernels == 8 + 2 * 3
     for k in ("log_abs_psi", "sign"):  # each walker's Psi~ is summed in a fixed order
         assert np.array_equal(got[k], whole[k]), k
+
+
+@pytest.mark.parametrize("full_lu,prec", [(False, pkg.PRECISION_FP64), (True, pkg.PRECISION_FP64), (False, pkg.PRECISION_MIXED)])
+def test_mos_of_very_different_scale(full_lu, prec):
+    """Psi does not change when a MO is scaled and the coefficients of the products that occupy it are divided
+    by the same power of two: every term of every sum is the same number as before, but rows of C and
+    ratios now range over 2^48 (four such MOs per spin), which a fixed-point form relative to the largest would
+    cut. Both agree within the rounding of the sums."""
+    wl = _workload(130, 70, 60)
+    ref = _occupied(wl, int(np.argmax(np.abs(wl.ci_coef))))
+    odd = np.array([m % 2 == 1 and m not in ref for m in range(wl.n_mo)])
+    power = np.array([12 * sum(odd[m] for m in _occupied(wl, k, True)) for k in range(wl.n_det)])
+    scaled = dataclasses.replace(wl, mo_coef=wl.mo_coef * np.where(odd, 2.0 ** 12, 1.0), ci_coef=np.ldexp(wl.ci_coef, -power))
+    got = []
+    for w in (wl, scaled):
+        ctx = pkg.Context.from_workload(w, device=0, precision=prec)
+        ctx.set_fallback(1e-30 if full_lu else 0.0)
+        got.append(_eval(ctx, wl.R))
+    want = oracle.evaluate(wl)
+    # as in test_residue_products_match_oracle_and_sparse_sums; pairs carry 2^-47 instead of 2^-53
+    u = 2.0 ** -53 if prec == pkg.PRECISION_FP64 else 2.0 ** -47
+    tol = 200 * u * np.maximum(want["kappa"], 1.0) + 4 * np.spacing(np.abs(want["log_abs_psi"]))
+    assert np.all(np.abs(got[0]["log_abs_psi"] - got[1]["log_abs_psi"]) <= tol)
+    assert np.array_equal(got[0]["sign"], got[1]["sign"])
+
+
+def _occupied(wl, k, twice=False):
+    """MOs of the two determinants of product k (twice: one entry per electron)."""
+    mos = []
+    for words in (wl.det_up[k], wl.det_dn[k]):
+        mos += [m for m in range(wl.n_mo) if int(words[m // 64]) >> (m % 64) & 1]
+    return mos if twice else set(mos)
