@@ -436,6 +436,28 @@ mdet_status spin_tables(mdet_ctx* c, int sp, int n_int, const std::vector<uint64
   return MDET_OK;
 }
 
+// Device memory that an evaluation can do without: a quarter of what is free at most, so that the arrays
+// that cannot be done without (allocated first), and other contexts' and the caller's, find room.
+int64_t optional_room() {
+  size_t free_b = 0, total_b = 0;
+  if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return (int64_t)(free_b / 4);
+}
+
+// Allocates from it; false (and *p null) when there is no room.
+template <class T>
+bool optional_alloc(T** p, size_t bytes) {
+  *p = nullptr;
+  if ((int64_t)bytes > optional_room()) return false;
+  if (cudaMalloc((void**)p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  *p = nullptr;
+  return false;
+}
+
 // The digits of B as operand tiles of the tcgen05 orbital product: per chunk of 32 MOs and slice of
 // 16 AOs, [AO / 8 mod 2][digit][MO][AO mod 8], so that the digits' MOs are rows of one operand. Mixed precision: the 7 digits `dig` of B_dig; FP64: 8
 // digits of B_am 2^(62 - fexp_m) (balanced base 256, the bytes of that integer + 0x80...80 less 128).
@@ -518,14 +540,13 @@ mdet_status build_dense(mdet_ctx* c) {
   if (!choose_moduli(mx.data(), &D)) return MDET_OK;
   for (int o = 0; o < 2; o++) {
     const size_t bytes = dense_plane_elems(D, o) * sizeof(uint16_t) * dense_planes(D, o);
-    void* p = nullptr;
-    if (bytes > kDenseMaxBytes || cudaMalloc(&p, bytes) != cudaSuccess) {
-      cudaGetLastError();  // no room: the sparse sums
+    if (bytes > kDenseMaxBytes || !optional_alloc(&D.planes[o], bytes)) {  // no room: the sparse sums
+      if (o) cudaFree(D.planes[0]);
+      D.planes[0] = D.planes[1] = nullptr;
       return MDET_OK;
     }
-    c->dev_problem_allocs.push_back(p);
-    D.planes[o] = static_cast<uint16_t*>(p);
   }
+  for (uint16_t* p : D.planes) c->dev_problem_allocs.push_back(p);
   CUDA_TRY(c, launch_dense_planes(P, D, nullptr));
   CUDA_TRY(c, cudaStreamSynchronize(nullptr));
   c->dense_ok = true;
@@ -745,53 +766,65 @@ mdet_status alloc_eval_arrays(mdet_ctx* c, DevScratch& S, int64_t W, bool df_tab
   if ((s = dalloc(c, &S.psit, (size_t)wp))) return s;
   if ((s = dalloc(c, &S.psia, (size_t)wp))) return s;
   if ((s = dalloc(c, &S.wstat, (size_t)W))) return s;
-  const bool main_scratch = df_tables || c->precision == MDET_PRECISION_FP64;  // not a re-evaluation's
-  if (main_scratch && scatter_group_walkers(P, W, df_tables) > 0 &&
-      cudaMalloc((void**)&S.W, sizeof(double) * W * N * M) != cudaSuccess) {  // no room: the epilogue's own scatter
-    cudaGetLastError();
-    S.W = nullptr;
+  S.cap_walk = W;
+  S.wp = wp;
+  return MDET_OK;
+}
+
+// The workspaces of a scratch that evaluations go faster with, each left out when there is no room: after
+// every array that has to be there. Those of the evaluation itself (not of a re-evaluation's scratch) first.
+mdet_status alloc_workspaces(mdet_ctx* c, DevScratch& S, bool df_tables, bool re_evaluation) {
+  const DevProblem& P = c->P;
+  const int64_t W = S.cap_walk, N = P.n_elec, M = P.n_mo;
+  auto drop = [](auto*& p) {
+    if (p) cudaFree(p);
+    p = nullptr;
+  };
+  // the residue products, for blocks of walkers that the workspace holds (a re-evaluation takes the
+  // sparse sums: see refine)
+  if (c->dense_ok && !re_evaluation) {
+    size_t x, y, ya;
+    dense_bytes(c->dense, &x, &y, &ya);
+    const int64_t work = std::min(c->product_bytes > 0 ? c->product_bytes : kDenseWorkBytes, optional_room());
+    const int64_t fit = work / (int64_t)(x + y + ya) / kWalkerPad * kWalkerPad;
+    S.dblk = std::min(S.wp, std::max<int64_t>(fit, kWalkerPad));
+    if (optional_alloc(&S.xmax, sizeof(uint32_t) * 2 * S.wp) && optional_alloc(&S.dx, x * S.dblk) &&
+        optional_alloc(&S.dy, y * S.dblk) && optional_alloc(&S.dyabs, ya * S.dblk) &&
+        optional_alloc(&S.derr, sizeof(int))) {
+      CUDA_TRY(c, cudaMemset(S.xmax, 0, sizeof(uint32_t) * 2 * S.wp));
+    } else {  // the sparse sums
+      drop(S.xmax);
+      drop(S.dx);
+      drop(S.dy);
+      drop(S.dyabs);
+      drop(S.derr);
+    }
   }
   if (mo_digits_supported(P, df_tables)) {  // digits of the AO values, for blocks of walkers
     const int64_t row_bytes = (int64_t)mo_digits_row_bytes(P, df_tables), per = 5 * N * row_bytes;
-    S.xd_walk = std::min(W, std::max<int64_t>(1, (c->digit_bytes > 0 ? c->digit_bytes : kDigitBytes) / per));
+    const int64_t work = std::min(c->digit_bytes > 0 ? c->digit_bytes : kDigitBytes, optional_room());
+    S.xd_walk = std::min(W, std::max<int64_t>(1, work / per));
     const int64_t rows = (S.xd_walk * 5 * N + 127) / 128 * 128;
-    if (cudaMalloc((void**)&S.xd, rows * row_bytes) != cudaSuccess ||
-        cudaMalloc((void**)&S.xer, sizeof(int) * rows) != cudaSuccess) {  // no room: the CUDA-core products
-      cudaGetLastError();
-      if (S.xd) cudaFree(S.xd);
-      S.xd = nullptr;
-      S.xer = nullptr;
+    if (!optional_alloc(&S.xd, rows * row_bytes) || !optional_alloc(&S.xer, sizeof(int) * rows)) {
+      drop(S.xd);  // the CUDA-core products
+      drop(S.xer);
     }
   }
-  // the workspace of the residue products, for blocks of walkers that it holds (a re-evaluation takes the
-  // sparse sums: see refine)
-  if (c->dense_ok && main_scratch) {
-    size_t x, y, ya;
-    dense_bytes(c->dense, &x, &y, &ya);
-    const int64_t work = c->product_bytes > 0 ? c->product_bytes : kDenseWorkBytes;
-    const int64_t fit = work / (int64_t)(x + y + ya) / kWalkerPad * kWalkerPad;
-    S.dblk = std::min(wp, std::max<int64_t>(fit, kWalkerPad));
-    bool ok = cudaMalloc((void**)&S.xmax, sizeof(uint32_t) * 2 * wp) == cudaSuccess &&
-              cudaMalloc((void**)&S.dx, x * S.dblk) == cudaSuccess &&
-              cudaMalloc((void**)&S.dy, y * S.dblk) == cudaSuccess &&
-              cudaMalloc((void**)&S.dyabs, ya * S.dblk) == cudaSuccess &&
-              cudaMalloc((void**)&S.derr, sizeof(int)) == cudaSuccess;
-    if (ok) {
-      CUDA_TRY(c, cudaMemset(S.xmax, 0, sizeof(uint32_t) * 2 * wp));
-    } else {  // no room: the sparse sums
-      cudaGetLastError();
-      void* p[] = {S.xmax, S.dx, S.dy, S.dyabs, S.derr};
-      for (void* q : p)
-        if (q) cudaFree(q);
-      S.xmax = nullptr;
-      S.dx = nullptr;
-      S.dy = nullptr;
-      S.dyabs = nullptr;
-      S.derr = nullptr;
+  if (!re_evaluation && scatter_group_walkers(P, W, df_tables) > 0)
+    optional_alloc(&S.W, sizeof(double) * W * N * M);  // (else the epilogue's own scatter)
+  if (S.fb && S.xmax && c->precision == MDET_PRECISION_FP64) {  // full LU's contraction as residue products
+    const int64_t ndt = (int64_t)P.n_det_sp[0] + P.n_det_sp[1];
+    const int64_t ldw = (P.fallback_cap + kWalkerPad - 1) / kWalkerPad * kWalkerPad;
+    if (optional_alloc(&S.fb_r, sizeof(double) * ndt * ldw) && optional_alloc(&S.fb_xmax, sizeof(uint32_t) * 2 * ldw) &&
+        optional_alloc(&S.fb_psi, sizeof(double) * ldw)) {
+      CUDA_TRY(c, cudaMemset(S.fb_r, 0, sizeof(double) * ndt * ldw));
+      CUDA_TRY(c, cudaMemset(S.fb_xmax, 0, sizeof(uint32_t) * 2 * ldw));
+    } else {
+      drop(S.fb_r);
+      drop(S.fb_xmax);
+      drop(S.fb_psi);
     }
   }
-  S.cap_walk = W;
-  S.wp = wp;
   return MDET_OK;
 }
 
@@ -803,19 +836,6 @@ mdet_status alloc_fallback(mdet_ctx* c, DevScratch& S) {
   mdet_status s;
   if ((s = dalloc(c, &S.fb, (size_t)P.fallback_cap * ndt * (3 + 4 * nmax)))) return s;
   if ((s = dalloc(c, &S.fb_list, (size_t)P.fallback_cap + 1))) return s;
-  if (S.xmax && c->precision == MDET_PRECISION_FP64) {
-    const int64_t ldw = (P.fallback_cap + kWalkerPad - 1) / kWalkerPad * kWalkerPad;
-    if (cudaMalloc((void**)&S.fb_r, sizeof(double) * ndt * ldw) != cudaSuccess ||
-        cudaMalloc((void**)&S.fb_xmax, sizeof(uint32_t) * 2 * ldw) != cudaSuccess ||
-        cudaMalloc((void**)&S.fb_psi, sizeof(double) * ldw) != cudaSuccess) {  // no room: the sparse sums
-      cudaGetLastError();
-      if (S.fb_r) cudaFree(S.fb_r);
-      S.fb_r = nullptr;
-    } else {
-      CUDA_TRY(c, cudaMemset(S.fb_r, 0, sizeof(double) * ndt * ldw));
-      CUDA_TRY(c, cudaMemset(S.fb_xmax, 0, sizeof(uint32_t) * 2 * ldw));
-    }
-  }
   return dalloc(c, &S.fb_acc, (size_t)P.fallback_cap * (3 + 8 * MDET_FALLBACK_MAX_SPIN));
 }
 
@@ -837,17 +857,15 @@ bool escalation_on(const mdet_ctx* c) {
   return ndt * n * n * n > 1e6;
 }
 
-mdet_status ensure_scratch(mdet_ctx* c, int64_t n_walk) {
+mdet_status alloc_scratch(mdet_ctx* c, int64_t n_walk) {
   DevScratch& S = c->S;
-  if (n_walk <= S.cap_walk) return MDET_OK;
-  free_scratch(c);
   const DevProblem& P = c->P;
   const bool mixed = c->precision == MDET_PRECISION_MIXED;
   mdet_status s;
   if ((s = alloc_eval_arrays(c, S, n_walk, mixed, mixed && c->contract_impl == 1))) return s;
   if ((s = dalloc(c, &S.queue, (size_t)kQueueWords * mdet_ctx::kMaxChunks))) return s;
   if (P.fallback_tol > 0.0 && P.n_up <= MDET_FALLBACK_MAX_SPIN) {
-    if (!mixed) return alloc_fallback(c, S);
+    if (!mixed) return (s = alloc_fallback(c, S)) ? s : alloc_workspaces(c, S, mixed, false);
     // mixed: the list of flagged walkers, then an FP64 re-evaluation of at most fallback_cap
     // of them (orbitals, optionally the ratio table, then full LU) on a scratch of their own
     const int cap = P.fallback_cap;
@@ -864,7 +882,17 @@ mdet_status ensure_scratch(mdet_ctx* c, int64_t n_walk) {
       return s;
     E.live = c->e_live;
   }
-  return MDET_OK;
+  if ((s = alloc_workspaces(c, S, mixed, false))) return s;
+  return c->E.fb ? alloc_workspaces(c, c->E, false, true) : MDET_OK;
+}
+
+// Scratch for n_walk walkers: all of it, or none.
+mdet_status ensure_scratch(mdet_ctx* c, int64_t n_walk) {
+  if (n_walk <= c->S.cap_walk) return MDET_OK;
+  free_scratch(c);
+  const mdet_status s = alloc_scratch(c, n_walk);
+  if (s != MDET_OK) free_scratch(c);
+  return s;
 }
 
 // Mixed precision: walkers whose estimate exceeds the tolerance (at most

@@ -63,3 +63,34 @@ def test_measured_fp64_rate_is_plausible():
     assert ms > 0 and 500 < mhz < 3000, (ms, mhz)
     assert 0.3 < a < 5.0, a
     assert abs(a - b) <= 0.1 * max(a, b), (a, b)
+
+
+def test_optional_workspaces_leave_room_for_what_is_needed():
+    """On a device that other allocations have nearly filled, the workspaces that only make an evaluation faster
+    are left out before an array that it needs is: with 1.8 to 4.2 GB free (1.6 GB are needed, 2.7 more are
+    wanted), every evaluation succeeds, with the results of one that has all the room."""
+    wl = synth.make_workload("room", 5, 5, 4, 9, (12, 6, 2), (0.05, 500.0), 30, 5000, 4, 64, n_unique=(300, 280))
+    R = torch.from_numpy(np.tile(wl.R, (625, 1, 1))).to("cuda:0")
+
+    def evaluate(free=None):
+        ctx = pkg.Context.from_workload(wl, device=0, precision=pkg.PRECISION_MIXED)
+        ctx.set_fallback(1e-5, 4096)
+        out = ctx.alloc_outputs(len(R))
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        filler = torch.empty(torch.cuda.mem_get_info()[0] - free, dtype=torch.uint8, device="cuda:0") if free else None
+        try:
+            got = {k: v[:64].cpu().numpy() for k, v in ctx.evaluate(R, out=out).items()}
+        finally:
+            del filler
+            ctx.close()
+            torch.cuda.empty_cache()
+        return got
+
+    want = evaluate()
+    ref = oracle.evaluate(wl)
+    for free in range(1800, 4300, 200):
+        got = evaluate(free << 20)
+        rep = compare(got, ref, tol_psi=1e-5, tol_der=1e-5)  # the fallback's tolerance
+        assert rep["ok"], (free, rep)
+        assert np.array_equal(got["sign"], want["sign"]), free
