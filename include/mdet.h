@@ -325,20 +325,25 @@ mdet_status mdet_get_last_launches(const mdet_ctx* ctx, int32_t* n_chunks, int32
 /*
  * Tile shapes of the evaluation kernels (tuning knobs with no counterpart in
  * the paper): spmm_chunk nonzeros of C per warp in the sparse contraction
- * (64..8192; the default, 512, is lowered to 16 for small expansions),
- * mo_ec electrons per thread block in the orbital kernels (4, 6 or 8),
+ * (64..8192; the default, 512, is lowered to 16 for small expansions, any other
+ * value is used as it is), mo_ec electrons per thread block in the CUDA-core
+ * orbital kernels (4, 6 or 8; in FP64, and in mixed precision beyond 112 AOs or
+ * 128 MOs, a value other than the default asks for them instead of the digit
+ * products),
  * walker_chunks as in mdet_set_walker_chunks, spmm_blocks the form of the
  * contraction (0: where C is dense enough, more than 1.2 % of at least 4,096
  * products, exact residue products on the tcgen05 tensor cores with one rounding
- * at the end, if the device has room for C's planes; elsewhere sparse FP64 sums,
+ * at the end, FP64 sums for rows that their fixed point would cut, if the device
+ * has room for C's planes; elsewhere sparse FP64 sums,
  * one warp per work item with one chunk, 4 blocks per SM with several; any other
  * value: the sparse sums on a persistent grid of at most that many 128-thread
  * blocks whose warps draw work items from a counter), mo_impl the orbital product
  * (2, the default: exact BF16 digit products on the tcgen05 tensor cores with
  * TMEM accumulators, in mixed precision accurate to about 2^-55 of the row and
- * column maxima and in FP64 to 2^-63; for small bases and the re-evaluation of
- * flagged walkers FP64 dot products; where the digits' sums could exceed 2^24 it
- * falls back to 1; 1: on the CUDA cores, the compensated FP32 dot product, accurate
+ * column maxima, in FP64 (and in mixed precision beyond 112 AOs or 128 MOs) with
+ * dot products for the elements that a dot product gives more accurately; for
+ * small bases and the re-evaluation of flagged walkers FP64 dot products; where
+ * the digits' sums could exceed 2^24 it falls back to 1; 1: on the CUDA cores, the compensated FP32 dot product, accurate
  * relative to each term, or the FP64 product; 0: mixed precision, the same digit
  * products on warp-level mma.sync),
  * contract_impl the CI contraction of the mixed path (0, the default: exact or
@@ -368,7 +373,8 @@ mdet_status mdet_set_tuning(mdet_ctx* ctx, const mdet_tuning* in);
  * pointer, [n_walk][n_up+n_dn][3]) with CUDA events on the context's stream and
  * picks the tile shapes by coordinate descent over spmm_chunk in
  * {256, 512, 1024, 2048}, mo_ec in {4, 6, 8} and (mixed precision)
- * walker_chunks in {1, 2, 3, 4}, stopping when budget_ms of GPU time is spent.
+ * walker_chunks in {1, 2, 3, 4}, stopping when budget_ms of GPU time is spent;
+ * a shape that this expansion's kernels do not have is left as it is.
  * The winner is stored in the context and returned in *out (may be null).
  * Allocates temporary output buffers; synchronous.
  */

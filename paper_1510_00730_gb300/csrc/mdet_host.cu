@@ -14,6 +14,13 @@
 
 using namespace mdet;
 
+namespace {
+constexpr int kDefaultChunk = 512;  // nonzeros per work item of the sparse contraction (pick_items)
+
+// measured best electron block of each CUDA-core orbital kernel
+int default_mo_ec(int precision) { return precision == MDET_PRECISION_MIXED ? 4 : 6; }
+}  // namespace
+
 struct mdet_ctx {
   int device = MDET_NO_DEVICE;
   int precision = MDET_PRECISION_FP64;
@@ -72,7 +79,7 @@ struct mdet_ctx {
   int escalate = MDET_ESCALATE_AUTO;
   bool in_batch = false;  // set while a batch enqueues this context's evaluation
   std::vector<int32_t> csr_ptr, csc_ptr;
-  int spmm_chunk = 512;  // tile shapes (mdet_set_tuning / mdet_autotune)
+  int spmm_chunk = kDefaultChunk;  // tile shapes (mdet_set_tuning / mdet_autotune)
   int spmm_blocks = 0;
   int mo_impl = 2;  // mixed orbitals: exact digit products on the tcgen05 tensor cores
   int mo_ec = 4;
@@ -344,15 +351,22 @@ bool use_items(const mdet_ctx* c, DevProblem& P, int chunk) {
   return false;
 }
 
-// The item size of one contraction: the tuned one, or shorter items when those are too few to fill
-// the chip with warps (each walks its nonzeros one after the other). The count is over groups of 256
-// walkers.
+// The item size of one contraction: the tuned one, or, instead of the default, shorter items when those
+// are too few to fill the chip with warps (each walks its nonzeros one after the other). The count is
+// over groups of 256 walkers.
 void pick_items(const mdet_ctx* c, DevProblem& P, int64_t n_walk) {
+  if (c->spmm_chunk != kDefaultChunk) return;
   const int64_t groups = (n_walk + kWalkerPad - 1) / kWalkerPad;
   int chunk = c->spmm_chunk;
   for (int small : kSmallChunks)
     if (small < chunk && P.nnz / chunk * groups < kItemWarps) chunk = small;
   use_items(c, P, chunk);  // (sets that were not built leave the tuned one)
+}
+
+// Whether the tuning asks for a block shape of the CUDA-core orbital kernels instead of the digit
+// products that serve by default (bases that have no choice between them keep the digits).
+bool mo_cores_asked(const mdet_ctx* c) {
+  return c->mo_ec != default_mo_ec(c->precision) && mo_repairs(c->P, c->precision == MDET_PRECISION_MIXED);
 }
 
 void free_arrays(DevScratch& S) {
@@ -568,6 +582,7 @@ mdet_status upload_problem(mdet_ctx* c) {
   P.spmm_chunk = c->spmm_chunk;
   P.spmm_blocks = c->spmm_blocks;
   P.mo_ec = c->mo_ec;
+  P.mo_cores = mo_cores_asked(c);
   P.mo_impl = c->mo_impl;
   P.n_sm = c->n_sm;
   P.phi_df = c->precision == MDET_PRECISION_MIXED;
@@ -916,6 +931,7 @@ mdet_status refine(mdet_ctx* c, bool table, int64_t n_walk, const double* R, dou
   // per block, whose few live walkers spread evenly over the SMs.
   DevProblem Pe = P;
   Pe.mo_ec = 1;
+  Pe.mo_cores = false;
   if (!table) Pe.mo_impl = 1;
   if (!use_items(c, Pe, kEscalationChunk)) return fail(c, MDET_E_STATE, "internal: escalation items missing");
   CUDA_TRY(c, launch_mo_f64(Pe, E, cap, c->e_R, st));
@@ -1007,7 +1023,7 @@ mdet_status mdet_create(mdet_ctx** out, int device, int precision) {
   // the accuracy targets of the two paths: 1e-5 (mixed) and 1e-8 (FP64) relative
   c->fallback_tol = precision == MDET_PRECISION_MIXED ? 1e-5 : 1e-8;
   c->fallback_cap = precision == MDET_PRECISION_MIXED ? 256 : 512;
-  c->mo_ec = precision == MDET_PRECISION_MIXED ? 4 : 6;  // measured best electron block of each orbital kernel
+  c->mo_ec = default_mo_ec(precision);
   if (device >= 0) {
     int n = 0;
     if (cudaGetDeviceCount(&n) != cudaSuccess || device >= n) {
@@ -1510,7 +1526,9 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
     const bool table = escalation_on(c);
     mdet_status es = refine(c, table, n_walk, R, log_abs_psi, sign, grad, lap, e_local, status, st);
     if (es != MDET_OK) return es;
-    c->last_kernels += 3 + 5 + (table ? mo_kernels(P, c->E, P.fallback_cap, false) + 4 : 1 + 1);
+    DevProblem Pe = P;
+    Pe.mo_cores = false;
+    c->last_kernels += 3 + 5 + (table ? mo_kernels(Pe, c->E, P.fallback_cap, false) + 4 : 1 + 1);
   } else {
     DevScratch Sb = c->S;
     if (!dense) Sb.xmax = nullptr;
@@ -1759,6 +1777,7 @@ mdet_status mdet_set_tuning(mdet_ctx* c, const mdet_tuning* t) {
   c->n_chunks_cfg = std::min(t->walker_chunks, (int)mdet_ctx::kMaxChunks);
   c->P.spmm_chunk = c->spmm_chunk;
   c->P.mo_ec = c->mo_ec;
+  c->P.mo_cores = mo_cores_asked(c);
   return MDET_OK;
 }
 
@@ -1811,6 +1830,8 @@ mdet_status mdet_autotune(mdet_ctx* c, int64_t n_walk, const double* R, double b
     const int* vals = param == 0 ? chunks : (param == 1 ? ecs : wcs);
     const int nv = param == 1 ? 3 : 4;
     if (param == 2 && !mixed) break;
+    if (param == 0 && use_dense(c) && c->S.xmax) continue;      // residue products have no items,
+    if (param == 1 && !mo_repairs(c->P, mixed)) continue;       // and these bases no other orbital kernel
     for (int q = 0; q < nv && s == MDET_OK && spent < budget_ms; q++) {
       mdet_tuning t = cur;
       int* field = param == 0 ? &t.spmm_chunk : (param == 1 ? &t.mo_ec : &t.walker_chunks);

@@ -95,7 +95,8 @@ struct DevProblem {
   int contract_impl;      // tuning: contraction in FP64 (0) or double-float on the FP32 pipe (1, mixed only)
   const float2* csr_val_df;  // C values as double-float pairs, row-major and column-major orders
   const float2* csc_val_df;
-  int mo_ec;              // tuning: electrons per CTA in the orbital kernels (4, 6 or 8)
+  int mo_ec;              // tuning: electrons per CTA in the CUDA-core orbital kernels (4, 6 or 8)
+  bool mo_cores;          //   whether it asks for those instead of the digit products
   int mo_impl;            // tuning: mixed orbitals by exact digit products on the tensor cores with tcgen05 (2),
                           // with warp-level mma.sync (0), or the compensated FP32 dot product (1)
   int n_sm;               // multiprocessors of the device (persistent grids)

@@ -639,7 +639,7 @@ bool mo_digits_supported(const DevProblem& P, bool df) {
 }
 
 bool use_mo_digits(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df) {
-  return P.mo_impl == 2 && S.xd && mo_digits_supported(P, df);
+  return P.mo_impl == 2 && !P.mo_cores && S.xd && mo_digits_supported(P, df);
 }
 
 bool mo_repairs(const DevProblem& P, bool df) { return !df || P.n_ao > kPlainAos || P.n_mo > kPlainMos; }
