@@ -250,13 +250,23 @@ cudaError_t launch_gemm_bf16(const GemmOperand& A, const GemmOperand& B, int64_t
                              cudaStream_t st) {
   if (A.rows <= 0 || B.rows <= 0 || A.cols <= 0) return cudaSuccess;
   const int64_t kc = std::max<int64_t>(kGK, (k_per_cta + kGK - 1) / kGK * kGK);
-  const dim3 grid((unsigned)((A.rows + kGM - 1) / kGM), (unsigned)((B.rows + kGN - 1) / kGN),
-                  (unsigned)((A.cols + kc - 1) / kc));
   static SmemOptIn opt;
   cudaError_t e = opt.ensure(k_gemm_bf16, kSmem);
-  if (e != cudaSuccess) return e;
-  k_gemm_bf16<<<grid, kThreads, kSmem, st>>>(A, B, kc, E);
-  return cudaGetLastError();
+  constexpr int64_t kSlab = (int64_t)32768 * kGN;  // rows of B per launch: a grid's y dimension is 65,535
+  for (int64_t n0 = 0; e == cudaSuccess && n0 < B.rows; n0 += kSlab) {
+    GemmOperand b = B;
+    GemmEpilogue ep = E;
+    b.rows = std::min(kSlab, B.rows - n0);
+    b.p = static_cast<const char*>(B.p) + n0 * B.rs * (B.bf16 ? 2 : 4);
+    ep.out = E.out + n0 * E.ldn;
+    if (E.bias) ep.bias = E.bias + n0;
+    if (E.h) ep.h = E.h + n0;
+    const dim3 grid((unsigned)((A.rows + kGM - 1) / kGM), (unsigned)((b.rows + kGN - 1) / kGN),
+                    (unsigned)((A.cols + kc - 1) / kc));
+    k_gemm_bf16<<<grid, kThreads, kSmem, st>>>(A, b, kc, ep);
+    e = cudaGetLastError();
+  }
+  return e;
 }
 
 }  // namespace mdet

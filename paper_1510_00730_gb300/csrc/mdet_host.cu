@@ -125,6 +125,7 @@ constexpr int kQueueWords = 6;
 // residue planes of C above this size; default workspaces of the residue products and of the
 // orbitals' AO digits (mdet_set_workspace)
 constexpr size_t kDenseMaxBytes = (size_t)8 << 30;
+constexpr int64_t kDenseMaxBlock = (int64_t)1 << 20;  // walkers of a block: 32,768 in the residues' grid
 constexpr int64_t kDenseWorkBytes = (int64_t)4 << 30, kDigitBytes = (int64_t)5 << 28;
 
 // weights of the first, each middle and the last walker chunk of the pipelined evaluation. The
@@ -802,7 +803,7 @@ mdet_status alloc_workspaces(mdet_ctx* c, DevScratch& S, bool df_tables, bool re
     dense_bytes(c->dense, &x, &y, &ya);
     const int64_t work = std::min(c->product_bytes > 0 ? c->product_bytes : kDenseWorkBytes, optional_room());
     const int64_t fit = work / (int64_t)(x + y + ya) / kWalkerPad * kWalkerPad;
-    S.dblk = std::min(S.wp, std::max<int64_t>(fit, kWalkerPad));
+    S.dblk = std::min({S.wp, std::max<int64_t>(fit, kWalkerPad), kDenseMaxBlock});
     if (optional_alloc(&S.xmax, sizeof(uint32_t) * 2 * S.wp) && optional_alloc(&S.dx, x * S.dblk) &&
         optional_alloc(&S.dy, y * S.dblk) && optional_alloc(&S.dyabs, ya * S.dblk) &&
         optional_alloc(&S.derr, sizeof(int))) {

@@ -656,10 +656,11 @@ mdet_status mdet_mlp_backward(mdet_mlp* m, int64_t n_walk, const float* dout, vo
     e = launch_gemm_bf16(GemmOperand{m->d2, H, 1, n_walk, H, 0}, GemmOperand{pb + m->oW2, H, 1, H, H, 1}, H,
                          GemmEpilogue{kEpiDtanh, m->d1, H, 1, nullptr, m->h1, H}, st);
   // weight gradients, summed over the walkers (the GEMMs' K), 256 walkers per CTA (with 1,024 a batch
-  // of 8,192 gave 16 CTAs, and the three products took 600 us):
+  // of 8,192 gave 16 CTAs, and the three products took 600 us), more where a grid dimension ends at 65,535:
   // gW3[k][j] = sum_w h2[w][k] dout[w][j], gW2[k][j] = sum_w h1[w][k] d2[w][j],
   // gW1[i][j] = sum_w x[w][i] d1[w][j] (computed as its transpose: rows j, columns i)
-  const int64_t kpc = 256;
+  constexpr int64_t kMaxGrid = 65535;
+  const int64_t kpc = std::max<int64_t>(256, (n_walk / kMaxGrid + 64) / 64 * 64);
   if (e == cudaSuccess)
     e = launch_gemm_bf16(GemmOperand{m->h2, 1, H, H, n_walk, 0}, GemmOperand{dout, 1, no, no, n_walk, 0}, kpc,
                          GemmEpilogue{kEpiAtomic, m->g + m->oW3, no, 1, nullptr, nullptr, 0}, st);
@@ -672,7 +673,7 @@ mdet_status mdet_mlp_backward(mdet_mlp* m, int64_t n_walk, const float* dout, vo
   if (e != cudaSuccess) return cuda_status(e);
   // bias gradients from the unrounded deltas
   const ColSumJobs jobs{{{dout, (int)no, m->g + m->ob3}, {m->d2, (int)H, m->g + m->ob2}, {m->d1, (int)H, m->g + m->ob1}}};
-  const int64_t per = 64;
+  const int64_t per = std::max<int64_t>(64, n_walk / kMaxGrid + 1);
   const dim3 grid(blocks(std::max(no, H), 128), (unsigned)((n_walk + per - 1) / per), 3);
   k_bias_grad<<<grid, 128, 0, st>>>(jobs, n_walk, per);
   return cuda_status(cudaGetLastError());

@@ -102,3 +102,32 @@ def test_empty_sum_and_refusals():
     assert L.mdet_gemm_bf16(2, 2, 4, p, 3, p, 4, p, 2, 0, 64, None) == 1  # lda below K
     assert L.mdet_gemm_bf16(2, 2, 4, None, 4, p, 4, p, 2, 0, 64, None) == 1  # null operand
     assert L.mdet_gemm_bf16(0, 2, 4, None, 4, None, 4, None, 2, 0, 64, None) == 0  # nothing to do
+
+
+def test_more_columns_than_a_grid_dimension_holds():
+    """N beyond 65,535 tiles of 128 columns."""
+    rng = np.random.default_rng(3)
+    N = 65535 * 128 + 300
+    a, b = _int_operands(rng, 3, 1000, 16)
+    A = torch.tensor(a, dtype=torch.float32, device=DEV)
+    B = torch.tensor(b, dtype=torch.float32, device=DEV).repeat(N // 1000 + 1, 1)[:N].contiguous()
+    D = pkg.gemm_bf16(A, B)
+    want = torch.tensor(a @ b.T, dtype=torch.float32, device=DEV).repeat(1, N // 1000 + 1)[:, :N]
+    assert torch.equal(D, want)
+
+
+def test_gradients_over_more_walkers_than_a_grid_dimension_holds():
+    """The bias gradients' grid has a block per 64 walkers: beyond 65,535 of them a block takes more. Every
+    walker's output derivative is the same small integer, so the last layer's bias gradients are exact."""
+    from paper_1510_00730_gb300 import binding
+
+    n = 65535 * 64 + 100
+    mlp = binding.MLP(0, 1, hidden=64, seed=1, s0=-1.5)
+    R = torch.zeros(n, 1, 3, dtype=torch.float64, device=DEV)
+    out = mlp.forward(R)
+    dout = torch.full_like(out, 2.0)
+    mlp.zero_grad()
+    mlp.backward(dout)
+    g = mlp.grads()
+    assert np.array_equal(g[-4:], np.full(4, 2.0 * n, np.float32))
+    assert np.all(np.isfinite(g))
