@@ -124,6 +124,26 @@ def test_dense_rows_take_smaller_moduli():
     assert ctx.last_kernels == 8 + 8  # the residue products, and the full-LU fallback with its own
 
 
+@pytest.mark.parametrize("prec", [pkg.PRECISION_FP64, pkg.PRECISION_MIXED])
+def test_more_than_eighteen_moduli(prec):
+    """Rows of 12,000 nonzeros: residues of a modulus p add up to about 12,000 p / 4 a row, so moduli above about
+    106 are excluded, and 124.6 bits take at least 19 (counted with 8 % of margin)."""
+    limit, moduli, bits = 1.08 * np.sqrt(8 * 2.0 ** 24 / 12000), [], 0.0
+    for p in range(256, 15, -1):
+        if p <= limit and bits < 124.6 and all(np.gcd(p, q) == 1 for q in moduli):
+            moduli.append(p)
+            bits += np.log2(p)
+    assert len(moduli) > 18
+    wl = synth.make_workload("mod", 12, 5, 4, 9, (12, 6, 2), (0.05, 500.0), 30, 12 * 12000, 4, 7, n_unique=(12, 12000))
+    ctx = pkg.Context.from_workload(wl, device=0, precision=prec)
+    if prec == pkg.PRECISION_MIXED:
+        ctx.set_fallback(1e-7)  # below the test tolerance, as the parity tests of this path
+    got = _eval(ctx, wl.R)
+    rep = compare(got, oracle.evaluate(wl), **TOL[prec])
+    assert rep["ok"], rep
+    assert ctx.last_kernels == (8 + 8 if prec == pkg.PRECISION_FP64 else 8 + 14)
+
+
 @pytest.mark.parametrize("n_walk", [5, 300])
 def test_full_lu_contraction(n_walk):
     """Every walker through full LU (a tolerance below any estimate): its contraction as residue
