@@ -28,17 +28,8 @@ UNIT = "walker-steps/s"
 CPU_SAMPLE_WALKERS = 96     # bounded oracle sample for the CPU baseline (~10-30 s of CPU work)
 CPU_SINGLE_CORE_WALKERS = 8  # the same oracle on one core, for the per-core figure
 # dram__bytes_read.sum + dram__bytes_write.sum of one k_mod_gemm launch on the 750k workload with 8,192
-# walkers, from one ncu capture per precision; null for a configuration that was not captured
-GEMM_TRAFFIC_750K = {}
-# The CI contraction as residue products (k_mod_gemm) keeps 124.6 bits in moduli of at most 8: at least
-# 16 planes of each order's C. The magnitude sum of the error estimate is not counted.
-MIN_RESIDUE_PLANES = 16
-
-
-def contraction_dense(n_det, n_up, n_dn):
-    """The library's rule for the residue products: dense enough that the tensor cores' dense products
-    take less time than the sparse FP64 sums."""
-    return n_det >= 4096 and n_det > 0.012 * n_up * n_dn
+# walkers, from one ncu capture per precision
+GEMM_TRAFFIC_750K = {"mixed": 4.48e9, "fp64": 4.47e9}
 
 
 def bf16_peak():
@@ -384,17 +375,17 @@ def run_ours(args):
     timed = ("mean over the timed steps of each launch's device duration, from its first block's start to its "
              "last warp's exit on the GPU global timer (written by the kernel)")
     traffic = args.traffic
-    if contraction_dense(st["n_det"], st["n_det_up"], st["n_det_dn"]):
+    moduli = ctxs[primary].last_moduli
+    if moduli:
         if traffic is None and args.workload == "chlorine_like_750k" and W == 8192:
             traffic = GEMM_TRAFFIC_750K.get(primary)
-        flops_launch = 2.0 * 2.0 * MIN_RESIDUE_PLANES * st["n_det_up"] * st["n_det_dn"] * W / main_chunks
+        flops_launch = 2.0 * 2.0 * moduli * st["n_det_up"] * st["n_det_dn"] * W / main_chunks
         launch_ms = kern["contract_timed"] / main_chunks
         tpeak, tsource = bf16_peak()
         achieved = flops_launch / (launch_ms / 1e3) / 1e12
         roofline = {"kernel": "k_mod_gemm", "bound": "tensor", "achieved": achieved, "peak": tpeak,
                     "unit": "TFLOP/s", "frac": achieved / tpeak, "peak_source": tsource, "peak_nominal": 2250.0,
-                    "flops_note": "BF16 operations of %d residue planes (the least any expansion has), without the "
-                                  "magnitude sums" % MIN_RESIDUE_PLANES}
+                    "flops_note": "BF16 operations of %d residue planes of each order, without the magnitude sums" % moduli}
     else:
         flops_launch = 4.0 * st["n_det"] * W / main_chunks
         launch_ms = kern["contract_timed"] / main_chunks
@@ -519,8 +510,7 @@ def measure_batched(precision, steps, warmup, streams=8, tune_ms=60.0, fallback_
         solo += a.elapsed_time(b)
         cms = c.profile()["contract"]
         c.set_profiling(False)
-        cst = c.stats()
-        if not contraction_dense(cst["n_det"], cst["n_det_up"], cst["n_det_dn"]):
+        if not c.last_moduli:
             contract_tf.append((4.0 * wl.n_det * wl.n_walk / (cms * 1e-3) / 1e12 if cms > 0 else float("nan"),
                                 4.0 * wl.n_det * wl.n_walk, cms))
     peak, _, _ = fp64_peak(dev.index, _gpu_index(dev.index))

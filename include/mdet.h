@@ -322,6 +322,11 @@ mdet_status mdet_set_walker_chunks(mdet_ctx* ctx, int n_chunks);
  * first evaluation. Either pointer may be null. */
 mdet_status mdet_get_last_launches(const mdet_ctx* ctx, int32_t* n_chunks, int32_t* n_kernels);
 
+/* The form of the last evaluation's contraction: *n_moduli residue planes of C and
+ * as many of its transpose (residue products), or 0 (sparse sums, and before the
+ * first evaluation). MDET_E_ARG for a null pointer. */
+mdet_status mdet_get_last_contraction(const mdet_ctx* ctx, int32_t* n_moduli);
+
 /*
  * Tile shapes of the evaluation kernels (tuning knobs with no counterpart in
  * the paper): spmm_chunk nonzeros of C per warp in the sparse contraction
@@ -343,8 +348,8 @@ mdet_status mdet_get_last_launches(const mdet_ctx* ctx, int32_t* n_chunks, int32
  * column maxima, in FP64 (and in mixed precision beyond 112 AOs or 128 MOs) with
  * dot products for the elements that a dot product gives more accurately; for
  * small bases and the re-evaluation of flagged walkers FP64 dot products; where
- * the digits' sums could exceed 2^24 it falls back to 1; 1: on the CUDA cores, the compensated FP32 dot product, accurate
- * relative to each term, or the FP64 product; 0: mixed precision, the same digit
+ * the digits' sums could exceed 2^24 it falls back to 1; 1: on the CUDA cores, the
+ * compensated FP32 dot product, accurate relative to each term, or the FP64 product; 0: mixed precision, the same digit
  * products on warp-level mma.sync),
  * contract_impl the CI contraction of the mixed path (0, the default: exact or
  * FP64 as above; 1: double-float pairs on the FP32 pipe with a compensated dot

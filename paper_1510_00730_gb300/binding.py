@@ -85,6 +85,7 @@ def load_library(build_if_missing: bool = True):
     L.mdet_set_profiling.argtypes = [vp, i32]
     L.mdet_set_walker_chunks.argtypes = [vp, i32]
     L.mdet_get_last_launches.argtypes = [vp, vp, vp]
+    L.mdet_get_last_contraction.argtypes = [vp, vp]
     L.mdet_set_escalation.argtypes = [vp, i32]
     L.mdet_set_fallback.argtypes = [vp, C.c_double, i32]
     L.mdet_set_workspace.argtypes = [vp, i64, i64]
@@ -107,7 +108,7 @@ def load_library(build_if_missing: bool = True):
     for name in ("mdet_create", "mdet_set_system", "mdet_set_orbitals", "mdet_set_ci_expansion", "mdet_evaluate",
                  "mdet_evaluate_host", "mdet_get_ratios", "mdet_get_stats", "mdet_get_spin_dets",
                  "mdet_get_ci_matrix", "mdet_omega_sort", "mdet_truncate_norm", "mdet_sm_chain", "mdet_set_ci_expansion_device", "mdet_set_profiling", "mdet_get_profile",
-                 "mdet_psi_tilde_noalloc", "mdet_set_walker_chunks", "mdet_get_last_launches", "mdet_set_escalation", "mdet_selftest_df32", "mdet_selftest_inv_r", "mdet_get_tuning",
+                 "mdet_psi_tilde_noalloc", "mdet_set_walker_chunks", "mdet_get_last_launches", "mdet_get_last_contraction", "mdet_set_escalation", "mdet_selftest_df32", "mdet_selftest_inv_r", "mdet_get_tuning",
                  "mdet_set_tuning", "mdet_autotune", "mdet_batch_evaluate", "mdet_batch_create", "mdet_batch_launch", "mdet_set_fallback", "mdet_set_workspace", "mdet_get_fallback",
                  "mdet_get_error_estimates", "mdet_measure_fp64_rate", "mdet_get_timeline"):
         getattr(L, name).restype = i32
@@ -486,6 +487,14 @@ class Context:
         ch, nk = C.c_int32(0), C.c_int32(0)
         self._check(self._L.mdet_get_last_launches(self._h, C.byref(ch), C.byref(nk)), "mdet_get_last_launches")
         return int(ch.value), int(nk.value)
+
+    @property
+    def last_moduli(self):
+        """Residue planes per order of the last evaluation's contraction, 0 for the sparse sums
+        (mdet_get_last_contraction)."""
+        n = C.c_int32()
+        self._check(self._L.mdet_get_last_contraction(self._h, C.byref(n)), "mdet_get_last_contraction")
+        return n.value
 
     @property
     def last_chunks(self):

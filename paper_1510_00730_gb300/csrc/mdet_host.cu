@@ -95,6 +95,7 @@ struct mdet_ctx {
   bool have_timeline = false;
   int prof_chunks = 0;
   int last_kernels = 0;  // kernels the last evaluation launched
+  int last_moduli = 0;   // and the moduli of its contraction (0: sparse sums)
   // per chunk: the start and end of every stage (stages of one chunk may run on
   // different streams, after waits)
   static constexpr int kEvPerChunk = 2 * MDET_N_STAGES;
@@ -474,9 +475,9 @@ bool optional_alloc(T** p, size_t bytes) {
 }
 
 // The digits of B as operand tiles of the tcgen05 orbital product: per chunk of 32 MOs and slice of
-// 16 AOs, [AO / 8 mod 2][digit][MO][AO mod 8], so that the digits' MOs are rows of one operand. Mixed precision: the 7 digits `dig` of B_dig; FP64: 8
-// digits of B_am 2^(62 - fexp_m) (balanced base 256, the bytes of that integer + 0x80...80 less 128).
-// *out is null when some order's sum could exceed 2^24, where the product's FP32 accumulators would
+// 16 AOs, [AO / 8 mod 2][digit][MO][AO mod 8], so that the digits' MOs are rows of one operand. Mixed
+// precision: the 7 digits `dig` of B_dig; FP64: 8 digits of B_am 2^(62 - fexp_m) (balanced base 256, the
+// bytes of that integer + 0x80...80 less 128). *out is null when some order's sum could exceed 2^24, where the product's FP32 accumulators would
 // no longer be exact (the AO digits are at most 256, the first of 7, else 128).
 mdet_status upload_digit_tiles(mdet_ctx* c, const std::vector<double>& B, const std::vector<uint16_t>& dig,
                                const std::vector<int>& fexp, const uint16_t** out) {
@@ -1514,13 +1515,14 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
     CUDA_TRY(c, cudaStreamWaitEvent(st, c->joined, 0));
   }
   c->prof_chunks = nch;
+  c->last_moduli = dense ? c->dense.nm : 0;
   // stability fallback over the whole batch, after every chunk has finished: mixed precision
   // escalates to FP64 first, FP64 goes to full LU directly
-  // kernels: 3 per chunk (reference, ratios, epilogue; 4 with the epilogue's separate scatter), its orbitals' (2 or 3 per walker block of the
-  // digit products, else 1) and its contraction's (1 for the sparse sums, 2 in double-float, 3 per walker
-  // block of the residue products); the full-LU
-  // fallback 5 (list, dets, scale, rows, out); the mixed refinement adds its list, gather,
-  // FP64 orbitals and scatter, and either the mark or the 4 FP64 table kernels
+  // kernels: 3 per chunk (reference, ratios, epilogue; 4 with the epilogue's separate scatter), its
+  // orbitals' (2 or 3 per walker block of the digit products, else 1) and its contraction's (1 for the
+  // sparse sums, 2 in double-float, 3 per walker block of the residue products); the full-LU fallback 5
+  // (list, dets, scale, rows, out), 8 with its own residue products; the mixed refinement adds its list,
+  // gather, FP64 orbitals and scatter, and either the mark or the 4 FP64 table kernels
   c->last_kernels = 3 * nch + orbital_kernels + contract_kernels + scatter_kernels;
   if (prof_all) CUDA_TRY(c, cudaEventRecord(c->ev_refine[0], st));
   if (mixed && c->E.fb && P.fallback_tol > 0.0) {
@@ -1661,6 +1663,12 @@ mdet_status mdet_get_last_launches(const mdet_ctx* c, int32_t* n_chunks, int32_t
   if (!c) return MDET_E_ARG;
   if (n_chunks) *n_chunks = c->last_walk > 0 ? c->prof_chunks : 0;
   if (n_kernels) *n_kernels = c->last_walk > 0 ? c->last_kernels : 0;
+  return MDET_OK;
+}
+
+mdet_status mdet_get_last_contraction(const mdet_ctx* c, int32_t* n_moduli) {
+  if (!c || !n_moduli) return MDET_E_ARG;
+  *n_moduli = c->last_walk > 0 ? c->last_moduli : 0;
   return MDET_OK;
 }
 

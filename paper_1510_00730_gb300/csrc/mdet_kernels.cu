@@ -861,7 +861,7 @@ __global__ void __launch_bounds__(512) k_scatter(DevProblem P, DevScratch S, int
 }
 
 // kSumLanes lanes to one sum over the MOs in k_final, their partial sums added in a fixed order. Two:
-// at 4096 walkers of 17 electrons and 100 MOs (pairs, 256 threads) the the last round of one lane to a sum
+// at 4096 walkers of 17 electrons and 100 MOs (pairs, 256 threads) the last round of one lane to a sum
 // leaves most threads idle (10% slower), and with four or eight the additions across lanes cost as much.
 constexpr int kSumLanes = 2;
 static __device__ __forceinline__ df32 lanes_sum(df32 v) {
@@ -900,10 +900,10 @@ static __device__ __forceinline__ T lanes_sum(T v) {
 // 0.43 ms at 8192 walkers of 17 electrons and 100 MOs in pairs, 1.09 -> 0.82 in FP64 (128 threads, one
 // kernel for both); 512 threads take 0.62 and 0.98.
 template <bool MIXED, int NT, bool SCAT>
-__global__ void __launch_bounds__(NT, SCAT ? (MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 1)) : 1) : 4) k_final(DevProblem P, DevScratch S, const double* __restrict__ R,
-                                               double* __restrict__ log_abs_psi, int8_t* __restrict__ sign,
-                                               double* __restrict__ grad, double* __restrict__ lap,
-                                               double* __restrict__ e_local, uint32_t* __restrict__ status) {
+__global__ void __launch_bounds__(NT, SCAT ? (MIXED ? (NT == 128 ? 5 : (NT == 256 ? 2 : 1)) : 1) : 4)
+    k_final(DevProblem P, DevScratch S, const double* __restrict__ R, double* __restrict__ log_abs_psi,
+            int8_t* __restrict__ sign, double* __restrict__ grad, double* __restrict__ lap,
+            double* __restrict__ e_local, uint32_t* __restrict__ status) {
   extern __shared__ double sm[];
   const int nu = P.n_up, nd = P.n_dn, N = nu + nd, M = P.n_mo;
   const int NM = N * M;

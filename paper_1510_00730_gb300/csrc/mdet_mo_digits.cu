@@ -226,17 +226,19 @@ __global__ void __launch_bounds__(256) k_mo_ao(DevProblem P, const double* __res
   for (int r = warp; r < 5 * NE; r += 8) {
     if (r % NE >= ne) continue;
     unsigned k = 0;
-    int at = 0;  // the AO of the lane's largest key
-    for (int a = lane; a < K; a += 32) {
-      const unsigned key = AoType<T>::key(*reinterpret_cast<const uint2*>(smx + r * stride + a * 8));
-      if (key > k) {
-        k = key;
-        at = a;
-      }
+    int at = 0;
+    auto key = [&](int a) { return AoType<T>::key(*reinterpret_cast<const uint2*>(smx + r * stride + a * 8)); };
+    if (P.B_top) {  // and the AO of the largest, for k_mo_repair
+      for (int a = lane; a < K; a += 32)
+        if (const unsigned x = key(a); x > k) {
+          k = x;
+          at = a;
+        }
+    } else {
+      for (int a = lane; a < K; a += 32) k = max(k, key(a));
     }
     const unsigned top = __reduce_max_sync(0xffffffffu, k);
-    if (P.B_top)  // for k_mo_repair
-      at = __shfl_sync(0xffffffffu, at, __ffs(__ballot_sync(0xffffffffu, k == top)) - 1);
+    if (P.B_top) at = __shfl_sync(0xffffffffu, at, __ffs(__ballot_sync(0xffffffffu, k == top)) - 1);
     if (lane == 0) {
       const int e = AoType<T>::row_exp(top);
       rexp[r] = e;
@@ -493,9 +495,9 @@ __global__ void __launch_bounds__(kOrderThreads, 1) k_mo_orders(DevProblem P, co
 // which mostly go to DRAM: 8,192 walkers of 17 electrons and 80 MOs, FP64, 0.50 ms with every small
 // element in the list, 0.18 with these (and no less with the 0.02 % that the two largest AOs leave).
 template <class T, class Out>
-__global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 4 : 3) k_mo_repair(DevProblem P, const double* __restrict__ R, int64_t w0, int64_t n_el,
-                                                   const uint8_t* __restrict__ xd, const int* __restrict__ xer,
-                                                   Out* __restrict__ phi) {
+__global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 4 : 3)
+    k_mo_repair(DevProblem P, const double* __restrict__ R, int64_t w0, int64_t n_el, const uint8_t* __restrict__ xd,
+                const int* __restrict__ xer, Out* __restrict__ phi) {
   constexpr int kABytes = AoType<T>::D * kSliceBytes;
   constexpr bool kDouble = std::is_same<T, double>::value;
   constexpr unsigned kAll = 0xffffffffu;
@@ -631,7 +633,9 @@ __global__ void __launch_bounds__(256, std::is_same<T, double>::value ? 4 : 3) k
 
 }  // namespace
 
-size_t mo_digits_row_bytes(const DevProblem& P, bool df) { return (size_t)(df ? AoType<df32>::D : AoType<double>::D) * 2 * P.tc_kp; }
+size_t mo_digits_row_bytes(const DevProblem& P, bool df) {
+  return (size_t)(df ? AoType<df32>::D : AoType<double>::D) * 2 * P.tc_kp;
+}
 int mo_bad_exponent() { return kBadRow; }
 
 bool mo_digits_supported(const DevProblem& P, bool df) {

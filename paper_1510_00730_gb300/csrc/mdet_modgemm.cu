@@ -22,7 +22,8 @@
 //    accumulator an exact integer. The accumulators are reduced mod p_q to one byte.
 //  - Reconstruction: X = sum_q y_q M_q - k P with M_q = (P / p_q) ((P / p_q)^-1 mod p_q),
 //    P = prod p_q > 2^124.6 and k = rint(sum_q y_q ((P / p_q)^-1 mod p_q) / p_q) (|X| / P < 0.36, and
-//    16-bit fractions put the sum within 0.05), in 128-bit wrap-around integers: X is exact, and v_i = RN(X) 2^(es_i + xe_w - 123).
+//    16-bit fractions put the sum within 0.05), in 128-bit wrap-around integers: X is exact, and
+//    v_i = RN(X) 2^(es_i + xe_w - 123).
 //  - The magnitude sums m = sum_j |c_ij| |r_j| 2^-(es_i + xe_w) ride along as one more product of each
 //    order: leading BF16 magnitudes; for the error estimate those of v as BF16 pairs h + l (2^-17
 //    relative), h h + h l + l h in one FP32 accumulator.
