@@ -517,18 +517,30 @@ mdet_status upload_digit_tiles(mdet_ctx* c, const std::vector<double>& B, const 
   return upload(c, tiles, out);
 }
 
-// Whether an expansion's contraction is taken as residue products on the tensor cores: a filled-in
-// C costs about 70 tensor flops per matrix element and walker, the sparse FP64 sums 4 flops per
-// nonzero at a thousandth of that rate. 8,192 walkers: 8.2 % of 3,015 x 3,015 filled takes 20.5 ms
-// sparse and 5.1 ms dense, so the two meet near 2 % by arithmetic; at 0.35 % the sparse sums take
-// 2.0 ms, and below a few thousand products the three launches cost more than the sums.
-bool dense_pays(int64_t nnz, int64_t nu, int64_t nd) { return nnz >= 4096 && (double)nnz > 0.012 * (double)nu * (double)nd; }
+// Whether an expansion's contraction of n_walk walkers is taken as residue products on the tensor cores.
+// Their time does not depend on the products; that of the sparse sums does, and for few walkers on the
+// latency of their chains. Times of both (us, FP64; 3,015 x 3,015 and 900 x 900 distinct determinants):
+//   density           0.33 %       0.66 %       1.2 %        2.2 %        4.4 %
+//   3,015, 256 w    196 / 291    203 / 412    198 / 659    219 / 634    196 / 610
+//   1,024           525 / 594    531 / 630    522 / 657    524 / 880    559 / 1,493
+//   8,192         3,713 / 1,574  3,714 / 2,012  3,713 / 3,213  3,716 / 5,645  3,728 / 10,958
+//   density           0.52 %       0.99 %       1.5 %        2.5 %        4.9 %
+//   900, 256 w       51 / 64      52 / 71      50 / 101     51 / 132     54 / 186
+//   1,024           113 / 97     113 / 107    114 / 133    112 / 228    117 / 247
+//   8,192           705 / 303    700 / 358    700 / 410    702 / 636    702 / 1,253
+// The line meets the 8,192-walker rows at 1.5 and 2.3 % and is at 1.2 % for a few walkers, where planes of
+// C (built when an evaluation of any size would use them) cost more than there is to gain. Below a few
+// thousand products the three launches cost more than the sums.
+bool dense_pays(int64_t nnz, int64_t nu, int64_t nd, int64_t n_walk) {
+  const double many = (double)std::min<int64_t>(n_walk, 8192) / 8192;
+  return nnz >= 4096 && (double)nnz > 0.012 * (double)nu * (double)nd + 5.0 * many * (double)(nu + nd);
+}
 
 // Residue planes of C for the tensor-core contraction, where they pay and fit; the sparse sums
 // serve every other expansion (and this one, when the device has no room for the planes).
 mdet_status build_dense(mdet_ctx* c) {
   DevProblem& P = c->P;
-  if (!dense_pays(P.nnz, P.n_det_sp[0], P.n_det_sp[1])) return MDET_OK;
+  if (!dense_pays(P.nnz, P.n_det_sp[0], P.n_det_sp[1], 1)) return MDET_OK;
   DenseContract& D = c->dense;
   D = DenseContract{};
   dense_shape(P.n_det_sp[0], P.n_det_sp[1], &D);
@@ -699,8 +711,9 @@ mdet_status upload_problem(mdet_ctx* c) {
   // contraction work items for the tuned size and for the short items of escalated re-evaluations
   // (and, where the sparse sums are what runs, for small contractions)
   if ((s = build_dense(c)) != MDET_OK) return s;
-  s = c->dense_ok ? ensure_items(c, {c->spmm_chunk, kEscalationChunk})
-                  : ensure_items(c, {c->spmm_chunk, kEscalationChunk, 256, 64, 32, 16});
+  s = c->dense_ok && dense_pays(P.nnz, P.n_det_sp[0], P.n_det_sp[1], INT64_MAX)
+          ? ensure_items(c, {c->spmm_chunk, kEscalationChunk})
+          : ensure_items(c, {c->spmm_chunk, kEscalationChunk, 256, 64, 32, 16});
   if (s != MDET_OK) return s;
   use_items(c, P, c->spmm_chunk);
   // the sequential chain of Sec. 2.2: distinct determinants in the order of the key of Eq. 3,
@@ -969,14 +982,17 @@ int mo_kernels(const DevProblem& P, const DevScratch& S, int64_t n_walk, bool df
 
 // Whether an evaluation's contraction runs as residue products: its expansion has them, its
 // scratch has their workspace, and no setting asks for a form of the sparse sums.
-bool use_dense(const mdet_ctx* c) { return c->dense_ok && c->contract_impl == 0 && c->spmm_blocks == 0; }
+bool use_dense(const mdet_ctx* c, int64_t n_walk) {
+  return c->dense_ok && c->contract_impl == 0 && c->spmm_blocks == 0 &&
+         dense_pays(c->P.nnz, c->P.n_det_sp[0], c->P.n_det_sp[1], n_walk);
+}
 
 // Walker chunks of a mixed-precision evaluation when none are configured: three
 // when the FP64 contraction is long enough to hide the FP32-pipe stages of the
 // other chunks (at least 100,000 products and 4 walker tiles per chunk), else one.
 int auto_chunks(const mdet_ctx* c, int64_t n_walk) {
   const int64_t tiles = (n_walk + kWalkerPad - 1) / kWalkerPad;
-  return (c->precision == MDET_PRECISION_MIXED && c->contract_impl == 0 && !use_dense(c) && c->P.nnz >= 100000 &&
+  return (c->precision == MDET_PRECISION_MIXED && c->contract_impl == 0 && !use_dense(c, n_walk) && c->P.nnz >= 100000 &&
           tiles >= 12)
              ? 3
              : 1;
@@ -1432,7 +1448,7 @@ mdet_status mdet_evaluate(mdet_ctx* c, int64_t n_walk, const double* R, double* 
     *off = t0 * kWalkerPad;
     *n = std::min<int64_t>(t1 * kWalkerPad, n_walk) - *off;
   };
-  const bool dense = use_dense(c) && c->S.xmax;
+  const bool dense = use_dense(c, n_walk) && c->S.xmax;
   int contract_kernels = 0, orbital_kernels = 0, scatter_kernels = 0;
   // stage i (MDET_STAGE_*) of chunk k on stream ks, bracketed by its two profiling events
   auto stage = [&](int k, int i, cudaStream_t ks, int persistent) -> mdet_status {
@@ -1839,7 +1855,7 @@ mdet_status mdet_autotune(mdet_ctx* c, int64_t n_walk, const double* R, double b
     const int* vals = param == 0 ? chunks : (param == 1 ? ecs : wcs);
     const int nv = param == 1 ? 3 : 4;
     if (param == 2 && !mixed) break;
-    if (param == 0 && use_dense(c) && c->S.xmax) continue;      // residue products have no items,
+    if (param == 0 && use_dense(c, n_walk) && c->S.xmax) continue;  // residue products have no items,
     if (param == 1 && !mo_repairs(c->P, mixed)) continue;       // and these bases no other orbital kernel
     for (int q = 0; q < nv && s == MDET_OK && spent < budget_ms; q++) {
       mdet_tuning t = cur;

@@ -236,3 +236,20 @@ def _occupied(wl, k, twice=False):
     for words in (wl.det_up[k], wl.det_dn[k]):
         mos += [m for m in range(wl.n_mo) if int(words[m // 64]) >> (m % 64) & 1]
     return mos if twice else set(mos)
+
+
+def test_the_form_depends_on_the_walkers():
+    """1.6 % of 700 x 700 filled: residue products for few walkers, sparse sums for many, with the same results."""
+    wl = _workload(700, 700, 64, n_det=8000)
+    ctx = pkg.Context.from_workload(wl, device=0)
+    ctx.set_fallback(0.0)
+    few = _eval(ctx, wl.R)
+    assert ctx.last_moduli >= 16
+    many = _eval(ctx, np.tile(wl.R, (128, 1, 1)))
+    assert ctx.last_moduli == 0
+    # as in test_residue_products_match_oracle_and_sparse_sums
+    tol = 1400 * 2.0 ** -53 * np.maximum(oracle.evaluate(wl)["kappa"], 1.0) + 4 * np.spacing(np.abs(few["log_abs_psi"]))
+    assert np.all(np.abs(few["log_abs_psi"] - many["log_abs_psi"][:64]) <= tol)
+    assert np.array_equal(few["sign"], many["sign"][:64]) and np.array_equal(few["status"], many["status"][:64])
+    again = _eval(ctx, wl.R)
+    assert ctx.last_moduli >= 16 and np.array_equal(again["log_abs_psi"], few["log_abs_psi"])
