@@ -465,16 +465,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1)
 // a warp per walker and product, four consecutive determinants per lane (one 4-byte load per
 // modulus, all issued before the arithmetic). Bound by instruction issue and the loads' latency at 24
 // warps an SM, not by its 25 bytes a determinant. The weighted sums run in 16-bit limbs with dp2a, two
-// moduli at a time, and each weight is fetched once for four determinants: an evaluation's two launches
-// (8192 walkers of 750000 determinants, and those it re-evaluates) 0.82 ms, of which the first is
-// 0.70, against 1.22 with 32-bit limbs in 64-bit multiply-adds and 1.15 with two determinants per
-// lane (the constant loads then bound it). Q, the pairs of moduli, is a template argument for the
-// usual counts: unrolled to the largest 0.88. (Before the choice of wide rows, which takes 0.1 ms.) Every
-// walker's Psi~ is summed in one warp, in a fixed order. Stores go through shared memory so that a
-// warp writes 256 consecutive bytes.
-// Few walkers (a re-evaluation, or too few for the warps of three blocks an SM): four warps to a walker
-// and product, so that each walks a quarter of the determinants: 67 of 256 slots with 900 + 900
-// determinants 44 -> 14 us, 87 with 3000 + 3000 120 -> 34, 1000 walkers of 900 + 900 46 -> 40.
+// moduli at a time, and each weight is fetched once for four determinants: 0.70 ms (8,192 walkers of
+// 750,000 products), against 1.1 with 32-bit limbs in 64-bit multiply-adds and 1.0 with two determinants
+// per lane (the constant loads then bound it), and 0.80 with the magnitudes read and the wide rows. Q, the
+// pairs of moduli, is a template argument for the usual counts (unrolled to the largest: a quarter more).
+// Every walker's Psi~ is summed in a fixed order. Stores go through shared memory so that a warp writes
+// 256 consecutive bytes.
+// Few walkers (full LU's, or too few for the warps of three blocks an SM): four warps to a walker and
+// product, so that each walks a quarter of the determinants: 1,000 walkers of 900 + 900 46 -> 40 us.
 constexpr int kCrtFewWalkers = 8;
 constexpr float kWideRow = 0x1p-13f;
 
@@ -653,8 +651,8 @@ __global__ void __launch_bounds__(256, 3) k_mod_crt(const __grid_constant__ Dens
   }
   if (lane == 0) {
     S.psit[w] = psi;
-    // a re-evaluation keeps the sum of the evaluation that flagged it. The columns' power of two, at least
-    // 2, is left to the end; the FP64 sum above carries none
+    // full LU, with a live count, has no use for the magnitude sum. The columns' power of two, at least 2, is
+    // left to the end; the FP64 sum above carries none
     if (!S.live) S.psia[w] = xb >= 0x7ff || failed ? pa : ldexpf(pa, xb - 1022);
   }
 }
