@@ -477,8 +477,9 @@ bool optional_alloc(T** p, size_t bytes) {
 // The digits of B as operand tiles of the tcgen05 orbital product: per chunk of 32 MOs and slice of
 // 16 AOs, [AO / 8 mod 2][digit][MO][AO mod 8], so that the digits' MOs are rows of one operand. Mixed
 // precision: the 7 digits `dig` of B_dig; FP64: 8 digits of B_am 2^(62 - fexp_m) (balanced base 256, the
-// bytes of that integer + 0x80...80 less 128). *out is null when some order's sum could exceed 2^24, where the product's FP32 accumulators would
-// no longer be exact (the AO digits are at most 256, the first of 7, else 128).
+// bytes of that integer + 0x80...80 less 128). *out is null when some order's sum could exceed 2^24, where
+// the product's FP32 accumulators would no longer be exact (the AO digits are at most 256, the first of
+// 7, else 128).
 mdet_status upload_digit_tiles(mdet_ctx* c, const std::vector<double>& B, const std::vector<uint16_t>& dig,
                                const std::vector<int>& fexp, const uint16_t** out) {
   const int D = c->precision == MDET_PRECISION_MIXED ? 7 : 8;
@@ -963,8 +964,9 @@ mdet_status refine(mdet_ctx* c, bool table, int64_t n_walk, const double* R, dou
   // few walkers: short work items keep the contraction's chains short, and the epilogue
   // spreads each walker's determinants over 512 threads. Sparse sums also where the evaluation took
   // residue products: these walkers are the ill-conditioned ones, which amplify any change of rounding
-  // (up to 7e-9 of grad Psi / Psi against 1e-11 to 1e-9 between two runs), and for the 60 to 140 of an
-  // evaluation the sparse sums take about as long.
+  // (up to 7e-9 of grad Psi / Psi against 1e-11 to 1e-9 between two runs). For the 60 to 140 of an
+  // evaluation the sparse sums take 0.08 ms (100,000 products) and 0.37 (750,000), the products 0.05 and
+  // 0.19.
   Pe.spmm_blocks = 0;
   CUDA_TRY(c, launch_contract_f64(Pe, E, cap, st));
   CUDA_TRY(c, launch_final(P, E, cap, c->e_R, o.log_abs_psi, o.sign, o.grad, o.lap, o.e_local, o.status, false, st,
@@ -1856,7 +1858,7 @@ mdet_status mdet_autotune(mdet_ctx* c, int64_t n_walk, const double* R, double b
     const int nv = param == 1 ? 3 : 4;
     if (param == 2 && !mixed) break;
     if (param == 0 && use_dense(c, n_walk) && c->S.xmax) continue;  // residue products have no items,
-    if (param == 1 && !mo_repairs(c->P, mixed)) continue;       // and these bases no other orbital kernel
+    if (param == 1 && !mo_repairs(c->P, mixed)) continue;           // and these bases no other orbital kernel
     for (int q = 0; q < nv && s == MDET_OK && spent < budget_ms; q++) {
       mdet_tuning t = cur;
       int* field = param == 0 ? &t.spmm_chunk : (param == 1 ? &t.mo_ec : &t.walker_chunks);
