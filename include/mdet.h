@@ -338,7 +338,8 @@ mdet_status mdet_get_last_contraction(const mdet_ctx* ctx, int32_t* n_moduli);
  * walker_chunks as in mdet_set_walker_chunks, spmm_blocks the form of the
  * contraction (0: where C is dense enough for the number of walkers, from 1.2 % of
  * at least 4,096 products, exact residue products on the tcgen05 tensor cores with one rounding
- * at the end, FP64 sums for rows that their fixed point would cut, if the device
+ * at the end, FP64 sums for rows that their fixed point would cut (most rows, and
+ * slower than the sparse sums, if MOs are scaled very differently), if the device
  * has room for C's planes; elsewhere sparse FP64 sums,
  * one warp per work item with one chunk, 4 blocks per SM with several; any other
  * value: the sparse sums on a persistent grid of at most that many 128-thread

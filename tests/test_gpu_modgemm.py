@@ -253,3 +253,26 @@ def test_the_form_depends_on_the_walkers():
     assert np.array_equal(few["sign"], many["sign"][:64]) and np.array_equal(few["status"], many["status"][:64])
     again = _eval(ctx, wl.R)
     assert ctx.last_moduli >= 16 and np.array_equal(again["log_abs_psi"], few["log_abs_psi"])
+
+
+@pytest.mark.parametrize("n_walk", [1217, 1300, 1303])
+def test_wide_rows_of_many_walkers(n_walk):
+    """As test_mos_of_very_different_scale, with more walkers than eight an SM, which the reconstruction takes
+    four to a block (the last block ragged): every fourth of them, and its neighbours, as in a small batch."""
+    wl = _workload(130, 70, 64)
+    ref = _occupied(wl, int(np.argmax(np.abs(wl.ci_coef))))
+    odd = np.array([m % 2 == 1 and m not in ref for m in range(wl.n_mo)])
+    power = np.array([12 * sum(odd[m] for m in _occupied(wl, k, True)) for k in range(wl.n_det)])
+    scaled = dataclasses.replace(wl, mo_coef=wl.mo_coef * np.where(odd, 2.0 ** 12, 1.0), ci_coef=np.ldexp(wl.ci_coef, -power))
+    ctx = pkg.Context.from_workload(scaled, device=0)
+    ctx.set_fallback(0.0)
+    few = _eval(ctx, wl.R)
+    many = _eval(ctx, np.tile(wl.R, (21, 1, 1))[:n_walk])
+    assert ctx.last_moduli >= 16
+    want = oracle.evaluate(wl)
+    tol = 200 * 2.0 ** -53 * np.maximum(want["kappa"], 1.0) + 4 * np.spacing(np.abs(want["log_abs_psi"]))
+    at = np.arange(n_walk) % 64
+    assert np.all(np.abs(many["log_abs_psi"] - few["log_abs_psi"][at]) <= tol[at])
+    assert np.array_equal(many["sign"], few["sign"][at])
+    rep = compare(few, want, **TOL[pkg.PRECISION_FP64])
+    assert rep["sign_ok"], rep
